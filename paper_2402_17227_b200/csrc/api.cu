@@ -34,6 +34,7 @@ size_t layout(Handle* h, uint8_t* base) {
   const size_t N = d.N, R = (size_t)d.N * d.T, DW = (size_t)d.d_out * d.d_in;
   uint8_t* cur = base;
   Workspace& w = h->ws;
+  w = Workspace();
   const size_t chunks = R / 32 + 2;
   w.a = carve<float>(cur, R);
   w.wc = carve<float>(cur, R);
@@ -60,12 +61,13 @@ size_t layout(Handle* h, uint8_t* base) {
     w.partial_tiles = carve<float>(cur, 3 * (size_t)h->max_units * 128 * 256);
     w.tickets = carve<int32_t>(cur, 6 * (size_t)h->max_units);
     w.sched = carve<int32_t>(cur, 8);
-  } else {
-    w.packG = nullptr;
-    w.packX = nullptr;
-    w.partial_tiles = nullptr;
-    w.tickets = nullptr;
-    w.sched = nullptr;
+  } else if (h->split_path) {
+    const bool fp32 = d.dtype == VCAS_DTYPE_F32;
+    w.packG = carve<__nv_bfloat16>(cur, 3 * (size_t)h->R_pad * d.d_out);
+    w.packX = carve<__nv_bfloat16>(cur, (fp32 ? 3 : 1) * (size_t)h->R_pad * d.d_in);
+    w.packY = carve<__nv_bfloat16>(cur, 3 * (size_t)h->R_pad * d.d_out);     // shared with the second set's packG
+    if (fp32) w.packW = carve<__nv_bfloat16>(cur, 3 * (size_t)((d.d_out + 63) / 64 * 64) * d.d_in);
+    w.partial_tiles = carve<float>(cur, 3 * (size_t)h->max_units * 128 * 256);
   }
   w.Gs = carve<float>(cur, DW);
   w.Gact = carve<float>(cur, DW);
@@ -93,10 +95,14 @@ size_t layout(Handle* h, uint8_t* base) {
   if (h->tensor_path) {
     v.packG = carve<__nv_bfloat16>(cur, (size_t)h->R_pad * d.d_out);
     v.packX = carve<__nv_bfloat16>(cur, (size_t)h->R_pad * d.d_in);
-    v.partial_tiles = w.partial_tiles + (size_t)h->max_units * 128 * 256;   // dW slot of this set = third slot
     v.tickets = w.tickets + 2 * (size_t)h->max_units;
     v.sched = w.sched + 2;
+  } else if (h->split_path) {
+    v.packG = w.packY;       // a probe reads packY only before a batch's draws fork, a sampled call has no second set
+    v.packX = carve<__nv_bfloat16>(cur, (d.dtype == VCAS_DTYPE_F32 ? 3 : 1) * (size_t)h->R_pad * d.d_in);
   }
+  if (w.partial_tiles != nullptr)
+    v.partial_tiles = w.partial_tiles + (size_t)h->max_units * 128 * 256;   // dW slot of this set = third slot
   v.Gact = carve<float>(cur, DW);
   h->sub_rows = carve<int32_t>(cur, SUB_MAX);
   h->sub_dY = carve<float>(cur, R * SUB_MAX * (d.dtype == VCAS_DTYPE_BF16 ? 2 : 4) / 4);
@@ -126,10 +132,12 @@ int sample_w_and_dw(Handle* h, const void* X, const void* dY, const SamplerArgs&
                     const Plan* plan, float* out, cudaStream_t st) {
   VCAS_CUDA(launch_scores_x(h, X, a, first_programmatic, st));
   VCAS_CUDA(launch_sample_w(h, a, st));
-  VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path, st));
-  if (h->tensor_path) {
-    const float keep = a.sample_w ? a.rho * a.nu : a.rho;
-    const int hint = (int)(keep * (float)(h->desc.N * h->desc.T)) + 1;
+  VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path || h->split_path, st));
+  const float keep = a.sample_w ? a.rho * a.nu : a.rho;
+  const int hint = (int)(keep * (float)(h->desc.N * h->desc.T)) + 1;
+  if (h->split_path) {
+    VCAS_CUDA(launch_split_dw(h, dY, X, false, hint, out, true, st));
+  } else if (h->tensor_path) {
     VCAS_CUDA(launch_umma_dw(h, h->ws.packG, h->ws.packX, h->R_pad, h->ws.counts + 1, hint, plan, out, st));
   } else {
     VCAS_CUDA(launch_fma_dw(h, dY, X, h->ws.idxW, h->ws.scaleW, h->ws.counts + 1, out, st));
@@ -155,9 +163,29 @@ inline void mark_dense(Handle* h, int k, cudaStream_t st) {
   if (h->prof_enabled && h->prof_dense_calls < PROF_RING) cudaEventRecord(h->ev_dense[h->prof_dense_calls * 4 + k], st);
 }
 
+// dX of a sampled call by the products that leave its row square-norms to a pass of their own
+int plain_dx(Handle* h, const void* dY, const void* W, float rho, const void* Hpre, void* dX, float* a_out, bool programmatic,
+             cudaStream_t st) {
+  if (h->split_path) {
+    const bool fp32 = h->desc.dtype == VCAS_DTYPE_F32;
+    VCAS_CUDA(launch_split_prep(h, dY, false, fp32 ? W : nullptr, h->ws.packW, h->desc.d_out, h->desc.d_in, dX, programmatic, st));
+    VCAS_CUDA(launch_split_dx(h, dY, W, false, rho, Hpre, dX, st));
+  } else {
+    VCAS_CUDA(launch_fma_dx(h, dY, W, h->ws.scaleA, Hpre, dX, st));
+  }
+  if (a_out != nullptr) VCAS_CUDA(launch_rownorm_out(h, dX, a_out, st));   // the zero rows are always written
+  return VCAS_OK;
+}
+
 // plan: the tiling made for a call whose dX product runs beside it (nullptr: planned alone)
-int dense_dw(Handle* h, const void* X, const void* dY, const Plan* plan, float* out, cudaStream_t st) {
-  if (h->tensor_path) {
+// y_ready: split path of an fp32 layer, the parts of dY are in place
+int dense_dw(Handle* h, const void* X, const void* dY, const Plan* plan, bool y_ready, float* out, cudaStream_t st) {
+  if (h->split_path) {
+    const int R = h->desc.N * h->desc.T;
+    const bool fp32 = h->desc.dtype == VCAS_DTYPE_F32;
+    if (fp32) VCAS_CUDA(launch_split_prep(h, y_ready ? nullptr : dY, true, X, h->ws.packX, R, h->desc.d_in, nullptr, false, st));
+    VCAS_CUDA(launch_split_dw(h, dY, X, true, R, out, fp32, st));
+  } else if (h->tensor_path) {
     VCAS_CUDA(launch_umma_dw(h, dY, X, h->desc.N * h->desc.T, h->ws.counts + 2, h->desc.N * h->desc.T, plan, out, st));
   } else {
     VCAS_CUDA(launch_fma_dw(h, dY, X, nullptr, nullptr, h->ws.counts + 2, out, st));
@@ -199,6 +227,7 @@ int vcas_create(vcas_handle* out, const vcas_layer_desc* desc, const vcas_config
   h->desc = *desc;
   if (cfg != nullptr) h->cfg = *cfg; else vcas_default_config(&h->cfg);
   h->tensor_path = tensor_ok && desc->gemm_path != VCAS_GEMM_FMA;
+  h->split_path = !h->tensor_path && desc->gemm_path == VCAS_GEMM_AUTO;
   h->R_pad = (desc->N * desc->T + 63) / 64 * 64;
   h->launches = 0;
   h->prof_enabled = false;
@@ -219,8 +248,8 @@ int vcas_create(vcas_handle* out, const vcas_layer_desc* desc, const vcas_config
     return VCAS_ERR_CUDA;
   }
   h->num_sms = prop.multiProcessorCount;
-  h->max_units = 2 * h->num_sms;
-  if (h->tensor_path && prop.major != 10) { delete h; return VCAS_ERR_CUDA; }
+  h->max_units = h->split_path ? split_max_units(*desc, h->num_sms) : 2 * h->num_sms;
+  if ((h->tensor_path || h->split_path) && prop.major != 10) { delete h; return VCAS_ERR_CUDA; }
   h->bytes = layout(h, nullptr);
   if (cudaMalloc(&h->base, h->bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -288,7 +317,7 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
   const int spare = 1;
   Plan px = {256, 1, 1}, pw = {256, 1, 1};
   if (h->tensor_path) plan_products(h, false, a.rho, hint, spare, a_out != nullptr, &px, &pw);
-  if (!h->tensor_path || h->prof_enabled) {
+  if (!(h->tensor_path || h->split_path) || h->prof_enabled) {
     // one stream, so that (with stage profiling) each pair of events brackets the kernels of one stage
     mark(h, 0, st);
     VCAS_CUDA(launch_rownorm_dy(h, dY, a, st));
@@ -299,15 +328,16 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
     mark(h, 2, st);
     if (h->tensor_path) {
       VCAS_CUDA(launch_umma_dx(h, dY, W, false, a.rho, Hpre, dX, a_out, skip_dropped, spare, &px, st));
-    } else {
-      VCAS_CUDA(launch_fma_dx(h, dY, W, h->ws.scaleA, Hpre, dX, st));     // always writes the zero rows
-      if (a_out != nullptr) VCAS_CUDA(launch_rownorm_out(h, dX, a_out, st));
+    } else if (plain_dx(h, dY, W, a.rho, Hpre, dX, a_out, false, st) != VCAS_OK) {
+      return VCAS_ERR_CUDA;
     }
     mark(h, 3, st);
     mark(h, 6, st);
-    VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path, st));
+    VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path || h->split_path, st));
     mark(h, 4, st);
-    if (h->tensor_path) {
+    if (h->split_path) {
+      VCAS_CUDA(launch_split_dw(h, dY, X, false, hint, dW, false, st));
+    } else if (h->tensor_path) {
       VCAS_CUDA(launch_umma_dw(h, h->ws.packG, h->ws.packX, h->R_pad, h->ws.counts + 1, hint, &pw, dW, st));
     } else {
       VCAS_CUDA(launch_fma_dw(h, dY, X, h->ws.idxW, h->ws.scaleW, h->ws.counts + 1, dW, st));
@@ -322,7 +352,8 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
     VCAS_CUDA(launch_sample_a(h, a, a.a_in == nullptr, st));
     VCAS_CUDA(cudaEventRecord(h->ev_fork, st));
     VCAS_CUDA(cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
-    VCAS_CUDA(launch_umma_dx(h, dY, W, false, a.rho, Hpre, dX, a_out, skip_dropped, spare, &px, st));
+    if (h->tensor_path) VCAS_CUDA(launch_umma_dx(h, dY, W, false, a.rho, Hpre, dX, a_out, skip_dropped, spare, &px, st));
+    else if (plain_dx(h, dY, W, a.rho, Hpre, dX, a_out, true, st) != VCAS_OK) return VCAS_ERR_CUDA;
     const int rc = sample_w_and_dw(h, X, dY, a, false, &pw, dW, h->side_stream);
     if (rc != VCAS_OK) return rc;
     VCAS_CUDA(cudaEventRecord(h->ev_join, h->side_stream));
@@ -421,7 +452,10 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
   cudaStream_t st = S(stream);
   if (join_pending(h, st) != VCAS_OK) return VCAS_ERR_CUDA;
   cudaStream_t sw = st;
-  const bool fork = h->tensor_path && !h->prof_enabled;
+  const bool fork = (h->tensor_path || h->split_path) && !h->prof_enabled;
+  const bool cut = h->split_path && h->desc.dtype == VCAS_DTYPE_F32;
+  mark_dense(h, 0, st);
+  if (cut) VCAS_CUDA(launch_split_prep(h, dY, true, W, h->ws.packW, h->desc.d_out, h->desc.d_in, nullptr, false, st));
   if (fork) {
     VCAS_CUDA(cudaEventRecord(h->ev_fork, st));
     VCAS_CUDA(cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
@@ -429,15 +463,16 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
   }
   Plan px = {256, 1, 1}, pw = {256, 1, 1};
   if (h->tensor_path) plan_products(h, true, 1.0f, h->desc.N * h->desc.T, 0, false, &px, &pw);
-  mark_dense(h, 0, st);
-  if (h->tensor_path) {
+  if (h->split_path) {
+    VCAS_CUDA(launch_split_dx(h, dY, W, true, 1.0f, Hpre, dX, st));
+  } else if (h->tensor_path) {
     VCAS_CUDA(launch_umma_dx(h, dY, W, true, 1.0f, Hpre, dX, nullptr, false, 0, &px, st));
   } else {
     VCAS_CUDA(launch_fma_dx(h, dY, W, nullptr, Hpre, dX, st));
   }
   mark_dense(h, 1, st);
   mark_dense(h, 3, sw);
-  const int rc = dense_dw(h, X, dY, h->tensor_path ? &pw : nullptr, dW, sw);
+  const int rc = dense_dw(h, X, dY, h->tensor_path ? &pw : nullptr, cut, dW, sw);
   mark_dense(h, 2, sw);
   if (fork) {
     VCAS_CUDA(cudaEventRecord(h->ev_join, sw));
@@ -509,7 +544,7 @@ int vcas_variance_probe(vcas_handle hh, int32_t M, const void* const* X_i, const
       VCAS_CUDA(launch_gather_cols(h, dY_i[i], h->desc.d_out, h->sub_rows, h->sub_k, h->sub_dY, st));
       dYp = h->sub_dY;
     }
-    int rc = dense_dw(hp, X_i[i], dYp, nullptr, h->ws.Gs, st);   // G_s,i
+    int rc = dense_dw(hp, X_i[i], dYp, nullptr, false, h->ws.Gs, st);   // G_s,i
     if (rc != VCAS_OK) return rc;
     VCAS_CUDA(launch_probe_welford(hp, i, st));
     SamplerArgs a = sampler_args(rho, nu, 0);

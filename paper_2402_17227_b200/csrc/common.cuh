@@ -35,8 +35,12 @@ struct Workspace {
   double* acc;     // [16] probe accumulators (0: V_act, 1: V_w, 2: p_lo, 3: p_hi, 4: V_s)
   double* partial; // [PARTIAL_SLOTS] block partial sums of the probe reductions
   // compact operands of the weight-gradient product (tensor path)
-  __nv_bfloat16* packG;  // [R_pad, d_out]
-  __nv_bfloat16* packX;  // [R_pad, d_in]
+  __nv_bfloat16* packG;  // [R_pad, d_out]; split path: [3][R_pad, d_out]
+  __nv_bfloat16* packX;  // [R_pad, d_in]; split path of an fp32 layer: [3][R_pad, d_in]
+  // split path: dY for the dX product (rows of kept data, compact; a dense product of an fp32 layer: all rows) and W,
+  // three parts each for an fp32 layer (a bf16 layer needs a compact copy of dY only)
+  __nv_bfloat16* packY;
+  __nv_bfloat16* packW;
   float* partial_tiles;  // [3][max_units][128 * 256] fp32 partial tiles of a split contraction: dX, dW, and the dW
                          // of the workspace's second set (see Handle::ws2)
   int32_t* tickets;      // [3][2 * max_units]: slices stored, slices finished, per tile
@@ -61,7 +65,8 @@ struct Handle {
   vcas_config cfg;
   int device;
   int num_sms;
-  bool tensor_path;
+  bool tensor_path;   // bf16 operands straight to the tensor cores (gemm_umma.cu)
+  bool split_path;    // operands cut into bf16 parts (gemm_split.cu); neither: fp32 FMA (gemm_fma.cu)
   int R_pad;
   int max_units;   // capacity of the split-contraction workspace, in (tile, slice) units
   void* base;
@@ -346,6 +351,19 @@ cudaError_t launch_fma_dx(Handle* h, const void* dY, const void* W, const float*
                           const void* H, void* dX, cudaStream_t st);
 cudaError_t launch_fma_dw(Handle* h, const void* dY, const void* X, const int32_t* idx,
                           const float* scale, const int32_t* cnt, float* dW, cudaStream_t st);
+
+// products of fp32 layers and of odd widths on the tensor cores, operands cut into bf16 parts
+int split_max_units(const vcas_layer_desc& d, int num_sms);      // (tile, slice) units their workspace holds
+// What they read: the rows of dY of kept data, compact (dense: all rows) into packY, a whole matrix M into Mp, and zeros in
+// the rows of dX_zero of dropped data; each may be nullptr.  programmatic: launched as a dependent of the kernel before it.
+cudaError_t launch_split_prep(Handle* h, const void* dY, bool dense, const void* M, __nv_bfloat16* Mp, int m_rows, int m_d,
+                              void* dX_zero, bool programmatic, cudaStream_t st);
+// dX from packY and packW (bf16: from packY, or dY itself when dense, and W)
+cudaError_t launch_split_dx(Handle* h, const void* dY, const void* W, bool dense, float rho_hint, const void* H, void* dX,
+                            cudaStream_t st);
+// dW from packG and packX (dense: from packY and packX, bf16 from dY and X); cnt_hint: expected number of rows
+cudaError_t launch_split_dw(Handle* h, const void* dY, const void* X, bool dense, int cnt_hint, float* dW, bool programmatic,
+                            cudaStream_t st);
 
 // tensor-core products
 // spare_sms: SMs the persistent grid leaves free (for a kernel of another stream that must run beside it);

@@ -9,7 +9,7 @@
 // Only the scalar fixed point and a scan over R/32 counts run on a single SM.
 #include <atomic>
 
-#include "common.cuh"
+#include "split.cuh"
 
 namespace vcas {
 namespace {
@@ -435,8 +435,9 @@ struct EmitParams {
   const int32_t* idxA; const int32_t* dropA;
   const int32_t* counts; const int32_t* chunk_off; const float* fix;
   float* w; float* q; float* scaleW; int32_t* idxW;
-  const __nv_bfloat16* dY; const __nv_bfloat16* X;       // operands to pack
+  const void* dY; const void* X;                         // operands to pack
   __nv_bfloat16* packG; __nv_bfloat16* packX;            // compact operands (nullptr: no packing)
+  size_t g_stride, x_stride;                             // elements between the parts of a cut operand
   int N, T, d_in, d_out;
   int sample_w;
   int parts;                                             // CTAs that share the packing of one chunk's rows
@@ -458,7 +459,10 @@ __device__ __forceinline__ uint4 scale8(const uint4& v, float sc) {
 // global row (by part 0); the operands of the chunk's kept rows j with j % parts == part are packed for the dW
 // product.  The rows of dropped data get w = q = 0, and the compact operands are padded with zero rows to a
 // multiple of 64 (the product's last k-block then adds nothing).
+// CUT: the operands for the products of gemm_split.cu: the rescaled rows of dY are kept to fp32 precision in three bf16
+// parts, and the rows of an fp32 X likewise (a bf16 X is its own single part).
 constexpr int EMIT_THREADS = 256;
+template <typename E, bool CUT>
 __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   __shared__ int s_r[32], s_pos[32], s_cnt;
   __shared__ float s_sc[32];
@@ -514,24 +518,37 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
         const int j = part + jj * parts;
         const size_t r = (size_t)s_r[j], pos = (size_t)s_pos[j];
         const float sc = s_sc[j];
-        const uint4* srcG = reinterpret_cast<const uint4*>(P.dY + r * P.d_out);
-        const uint4* srcX = reinterpret_cast<const uint4*>(P.X + r * P.d_in) - vo;
-        uint4* dstG = reinterpret_cast<uint4*>(P.packG + pos * P.d_out);
-        uint4* dstX = reinterpret_cast<uint4*>(P.packX + pos * P.d_in) - vo;
+        const E* srcG = reinterpret_cast<const E*>(P.dY) + r * P.d_out;
+        const E* srcX = reinterpret_cast<const E*>(P.X) + r * P.d_in - (size_t)P.d_out;
+        __nv_bfloat16* dstG = P.packG + pos * P.d_out;
+        __nv_bfloat16* dstX = P.packX + pos * P.d_in - (size_t)P.d_out;
         const int p0 = (seg << 7) + lane;
-        uint4 v[4];
+        Vec8<E> v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int piece = p0 + 32 * q;
-          if (piece < vt) v[q] = __ldg(piece < vo ? srcG + piece : srcX + piece);
+          if (piece < vt) v[q].load((piece < vo ? srcG : srcX) + piece * 8);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int piece = p0 + 32 * q;
-          if (piece < vt) {
-            if (piece < vo) dstG[piece] = scale8(v[q], sc);
-            else dstX[piece] = v[q];
+          if (piece >= vt) break;
+          const bool g = piece < vo;
+          __nv_bfloat16* dst = (g ? dstG : dstX) + piece * 8;
+          if constexpr (CUT) {
+            if (sizeof(E) == 4 || g) {
+              float f[8];
+              v[q].get(f);
+              if (g) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) f[e] *= sc;
+              }
+              store_parts3(f, dst, g ? P.g_stride : P.x_stride);
+              continue;
+            }
           }
+          if constexpr (sizeof(E) == 2)
+            *reinterpret_cast<uint4*>(dst) = g ? scale8(v[q].v, sc) : v[q].v;
         }
       }
       __syncthreads();
@@ -548,11 +565,16 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   // zero rows up to the next multiple of 64
   if (pack) {
     const int padded = (cntW + 63) / 64 * 64;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
     for (int k = cntW + (int)blockIdx.x; k < padded; k += gridDim.x) {
-      for (int i = tid; i < P.d_out / 8; i += EMIT_THREADS)
-        reinterpret_cast<uint4*>(P.packG + (size_t)k * P.d_out)[i] = make_uint4(0u, 0u, 0u, 0u);
-      for (int i = tid; i < P.d_in / 8; i += EMIT_THREADS)
-        reinterpret_cast<uint4*>(P.packX + (size_t)k * P.d_in)[i] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int part = 0; part < (CUT ? 3 : 1); ++part)
+        for (int i = tid; i < P.d_out / 8; i += EMIT_THREADS)
+          reinterpret_cast<uint4*>(P.packG + part * P.g_stride + (size_t)k * P.d_out)[i] = z;
+#pragma unroll
+      for (int part = 0; part < (CUT && sizeof(E) == 4 ? 3 : 1); ++part)
+        for (int i = tid; i < P.d_in / 8; i += EMIT_THREADS)
+          reinterpret_cast<uint4*>(P.packX + part * P.x_stride + (size_t)k * P.d_in)[i] = z;
     }
   }
 }
@@ -636,7 +658,8 @@ cudaError_t launch_emit_pack(Handle* h, const void* dY, const void* X, const Sam
   P.wc = ws.wc; P.uc = ws.uc; P.q_in = a.q_in; P.scaleA = ws.scaleA; P.idxA = ws.idxA; P.dropA = ws.dropA;
   P.counts = ws.counts; P.chunk_off = ws.chunk_off; P.fix = ws.fix;
   P.w = ws.w; P.q = ws.q; P.scaleW = ws.scaleW; P.idxW = ws.idxW;
-  P.dY = (const __nv_bfloat16*)dY; P.X = (const __nv_bfloat16*)X;
+  P.dY = dY; P.X = X;
+  P.g_stride = (size_t)h->R_pad * d.d_out; P.x_stride = (size_t)h->R_pad * d.d_in;
   P.packG = pack ? ws.packG : nullptr;
   P.packX = pack ? ws.packX : nullptr;
   P.N = d.N; P.T = d.T; P.d_in = d.d_in; P.d_out = d.d_out;
@@ -652,7 +675,10 @@ cudaError_t launch_emit_pack(Handle* h, const void* dY, const void* X, const Sam
   P.parts = (int)parts;
   long blocks = ((R + 31) / 32) * parts;
   if (blocks > cap) blocks = cap;
-  const cudaError_t e = launch_after(emit_pack_kernel, dim3((unsigned)blocks), dim3(EMIT_THREADS), 0, st, P);
+  const dim3 grid((unsigned)blocks), threads(EMIT_THREADS);
+  const cudaError_t e = !(pack && h->split_path) ? launch_after(emit_pack_kernel<__nv_bfloat16, false>, grid, threads, 0, st, P)
+      : d.dtype == VCAS_DTYPE_F32                ? launch_after(emit_pack_kernel<float, true>, grid, threads, 0, st, P)
+                                                 : launch_after(emit_pack_kernel<__nv_bfloat16, true>, grid, threads, 0, st, P);
   h->launches += 1;
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -1,0 +1,75 @@
+"""Products with operands cut into bf16 parts: fp32 layers, and bf16 layers whose widths are not multiples of 64.
+
+Tolerances: fp32 results within 1e-6 of the float64 oracle (the parts are exact, products below 2^-26 are left out,
+sums of a stage of 32 or 64 terms are truncated to 24 bits and added up in fp32: measured below 4e-7); a bf16 layer's dW,
+whose rescaled rows are not rounded to bf16, meets the same, its dX carries one bf16 rounding (2^-9 / sqrt(3) of its norm)."""
+import pytest
+import torch
+
+from oracle import vcas_oracle as o
+from paper_2402_17227_b200 import binding as vb
+from paper_2402_17227_b200 import build as vbuild
+from paper_2402_17227_b200 import inputs
+from tests.util import np64, rel_fro
+
+pytestmark = pytest.mark.gpu
+F32, BF16 = torch.float32, torch.bfloat16
+
+
+# one row, one k-block, tiles that span data (T below and above 128, not dividing it), ragged widths, contractions cut
+# into slices (few tiles, many k-blocks), more tiles than SMs
+@pytest.mark.parametrize("shape", [(1, 1, 8, 8), (4, 64, 256, 256), (3, 50, 72, 200), (5, 197, 128, 1000), (2, 130, 64, 4096),
+                                   (16, 256, 72, 64), (33, 150, 776, 1000), (9, 333, 1032, 520), (40, 128, 1288, 72)])
+@pytest.mark.parametrize("dtype", [F32, BF16])
+def test_split_products_match_oracle(dtype, shape):
+    vbuild.build()
+    N, T, d_in, d_out = shape
+    if dtype == BF16 and d_in % 64 == 0 and d_out % 64 == 0:
+        d_out += 8                                     # multiples of 64 take the other tensor-core kernels
+    X, dY, W = inputs.make_layer(inputs.LayerCase("t", N, T, d_in, d_out, dtype, 1.5, 1.0, 0.5, 0.5))
+    H = (2.0 * torch.randn(N * T, d_in, generator=torch.Generator().manual_seed(3))).to(dtype)
+    layer = vb.Layer(N, T, d_in, d_out, dtype)
+    Xc, dYc, Wc, Hc = [t.cuda() for t in (X, dY, W, H)]
+    gp = o.gelu_prime(np64(H))
+    tol_x, tol_w = (1e-6 if dtype == F32 else 2.5e-3), 1e-6
+    for seed, rho, nu in [(3, 0.5, 0.5), (11, 0.3, 0.4), (5, 1.0, 1.0)]:
+        ref = o.linear_bwd(np64(X), np64(dY), np64(W), N, T, rho, nu, seed)
+        p_in, q_in = torch.from_numpy(ref["p32"]).cuda(), torch.from_numpy(ref["q32"]).cuda()
+        dX, dW = layer.linear_bwd(Xc, dYc, Wc, rho, nu, seed, p_in=p_in, q_in=q_in, H=Hc)
+        assert rel_fro(np64(dX), ref["dX"] * gp) <= tol_x and rel_fro(np64(dW), ref["dW"]) <= tol_w
+        assert not np64(dX)[~ref["keepA"].repeat(T)].any()
+        again = layer.linear_bwd(Xc, dYc, Wc, rho, nu, seed, p_in=p_in, q_in=q_in, H=Hc)
+        assert torch.equal(dX, again[0]) and torch.equal(dW, again[1])
+    dXd, dWd = o.dense_bwd(np64(X), np64(dY), np64(W))
+    dX, dW = layer.dense_bwd(Xc, dYc, Wc)
+    assert rel_fro(np64(dX), dXd) <= tol_x and rel_fro(np64(dW), dWd) <= tol_w
+    assert layer.device_status() == 0
+    # a wait that runs out is reported and the handle recovers
+    layer.set_wait_limit(2_000_000, stall_once=True)
+    layer.dense_bwd(Xc, dYc, Wc)
+    assert layer.device_status() == -6
+    layer.set_wait_limit(2_000_000_000, stall_once=False)
+    again = layer.dense_bwd(Xc, dYc, Wc)
+    assert torch.equal(dX, again[0]) and torch.equal(dW, again[1]) and layer.device_status() == 0
+    layer.close()
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan"), 3.4e38])
+def test_split_products_of_values_without_a_finite_bf16_part(value):
+    """An infinite, NaN or nearly overflowing weight gives what fp32 arithmetic gives: only its own column is not finite."""
+    vbuild.build()
+    N, T, d_in, d_out = 2, 40, 72, 64
+    X, dY, W = inputs.make_layer(inputs.LayerCase("t", N, T, d_in, d_out, F32, 1.0, 0.5, 0.5, 0.5))
+    dY, W = dY.abs() + 0.5, W.clone()
+    W[5, 7] = value
+    layer = vb.Layer(N, T, d_in, d_out, F32)
+    dX, dW = layer.dense_bwd(X.cuda(), dY.cuda(), W.cuda())
+    col = dX[:, 7].cpu()
+    if value != value:
+        assert torch.isnan(col).all()
+    else:
+        assert (torch.isinf(col) | (col > 1e37)).all()
+    keep = [c for c in range(d_in) if c != 7]
+    ref = np64(dY) @ np64(W)[:, keep]
+    assert rel_fro(np64(dX[:, keep]), ref) <= 1e-6
+    layer.close()
