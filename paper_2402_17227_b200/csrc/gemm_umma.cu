@@ -406,7 +406,10 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
   } else if (warp == 5) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // The whole warp runs the loop and one lane issues: with warp-uniform control flow the descriptors stay in uniform
+    // registers (a branch into one lane cost 2 % of the 256-row products).
+    const bool leader = elect_one();
+    {
       constexpr uint32_t idesc = make_idesc(BN, MODE == MODE_DW, true);
       constexpr uint32_t a_step = MODE == MODE_DW ? (UMMA_K * 128 >> 4) : (UMMA_K * 2 >> 4);
       int stage = 0; uint32_t phase = 0; int lt = 0;
@@ -414,9 +417,10 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       int qi = 0; uint32_t qph = 0;
       auto next_unit = [&](int prev) -> int {
         if constexpr (DYN) {
-          if (!mbar_wait(&s.q_full[qi], qph, abort_flag, P.status)) { ok = false; return -1; }
+          if (!__all_sync(0xffffffffu, mbar_wait(&s.q_full[qi], qph, abort_flag, P.status))) { ok = false; return -1; }
           const int t = *(volatile int*)&s.tile_q[qi];
-          mbar_arrive(&s.q_empty[qi]);
+          __syncwarp();
+          if (leader) mbar_arrive(&s.q_empty[qi]);
           if (++qi == QD) { qi = 0; qph ^= 1u; }
           return t;
         } else if constexpr (LEAN) {
@@ -433,12 +437,12 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const int slice = u % D.S;
         const int nkb = min(D.kblocks, (slice + 1) * D.kb_per) - slice * D.kb_per;
         const int buf = lt_now % NACC; const uint32_t use = (uint32_t)(lt_now / NACC) & 1u;
-        ok = mbar_wait(&s.tmem_empty[buf], use ^ 1u, abort_flag, P.status);
+        ok = __all_sync(0xffffffffu, mbar_wait(&s.tmem_empty[buf], use ^ 1u, abort_flag, P.status));
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);   // half hh of a 256-row tile: + hh * BN
         for (int kb = 0; kb < nkb; ++kb) {
-          ok = mbar_wait(&s.full[stage], phase, abort_flag, P.status);
+          ok = __all_sync(0xffffffffu, mbar_wait(&s.full[stage], phase, abort_flag, P.status));
           if (!ok) break;
           tc_fence_after();
           const uint32_t sa = smem_u32(s.stages + stage * C::STAGE_BYTES);
@@ -448,14 +452,15 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const uint64_t da = MODE == MODE_DW ? desc_mnmajor(sa + hh * A_BYTES) : desc_kmajor(sa + hh * A_BYTES);
 #pragma unroll
             for (int k4 = 0; k4 < BK / UMMA_K; ++k4)
-              umma_bf16(d_tmem + (uint32_t)(hh * BN), da + (uint64_t)(k4 * a_step),
-                        db + (uint64_t)(k4 * (UMMA_K * 128 >> 4)), idesc, (kb | k4) != 0 ? 1u : 0u);
+              if (leader)
+                umma_bf16(d_tmem + (uint32_t)(hh * BN), da + (uint64_t)(k4 * a_step),
+                          db + (uint64_t)(k4 * (UMMA_K * 128 >> 4)), idesc, (kb | k4) != 0 ? 1u : 0u);
           }
-          umma_commit(&s.empty[stage]);
+          if (leader) umma_commit(&s.empty[stage]);
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit(&s.tmem_full[buf]);
+        if (leader) umma_commit(&s.tmem_full[buf]);
       }
     }
   } else {
