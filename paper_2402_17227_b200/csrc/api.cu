@@ -419,7 +419,7 @@ int vcas_layernorm_bwd(vcas_handle hh, const void* X, const void* gamma, const v
   if (join_pending(h, st) != VCAS_OK) return VCAS_ERR_CUDA;
   VCAS_CUDA(launch_rownorm_dy(h, dY, a, st));
   VCAS_CUDA(launch_sample_a(h, a, a.a_in == nullptr, st));
-  VCAS_CUDA(launch_layernorm_bwd(h, X, gamma, dY, eps, dX, a_out, skip, dgamma, dbeta, rho, st));
+  VCAS_CUDA(launch_layernorm_bwd(h, X, gamma, dY, eps, dX, a_out, skip, dgamma, dbeta, st));
   return VCAS_OK;
 }
 

@@ -1,7 +1,7 @@
 // SampleA in front of a layer that is not a matrix product (Sec. 4: SampleA sits at every layer; App. E: the
 // sampled, rescaled gradient is multiplied by the layer's exact Jacobian): the backward of
 // Y = LayerNorm(X) * gamma + beta.  Only the rows of kept data are read and computed; rows of dropped data
-// get dX = 0.  HBM-bound row-wise and column-wise passes, fixed summation orders.
+// get dX = 0.  HBM-bound: every kept row of X and dY is read once and held in registers; fixed summation orders.
 #include "common.cuh"
 
 namespace vcas {
@@ -46,14 +46,177 @@ template <> struct Ld<float> {
 struct LnParams {
   const void* X; const void* gamma; const void* dY; void* dX;
   const float* scaleA; const int32_t* idxA; const int32_t* dropA; const int32_t* counts;
-  float* mu; float* rstd;          // [R] per-row statistics kept for the column pass
+  float* mu; float* rstd;          // [R] per-row statistics kept for the column pass of wide rows
   float* a_out; int a_parts;       // optional row square-norms of the stored dX (first part; the others 0)
-  float* partial;                  // [2][chunks][d] column partial sums
+  float* partial;                  // [2][CTAs or row ranges][d] column partial sums
   float* dgamma; float* dbeta;
-  int N, T, d, chunks, skip_dropped;
+  int N, T, d, skip_dropped;
   float eps;
 };
 
+constexpr int LN_WARPS = 8;
+constexpr int LN_VPL = 4;          // 16-byte vectors of a row that a lane holds
+
+// Sum of one float over the G warps of a row group, in a fixed order; result in every lane.  slot: G floats per group.
+template <int G>
+__device__ __forceinline__ void group_sum(float (&v)[3], int n, float* slot, int gw, int group) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    if (i < n) v[i] = warp_sum(v[i]);
+  if (G > 1) {
+    if ((threadIdx.x & 31) == 0)
+      for (int i = 0; i < n; ++i) slot[gw * 3 + i] = v[i];
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(32 * G) : "memory");
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < n) {
+        float t = 0.f;
+        for (int w = 0; w < G; ++w) t += slot[w * 3 + i];
+        v[i] = t;
+      }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(32 * G) : "memory");
+  }
+}
+
+// G warps per row (a lane holds up to four vectors of it, so G = ceil(d / 1024) for bf16), the kept rows dealt out to the
+// row groups of the grid in turn.  The row's statistics, dX and its share of the column sums dgamma = sum_r G_hat_r x_hat_r,
+// dbeta = sum_r G_hat_r come from one read of X and dY; a lane keeps the column sums of its columns in registers over
+// all its rows, the CTA adds its groups in order and stores one partial sum per column.  (With a second, column-wise
+// pass over the rows the call on 16384 x 1024 at ratio 0.5 took 87 us, 17 for the rows and 40 for the columns, one
+// dependent load at a time; now 35, 19 of them here.)
+template <typename T, int G>
+__global__ void __launch_bounds__(LN_WARPS * 32, 2) ln_kernel(LnParams P) {
+  using L = Ld<T>;
+  using V = typename L::V;
+  constexpr int VN = L::N;
+  constexpr int GROUPS = LN_WARPS / G;
+  __shared__ float s_slot[GROUPS][G * 3];
+  extern __shared__ float s_col[];                   // [GROUPS][2][32 * VN] column sums on their way to the CTA's sum
+  pdl_wait();      // the kept data come from the SampleA kernel
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / G, gw = warp % G;
+  const int cntA = P.counts[0], Tn = P.T, d = P.d;
+  const int kept_rows = cntA * Tn;
+  const int nv = d / VN;
+  const float inv_d = 1.0f / (float)d;
+  const int v0 = gw * 32 + lane;                     // this lane's vectors: v0, v0 + 32 G, ...
+  float ag[LN_VPL][VN], ab[LN_VPL][VN];
+#pragma unroll
+  for (int q = 0; q < LN_VPL; ++q)
+#pragma unroll
+    for (int e = 0; e < VN; ++e) { ag[q][e] = 0.f; ab[q][e] = 0.f; }
+  const int groups = gridDim.x * GROUPS, me = blockIdx.x * GROUPS + group;
+  for (int c = me; c < kept_rows; c += groups) {
+    const int k = c / Tn;
+    const int n = P.idxA[k];
+    const size_t r = (size_t)n * Tn + (c - k * Tn);
+    const float sc = P.scaleA[n];
+    const V* xv = reinterpret_cast<const V*>((const T*)P.X + r * d);
+    const V* gv = reinterpret_cast<const V*>((const T*)P.dY + r * d);
+    const V* wv = reinterpret_cast<const V*>((const T*)P.gamma);
+    V x[LN_VPL], g[LN_VPL];
+#pragma unroll
+    for (int q = 0; q < LN_VPL; ++q)
+      if (v0 + q * 32 * G < nv) x[q] = __ldg(xv + v0 + q * 32 * G);
+#pragma unroll
+    for (int q = 0; q < LN_VPL; ++q)
+      if (v0 + q * 32 * G < nv) g[q] = __ldg(gv + v0 + q * 32 * G);
+    float sums[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < LN_VPL; ++q)
+      if (v0 + q * 32 * G < nv) {
+        float f[VN];
+        L::unpack(x[q], f);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) sums[0] += f[e];
+      }
+    group_sum<G>(sums, 1, s_slot[group], gw, group);
+    const float mean = sums[0] * inv_d;
+    // variance, and the two row sums of g_hat = G_hat * gamma that the Jacobian needs
+    sums[0] = sums[1] = sums[2] = 0.f;
+#pragma unroll
+    for (int q = 0; q < LN_VPL; ++q)
+      if (v0 + q * 32 * G < nv) {
+        float f[VN], y[VN], w[VN];
+        L::unpack(x[q], f);
+        L::unpack(g[q], y);
+        L::unpack(__ldg(wv + v0 + q * 32 * G), w);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) {
+          const float xc = f[e] - mean, gh = sc * y[e] * w[e];
+          sums[0] = fmaf(xc, xc, sums[0]);
+          sums[1] += gh;
+          sums[2] = fmaf(gh, xc, sums[2]);
+        }
+      }
+    group_sum<G>(sums, 3, s_slot[group], gw, group);
+    const float rstd = rsqrtf(sums[0] * inv_d + P.eps);
+    const float m1 = sums[1] * inv_d, m2 = sums[2] * rstd * inv_d;     // mean(g_hat), mean(g_hat * x_hat)
+    float sq[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < LN_VPL; ++q)
+      if (v0 + q * 32 * G < nv) {
+        float f[VN], y[VN], w[VN], o[VN];
+        L::unpack(x[q], f);
+        L::unpack(g[q], y);
+        L::unpack(__ldg(wv + v0 + q * 32 * G), w);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) {
+          const float xh = (f[e] - mean) * rstd, gs = sc * y[e], gh = gs * w[e];
+          o[e] = (gh - m1 - xh * m2) * rstd;
+          ag[q][e] = fmaf(gs, xh, ag[q][e]);
+          ab[q][e] += gs;
+        }
+        V ov;
+        sq[0] += L::pack(o, ov);
+        reinterpret_cast<V*>((T*)P.dX + r * d)[v0 + q * 32 * G] = ov;
+      }
+    if (P.a_out != nullptr) {                        // the same for the whole grid
+      group_sum<G>(sq, 1, s_slot[group], gw, group);
+      if (gw == 0)
+        for (int j = lane; j < P.a_parts; j += 32) P.a_out[r * P.a_parts + j] = j == 0 ? sq[0] : 0.f;
+    }
+  }
+  // rows of dropped data
+  if (!P.skip_dropped) {
+    const int drop_rows = (P.N - cntA) * Tn;
+    for (int i = me; i < drop_rows; i += groups) {
+      const int k = i / Tn;
+      const size_t r = (size_t)P.dropA[k] * Tn + (i - k * Tn);
+      V z;
+      float zero[VN];
+#pragma unroll
+      for (int e = 0; e < VN; ++e) zero[e] = 0.f;
+      L::pack(zero, z);
+      for (int j = v0; j < nv; j += 32 * G) reinterpret_cast<V*>((T*)P.dX + r * d)[j] = z;
+      if (P.a_out != nullptr && gw == 0)
+        for (int j = lane; j < P.a_parts; j += 32) P.a_out[r * P.a_parts + j] = 0.f;
+    }
+  }
+  // the CTA's column sums, groups in order
+  constexpr int W = 32 * G * VN;                     // columns of one q
+#pragma unroll
+  for (int q = 0; q < LN_VPL; ++q) {
+    if (q * 32 * G >= nv) break;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < VN; ++e) {
+      s_col[(group * 2 + 0) * W + (gw * 32 + lane) * VN + e] = ag[q][e];
+      s_col[(group * 2 + 1) * W + (gw * 32 + lane) * VN + e] = ab[q][e];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * W; i += LN_WARPS * 32) {
+      const int which = i / W, col = q * W + (i - which * W);
+      if (col >= d) continue;
+      float t = 0.f;
+#pragma unroll
+      for (int gr = 0; gr < GROUPS; ++gr) t += s_col[(gr * 2 + which) * W + (i - which * W)];
+      P.partial[((size_t)which * gridDim.x + blockIdx.x) * d + col] = t;
+    }
+  }
+}
+
+// Rows wider than eight warps hold in registers: two passes, one over rows and one over columns.
 // One warp per row.  Work item c < cntA*T: token of a kept datum (compact order); the items after those are the
 // rows of dropped data, which are zeroed (unless the caller's consumer never reads them).
 template <typename T>
@@ -79,7 +242,8 @@ __global__ void __launch_bounds__(256) ln_row_kernel(LnParams P) {
       for (int e = 0; e < VN; ++e) zero[e] = 0.f;
       L::pack(zero, z);
       for (int j = lane; j < nv; j += 32) reinterpret_cast<V*>((T*)P.dX + r * d)[j] = z;
-      if (P.a_out != nullptr && lane < P.a_parts) P.a_out[r * P.a_parts + lane] = 0.f;
+      if (P.a_out != nullptr)
+        for (int j = lane; j < P.a_parts; j += 32) P.a_out[r * P.a_parts + j] = 0.f;
       continue;
     }
     const int k = c / Tn;
@@ -136,14 +300,13 @@ __global__ void __launch_bounds__(256) ln_row_kernel(LnParams P) {
     if (lane == 0) {
       P.mu[r] = mean;
       P.rstd[r] = rstd;
-      if (P.a_out != nullptr) P.a_out[r * P.a_parts] = sq;
-    } else if (P.a_out != nullptr && lane < P.a_parts) {
-      P.a_out[r * P.a_parts + lane] = 0.f;
     }
+    if (P.a_out != nullptr)
+      for (int j = lane; j < P.a_parts; j += 32) P.a_out[r * P.a_parts + j] = j == 0 ? sq : 0.f;
   }
 }
 
-// One thread per column, the kept rows cut into `chunks` contiguous ranges (blockIdx.y): partial sums of
+// One thread per column, the kept rows cut into contiguous ranges (blockIdx.y): partial sums of
 // dgamma = sum_r G_hat_r * x_hat_r and dbeta = sum_r G_hat_r in row order.
 template <typename T>
 __global__ void __launch_bounds__(256) ln_col_kernel(LnParams P) {
@@ -152,7 +315,7 @@ __global__ void __launch_bounds__(256) ln_col_kernel(LnParams P) {
   const int col = blockIdx.x * blockDim.x + threadIdx.x;
   const int Tn = P.T, d = P.d;
   const int rows = P.counts[0] * Tn;
-  const int per = (rows + P.chunks - 1) / P.chunks;
+  const int per = (rows + (int)gridDim.y - 1) / (int)gridDim.y;
   const int c0 = blockIdx.y * per, c1 = min(rows, c0 + per);
   if (col >= d) return;
   float ag = 0.f, ab = 0.f;
@@ -166,27 +329,74 @@ __global__ void __launch_bounds__(256) ln_col_kernel(LnParams P) {
     ab += g;
   }
   P.partial[(size_t)blockIdx.y * d + col] = ag;
-  P.partial[(size_t)(P.chunks + blockIdx.y) * d + col] = ab;
+  P.partial[(size_t)((int)gridDim.y + blockIdx.y) * d + col] = ab;
 }
 
-__global__ void __launch_bounds__(256) ln_col_reduce_kernel(LnParams P) {
+// Adds the partial sums of CTAs or row ranges: 32 columns per CTA, 32 warps over 32 ranges of them, the ranges in order.
+// Latency-bound (a few hundred partial sums of a column, a row apart): a warp has eight loads in flight.
+constexpr int ADD_WARPS = 32;
+__global__ void __launch_bounds__(ADD_WARPS * 32) ln_add_kernel(LnParams P, int blocks) {
+  __shared__ float s[ADD_WARPS][32];
   pdl_wait();
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= P.d) return;
-  float ag = 0.f, ab = 0.f;
-  for (int ch = 0; ch < P.chunks; ++ch) {      // chunks in order
-    ag += P.partial[(size_t)ch * P.d + col];
-    ab += P.partial[(size_t)(P.chunks + ch) * P.d + col];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tiles = (P.d + 31) / 32;
+  const int which = blockIdx.x / tiles, col = (blockIdx.x - which * tiles) * 32 + lane;
+  const int per = (blocks + ADD_WARPS - 1) / ADD_WARPS, b0 = warp * per, b1 = min(blocks, b0 + per);
+  float t = 0.f;
+  if (col < P.d) {
+    const float* src = P.partial + (size_t)which * blocks * P.d + col;
+    for (int b = b0; b < b1; b += 8) {
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = b + q < b1 ? __ldcg(src + (size_t)(b + q) * P.d) : 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) t += v[q];
+    }
   }
-  P.dgamma[col] = ag;
-  P.dbeta[col] = ab;
+  s[warp][lane] = t;
+  __syncthreads();
+  if (warp == 0 && col < P.d) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < ADD_WARPS; ++w) v += s[w][lane];
+    (which == 0 ? P.dgamma : P.dbeta)[col] = v;
+  }
+}
+
+template <typename T, int G>
+cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
+  // Two CTAs per SM, fewer when there are fewer rows than row groups or the scratch (4 d^2 floats) is small
+  long blocks = (rows + LN_WARPS / G - 1) / (LN_WARPS / G);
+  if (blocks > 2 * h->num_sms) blocks = 2 * h->num_sms;
+  if (blocks > 2l * P.d) blocks = 2l * P.d;
+  const size_t smem = (size_t)LN_WARPS * 2 * 32 * Ld<T>::N * sizeof(float);
+  cudaError_t e = launch_after(ln_kernel<T, G>, dim3((unsigned)blocks), dim3(LN_WARPS * 32), smem, st, P);
+  if (e == cudaSuccess)
+    e = launch_after(ln_add_kernel, dim3(2 * ((P.d + 31) / 32)), dim3(ADD_WARPS * 32), 0, st, P, (int)blocks);
+  h->launches += 2;
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+template <typename T>
+cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
+  const int per_warp = 32 * LN_VPL * Ld<T>::N;       // columns one warp can hold
+  if (P.d <= per_warp) return run_ln<T, 1>(h, P, rows, st);
+  if (P.d <= 2 * per_warp) return run_ln<T, 2>(h, P, rows, st);
+  if (P.d <= 4 * per_warp) return run_ln<T, 4>(h, P, rows, st);
+  if (P.d <= 8 * per_warp) return run_ln<T, 8>(h, P, rows, st);
+  const int col_blocks = (P.d + 255) / 256;
+  const int chunks = 4 * h->num_sms > col_blocks ? 4 * h->num_sms / col_blocks : 1;
+  const long blocks = (rows + 7) / 8 < (1l << 20) ? (rows + 7) / 8 : (1l << 20);
+  cudaError_t e = launch_after(ln_row_kernel<T>, dim3((unsigned)blocks), dim3(256), 0, st, P);
+  if (e == cudaSuccess) e = launch_after(ln_col_kernel<T>, dim3(col_blocks, chunks), dim3(256), 0, st, P);
+  if (e == cudaSuccess) e = launch_after(ln_add_kernel, dim3(2 * ((P.d + 31) / 32)), dim3(ADD_WARPS * 32), 0, st, P, chunks);
+  h->launches += 3;
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_layernorm_bwd(Handle* h, const void* X, const void* gamma, const void* dY, float eps, void* dX,
-                                 float* a_out, bool skip_dropped, float* dgamma, float* dbeta, float rho_hint,
-                                 cudaStream_t st) {
+                                 float* a_out, bool skip_dropped, float* dgamma, float* dbeta, cudaStream_t st) {
   const vcas_layer_desc& d = h->desc;
   const Workspace& ws = h->ws;
   LnParams P;
@@ -194,31 +404,12 @@ cudaError_t launch_layernorm_bwd(Handle* h, const void* X, const void* gamma, co
   P.scaleA = ws.scaleA; P.idxA = ws.idxA; P.dropA = ws.dropA; P.counts = ws.counts;
   P.mu = ws.w; P.rstd = ws.q;
   P.a_out = a_out; P.a_parts = a_out_parts(d.d_in);
-  P.partial = ws.Gs;
+  P.partial = ws.Gs;                                 // Gs, Gact, mean and m2 are neighbours: 4 d^2 floats
   P.dgamma = dgamma; P.dbeta = dbeta;
   P.N = d.N; P.T = d.T; P.d = d.d_in; P.skip_dropped = skip_dropped ? 1 : 0;
   P.eps = eps;
-  const int col_blocks = (d.d_in + 255) / 256;
-  int chunks = (h->num_sms * 4) / col_blocks;
-  if (chunks > d.d_in / 2) chunks = d.d_in / 2;       // the scratch holds d * d floats
-  const long exp_rows = (long)((double)rho_hint * d.N * d.T) + 1;
-  if (chunks > exp_rows / 16 + 1) chunks = (int)(exp_rows / 16 + 1);
-  if (chunks < 1) chunks = 1;
-  P.chunks = chunks;
-  const long R = (long)d.N * d.T;
-  long rb = (R + 7) / 8;
-  if (rb > (1l << 20)) rb = 1l << 20;
-  cudaError_t e;
-  if (d.dtype == VCAS_DTYPE_BF16) {
-    e = launch_after(ln_row_kernel<__nv_bfloat16>, dim3((unsigned)rb), dim3(256), 0, st, P);
-    if (e == cudaSuccess) e = launch_after(ln_col_kernel<__nv_bfloat16>, dim3(col_blocks, chunks), dim3(256), 0, st, P);
-  } else {
-    e = launch_after(ln_row_kernel<float>, dim3((unsigned)rb), dim3(256), 0, st, P);
-    if (e == cudaSuccess) e = launch_after(ln_col_kernel<float>, dim3(col_blocks, chunks), dim3(256), 0, st, P);
-  }
-  if (e == cudaSuccess) e = launch_after(ln_col_reduce_kernel, dim3(col_blocks), dim3(256), 0, st, P);
-  h->launches += 3;
-  return e != cudaSuccess ? e : cudaGetLastError();
+  const long rows = (long)d.N * d.T;
+  return d.dtype == VCAS_DTYPE_BF16 ? run_ln<__nv_bfloat16>(h, P, rows, st) : run_ln<float>(h, P, rows, st);
 }
 
 }  // namespace vcas
