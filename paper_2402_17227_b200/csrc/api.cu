@@ -532,6 +532,11 @@ int vcas_variance_probe(vcas_handle hh, int32_t M, const void* const* X_i, const
   // on sub_k rows of the parameter gradient only: the products run through a copy of the handle whose d_out is
   // sub_k, on those columns of dY; scoring and sampling still see the whole of dY.
   const bool sub = h->sub_k > 0;
+  const double scale = sub ? (double)h->desc.d_out / (double)h->sub_k : 1.0;
+  if (probe_fused_ok(h, M)) {
+    VCAS_CUDA(launch_probe_fused(h, M, X_i, dY_i, rho, nu, s_lo, s_hi, seed, scale, V_s, V_act, V_w, p_lo, p_hi, st));
+    return VCAS_OK;
+  }
   Handle hs = *h;
   if (sub) hs.desc.d_out = h->sub_k;
   hs.plan_valid = false;
@@ -577,7 +582,6 @@ int vcas_variance_probe(vcas_handle hh, int32_t M, const void* const* X_i, const
     VCAS_CUDA(cudaEventRecord(h->ev_join, h->side_stream));
     VCAS_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
   }
-  const double scale = sub ? (double)h->desc.d_out / (double)h->sub_k : 1.0;
   VCAS_CUDA(launch_probe_finalize(hp, M, scale, V_s, V_act, V_w, p_lo, p_hi, st));
   if (sub) h->launches += hs.launches - launches0;
   return VCAS_OK;

@@ -23,7 +23,7 @@ namespace {
 
 constexpr int MODE_DX = 0, MODE_DW = 1;
 constexpr int SPLIT_THREADS = 10 * 32;
-constexpr int ACC_THREADS = 256;
+constexpr int ACC_WARPS = 8;
 constexpr int BN = 256;                      // tile columns
 constexpr int MAX_SPLIT = 16;
 
@@ -114,7 +114,7 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < C::STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], ACC_THREADS); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], ACC_WARPS); }
     *abort_flag = 0;
     *reinterpret_cast<volatile unsigned long long*>(abort_flag + 5) = P.wait_limit_ns;     // read by mbar_wait
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -218,8 +218,8 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       for (int e = 0; e < CW; ++e) acc[e] = 0.f;
       for (int j = 0; j < n; ++j, ++it) {
         const uint32_t buf = it & 1u;
-        // the lanes of a warp leave together
-        ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[buf], (it >> 1) & 1u, abort_flag, P.status));
+        // The lanes of a warp leave together.  No call here: it would put the sums held in registers into local memory.
+        ok = __all_sync(0xffffffffu, mbar_wait_spin(&acc_full[buf], (it >> 1) & 1u, abort_flag, P.status));
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
@@ -229,8 +229,10 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 #pragma unroll
           for (int e = 0; e < 32; ++e) acc[h * 32 + e] += __uint_as_float(v[e]);
         }
+        // one arrival per warp: the arrivals of all threads at one barrier are served one after the other
         tc_fence_before();
-        mbar_arrive(&acc_empty[buf]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[buf]);
       }
       const int row = eq * 32 + lane, r0 = tile / W.ntiles * BM + row;
       const int col0 = tile % W.ntiles * BN + eg * CW;

@@ -120,24 +120,6 @@ __device__ __forceinline__ float gelu_prime(float x) {
   for (int k = 10; k >= 0; --k) p = fmaf(p, t, GP_C[k]);
   return fmaf(copysignf(ax, x), p, 0.5f);
 }
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 // r[e] *= GELU'(h_e) for the eight bf16 pre-activations in hv: the same polynomial as gelu_prime, the four pairs
 // side by side and every step of Horner's rule issued for all of them before the next (independent chains).
 __device__ __forceinline__ void gelu_prime8(const uint4& hv, float (&r)[8]) {

@@ -10,12 +10,11 @@
 #include <atomic>
 
 #include "split.cuh"
+#include "water.cuh"
 
 namespace vcas {
 namespace {
 
-constexpr int SAMPLER_THREADS = 1024;
-constexpr int WATER_ROUNDS = 128;     // rounds of the water-filling before it is reported as not converged
 
 struct Scratch {
   double d[32];
@@ -237,22 +236,6 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) sample_a_big_kernel(SampleAPa
 }
 
 // ------------------------------------------------------------------------------ SampleW
-// How q follows from a row's score once sample_w_kernel has run: fix[1] = mode, fix[0] = c.
-constexpr int Q_ZERO = 0;     // nothing to keep (no score is positive, or the budget is 0)
-constexpr int Q_ONES = 1;     // the budget covers every positive score: q = [w > 0]
-constexpr int Q_CAPPED = 2;   // q = min(1, c w)
-constexpr int Q_GIVEN = 3;    // q is read from the caller's q_in
-
-__device__ __forceinline__ float q_of(int mode, float c, float w, const float* q_in, int r) {
-  if (mode == Q_CAPPED) {
-    if (!(w > 0.f)) return 0.f;
-    const float cx = c * w;
-    return cx >= 1.0f ? 1.f : cx;
-  }
-  if (mode == Q_ONES) return w > 0.f ? 1.f : 0.f;
-  if (mode == Q_GIVEN) return q_in[r];
-  return 0.f;
-}
 __device__ __forceinline__ bool row_kept(int sample_w, float q, uint32_t u) {
   return sample_w ? (q > 0.f && u < (uint32_t)floorf(q * 16777216.0f)) : true;
 }
@@ -268,28 +251,6 @@ struct SampleWParams {
   int sample_w, accumulate_vw;
   int smem_rows;                            // scores that fit the kernel's shared memory
 };
-
-struct WShared {
-  float part_f[2][32];
-  int part_i[2][32];
-  int scan[33];
-};
-
-// Block-wide sum of one float and one int in a fixed order (lanes by shuffle tree, then the 32
-// warp totals by the same tree, which every warp runs for itself so that one barrier suffices; the
-// buffers alternate with `parity`, and a buffer is rewritten only after a later barrier).  fp32 on
-// purpose: this is a single-CTA kernel, and double-precision arithmetic concentrated on one SM was
-// measured to dominate its run time; a tree sum of non-negative fp32 terms is accurate to about
-// 1e-6, inside the 2e-5 the probabilities are specified to.
-__device__ __forceinline__ void fast_sum(float& s, int& c, WShared* sh, int parity) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  s = warp_sum(s);
-  c = __reduce_add_sync(0xffffffffu, c);
-  if (lane == 0) { sh->part_f[parity][warp] = s; sh->part_i[parity][warp] = c; }
-  __syncthreads();
-  s = warp_sum(sh->part_f[parity][lane]);
-  c = __reduce_add_sync(0xffffffffu, sh->part_i[parity][lane]);
-}
 
 // SampleW's single-CTA part (Sec. 4.2, Eq. 3).  The n = T * (#kept data) scores sit in shared memory (in
 // global memory beyond smem_rows: same code, slower loads).  1. c with sum_r min(1, c w_r) = nu * n by
@@ -318,43 +279,8 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) sample_w_kernel(SampleWParams
   int mode = Q_GIVEN;
   float c = 0.f;
   if (P.q_in == nullptr) {
-    const float budget = P.nu * (float)T * (float)cntA;
-    float S = 0.f;
-    int nz = 0;
-    for (int i = tid; i < n; i += SAMPLER_THREADS) {
-      const float x = w[i];
-      if (x > 0.f) { S += x; ++nz; }
-    }
-    int parity = 0;
-    fast_sum(S, nz, &sh, parity); parity ^= 1;
-    if (nz == 0 || budget <= 0.f) {
-      mode = Q_ZERO;
-    } else if ((float)nz <= budget) {
-      mode = Q_ONES;
-    } else {
-      mode = Q_CAPPED;
-      c = budget / S;
-      int k = 0;
-      bool converged = false;
-      for (int iter = 0; iter < WATER_ROUNDS; ++iter) {
-        float Su = 0.f;
-        int ks = 0;
-        for (int i = tid; i < n; i += SAMPLER_THREADS) {
-          const float x = w[i];
-          if (x > 0.f) {
-            if (c * x >= 1.0f) ++ks; else Su += x;
-          }
-        }
-        fast_sum(Su, ks, &sh, parity); parity ^= 1;
-        if (ks == k) { converged = true; break; }
-        k = ks;
-        if (Su > 0.f) {
-          const float cn = (budget - (float)k) / Su;
-          c = cn > c ? cn : c;
-        }
-      }
-      if (!converged && tid == 0) atomicExch(P.status, (int32_t)VCAS_ERR_INTERNAL);
-    }
+    if (!water_fill(w, n, P.nu * (float)T * (float)cntA, &sh, mode, c) && tid == 0)
+      atomicExch(P.status, (int32_t)VCAS_ERR_INTERNAL);
   }
   __syncthreads();      // the reduction buffers are free again
 
@@ -592,8 +518,6 @@ mask_kernel(const float* __restrict__ p, int n, uint64_t seed, int sampler, uint
       [&](int i, int pos) { if (idx != nullptr) idx[pos] = i; }, &sc);
   if (threadIdx.x == 0 && cnt != nullptr) *cnt = c;
 }
-
-constexpr int SAMPLE_W_SMEM_ROWS = 56 * 1024;     // 224 KB of scores
 
 }  // namespace
 
