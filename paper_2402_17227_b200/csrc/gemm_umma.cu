@@ -792,13 +792,14 @@ __global__ void __launch_bounds__(REDUCE_THREADS) slice_reduce_kernel(GemmParams
 // ------------------------------------------------------------------------------ host side
 // Tile shape and number of contraction slices from a small cost model of the kernel instances (per
 // unit of work, so independent of the layer's shape), fitted to serialised stage times of every tiling
-// on five layer shapes on B200: a k-block costs about 0.50 / 0.45 / 0.43 us for 256 / 128 / 64 wide
-// 128-row tiles (the shared-memory fill rate of one SM bounds it, so narrow tiles only pay off when
-// they fill more SMs); a unit costs about 4 us of set-up, pipeline fill and output store; a sliced unit
-// stores its partial tile instead, and the reduction launch that follows adds the slices on all SMs:
-// together about 11 us + 1 us per slice; a 256 x 256 tile (mh = 2) costs about 0.66 us per k-block for
-// twice the work, and 7 us per tile.
-constexpr double SLICED_US = 11.0, SLICED_PER_SLICE_US = 1.0;
+// on eight layer shapes on B200: a k-block costs about 0.385 / 0.32 / 0.28 us for 256 / 128 / 64 wide
+// 128-row tiles (four products of 0.08 us each at the clock under load; the rest is the hand-over of a stage, so narrow
+// tiles only pay off when they fill more SMs); a unit costs about 2 us of set-up, pipeline fill and output store; a sliced
+// unit stores its partial tile instead, and the reduction launch that follows adds the slices on all SMs: together
+// about 4 us and 0.05 us per 256-wide unit for the traffic of the partial tiles; a 256 x 256 tile (mh = 2) costs about
+// 0.62 us per k-block for twice the work, and 4.5 us per tile, whose epilogue nothing overlaps.
+constexpr double KB_US[3] = {0.385, 0.32, 0.28}, UNIT_US = 2.0, KB2_US = 0.62, UNIT2_US = 4.5;
+inline double sliced_us(long units, int bn) { return 4.0 + 0.05 * (double)units * bn / 256.0; }
 struct Cand {
   Plan plan;
   long units;      // (tile, slice) units
@@ -813,7 +814,6 @@ constexpr int MAX_DEVICES = 64;
 int enumerate_plans(long row_tiles128, long row_tiles256, int n_extent, int kblocks, int num_sms, int max_units,
                     int force_bn, int force_split, bool remainder_ok, Cand* out) {
   const int widths[3] = {256, 128, 64};
-  const double c_kb[3] = {0.50, 0.45, 0.43};
   int n = 0;
   if (kblocks < 1) kblocks = 1;
   for (int i = 0; i < 3; ++i) {
@@ -828,12 +828,12 @@ int enumerate_plans(long row_tiles128, long row_tiles256, int n_extent, int kblo
       if (sp > 1 && force_split == 0 && kblocks / sp < 4) continue;   // slices too short to pay off
       const long units = tiles * sp;
       const double waves = (double)((units + num_sms - 1) / num_sms);
-      const double unit = (double)((kblocks + sp - 1) / sp) * c_kb[i] + (sp > 1 ? SLICED_US + SLICED_PER_SLICE_US * sp : 4.0);
+      const double unit = (double)((kblocks + sp - 1) / sp) * KB_US[i] + (sp > 1 ? sliced_us(units, widths[i]) : UNIT_US);
       if (n < MAX_CANDS) out[n++] = {{widths[i], sp, 1}, units, unit, waves * unit};
     }
     if (widths[i] == 256 && force_split <= 1) {                        // 256 x 256 tiles, never sliced
       const long units = row_tiles256 * ntiles;
-      const double wave = (double)kblocks * 0.66 + 7.0;
+      const double wave = (double)kblocks * KB2_US + UNIT2_US;
       if (n < MAX_CANDS) out[n++] = {{256, 1, 2}, units, wave, (double)((units + num_sms - 1) / num_sms) * wave};
       const long frac = units % num_sms;
       if (remainder_ok && frac > 0 && 2 * frac <= num_sms) {            // whole waves, then the rest as sliced 128-row tiles
@@ -843,7 +843,7 @@ int enumerate_plans(long row_tiles128, long row_tiles256, int n_extent, int kblo
         if (sp < 1) sp = 1;
         // the second launch always runs the sliced instance (its tiles go through the slice exchange even when
         // a contraction ends up in one slice), and costs a launch of its own
-        const double tail = (double)((kblocks + sp - 1) / sp) * 0.50 + SLICED_US + SLICED_PER_SLICE_US * (double)sp + 4.0;
+        const double tail = (double)((kblocks + sp - 1) / sp) * KB_US[0] + sliced_us(2 * frac * sp, 256) + 4.0;
         if (n < MAX_CANDS) out[n++] = {{256, 1, 3}, units, wave, (double)(units / num_sms) * wave + tail};
       }
     }
@@ -874,7 +874,7 @@ Plan best_alone(const Cand* c, int n) {
 // up and draws units until none are left.  (Measured on the BERT-base layer: a dense call takes 63 us when the
 // two grids together exceed the SMs and every unit of the second waits for the first, 52 us when the dW product
 // runs as 36 tiles of 256 x 256 beside the 96 CTAs of the dX product.)
-constexpr double KERNEL_US = 3.0;   // launch ramp and exit of a product kernel, on top of its units (timeline measurements)
+constexpr double KERNEL_US = 4.0;   // launch ramp and exit of a product kernel, on top of its units (timeline measurements)
 
 // Finish time of the second product: `units` units of `unit` us each, ready at `ready`, on the SMs the first
 // product (g1 CTAs, `units1` units of `unit1` us) leaves free.
@@ -882,36 +882,38 @@ constexpr double KERNEL_US = 3.0;   // launch ramp and exit of a product kernel,
 // CTAs that start first are also the ones with the most units.
 double second_end(long units, double unit, long g2, int slices, double ready, long g1, long units1, double unit1,
                   int num_sms) {
+  if (units <= 0) return ready + KERNEL_US;
   const long full = units1 / g1, rest = units1 % g1;
-  // phases of the first product: [0, full * unit1) all g1 CTAs busy; [full * unit1, (full + 1) * unit1) only
-  // `rest` of them (if any); afterwards none
-  const double t_a = (double)full * unit1 + KERNEL_US;
-  const double t_b = rest > 0 ? t_a + unit1 : t_a;
-  const long busy[3] = {g1, rest, 0};
-  const double from[3] = {0.0, t_a, t_b};
-  const double to[3] = {t_a, t_b, 1e30};
-  long left = units;
-  double end = ready;
-  bool started = false;
-  for (int ph = 0; ph < 3 && left > 0; ++ph) {
-    long sms = num_sms - busy[ph];
-    if (sms > g2) sms = g2;
-    const double t0 = ready > from[ph] ? ready : from[ph];
-    if (sms <= 0 || t0 >= to[ph]) continue;
-    if (!started && slices > 1) {
-      const long upi = (g2 / slices) * slices;
-      const long most = upi > 0 ? (units + upi - 1) / upi : units;
-      end = t0 + (double)most * unit;
+  // SMs by the time they are free for the second product: those without a CTA of the first, those whose CTA has no unit
+  // in the first product's last, partial wave, and the others
+  const double t_a = (double)full * unit1 + KERNEL_US, t_b = rest > 0 ? t_a + unit1 : t_a;
+  const double at[3] = {ready, ready > t_a ? ready : t_a, ready > t_b ? ready : t_b};
+  long sms[3] = {num_sms - g1, rest > 0 ? g1 - rest : 0, rest > 0 ? rest : g1};
+  long left = g2;
+  for (int i = 0; i < 3; ++i) {
+    if (sms[i] > left) sms[i] = left;
+    left -= sms[i];
+  }
+  if (slices > 1) {       // the units are assigned in advance: the last CTA to start has its share still to do
+    const long upi = (g2 / slices) * slices;
+    const long most = upi > 0 ? (units + upi - 1) / upi : units;
+    int last = 0;
+    for (int i = 0; i < 3; ++i)
+      if (sms[i] > 0) last = i;
+    return at[last] + (double)most * unit + KERNEL_US;
+  }
+  // the earliest time by which the SMs, each from when it is free, have worked all units off
+  double end = 1e30;
+  for (int i = 0; i < 3; ++i) {
+    if (sms[i] <= 0) continue;
+    for (long k = 1; k <= units; ++k) {
+      const double t = at[i] + (double)k * unit;
+      if (t >= end) break;
+      long done = 0;
+      for (int j = 0; j < 3; ++j)
+        if (sms[j] > 0 && t > at[j]) done += sms[j] * (long)((t - at[j]) / unit + 1e-9);
+      if (done >= units) { end = t; break; }
     }
-    started = true;
-    // units that start in this phase (a unit started before the phase ends is finished by its CTA)
-    const double span = to[ph] - t0;
-    long rounds = ph == 2 ? (left + sms - 1) / sms : (long)(span / unit) + 1;
-    long can = rounds * sms;
-    if (can > left) { can = left; rounds = (left + sms - 1) / sms; }
-    left -= can;
-    const double e = t0 + (double)rounds * unit;
-    if (e > end) end = e;
   }
   return end + KERNEL_US;
 }
@@ -919,10 +921,14 @@ double second_end(long units, double unit, long g2, int slices, double ready, lo
 void best_pair(const Cand* c1, int n1, int ctas1, const Cand* c2, int n2, int ctas2, int num_sms, double offset,
                Plan* p1, Plan* p2) {
   double best = 1e30;
+  const double alone_offset = offset;
   *p1 = c1[0].plan; *p2 = c2[0].plan;
   for (int i = 0; i < n1; ++i) {
     const bool split1 = c1[i].plan.mh == 3;
     const long g1 = split1 || c1[i].units > ctas1 ? ctas1 : c1[i].units;
+    // The kernels in front of the second product share the SMs with the first: on the BERT-base layer the call takes 31 us
+    // with 30 CTAs of the first product and 34 with 120, although these finish earlier.
+    offset = alone_offset * (1.0 + 0.25 * (double)g1 / num_sms);
     const double d1 = (split1 ? c1[i].alone : (double)((c1[i].units + g1 - 1) / g1) * c1[i].unit) + KERNEL_US;
     for (int j = 0; j < n2; ++j) {
       const bool split2 = c2[j].plan.mh == 3;
@@ -936,6 +942,8 @@ void best_pair(const Cand* c1, int n1, int ctas1, const Cand* c2, int n2, int ct
       } else {
         end2 = second_end(c2[j].units, c2[j].unit, g2, c2[j].plan.split, offset, g1, c1[i].units, c1[i].unit, num_sms);
       }
+      // the launch that adds the first product's slices takes SMs and L2 bandwidth from the kernels of the other branch
+      if (c1[i].plan.split > 1) end2 += 3.0;
       const double end = d1 > end2 ? d1 : end2;
       // ties: the pair whose products finish earlier, then the one with less SM time
       const double sm_time = (double)c1[i].units * c1[i].unit + (double)c2[j].units * c2[j].unit;
