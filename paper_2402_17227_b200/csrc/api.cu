@@ -316,7 +316,7 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
   // stream, needs a whole SM's shared memory.
   const int spare = 1;
   Plan px = {256, 1, 1}, pw = {256, 1, 1};
-  if (h->tensor_path) plan_products(h, false, a.rho, hint, spare, a_out != nullptr, &px, &pw);
+  if (h->tensor_path) plan_products(h, false, a.rho, hint, spare, a_out != nullptr, Hpre != nullptr, &px, &pw);
   if (!(h->tensor_path || h->split_path) || h->prof_enabled) {
     // one stream, so that (with stage profiling) each pair of events brackets the kernels of one stage
     mark(h, 0, st);
@@ -462,7 +462,7 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
     sw = h->side_stream;
   }
   Plan px = {256, 1, 1}, pw = {256, 1, 1};
-  if (h->tensor_path) plan_products(h, true, 1.0f, h->desc.N * h->desc.T, 0, false, &px, &pw);
+  if (h->tensor_path) plan_products(h, true, 1.0f, h->desc.N * h->desc.T, 0, false, Hpre != nullptr, &px, &pw);
   if (h->split_path) {
     VCAS_CUDA(launch_split_dx(h, dY, W, true, 1.0f, Hpre, dX, st));
   } else if (h->tensor_path) {

@@ -382,7 +382,7 @@ cudaError_t launch_umma_dw(Handle* h, const void* A_rows, const void* B_rows, in
 // Tilings of the dX and dW products of one call, chosen together because they share the SMs (cached in the
 // handle until the expected kept counts or the tuning overrides change).
 // row_norms_out: the dX product must emit row square-norms from its epilogue (unsliced 256-wide tiles only)
-void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spare_sms, bool row_norms_out, Plan* dx,
+void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spare_sms, bool row_norms_out, bool gelu, Plan* dx,
                    Plan* dw);
 
 // LayerNorm backward over the rows of kept data (after SampleA): dX, optional row square-norms of dX, dgamma, dbeta

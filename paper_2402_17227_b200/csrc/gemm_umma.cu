@@ -33,12 +33,13 @@ constexpr int EPI_BYTES = 8 * EPI_WARP_BYTES;           // one buffer for each o
 // accumulators, which cuts the shared-memory fill per FLOP by a third (the fill rate of one SM is
 // what bounds a 128 x 256 tile); it uses all 512 TMEM columns, so its epilogue does not overlap the
 // next main loop.  It is used for large problems only and never with a sliced contraction.
-template <int BN, int MH> struct TileCfg {
+// GELU: the instance whose epilogue multiplies by GELU'(H) gives up a stage for one more 4 KB buffer per epilogue warp.
+template <int BN, int MH, bool GELU> struct TileCfg {
   static constexpr int B_BYTES = BN * BK * 2;
   static constexpr int AT_BYTES = MH * A_BYTES;                       // the A part of a stage
   static constexpr int STAGE_BYTES = AT_BYTES + B_BYTES;
-  static constexpr int STAGES = MH == 2 ? 3 : (BN == 256 ? 4 : (BN == 128 ? 6 : 8));
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + EPI_BYTES + 256 /*barriers*/;
+  static constexpr int STAGES = (MH == 2 ? 3 : (BN == 256 ? 4 : (BN == 128 ? 6 : 8))) - (GELU ? (BN == 64 ? 2 : 1) : 0);
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + (GELU ? 2 : 1) * EPI_BYTES + 384 /*barriers*/;
 };
 
 constexpr int QD = 2;   // depth of the work queue: the producer may be this many items ahead of the other roles
@@ -54,37 +55,43 @@ struct SmemLayout {
   int* abort_flag;
   int* flag;          // epilogue broadcast slot
   int* tile_q;        // [QD] work items handed from the producer thread to the other roles
-  uint8_t* epi;       // [4 warps][2][32 rows][128 B] staging for bulk / TMA stores
+  uint8_t* epi;       // [8 warps][32 rows][128 B] staging for bulk / TMA stores
+  uint8_t* hbuf;      // GELU: [8 warps][32 rows][128 B] pre-activations of a warp's next chunk
+  uint64_t* h_full;   // GELU: [8 warps]
 };
 
-template <int BN, int MH>
+template <int BN, int MH, bool GELU>
 __device__ __forceinline__ SmemLayout carve(uint8_t* raw) {
-  using C = TileCfg<BN, MH>;
+  using C = TileCfg<BN, MH, GELU>;
   SmemLayout s;
   uint8_t* base = (uint8_t*)(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
   s.stages = base;
   s.epi = base + C::STAGES * C::STAGE_BYTES;                       // 1024-byte aligned (swizzle atom)
-  uint64_t* bars = (uint64_t*)(s.epi + EPI_BYTES);
+  s.hbuf = s.epi + EPI_BYTES;
+  uint64_t* bars = (uint64_t*)(s.epi + (GELU ? 2 : 1) * EPI_BYTES);
   s.full = bars;
   s.empty = bars + C::STAGES;
   s.tmem_full = bars + 2 * C::STAGES;
   s.tmem_empty = bars + 2 * C::STAGES + 2;
   s.q_full = bars + 2 * C::STAGES + 4;
   s.q_empty = bars + 2 * C::STAGES + 4 + QD;
-  s.tmem_holder = (uint32_t*)(bars + 2 * C::STAGES + 4 + 2 * QD);
+  s.h_full = bars + 2 * C::STAGES + 4 + 2 * QD;
+  s.tmem_holder = (uint32_t*)(s.h_full + (GELU ? 8 : 0));
   s.abort_flag = (int*)(s.tmem_holder + 1);
   s.flag = s.abort_flag + 1;
   s.tile_q = s.flag + 1;
   return s;
 }
 
-template <int BN, int MH>
+template <int BN, int MH, bool GELU>
 __device__ __forceinline__ uint32_t setup(const SmemLayout& s, int warp, int tid, bool with_queue,
                                           unsigned long long wait_limit_ns) {
-  using C = TileCfg<BN, MH>;
+  using C = TileCfg<BN, MH, GELU>;
   if (tid == 0) {
     for (int i = 0; i < C::STAGES; ++i) { mbar_init(&s.full[i], 1); mbar_init(&s.empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&s.tmem_full[i], 1); mbar_init(&s.tmem_empty[i], EPI_THREADS); }
+    if (GELU)
+      for (int i = 0; i < 8; ++i) mbar_init(&s.h_full[i], 1);
     if (with_queue)
       for (int i = 0; i < QD; ++i) { mbar_init(&s.q_full[i], 1); mbar_init(&s.q_empty[i], EPI_THREADS + 1); }
     *s.abort_flag = 0;
@@ -119,6 +126,11 @@ __device__ __forceinline__ float gelu_prime(float x) {
 #pragma unroll
   for (int k = 10; k >= 0; --k) p = fmaf(p, t, GP_C[k]);
   return fmaf(copysignf(ax, x), p, 0.5f);
+}
+__device__ __forceinline__ uint4 lds16(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
+  return v;
 }
 // r[e] *= GELU'(h_e) for the eight bf16 pre-activations in hv: the same polynomial as gelu_prime, the four pairs
 // side by side and every step of Horner's rule issued for all of them before the next (independent chains).
@@ -194,6 +206,7 @@ struct GemmParams {
   const int32_t* counts;   // counts[0] = number of kept data
   const float* scaleA;     // 1/p_n per datum
   const __nv_bfloat16* H;  // optional GELU pre-activation [R, d_in]
+  int h_tx_bytes;          // bytes one box of it delivers (min(T, 32) rows of 128 B)
   __nv_bfloat16* dX;       // [R, d_in]
   float* a_out;            // optional [R][a_parts]: square-norm of the stored row of dX, one partial sum per 256-column
   int a_parts;             // tile (unsliced 256-wide tiles only); the layer below adds the partials in order
@@ -300,17 +313,18 @@ __device__ __forceinline__ void tile_coords(const GemmParams& P, const Decomp& D
 // KIND_SLICED has only the slice exchange (a contraction that ends up in one slice still goes through it).
 // Separate instances because the product kernels are short: code that a launch never runs still costs it
 // time.
-template <int MODE, int BN, int MH, int KIND>
+// GELU: the dX epilogue multiplies by GELU'(H) (unsliced instances; a sliced product leaves it to the reduction launch).
+template <int MODE, int BN, int MH, int KIND, bool GELU>
 __global__ void __maxnreg__(MAX_REGS)
 umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-            const __grid_constant__ CUtensorMap tmC, GemmParams P) {
-  using C = TileCfg<BN, MH>;
+            const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmH, GemmParams P) {
+  using C = TileCfg<BN, MH, GELU>;
   constexpr int BMT = BM * MH;          // rows of a tile
   constexpr int NACC = MH == 2 ? 1 : 2;  // accumulator sets in TMEM
   extern __shared__ uint8_t smem_raw[];
-  const SmemLayout s = carve<BN, MH>(smem_raw);
+  const SmemLayout s = carve<BN, MH, GELU>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t tmem_base = setup<BN, MH>(s, warp, tid, KIND == KIND_DYNAMIC, P.wait_limit_ns);
+  const uint32_t tmem_base = setup<BN, MH, GELU>(s, warp, tid, KIND == KIND_DYNAMIC, P.wait_limit_ns);
   volatile int* abort_flag = s.abort_flag;
   pdl_wait();      // barriers and TMEM are set up; the counts and operands come from earlier kernels
   constexpr bool LEAN = KIND != KIND_SLICED;
@@ -483,6 +497,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
     };
     const uint32_t swz = (uint32_t)(lane & 7);                   // 128-byte swizzle: 16-byte slot ^= row & 7
+    uint32_t h_phase = 0;
     int lt = 0;
     bool ok = true;
     int qi = 0; uint32_t qph = 0;
@@ -542,21 +557,21 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       size_t row0; int rows_valid, col0, n_out, t_out; float sc;
       geometry(tile, true, row0, rows_valid, col0, sc, n_out, t_out);
       const int buf = lt_now % NACC; const uint32_t use = (uint32_t)(lt_now / NACC) & 1u;
-      if constexpr (LEAN && MODE == MODE_DX) {
-        // GELU' epilogue: while the tile's products are still running, ask L2 for the pre-activations of this
-        // thread's rows
-        if (P.H != nullptr) {
-#pragma unroll
-          for (int hh = 0; hh < MH; ++hh) {
-            const int hrow = hh * BM + row;
-            if (hrow < rows_valid) {
-              const __nv_bfloat16* hp = P.H + (row0 + hrow) * ld + col0;
-#pragma unroll
-              for (int j = eg; j < BN / 64; j += 2)
-                if (col0 + j * 64 < P.d_in) asm volatile("prefetch.global.L2 [%0];" ::"l"(hp + j * 64));
-            }
+      // GELU': this warp's pre-activations (32 rows x 128 bytes of chunk hj) come by TMA while the products or the chunk before
+      // are worked on; rows past T and columns past d_in are zero-filled.
+      auto load_h = [&](int hj) {
+        if constexpr (GELU) {
+          const int hh = hj / (BN / 64), j = hj % (BN / 64);
+          if (lane == 0) {
+            mbar_expect_tx(&s.h_full[eg * 4 + eq], (uint32_t)P.h_tx_bytes);
+            tma_load_3d(s.hbuf + (eg * 4 + eq) * EPI_WARP_BYTES, &tmH, col0 + j * 64, t_out + hh * BM + eq * 32, n_out, &s.h_full[eg * 4 + eq]);
           }
         }
+      };
+      if constexpr (GELU) {
+        int first = eg;
+        while (first < MH * (BN / 64) && col0 + first % (BN / 64) * 64 >= P.d_in) first += 2;
+        if (first < MH * (BN / 64)) load_h(first);
       }
       bool got = mbar_wait(&s.tmem_full[buf], use, abort_flag, P.status);
       if constexpr (!LEAN) {
@@ -582,11 +597,6 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         float rowsq[MH];                                            // square-norm of this thread's row(s), as stored
 #pragma unroll
         for (int hh = 0; hh < MH; ++hh) rowsq[hh] = 0.f;
-        // GELU' epilogue: this thread's 64 pre-activations of a chunk (eight 16-byte loads, its own row) are
-        // requested at the top of the chunk, in front of the TMEM load; they were prefetched to L2 before the
-        // wait for the accumulator, and the other warp of this quarter covers what latency is left.  (Staging
-        // them through shared memory with coalesced copies was measured slower.)
-        uint4 hq[8];
 #pragma unroll 1
         for (int hj = eg; hj < MH * (BN / COLS); hj += 2, ++nbuf) {      // this group's chunks
           const int hh = hj / (BN / COLS), j = hj % (BN / COLS);    // 128-row half of the tile, column chunk
@@ -597,13 +607,21 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           // the store of this warp's chunk before must have read the buffer before it is refilled (the wait sits
           // behind the TMEM load, where it costs little; the other warp of this quarter works meanwhile)
           auto buffer_free = [&]() { if (nbuf >= 1) { if (lane == 0) bulk_wait_read_0(); __syncwarp(); } };
-          const bool with_h = MODE == MODE_DX && P.H != nullptr;
-          if (with_h) {
-            // rows beyond the tile's valid rows read a valid row instead: their outputs are clipped by the store
-            const int hrow = min(hh * BM + row, rows_valid - 1);
-            const uint4* src = reinterpret_cast<const uint4*>(P.H + (row0 + hrow) * ld + col0 + j * 64);
+          // GELU': a thread's 64 pre-activations of the chunk from the swizzled buffer, which then takes the next chunk's.
+          // (Sixteen-byte loads of its own row by every thread cost 32 cache-line look-ups an instruction: with them the dX
+          // product of 5000 kept rows, 768 -> 3072 took 76 us instead of 54.)
+          uint4 hq[8];
+          if constexpr (GELU) {
+            if (!__all_sync(0xffffffffu, mbar_wait(&s.h_full[eg * 4 + eq], h_phase, abort_flag, P.status))) { ok = false; break; }
+            h_phase ^= 1u;
+            const uint4* src = reinterpret_cast<const uint4*>(s.hbuf + (eg * 4 + eq) * EPI_WARP_BYTES + lane * 128);
 #pragma unroll
-            for (int k8 = 0; k8 < 8; ++k8) hq[k8] = __ldg(src + k8);
+            for (int k8 = 0; k8 < 8; ++k8) hq[k8] = lds16(src + ((uint32_t)k8 ^ swz));
+            fence_async_smem();     // the reads are done before the copy engine writes the buffer again
+            __syncwarp();
+            int next = hj + 2;
+            while (next < MH * (BN / 64) && col0 + next % (BN / 64) * 64 >= P.d_in) next += 2;
+            if (next < MH * (BN / 64)) load_h(next);
           }
           if (MODE == MODE_DX) {
 #pragma unroll
@@ -616,7 +634,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 float r[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) r[e] = sc * __uint_as_float(v[g8 * 8 + e]);
-                if (with_h) gelu_prime8(hq[half * 4 + g8], r);
+                if constexpr (GELU) gelu_prime8(hq[half * 4 + g8], r);
                 uint4 o;
                 o.x = pack_bf16(r[0], r[1]); o.y = pack_bf16(r[2], r[3]);
                 o.z = pack_bf16(r[4], r[5]); o.w = pack_bf16(r[6], r[7]);
@@ -652,6 +670,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             bulk_commit();
           }
         }
+        if (GELU && !ok) break;
         tc_fence_before();
         mbar_arrive(&s.tmem_empty[buf]);
         if (MODE == MODE_DX && P.a_out != nullptr) {
@@ -811,8 +830,9 @@ constexpr int MAX_DEVICES = 64;
 
 // row_tiles128: number of 128-row tile rows (for dX: kept data x 128-token chunks); a 256-row tile covers two.
 // remainder_ok: 256-row tiles may leave a last partial wave to a second launch with 128-row tiles (mh = 3).
+// gelu: the epilogue multiplies by GELU'.
 int enumerate_plans(long row_tiles128, long row_tiles256, int n_extent, int kblocks, int num_sms, int max_units,
-                    int force_bn, int force_split, bool remainder_ok, Cand* out) {
+                    int force_bn, int force_split, bool remainder_ok, bool gelu, Cand* out) {
   const int widths[3] = {256, 128, 64};
   int n = 0;
   if (kblocks < 1) kblocks = 1;
@@ -831,7 +851,9 @@ int enumerate_plans(long row_tiles128, long row_tiles256, int n_extent, int kblo
       const double unit = (double)((kblocks + sp - 1) / sp) * KB_US[i] + (sp > 1 ? sliced_us(units, widths[i]) : UNIT_US);
       if (n < MAX_CANDS) out[n++] = {{widths[i], sp, 1}, units, unit, waves * unit};
     }
-    if (widths[i] == 256 && force_split <= 1) {                        // 256 x 256 tiles, never sliced
+    // 256 x 256 tiles, never sliced; not with GELU', whose epilogue only hides behind the next tile's products in 128-row
+    // tiles (two accumulators)
+    if (widths[i] == 256 && force_split <= 1 && !gelu) {
       const long units = row_tiles256 * ntiles;
       const double wave = (double)kblocks * KB2_US + UNIT2_US;
       if (n < MAX_CANDS) out[n++] = {{256, 1, 2}, units, wave, (double)((units + num_sms - 1) / num_sms) * wave};
@@ -953,15 +975,15 @@ void best_pair(const Cand* c1, int n1, int ctas1, const Cand* c2, int n2, int ct
   }
 }
 
-template <int MODE, int BN, int MH, int KIND>
-cudaError_t run_gemm_k(Handle* h, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, const GemmParams& P0,
-                     long max_items, int ctas, bool pdl, cudaStream_t st) {
+template <int MODE, int BN, int MH, int KIND, bool GELU = false>
+cudaError_t run_gemm_k(Handle* h, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, const CUtensorMap& hm,
+                       const GemmParams& P0, long max_items, int ctas, bool pdl, cudaStream_t st) {
   // the opt-in to large dynamic shared memory is a per-device attribute of the kernel
   static std::atomic<bool> attr_set[MAX_DEVICES];
   if (h->device < 0 || h->device >= MAX_DEVICES) return cudaErrorInvalidDevice;
   if (!attr_set[h->device].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(umma_kernel<MODE, BN, MH, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         TileCfg<BN, MH>::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(umma_kernel<MODE, BN, MH, KIND, GELU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         TileCfg<BN, MH, GELU>::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[h->device].store(true, std::memory_order_release);
   }
@@ -970,7 +992,7 @@ cudaError_t run_gemm_k(Handle* h, const CUtensorMap& a, const CUtensorMap& b, co
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = (size_t)TileCfg<BN, MH>::SMEM_BYTES;
+  cfg.dynamicSmemBytes = (size_t)TileCfg<BN, MH, GELU>::SMEM_BYTES;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 0;
@@ -981,7 +1003,7 @@ cudaError_t run_gemm_k(Handle* h, const CUtensorMap& a, const CUtensorMap& b, co
     cfg.numAttrs += 1;
   }
   cfg.gridDim = dim3((unsigned)grid);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, umma_kernel<MODE, BN, MH, KIND>, a, b, c, P);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, umma_kernel<MODE, BN, MH, KIND, GELU>, a, b, c, hm, P);
   h->launches += 1;
   if (e != cudaSuccess) return e;
   if constexpr (KIND == KIND_SLICED) {
@@ -1000,22 +1022,28 @@ cudaError_t run_gemm_k(Handle* h, const CUtensorMap& a, const CUtensorMap& b, co
 }
 
 template <int MODE, int BN, int MH>
-cudaError_t run_gemm(Handle* h, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, const GemmParams& P,
-                     long max_items, int ctas, bool pdl, cudaStream_t st) {
+cudaError_t run_gemm(Handle* h, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, const CUtensorMap& hm,
+                     const GemmParams& P, long max_items, int ctas, bool pdl, cudaStream_t st) {
   const bool many = max_items > ctas;      // more work items than CTAs: dynamic order
+  if constexpr (MODE == MODE_DX) {
+    if (P.H != nullptr && (MH == 2 || P.split_k == 1)) {
+      if (many) return run_gemm_k<MODE, BN, MH, KIND_DYNAMIC, true>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
+      return run_gemm_k<MODE, BN, MH, KIND_STATIC, true>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
+    }
+  }
   if constexpr (MH == 2) {
-    if (many) return run_gemm_k<MODE, BN, MH, KIND_DYNAMIC>(h, a, b, c, P, max_items, ctas, pdl, st);
-    return run_gemm_k<MODE, BN, MH, KIND_STATIC>(h, a, b, c, P, max_items, ctas, pdl, st);
+    if (many) return run_gemm_k<MODE, BN, MH, KIND_DYNAMIC>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
+    return run_gemm_k<MODE, BN, MH, KIND_STATIC>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
   } else {
-    if (P.split_k != 1) return run_gemm_k<MODE, BN, MH, KIND_SLICED>(h, a, b, c, P, max_items, ctas, pdl, st);
-    if (many) return run_gemm_k<MODE, BN, MH, KIND_DYNAMIC>(h, a, b, c, P, max_items, ctas, pdl, st);
-    return run_gemm_k<MODE, BN, MH, KIND_STATIC>(h, a, b, c, P, max_items, ctas, pdl, st);
+    if (P.split_k != 1) return run_gemm_k<MODE, BN, MH, KIND_SLICED>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
+    if (many) return run_gemm_k<MODE, BN, MH, KIND_DYNAMIC>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
+    return run_gemm_k<MODE, BN, MH, KIND_STATIC>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
   }
 }
 
 template <int MODE>
 cudaError_t run_gemm_bn(Handle* h, const Plan& plan, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
-                        const GemmParams& P, long max_items, int ctas, bool pdl, cudaStream_t st) {
+                        const CUtensorMap& hm, const GemmParams& P, long max_items, int ctas, bool pdl, cudaStream_t st) {
   if (plan.mh == 3) {
     // whole waves of 256-row tiles, then the remaining tiles as 128-row tiles with a sliced contraction
     // (both launches derive the same division from the device-resident counts)
@@ -1023,17 +1051,17 @@ cudaError_t run_gemm_bn(Handle* h, const Plan& plan, const CUtensorMap& a, const
     Q.split_k = 1;
     Q.part = 1;
     Q.head_ctas = (int)(max_items < ctas ? max_items : ctas);
-    const cudaError_t e = run_gemm<MODE, 256, 2>(h, a, b, c, Q, max_items, ctas, pdl, st);
+    const cudaError_t e = run_gemm<MODE, 256, 2>(h, a, b, c, hm, Q, max_items, ctas, pdl, st);
     if (e != cudaSuccess) return e;
     Q.part = 2;
     Q.split_k = 0;
-    return run_gemm<MODE, 256, 1>(h, a, b, c, Q, (long)ctas, ctas, true, st);
+    return run_gemm<MODE, 256, 1>(h, a, b, c, hm, Q, (long)ctas, ctas, true, st);
   }
-  if (plan.mh == 2) return run_gemm<MODE, 256, 2>(h, a, b, c, P, max_items, ctas, pdl, st);
+  if (plan.mh == 2) return run_gemm<MODE, 256, 2>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
   switch (plan.bn) {
-    case 256: return run_gemm<MODE, 256, 1>(h, a, b, c, P, max_items, ctas, pdl, st);
-    case 128: return run_gemm<MODE, 128, 1>(h, a, b, c, P, max_items, ctas, pdl, st);
-    default: return run_gemm<MODE, 64, 1>(h, a, b, c, P, max_items, ctas, pdl, st);
+    case 256: return run_gemm<MODE, 256, 1>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
+    case 128: return run_gemm<MODE, 128, 1>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
+    default: return run_gemm<MODE, 64, 1>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
   }
 }
 
@@ -1072,12 +1100,12 @@ bool dw_remainder_ok(const Handle* h) {
 }
 }  // namespace
 
-void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spare_sms, bool row_norms_out, Plan* dx,
+void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spare_sms, bool row_norms_out, bool gelu, Plan* dx,
                    Plan* dw) {
   const vcas_layer_desc& d = h->desc;
   const DxShape g = dx_shape(h, dense, rho_hint);
   const int kb_w = (cnt_hint + BK - 1) / BK;
-  const int key[PLAN_KEY_INTS] = {(dense ? 1 : 0) | (row_norms_out ? 2 : 0), (int)g.row_tiles128, kb_w, spare_sms,
+  const int key[PLAN_KEY_INTS] = {(dense ? 1 : 0) | (row_norms_out ? 2 : 0) | (gelu ? 4 : 0), (int)g.row_tiles128, kb_w, spare_sms,
                                   h->tune_dx_tile_n, h->tune_dw_tile_n, h->tune_dx_split_k, h->tune_dw_split_k,
                                   h->tune_dx_tile_m + 4 * h->tune_dw_tile_m};
   bool hit = h->plan_valid;
@@ -1101,10 +1129,10 @@ void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spar
     // the epilogue emits row square-norms of dX only from unsliced 256-wide tiles (one partial sum per tile)
     const int nx = enumerate_plans(g.row_tiles128, g.row_tiles256, d.d_in, g.kblocks, ctas, h->max_units,
                                    row_norms_out ? 256 : h->tune_dx_tile_n, row_norms_out ? 1 : h->tune_dx_split_k,
-                                   g.rem_ok && !row_norms_out, cx);
+                                   g.rem_ok && !row_norms_out, gelu, cx);
     const bool rem_w = dw_remainder_ok(h);
     const int nw = enumerate_plans((d.d_out + BM - 1) / BM, (d.d_out + 2 * BM - 1) / (2 * BM), d.d_in, kb_w, h->num_sms,
-                                   h->max_units, h->tune_dw_tile_n, h->tune_dw_split_k, rem_w, cw);
+                                   h->max_units, h->tune_dw_tile_n, h->tune_dw_split_k, rem_w, false, cw);
     // A sampled dW product becomes ready later than the dX product by the time of the kernels in front of it
     // on the side stream (fitted to their ncu durations on three layer shapes): the norms of the kept rows of X
     // (HBM-bound), SampleW's single-CTA fixed point over the rows of kept data, and the emit + pack pass, which
@@ -1138,7 +1166,7 @@ cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense,
                            void* dX, float* a_out, bool skip_dropped, int spare_sms, const Plan* pair_plan,
                            cudaStream_t st) {
   const vcas_layer_desc& d = h->desc;
-  CUtensorMap tmA, tmB, tmC;
+  CUtensorMap tmA, tmB, tmC, tmH;
   {
     const uint64_t dims[3] = {(uint64_t)d.d_out, (uint64_t)d.T, (uint64_t)d.N};
     const uint64_t strides[2] = {(uint64_t)d.d_out * 2, (uint64_t)d.T * d.d_out * 2};
@@ -1156,12 +1184,15 @@ cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense,
     const uint64_t strides[2] = {(uint64_t)d.d_in * 2, (uint64_t)d.T * d.d_in * 2};
     const uint32_t box[3] = {64, (uint32_t)(d.T < 32 ? d.T : 32), 1};
     if (!make_map(&tmC, dX, 3, dims, strides, box)) return cudaErrorInvalidValue;
+    tmH = tmC;
+    if (H != nullptr && !make_map(&tmH, H, 3, dims, strides, box)) return cudaErrorInvalidValue;
   }
   GemmParams P;
   common_params(h, P, 0);
   P.idxA = h->ws.idxA; P.dropA = h->ws.dropA; P.counts = h->ws.counts; P.scaleA = h->ws.scaleA;
   P.a_out = a_out; P.a_parts = a_out_parts(d.d_in);
   P.H = (const __nv_bfloat16*)H; P.dX = (__nv_bfloat16*)dX;
+  P.h_tx_bytes = (d.T < 32 ? d.T : 32) * 128;
   P.N = d.N; P.T = d.T; P.dense = dense ? 1 : 0;
   P.skip_dropped = skip_dropped ? 1 : 0;
   P.a_tx_bytes = (d.T < BM ? d.T : BM) * BK * 2;
@@ -1175,13 +1206,13 @@ cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense,
     Cand cands[MAX_CANDS];
     const bool rn = a_out != nullptr;
     const int n = enumerate_plans(g.row_tiles128, g.row_tiles256, d.d_in, g.kblocks, ctas, h->max_units,
-                                  rn ? 256 : h->tune_dx_tile_n, rn ? 1 : h->tune_dx_split_k, g.rem_ok && !rn, cands);
+                                  rn ? 256 : h->tune_dx_tile_n, rn ? 1 : h->tune_dx_split_k, g.rem_ok && !rn, H != nullptr, cands);
     plan = apply_tile_m(h->tune_dx_tile_m, best_alone(cands, n), g.rem_ok && !rn);
   }
   P.split_k = plan.split;
   // upper bound of work items: every datum kept and split, or every datum a zero tile
   const long max_items = (long)d.N * (plan.mh >= 2 ? chunks2 : chunks) * ((d.d_in + plan.bn - 1) / plan.bn) * plan.split;
-  return run_gemm_bn<MODE_DX>(h, plan, tmA, tmB, tmC, P, max_items, ctas, true, st);
+  return run_gemm_bn<MODE_DX>(h, plan, tmA, tmB, tmC, tmH, P, max_items, ctas, true, st);
 }
 
 cudaError_t launch_umma_dw(Handle* h, const void* A_rows, const void* B_rows, int rows_capacity, const int32_t* cnt,
@@ -1217,12 +1248,12 @@ cudaError_t launch_umma_dw(Handle* h, const void* A_rows, const void* B_rows, in
     const bool rem_ok = dw_remainder_ok(h);
     Cand cands[MAX_CANDS];
     const int n = enumerate_plans(mtiles, mtiles2, d.d_in, (cnt_hint + BK - 1) / BK, h->num_sms, h->max_units,
-                                  h->tune_dw_tile_n, h->tune_dw_split_k, rem_ok, cands);
+                                  h->tune_dw_tile_n, h->tune_dw_split_k, rem_ok, false, cands);
     plan = apply_tile_m(h->tune_dw_tile_m, best_alone(cands, n), rem_ok);
   }
   P.split_k = plan.split;
   const long max_items = (plan.mh >= 2 ? mtiles2 : mtiles) * ((d.d_in + plan.bn - 1) / plan.bn) * plan.split;
-  return run_gemm_bn<MODE_DW>(h, plan, tmA, tmB, tmC, P, max_items, h->num_sms, true, st);
+  return run_gemm_bn<MODE_DW>(h, plan, tmA, tmB, tmC, tmC, P, max_items, h->num_sms, true, st);
 }
 
 }  // namespace vcas
