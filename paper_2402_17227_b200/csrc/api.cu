@@ -46,6 +46,7 @@ size_t layout(Handle* h, uint8_t* base) {
   w.scaleA = carve<float>(cur, N);
   w.scaleW = carve<float>(cur, R);
   w.sorted = carve<float>(cur, N);
+  w.gk = carve<float>(cur, N);
   w.idxA = carve<int32_t>(cur, N);
   w.dropA = carve<int32_t>(cur, N);
   w.idxW = carve<int32_t>(cur, R);
@@ -79,6 +80,7 @@ size_t layout(Handle* h, uint8_t* base) {
   v.wc = carve<float>(cur, R);
   v.uc = carve<uint32_t>(cur, R);
   v.g = carve<float>(cur, N);
+  v.gk = carve<float>(cur, N);
   v.p = carve<float>(cur, N);
   v.w = carve<float>(cur, R);
   v.q = carve<float>(cur, R);

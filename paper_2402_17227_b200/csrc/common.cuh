@@ -25,12 +25,13 @@ struct Workspace {
   float* scaleA;   // [N]  1/p_n for kept data, 0 for dropped data
   float* scaleW;   // [R]  1/(p_n q_r) per compacted row
   float* sorted;   // [N]  data norms in descending order (Eq. 4)
+  float* gk;       // [N]  SampleA: norms of the alive data, in the order of their list
   int32_t* idxA;   // [N]  kept data, ascending
   int32_t* dropA;  // [N]  dropped data, ascending
   int32_t* idxW;   // [R]  kept rows, ascending
   int32_t* chunk_off;  // [R/32 + 2] position in idxW of the first kept row of every chunk of 32 compact rows
   float* fix;      // [4]  0: the factor c of q = min(1, c w) found by the water-filling, 1: mode (see sample_w_kernel)
-  int32_t* counts; // [8]  0: cntA, 1: cntW, 2: R (constant, for dense launches), 4: reduction ticket
+  int32_t* counts; // [8]  0: cntA, 1: cntW, 2: R (constant, for dense launches), 4: reduction ticket, 5: SampleA's ticket
   int32_t* status; // [1]  device status word
   double* acc;     // [16] probe accumulators (0: V_act, 1: V_w, 2: p_lo, 3: p_hi, 4: V_s)
   double* partial; // [PARTIAL_SLOTS] block partial sums of the probe reductions

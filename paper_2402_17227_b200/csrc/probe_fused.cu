@@ -620,8 +620,12 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
     PROBE_CUDA(cudaGetLastError());
     Q.first_batch = i0;
     const dim3 draw_grid((unsigned)(PD * passes + 1), (unsigned)batches);
-    PROBE_CUDA(d.N <= 32 ? launch_after(probe_draw_kernel<1>, draw_grid, dim3(DRAW_THREADS), 0, st, Q)
-                         : launch_after(probe_draw_kernel<32>, draw_grid, dim3(DRAW_THREADS), 0, st, Q));
+    const dim3 threads(DRAW_THREADS);
+    PROBE_CUDA(d.N <= 32    ? launch_after(probe_draw_kernel<1>, draw_grid, threads, 0, st, Q)
+               : d.N <= 64  ? launch_after(probe_draw_kernel<2>, draw_grid, threads, 0, st, Q)
+               : d.N <= 128 ? launch_after(probe_draw_kernel<4>, draw_grid, threads, 0, st, Q)
+               : d.N <= 256 ? launch_after(probe_draw_kernel<8>, draw_grid, threads, 0, st, Q)
+                            : launch_after(probe_draw_kernel<32>, draw_grid, threads, 0, st, Q));
     PROBE_CUDA(cudaEventRecord(h->ev_fork, st));
     PROBE_CUDA(cudaStreamWaitEvent(side, h->ev_fork, 0));
     PROBE_CUDA(launch_maybe_after(false, probe_vw_kernel, dim3((unsigned)M, (unsigned)batches), dim3(SAMPLER_THREADS), vw_smem, side, Q));

@@ -140,41 +140,87 @@ struct SampleAParams {
   int32_t* idxA; int32_t* dropA; int32_t* counts;
   int32_t* kept_out; int32_t* kept_cnt_out;
   int32_t* status;
+  float* gk;                       // [N] norms of the alive data, in the order of their list
+  int32_t* ticket;                 // CTAs that have finished; zero between launches
 };
 
-// SampleA (Sec. 4.1) for N <= 32 * SLOTS data: one warp per datum sums its T row square-norms (only the alive
-// data are read; the others have norm 0), then warp 0 finds p, draws the masks and writes the lists.
-constexpr int SAMPLE_A_THREADS = 512;
+constexpr int SAMPLE_A_THREADS = 256;
+constexpr int SAMPLE_A_WARP_LEN = 1024;    // longest sum one warp takes
+
+// Sum of the len floats of one datum by a CTA, in a fixed order; result in thread 0.
+__device__ __forceinline__ float datum_sqnorm_cta(const float* an, int len, float* s_part) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  int t = threadIdx.x;
+  for (; t + 3 * SAMPLE_A_THREADS < len; t += 4 * SAMPLE_A_THREADS)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] += __ldcg(an + t + k * SAMPLE_A_THREADS);
+  for (; t < len; t += SAMPLE_A_THREADS) s[0] += __ldcg(an + t);
+  const float w = warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+  if (lane == 0) s_part[warp] = w;
+  __syncthreads();
+  float r = 0.f;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < SAMPLE_A_THREADS / 32; ++i) r += s_part[i];
+  __syncthreads();
+  return r;
+}
+
+// SampleA (Sec. 4.1) for N <= 32 * SLOTS data.  The CTAs share the data (only the alive ones are read; the others have norm
+// 0): one warp sums a datum's T row square-norms, or, where a producer's partial sums make that many more, a CTA.  The CTA
+// that finishes last finds p, draws the masks and writes the lists in one warp, whose lanes hold SLOTS data each: the
+// smallest SLOTS that fits, since every slot costs a Philox block and a term in every round.  (With one CTA for all sums a
+// chained layer's 1 MB of partial sums took 30 us, and 64 data in 32 slots 18 us instead of 5.)
 template <int SLOTS>
 __global__ void __launch_bounds__(SAMPLE_A_THREADS) sample_a_kernel(SampleAParams P) {
   __shared__ float s_g[32 * SLOTS];
+  __shared__ float s_part[SAMPLE_A_THREADS / 32];
+  __shared__ int s_last;
   pdl_wait();      // the row norms come from the kernel before this one
   pdl_trigger();   // the dX product kernel may set itself up meanwhile
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int n = threadIdx.x; n < 32 * SLOTS; n += SAMPLE_A_THREADS) s_g[n] = 0.f;
-  __syncthreads();
   // a caller's list of alive data is not trusted: a length outside [0, N] or an entry outside [0, N) is reported
   // as VCAS_ERR_BAD_ARG in the status word and not followed
   int nd = P.N;
   if (P.alive != nullptr) {
     nd = *P.alive_cnt;
     if (nd < 0 || nd > P.N) {
-      if (threadIdx.x == 0) atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
+      if (threadIdx.x == 0 && blockIdx.x == 0) atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
       nd = min(max(nd, 0), P.N);
     }
   }
   const int len = P.T * P.a_parts;
-  for (int k = warp; k < nd; k += SAMPLE_A_THREADS / 32) {
-    const int n = P.alive != nullptr ? P.alive[k] : k;
-    if ((unsigned)n >= (unsigned)P.N) {
-      if (lane == 0) atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
-      continue;
+  if (len <= SAMPLE_A_WARP_LEN) {
+    for (int k = blockIdx.x * (SAMPLE_A_THREADS / 32) + warp; k < nd; k += gridDim.x * (SAMPLE_A_THREADS / 32)) {
+      const int n = P.alive != nullptr ? P.alive[k] : k;
+      const float s = (unsigned)n < (unsigned)P.N ? datum_sqnorm_warp(P.a + (size_t)n * len, len, lane) : 0.f;
+      if (lane == 0) P.gk[k] = sqrtf(s);
     }
-    const float s = datum_sqnorm_warp(P.a + (size_t)n * len, len, lane);
-    if (lane == 0) s_g[n] = sqrtf(s);
+  } else {
+    for (int k = blockIdx.x; k < nd; k += gridDim.x) {
+      const int n = P.alive != nullptr ? P.alive[k] : k;
+      if ((unsigned)n >= (unsigned)P.N) continue;
+      const float s = datum_sqnorm_cta(P.a + (size_t)n * len, len, s_part);
+      if (threadIdx.x == 0) P.gk[k] = sqrtf(s);
+    }
+  }
+  if (gridDim.x > 1) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(P.ticket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *P.ticket = 0;
+  }
+  for (int n = threadIdx.x; n < 32 * SLOTS; n += SAMPLE_A_THREADS) s_g[n] = 0.f;
+  __syncthreads();
+  for (int k = threadIdx.x; k < nd; k += SAMPLE_A_THREADS) {
+    const int n = P.alive != nullptr ? P.alive[k] : k;
+    if ((unsigned)n < (unsigned)P.N) s_g[n] = __ldcg(P.gk + k);
+    else atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
   }
   __syncthreads();
-  for (int n = threadIdx.x; n < P.N; n += SAMPLE_A_THREADS) P.g[n] = s_g[n];
   if (warp == 0) {
     SampleAOut o;
     o.p = P.p; o.scaleA = P.scaleA; o.idxA = P.idxA; o.dropA = P.dropA; o.idx_copy = P.kept_out;
@@ -183,6 +229,8 @@ __global__ void __launch_bounds__(SAMPLE_A_THREADS) sample_a_kernel(SampleAParam
       P.counts[0] = kept;
       if (P.kept_cnt_out != nullptr) *P.kept_cnt_out = kept;
     }
+  } else {
+    for (int n = threadIdx.x - 32; n < P.N; n += SAMPLE_A_THREADS - 32) P.g[n] = s_g[n];
   }
 }
 
@@ -532,11 +580,23 @@ cudaError_t launch_sample_a(Handle* h, const SamplerArgs& a, bool programmatic, 
   P.g = ws.g; P.p = ws.p; P.scaleA = ws.scaleA; P.idxA = ws.idxA; P.dropA = ws.dropA; P.counts = ws.counts;
   P.kept_out = a.kept_out; P.kept_cnt_out = a.kept_cnt_out;
   P.status = ws.status;
+  P.gk = ws.gk; P.ticket = ws.counts + 5;
+  const int per_cta = d.T * P.a_parts <= SAMPLE_A_WARP_LEN ? SAMPLE_A_THREADS / 32 : 1;
+  int ctas = (d.N + per_cta - 1) / per_cta;
+  const int cap = h->num_sms > 0 ? h->num_sms : 148;
+  if (ctas > cap) ctas = cap;
+  const dim3 grid((unsigned)ctas), threads(SAMPLE_A_THREADS);
   cudaError_t e;
   if (d.N <= 32)
-    e = launch_maybe_after(programmatic, sample_a_kernel<1>, dim3(1), dim3(SAMPLE_A_THREADS), 0, st, P);
+    e = launch_maybe_after(programmatic, sample_a_kernel<1>, grid, threads, 0, st, P);
+  else if (d.N <= 64)
+    e = launch_maybe_after(programmatic, sample_a_kernel<2>, grid, threads, 0, st, P);
+  else if (d.N <= 128)
+    e = launch_maybe_after(programmatic, sample_a_kernel<4>, grid, threads, 0, st, P);
+  else if (d.N <= 256)
+    e = launch_maybe_after(programmatic, sample_a_kernel<8>, grid, threads, 0, st, P);
   else if (d.N <= WARP_MAX_N)
-    e = launch_maybe_after(programmatic, sample_a_kernel<32>, dim3(1), dim3(SAMPLE_A_THREADS), 0, st, P);
+    e = launch_maybe_after(programmatic, sample_a_kernel<32>, grid, threads, 0, st, P);
   else
     e = launch_maybe_after(programmatic, sample_a_big_kernel, dim3(1), dim3(SAMPLER_THREADS), 0, st, P);
   h->launches += 1;

@@ -12,7 +12,7 @@ namespace {
 constexpr int STATIC_MAX_R = 16384;   // rows (N*T) the fixed scratch can serve
 constexpr int STATIC_MAX_N = 4096;    // data
 constexpr size_t kRowArrays = 8;      // a, wc, w, q, scaleW (float), idxW, chunk_off (int32), uc (uint32), each [STATIC_MAX_R]
-constexpr size_t kDatumArrays = 6;    // g, p, scaleA, sorted (float) and idxA, dropA (int32), each [STATIC_MAX_N]
+constexpr size_t kDatumArrays = 6;    // g, p, scaleA, gk (float) and idxA, dropA (int32), each [STATIC_MAX_N]
 constexpr size_t kTailBytes = 768;    // counts [8] int32, acc [16] double, fix [4] float + status word, 256-byte slots
 constexpr size_t kScratchBytes = kRowArrays * STATIC_MAX_R * 4 + kDatumArrays * STATIC_MAX_N * 4 + kTailBytes;
 
@@ -74,7 +74,7 @@ extern "C" int vcas_score_static(int32_t N, int32_t T, int32_t d_in, int32_t d_o
   ws.g = fn + 0 * STATIC_MAX_N;
   ws.p = fn + 1 * STATIC_MAX_N;
   ws.scaleA = fn + 2 * STATIC_MAX_N;
-  ws.sorted = fn + 3 * STATIC_MAX_N;
+  ws.gk = fn + 3 * STATIC_MAX_N;
   ws.idxA = reinterpret_cast<int32_t*>(fn + 4 * STATIC_MAX_N);
   ws.dropA = reinterpret_cast<int32_t*>(fn + 5 * STATIC_MAX_N);
   unsigned char* tail = reinterpret_cast<unsigned char*>(fn + kDatumArrays * STATIC_MAX_N);
