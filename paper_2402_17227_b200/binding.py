@@ -56,6 +56,29 @@ class ChainArgs(C.Structure):
                 ("kept_cnt_out", C.c_void_p), ("skip_dropped_rows", C.c_int32), ("defer_join", C.c_int32)]
 
 
+_P, _I, _F, _U64 = C.c_void_p, C.c_int32, C.c_float, C.c_uint64
+# argument types, so that plain numbers and addresses can be passed (void pointers take an int or None)
+_SAMPLING_OUT = [_P] * 8
+ARGTYPES = {
+    "vcas_default_config": [_P], "vcas_create": [_P] * 3, "vcas_destroy": [_P], "vcas_workspace_bytes": [_P] * 2,
+    "vcas_linear_bwd": [_P] * 4 + [_F, _F, _U64] + [_P] * 3,
+    "vcas_linear_bwd_ex": [_P] * 4 + [_F, _F, _U64] + [_P] * 6,
+    "vcas_linear_bwd_chain": [_P] * 4 + [_F, _F, _U64] + [_P] * 4,
+    "vcas_chain_parts": [_P] * 2,
+    "vcas_layernorm_bwd": [_P] * 4 + [_F, _F, _U64] + [_P] * 5,
+    "vcas_join": [_P] * 2, "vcas_dense_bwd": [_P] * 7, "vcas_dense_bwd_ex": [_P] * 8,
+    "vcas_score": [_P] * 3 + [_F, _F, _U64] + _SAMPLING_OUT + [_P],
+    "vcas_last_sampling": [_P] + _SAMPLING_OUT + [_P],
+    "vcas_mask_from_probs": [_P, _P, _I, _U64, _I] + [_P] * 4,
+    "vcas_variance_probe": [_P, _I] + [_P] * 3 + [_F, _F, _F, _U64] + [_P] * 6,
+    "vcas_update_ratios": [_P, _I] + [_P] * 6,
+    "vcas_last_device_status": [_P] * 2, "vcas_launch_count": [_P] * 2,
+    "vcas_set_profiling": [_P, _I], "vcas_stage_times": [_P] * 3, "vcas_set_wait_limit": [_P, _U64, _I],
+    "vcas_set_probe_subsample": [_P, _I, _U64], "vcas_get_probe_subsample": [_P] * 3,
+    "vcas_score_static": [_I] * 5 + [_P, _P, _F, _F, _U64] + _SAMPLING_OUT + [_P],
+    "vcas_set_tuning": [_P] + [_I] * 6, "vcas_last_plan": [_P] * 2, "vcas_version": [],
+}
+
 _lib = None
 
 
@@ -69,7 +92,8 @@ def lib() -> C.CDLL:
                                "there is no CPU implementation")
         l = C.CDLL(LIB_PATH)
         for name in EXPORTS:
-            getattr(l, name).restype = C.c_int
+            fn = getattr(l, name)
+            fn.restype, fn.argtypes = C.c_int, ARGTYPES[name]
         _lib = l
     return _lib
 
@@ -81,13 +105,19 @@ def _check(code: int, where: str) -> None:
 
 def _ptr(t):
     if t is None:
-        return C.c_void_p(None)
+        return None
     assert t.is_cuda and t.is_contiguous(), "device-resident contiguous tensors only"
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# the current stream's handle without the Python stream object around it (0.3 us instead of 3)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def default_config() -> Config:
@@ -106,6 +136,19 @@ class Sampling:
     cntA: int
     idxW: torch.Tensor
     cntW: int
+
+
+def _sampling_buffers(N: int, R: int, dev):
+    """g, p, w, q, idxA, idxW and the two counts: the outputs of a scoring call, which writes all of them."""
+    f, i = torch.float32, torch.int32
+    return (torch.empty(N, dtype=f, device=dev), torch.empty(N, dtype=f, device=dev), torch.empty(R, dtype=f, device=dev),
+            torch.empty(R, dtype=f, device=dev), torch.empty(N, dtype=i, device=dev), torch.empty(R, dtype=i, device=dev),
+            torch.empty(2, dtype=i, device=dev))
+
+
+def _sampling_ptrs(b):
+    g, p, w, q, idxA, idxW, cnt = [t.data_ptr() for t in b]
+    return g, p, w, q, idxA, cnt, idxW, cnt + 4
 
 
 class Layer:
@@ -144,8 +187,8 @@ class Layer:
     def linear_bwd(self, X, dY, W, rho: float, nu: float, seed: int, *, p_in=None, q_in=None, H=None,
                    dX=None, dW=None):
         dX, dW = self._outs(dX, dW, X.device)
-        rc = lib().vcas_linear_bwd_ex(self._h, _ptr(X), _ptr(dY), _ptr(W), C.c_float(rho), C.c_float(nu),
-                                      C.c_uint64(seed), _ptr(p_in), _ptr(q_in), _ptr(H), _ptr(dX), _ptr(dW),
+        rc = lib().vcas_linear_bwd_ex(self._h, _ptr(X), _ptr(dY), _ptr(W), rho, nu,
+                                      seed, _ptr(p_in), _ptr(q_in), _ptr(H), _ptr(dX), _ptr(dW),
                                       _stream())
         _check(rc, "vcas_linear_bwd_ex")
         return dX, dW
@@ -158,8 +201,8 @@ class Layer:
         dp = lambda t: None if t is None else t.data_ptr()
         args = ChainArgs(dp(H), dp(a_in), a_in_parts, dp(alive_in), dp(alive_cnt_in), dp(a_out), dp(kept_out),
                          dp(kept_cnt_out), 1 if skip_dropped_rows else 0, 1 if defer_join else 0)
-        _check(lib().vcas_linear_bwd_chain(self._h, _ptr(X), _ptr(dY), _ptr(W), C.c_float(rho), C.c_float(nu),
-                                           C.c_uint64(seed), C.byref(args), _ptr(dX), _ptr(dW), _stream()),
+        _check(lib().vcas_linear_bwd_chain(self._h, _ptr(X), _ptr(dY), _ptr(W), rho, nu,
+                                           seed, C.byref(args), _ptr(dX), _ptr(dW), _stream()),
                "vcas_linear_bwd_chain")
 
     def layernorm_bwd(self, X, gamma, dY, rho: float, seed: int, eps: float = 1e-5, *, dX=None, a_in=None,
@@ -174,8 +217,8 @@ class Layer:
         dp = lambda t: None if t is None else t.data_ptr()
         args = ChainArgs(None, dp(a_in), a_in_parts, dp(alive_in), dp(alive_cnt_in), dp(a_out), dp(kept_out),
                          dp(kept_cnt_out), 1 if skip_dropped_rows else 0, 0)
-        _check(lib().vcas_layernorm_bwd(self._h, _ptr(X), _ptr(gamma), _ptr(dY), C.c_float(eps), C.c_float(rho),
-                                        C.c_uint64(seed), C.byref(args), _ptr(dX), _ptr(dg), _ptr(db), _stream()),
+        _check(lib().vcas_layernorm_bwd(self._h, _ptr(X), _ptr(gamma), _ptr(dY), eps, rho,
+                                        seed, C.byref(args), _ptr(dX), _ptr(dg), _ptr(db), _stream()),
                "vcas_layernorm_bwd")
         return dX, dg, db
 
@@ -189,8 +232,8 @@ class Layer:
 
     def linear_bwd_plain(self, X, dY, W, rho: float, nu: float, seed: int, dX, dW):
         """vcas_linear_bwd with caller-provided outputs (the call a training loop makes)."""
-        _check(lib().vcas_linear_bwd(self._h, _ptr(X), _ptr(dY), _ptr(W), C.c_float(rho), C.c_float(nu),
-                                     C.c_uint64(seed), _ptr(dX), _ptr(dW), _stream()), "vcas_linear_bwd")
+        _check(lib().vcas_linear_bwd(self._h, _ptr(X), _ptr(dY), _ptr(W), rho, nu,
+                                     seed, _ptr(dX), _ptr(dW), _stream()), "vcas_linear_bwd")
 
     def dense_bwd(self, X, dY, W, *, H=None, dX=None, dW=None):
         dX, dW = self._outs(dX, dW, X.device)
@@ -200,27 +243,23 @@ class Layer:
 
     # ------------------------------------------------------------------ sampling
     def _sampling_buffers(self, dev):
-        f = dict(dtype=torch.float32, device=dev)
-        i = dict(dtype=torch.int32, device=dev)
-        return (torch.empty(self.N, **f), torch.empty(self.N, **f), torch.empty(self.R, **f),
-                torch.empty(self.R, **f), torch.empty(self.N, **i), torch.zeros(1, **i),
-                torch.empty(self.R, **i), torch.zeros(1, **i))
+        return _sampling_buffers(self.N, self.R, dev)
 
     @staticmethod
     def _pack_sampling(b) -> Sampling:
-        g, p, w, q, idxA, cntA, idxW, cntW = b
-        ca, cw = int(cntA.item()), int(cntW.item())
+        g, p, w, q, idxA, idxW, cnt = b
+        ca, cw = cnt.tolist()           # one wait for both counts
         return Sampling(g, p, w, q, idxA[:ca], ca, idxW[:cw], cw)
 
     def score(self, X, dY, rho: float, nu: float, seed: int) -> Sampling:
         b = self._sampling_buffers(X.device)
-        _check(lib().vcas_score(self._h, _ptr(X), _ptr(dY), C.c_float(rho), C.c_float(nu), C.c_uint64(seed),
-                                *[_ptr(t) for t in b], _stream()), "vcas_score")
+        _check(lib().vcas_score(self._h, _ptr(X), _ptr(dY), rho, nu, seed,
+                                *_sampling_ptrs(b), _stream()), "vcas_score")
         return self._pack_sampling(b)
 
     def last_sampling(self, device=None) -> Sampling:
         b = self._sampling_buffers(device or torch.device("cuda", torch.cuda.current_device()))
-        _check(lib().vcas_last_sampling(self._h, *[_ptr(t) for t in b], _stream()), "vcas_last_sampling")
+        _check(lib().vcas_last_sampling(self._h, *_sampling_ptrs(b), _stream()), "vcas_last_sampling")
         return self._pack_sampling(b)
 
     def mask_from_probs(self, p, seed: int, sampler_id: int):
@@ -228,7 +267,7 @@ class Layer:
         keep = torch.empty(n, dtype=torch.uint8, device=p.device)
         idx = torch.empty(n, dtype=torch.int32, device=p.device)
         cnt = torch.zeros(1, dtype=torch.int32, device=p.device)
-        _check(lib().vcas_mask_from_probs(self._h, _ptr(p), C.c_int32(n), C.c_uint64(seed), C.c_int32(sampler_id),
+        _check(lib().vcas_mask_from_probs(self._h, _ptr(p), n, seed, sampler_id,
                                           _ptr(keep), _ptr(idx), _ptr(cnt), _stream()), "vcas_mask_from_probs")
         c = int(cnt.item())
         return keep, idx[:c], c
@@ -242,8 +281,8 @@ class Layer:
         xa = (C.c_void_p * M)(*[x.data_ptr() for x in Xs])
         ya = (C.c_void_p * M)(*[y.data_ptr() for y in dYs])
         base, st = out.data_ptr(), 4
-        rc = lib().vcas_variance_probe(self._h, C.c_int32(M), xa, ya, _ptr(W), C.c_float(rho), C.c_float(nu),
-                                       C.c_float(s), C.c_uint64(seed), *[C.c_void_p(base + st * k) for k in range(5)],
+        rc = lib().vcas_variance_probe(self._h, M, xa, ya, _ptr(W), rho, nu,
+                                       s, seed, *[base + st * k for k in range(5)],
                                        _stream())
         _check(rc, "vcas_variance_probe")
         return out
@@ -257,9 +296,9 @@ class Layer:
     def set_tuning(self, dx_tile_n: int = 0, dw_tile_n: int = 0, dx_split_k: int = 0, dw_split_k: int = 0,
                    tile_m: int = 0, dw_tile_m: int | None = None) -> None:
         """tile_m: tile height of the dX product, and of the dW product too unless dw_tile_m is given."""
-        _check(lib().vcas_set_tuning(self._h, C.c_int32(dx_tile_n), C.c_int32(dw_tile_n), C.c_int32(dx_split_k),
-                                     C.c_int32(dw_split_k), C.c_int32(tile_m),
-                                     C.c_int32(tile_m if dw_tile_m is None else dw_tile_m)), "vcas_set_tuning")
+        _check(lib().vcas_set_tuning(self._h, dx_tile_n, dw_tile_n, dx_split_k,
+                                     dw_split_k, tile_m,
+                                     tile_m if dw_tile_m is None else dw_tile_m), "vcas_set_tuning")
 
     def last_plan(self):
         """((width, slices, height code) of the dX product, the same of the dW product) of the last call."""
@@ -268,7 +307,7 @@ class Layer:
         return tuple(a[0:3]), tuple(a[3:6])
 
     def set_probe_subsample(self, rows: int, seed: int = 0) -> None:
-        _check(lib().vcas_set_probe_subsample(self._h, C.c_int32(rows), C.c_uint64(seed)), "vcas_set_probe_subsample")
+        _check(lib().vcas_set_probe_subsample(self._h, rows, seed), "vcas_set_probe_subsample")
 
     def probe_subsample(self):
         """The rows of the parameter gradient the probe samples (host list; empty when it uses all rows)."""
@@ -279,11 +318,11 @@ class Layer:
         return list(rows)[:n.value]
 
     def set_wait_limit(self, limit_ns: int, stall_once: bool = False) -> None:
-        _check(lib().vcas_set_wait_limit(self._h, C.c_uint64(limit_ns), C.c_int32(1 if stall_once else 0)),
+        _check(lib().vcas_set_wait_limit(self._h, limit_ns, 1 if stall_once else 0),
                "vcas_set_wait_limit")
 
     def set_profiling(self, enable: bool) -> None:
-        _check(lib().vcas_set_profiling(self._h, C.c_int32(1 if enable else 0)), "vcas_set_profiling")
+        _check(lib().vcas_set_profiling(self._h, 1 if enable else 0), "vcas_set_profiling")
 
     def stage_times(self):
         """(ms[8], calls[2]) summed over the calls recorded since profiling was enabled or last read."""
@@ -309,7 +348,7 @@ def update_ratios(s: float, rho, nu, V_s, V_act, V_w, p_lo, p_hi, config: Config
     arr = lambda v: (C.c_float * L)(*[float(x) for x in v])
     rho_a, nu_a = arr(rho), arr(nu)
     st = State(float(s), int(t), L, C.cast(rho_a, C.POINTER(C.c_float)), C.cast(nu_a, C.POINTER(C.c_float)))
-    rc = lib().vcas_update_ratios(C.byref(st), C.c_int32(L), arr(V_s), arr(V_act), arr(V_w), arr(p_lo), arr(p_hi),
+    rc = lib().vcas_update_ratios(C.byref(st), L, arr(V_s), arr(V_act), arr(V_w), arr(p_lo), arr(p_hi),
                                   C.byref(config))
     _check(rc, "vcas_update_ratios")
     return st.s, list(rho_a), list(nu_a)
@@ -319,15 +358,11 @@ def score_static(X, dY, N: int, T: int, rho: float, nu: float, seed: int) -> Sam
     """vcas_score_static: scores, probabilities and index lists without a handle or any device
     allocation by the library (the output tensors below are the caller's, made by torch).
     Limits: N <= 4096, N*T <= 16384.  Calls sharing a device must not overlap on the GPU."""
-    R, dev = N * T, X.device
-    f = dict(dtype=torch.float32, device=dev)
-    i = dict(dtype=torch.int32, device=dev)
-    b = (torch.empty(N, **f), torch.empty(N, **f), torch.empty(R, **f), torch.empty(R, **f),
-         torch.empty(N, **i), torch.zeros(1, **i), torch.empty(R, **i), torch.zeros(1, **i))
+    b = _sampling_buffers(N, N * T, X.device)
     dt = {torch.float32: DTYPE_F32, torch.bfloat16: DTYPE_BF16}[X.dtype]
-    rc = lib().vcas_score_static(C.c_int32(N), C.c_int32(T), C.c_int32(X.shape[1]), C.c_int32(dY.shape[1]),
-                                 C.c_int32(dt), _ptr(X), _ptr(dY), C.c_float(rho), C.c_float(nu), C.c_uint64(seed),
-                                 *[_ptr(t) for t in b], _stream())
+    rc = lib().vcas_score_static(N, T, X.shape[1], dY.shape[1],
+                                 dt, _ptr(X), _ptr(dY), rho, nu, seed,
+                                 *_sampling_ptrs(b), _stream())
     _check(rc, "vcas_score_static")
     return Layer._pack_sampling(b)
 

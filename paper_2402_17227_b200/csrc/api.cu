@@ -111,19 +111,10 @@ size_t layout(Handle* h, uint8_t* base) {
   return (size_t)(cur - base);
 }
 
+// programmatic: behind the kernel before it in `st`
 int copy_out(Handle* h, float* g, float* p, float* w, float* q, int32_t* idxA, int32_t* cntA, int32_t* idxW,
-             int32_t* cntW, cudaStream_t st) {
-  const size_t N = h->desc.N, R = (size_t)h->desc.N * h->desc.T;
-  const Workspace& ws = h->ws;
-  const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-  if (g) VCAS_CUDA(cudaMemcpyAsync(g, ws.g, N * sizeof(float), k, st));
-  if (p) VCAS_CUDA(cudaMemcpyAsync(p, ws.p, N * sizeof(float), k, st));
-  if (w) VCAS_CUDA(cudaMemcpyAsync(w, ws.w, R * sizeof(float), k, st));
-  if (q) VCAS_CUDA(cudaMemcpyAsync(q, ws.q, R * sizeof(float), k, st));
-  if (idxA) VCAS_CUDA(cudaMemcpyAsync(idxA, ws.idxA, N * sizeof(int32_t), k, st));
-  if (cntA) VCAS_CUDA(cudaMemcpyAsync(cntA, ws.counts + 0, sizeof(int32_t), k, st));
-  if (idxW) VCAS_CUDA(cudaMemcpyAsync(idxW, ws.idxW, R * sizeof(int32_t), k, st));
-  if (cntW) VCAS_CUDA(cudaMemcpyAsync(cntW, ws.counts + 1, sizeof(int32_t), k, st));
+             int32_t* cntW, bool programmatic, cudaStream_t st) {
+  VCAS_CUDA(launch_copy_out(h, g, p, w, q, idxA, cntA, idxW, cntW, programmatic, st));
   return VCAS_OK;
 }
 
@@ -244,14 +235,15 @@ int vcas_create(vcas_handle* out, const vcas_layer_desc* desc, const vcas_config
   h->sub_k = 0;
   h->join_pending = false;
   h->stall_once = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&h->device) != cudaSuccess || cudaGetDeviceProperties(&prop, h->device) != cudaSuccess) {
+  int major = 0;
+  if (cudaGetDevice(&h->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, h->device) != cudaSuccess) {
     delete h;
     return VCAS_ERR_CUDA;
   }
-  h->num_sms = prop.multiProcessorCount;
   h->max_units = h->split_path ? split_max_units(*desc, h->num_sms) : 2 * h->num_sms;
-  if ((h->tensor_path || h->split_path) && prop.major != 10) { delete h; return VCAS_ERR_CUDA; }
+  if ((h->tensor_path || h->split_path) && major != 10) { delete h; return VCAS_ERR_CUDA; }
   h->bytes = layout(h, nullptr);
   if (cudaMalloc(&h->base, h->bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -498,14 +490,14 @@ int vcas_score(vcas_handle hh, const void* X, const void* dY, float rho, float n
   VCAS_CUDA(launch_scores_x(h, X, a, true, st));
   VCAS_CUDA(launch_sample_w(h, a, st));
   VCAS_CUDA(launch_emit_pack(h, dY, X, a, false, st));
-  return copy_out(h, g, p, w, q, idxA, cntA, idxW, cntW, st);
+  return copy_out(h, g, p, w, q, idxA, cntA, idxW, cntW, true, st);
 }
 
 int vcas_last_sampling(vcas_handle hh, float* g, float* p, float* w, float* q, int32_t* idxA, int32_t* cntA,
                        int32_t* idxW, int32_t* cntW, vcas_stream stream) {
   if (hh == nullptr) return VCAS_ERR_BAD_ARG;
   if (join_pending(H(hh), S(stream)) != VCAS_OK) return VCAS_ERR_CUDA;
-  return copy_out(H(hh), g, p, w, q, idxA, cntA, idxW, cntW, S(stream));
+  return copy_out(H(hh), g, p, w, q, idxA, cntA, idxW, cntW, false, S(stream));
 }
 
 int vcas_mask_from_probs(vcas_handle hh, const float* p, int32_t n, uint64_t seed, int32_t sampler_id,

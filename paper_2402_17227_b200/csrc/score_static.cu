@@ -92,18 +92,6 @@ extern "C" int vcas_score_static(int32_t N, int32_t T, int32_t d_in, int32_t d_o
   if (launch_sample_w(&h, a, st) != cudaSuccess) return VCAS_ERR_CUDA;
   if (launch_emit_pack(&h, dY, X, a, false, st) != cudaSuccess) return VCAS_ERR_CUDA;
 
-  const size_t R = (size_t)N * T;
-  const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-#define COPY_OUT(dst, src, bytes) \
-  if ((dst) != nullptr && cudaMemcpyAsync((dst), (src), (bytes), k, st) != cudaSuccess) return VCAS_ERR_CUDA
-  COPY_OUT(g, ws.g, N * sizeof(float));
-  COPY_OUT(p, ws.p, N * sizeof(float));
-  COPY_OUT(w, ws.w, R * sizeof(float));
-  COPY_OUT(q, ws.q, R * sizeof(float));
-  COPY_OUT(idxA, ws.idxA, N * sizeof(int32_t));
-  COPY_OUT(cntA, ws.counts + 0, sizeof(int32_t));
-  COPY_OUT(idxW, ws.idxW, R * sizeof(int32_t));
-  COPY_OUT(cntW, ws.counts + 1, sizeof(int32_t));
-#undef COPY_OUT
+  if (launch_copy_out(&h, g, p, w, q, idxA, cntA, idxW, cntW, true, st) != cudaSuccess) return VCAS_ERR_CUDA;
   return VCAS_OK;
 }
