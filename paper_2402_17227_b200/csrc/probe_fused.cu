@@ -11,7 +11,7 @@
 //
 // Four launches serve up to four batches: norms of the rows of dY and X (which also gathers the sampled columns of dY), one
 // CTA per draw for p, mask and c, one CTA per draw for Eq. 3 (beside the product, on the side stream), the product.
-// Measured on B200: 4096 rows, 768 -> 3072, M = 4: 664 -> 223 us; 16384 rows, 4096 -> 128 of 11008, M = 2: 521 -> 317 us.
+// Measured on B200: 4096 rows, 768 -> 3072, M = 4: 664 -> 219 us; 16384 rows, 4096 -> 128 of 11008, M = 2: 521 -> 254 us.
 #include <atomic>
 
 #include "rows.cuh"
@@ -43,10 +43,42 @@ struct ProbeGroup {
 };
 
 // ------------------------------------------------------------------------------------- row norms
-// One warp per row, HBM-bound: of every batch first the R rows of dY, then those of X.  With cols the k sampled columns of
-// every row of dY are copied out while the row is in the caches.
-__global__ void __launch_bounds__(256) probe_norms_kernel(ProbeGroup G, int batches, int R, int d_out, int d_in,
-                                                          const int32_t* __restrict__ cols, int k) {
+// Sum of squares of a row by one warp, and its k elements at the ascending columns `cols` copied to dst.  The columns are
+// picked after every 4 KB, from L1: with 48 rows in flight an SM has a megabyte of rows open, so that a pass over the row when
+// it ends finds its start neither in L1 nor surely in L2 (16384 rows of 11008 twice, 128 columns, with the rows of X:
+// 198 -> 155 us, 6.4 TB/s, which also took the operands' addresses out of local memory).
+__device__ __forceinline__ float row_partial_pick(const __nv_bfloat16* __restrict__ row, int d, int lane,
+                                                  const int32_t* __restrict__ cols, int k, __nv_bfloat16* __restrict__ dst) {
+  const uint4* v = reinterpret_cast<const uint4*>(row);
+  const int nv = d / 8;                              // d is a multiple of 64
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int v0 = 0, q = 0; v0 < nv; v0 += 256) {
+    uint4 x[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int i = v0 + lane + 32 * e;
+      x[e] = i < nv ? __ldg(v + i) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e % 4] += sq8(x[e]);
+    const int end = min((v0 + 256) * 8, d);
+    for (;;) {
+      const int col = q + lane < k ? __ldg(cols + q + lane) : INT32_MAX;
+      const bool in = col < end;
+      if (in) reinterpret_cast<unsigned short*>(dst)[q + lane] = __ldg(reinterpret_cast<const unsigned short*>(row) + col);
+      const int n = __popc(__ballot_sync(0xffffffffu, in));
+      q += n;
+      if (n < 32) break;
+    }
+  }
+  return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+
+// One warp per row, HBM-bound: of every batch first the R rows of dY, then those of X.  PICK: the k sampled columns of every
+// row of dY are copied out on the way.
+template <bool PICK>
+__global__ void __launch_bounds__(256) probe_norms_kernel(const __grid_constant__ ProbeGroup G, int batches, int R, int d_out,
+                                                          int d_in, const int32_t* __restrict__ cols, int k) {
   pdl_trigger();
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < 2 * R * batches; i += gridDim.x * wpb) {
@@ -54,14 +86,9 @@ __global__ void __launch_bounds__(256) probe_norms_kernel(ProbeGroup G, int batc
     const bool y = c < R;
     const int r = y ? c : c - R, d = y ? d_out : d_in;
     const __nv_bfloat16* row = (y ? G.dY[g] : G.X[g]) + (size_t)r * d;
-    const float s = warp_sum(row_partial<__nv_bfloat16>(row, d, lane));
+    const float s = warp_sum(PICK && y ? row_partial_pick(row, d, lane, cols, k, G.sub + ((size_t)g * R + r) * k)
+                                       : row_partial<__nv_bfloat16>(row, d, lane));
     if (lane == 0) (y ? G.a : G.b)[(size_t)g * R + r] = s;
-    if (y && cols != nullptr)
-      for (int q = lane * 2; q < k; q += 64) {
-        const uint32_t lo = __ldg(reinterpret_cast<const unsigned short*>(row) + cols[q]);
-        const uint32_t hi = __ldg(reinterpret_cast<const unsigned short*>(row) + cols[q + 1]);
-        *reinterpret_cast<uint32_t*>(G.sub + ((size_t)g * R + r) * k + q) = lo | (hi << 16);
-      }
   }
 }
 
@@ -432,9 +459,11 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
     }
   }
   __syncwarp();
-  pdl_trigger();
   tc_fence_before();
   __syncthreads();
+  // Not before all warps are here: the first thread to say so speaks for the CTA, and the CTAs of the kernel that adds slices
+  // would wait on the SMs left to Eq. 3, whose CTAs need all of an SM's registers (20 us at the end of a probe).
+  pdl_trigger();
   if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem_base, PBUFS * PBN); }
 }
 
@@ -616,7 +645,8 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
     if (i0 > 0) PROBE_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));       // Eq. 3 of the group before reads its scratch
     long blocks = (2l * R * batches + 7) / 8;
     if (blocks > (1l << 20)) blocks = 1l << 20;
-    probe_norms_kernel<<<(unsigned)blocks, 256, 0, st>>>(G, batches, R, d.d_out, d.d_in, sub > 0 ? h->sub_rows : nullptr, sub);
+    if (sub > 0) probe_norms_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(G, batches, R, d.d_out, d.d_in, h->sub_rows, sub);
+    else probe_norms_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(G, batches, R, d.d_out, d.d_in, nullptr, 0);
     PROBE_CUDA(cudaGetLastError());
     Q.first_batch = i0;
     const dim3 draw_grid((unsigned)(PD * passes + 1), (unsigned)batches);

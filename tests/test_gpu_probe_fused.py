@@ -56,3 +56,20 @@ def test_fused_probe_matches_oracle(N, T, d_in, d_out, M, rows):
     assert np.array_equal(got.cpu().numpy(), out)
     del g
     layer.close()
+
+
+@pytest.mark.parametrize("d_out,rows", [(2048, 64), (2112, 256), (4160, 192), (6208, 64)])
+def test_sampled_columns_over_several_chunks_of_a_row(d_out, rows):
+    """The columns are picked 2048 at a time, 32 per step: one to eight steps in a chunk, a last chunk of 64."""
+    vbuild.build()
+    N, T, d_in, M = 3, 64, 64, 2
+    case = inputs.LayerCase("pc", N, T, d_in, d_out, torch.bfloat16, 1.0, 0.5, 0.5, 0.5)
+    batches = [inputs.make_layer(case, batch=i) for i in range(M)]
+    layer = vb.Layer(N, T, d_in, d_out, torch.bfloat16, vb.GEMM_TENSOR)
+    layer.set_probe_subsample(rows, 3)
+    out = layer.variance_probe([b[0].cuda() for b in batches], [b[1].cuda() for b in batches], batches[0][2].cuda(), 0.4, 0.5,
+                               0.75, 42).cpu().numpy()
+    ref = o.variance_probe([np64(b[0]) for b in batches], [np64(b[1]) for b in batches], np64(batches[0][2]), N, T, f32(0.4), 0.5,
+                           s=0.75, alpha=0.05, seed=42, param_rows=layer.probe_subsample())
+    assert out[:3] == pytest.approx([ref["V_s"], ref["V_act"], ref["V_w"]], rel=1e-4)
+    layer.close()
