@@ -11,7 +11,7 @@
 //
 // Four launches serve up to four batches: norms of the rows of dY and X (which also gathers the sampled columns of dY), one
 // CTA per draw for p, mask and c, one CTA per draw for Eq. 3 (beside the product, on the side stream), the product.
-// Measured on B200: 4096 rows, 768 -> 3072, M = 4: 664 -> 219 us; 16384 rows, 4096 -> 128 of 11008, M = 2: 521 -> 254 us.
+// Measured on B200: 4096 rows, 768 -> 3072, M = 4: 664 -> 203 us; 16384 rows, 4096 -> 128 of 11008, M = 2: 521 -> 241 us.
 #include <atomic>
 
 #include "rows.cuh"
@@ -209,9 +209,9 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) probe_vw_kernel(DrawParams P)
 struct ProbeMaps { CUtensorMap a[PG], b[PG]; };      // per batch: dY (or its sampled columns) and X
 struct ProbeParams {
   const float4* c;                 // [batch][pass][N] of PD draws
-  float* mean; float* m2;          // [d_out, d_in] running mean and squared deviation of G_s
+  float* mean; float* m2;          // d_out x d_in, by tiles: running mean and squared deviation of G_s
   double* pact; double* ps;        // [tiles] sum of squares of the differences so far; sum of m2 (last batch)
-  float* partial;                  // [batch][unit][1 + D][128][64] when a tile's data are cut into slices
+  float* partial;                  // [batch][unit][1 + D][128 x 64] when a tile's data are cut into slices
   int N, T, d_in, d_out, kT, steps, S, per, ntiles, units;    // kT: steps of a datum
   int first_batch, batches, M;
   int pass, passes;                // the draws of this pass are pass * PD ...
@@ -229,15 +229,22 @@ __device__ __forceinline__ float welford(float x, int i, int M, float& mean, flo
   m2 = fmaf(d, x - mean, m2);
   return i == M - 1 ? m2 : 0.f;
 }
-// W consecutive elements at o: G_s of batch i into the running moments, all loads before the first store.  m2 of the first
-// batch is 0 and not stored, neither is anything of the last.
+// Where a tile's columns 4 q .. 4 q + 3 of `row` are in a scratch tile of `rows` rows.  The threads of a warp have consecutive
+// rows, so they take 512 consecutive bytes: in rows of 64 columns an instruction met 32 cache lines, and the moments of a tile
+// and batch took 4 us in which the products could run eight data ahead at most (189 -> 176 us for 768 -> 3072, M = 4).
+__device__ __forceinline__ size_t scratch_at(int q, int rows, int row) { return ((size_t)q * rows + row) * 4; }
+// G_s of batch i at W columns from 4 q0 on into the running moments, all loads before the first store.  m2 of the first batch
+// is 0 and not stored, neither is anything of the last.  The moments of a tile have its rows below d_out.
 template <int W>
-__device__ __forceinline__ float welford_row(const ProbeParams& P, int i, size_t o, const float (&x)[W]) {
+__device__ __forceinline__ float welford_row(const ProbeParams& P, int i, int tile, int row, int q0, const float (&x)[W]) {
   float4 mean[W / 4], m2[W / 4];
+  const int r0 = tile / P.ntiles * BM, rows = min(BM, P.d_out - r0);
+  const size_t o = (size_t)r0 * P.d_in + (size_t)(tile % P.ntiles) * rows * PBN + scratch_at(q0, rows, row);
+  const size_t step = (size_t)rows * 4;
 #pragma unroll
   for (int e = 0; e < W / 4; ++e) {
-    mean[e] = i > 0 ? *reinterpret_cast<const float4*>(P.mean + o + 4 * e) : make_float4(0.f, 0.f, 0.f, 0.f);
-    m2[e] = i > 1 ? *reinterpret_cast<const float4*>(P.m2 + o + 4 * e) : make_float4(0.f, 0.f, 0.f, 0.f);
+    mean[e] = i > 0 ? *reinterpret_cast<const float4*>(P.mean + o + e * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+    m2[e] = i > 1 ? *reinterpret_cast<const float4*>(P.m2 + o + e * step) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   float r = 0.f;
 #pragma unroll
@@ -245,8 +252,8 @@ __device__ __forceinline__ float welford_row(const ProbeParams& P, int i, size_t
     r += (welford(x[4 * e], i, P.M, mean[e].x, m2[e].x) + welford(x[4 * e + 1], i, P.M, mean[e].y, m2[e].y)) +
          (welford(x[4 * e + 2], i, P.M, mean[e].z, m2[e].z) + welford(x[4 * e + 3], i, P.M, mean[e].w, m2[e].w));
     if (i < P.M - 1) {
-      *reinterpret_cast<float4*>(P.mean + o + 4 * e) = mean[e];
-      if (i > 0) *reinterpret_cast<float4*>(P.m2 + o + 4 * e) = m2[e];
+      *reinterpret_cast<float4*>(P.mean + o + e * step) = mean[e];
+      if (i > 0) *reinterpret_cast<float4*>(P.m2 + o + e * step) = m2[e];
     }
   }
   return r;
@@ -434,14 +441,14 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
 #pragma unroll
           for (int j = 0; j < D; ++j) unpack2(df2[j][e], df[j][2 * e], df[j][2 * e + 1]);
         }
-        float* part = P.partial + (((size_t)g * P.units + u) * (1 + D) * BM + row) * PBN + eg * CW;
+        float* part = P.partial + ((size_t)g * P.units + u) * (1 + D) * BM * PBN + scratch_at(eg * (CW / 4), BM, row);
         if (P.S > 1) {
 #pragma unroll
           for (int e = 0; e < CW; e += 4) {
-            if (EXACT) *reinterpret_cast<float4*>(part + e) = make_float4(gs[e], gs[e + 1], gs[e + 2], gs[e + 3]);
+            if (EXACT) *reinterpret_cast<float4*>(part + scratch_at(e / 4, BM, 0)) = make_float4(gs[e], gs[e + 1], gs[e + 2], gs[e + 3]);
 #pragma unroll
             for (int j = 0; j < D; ++j)
-              *reinterpret_cast<float4*>(part + (size_t)(1 + j) * BM * PBN + e) = make_float4(df[j][e], df[j][e + 1], df[j][e + 2], df[j][e + 3]);
+              *reinterpret_cast<float4*>(part + (size_t)(1 + j) * BM * PBN + scratch_at(e / 4, BM, 0)) = make_float4(df[j][e], df[j][e + 1], df[j][e + 2], df[j][e + 3]);
           }
         } else if (r0 < P.d_out) {
 #pragma unroll
@@ -451,7 +458,7 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
             for (int e = 0; e < CW; ++e) t = fmaf(df[j][e], df[j][e], t);
             act += (double)t;
           }
-          if (EXACT) sq += (double)welford_row<CW>(P, P.first_batch + g, (size_t)r0 * P.d_in + tile % P.ntiles * PBN + eg * CW, gs);
+          if (EXACT) sq += (double)welford_row<CW>(P, P.first_batch + g, tile, row, eg * (CW / 4), gs);
         }
       }
       if (!ok) break;
@@ -478,14 +485,13 @@ __global__ void __launch_bounds__(ADD_THREADS) probe_add_kernel(ProbeParams P) {
   const int tile = blockIdx.x / ADD_PARTS, rows = BM / ADD_PARTS, first = blockIdx.x % ADD_PARTS * rows;
   double act = 0.0, sq = 0.0;
   for (int i = threadIdx.x; i < rows * BN / 4; i += ADD_THREADS) {
-    const int row = first + i / (BN / 4), c4 = i % (BN / 4) * 4;
-    const int r0 = tile / P.ntiles * BM + row, col = tile % P.ntiles * BN + c4;
-    if (r0 >= P.d_out || col >= P.d_in) continue;
+    const int row = first + i % rows, q0 = i / rows;
+    if (tile / P.ntiles * BM + row >= P.d_out) continue;
     for (int g = 0; g < P.batches; ++g) {
       float x[1 + D][4] = {};
 #pragma unroll 4
       for (int s = 0; s < P.S; ++s) {
-        const float* part = P.partial + (((size_t)g * P.units + tile * P.S + s) * (1 + D) * BM + row) * BN + c4;
+        const float* part = P.partial + ((size_t)g * P.units + tile * P.S + s) * (1 + D) * BM * BN + scratch_at(q0, BM, row);
 #pragma unroll
         for (int q = EXACT ? 0 : 1; q <= D; ++q) {
           const float4 v = __ldcg(reinterpret_cast<const float4*>(part + (size_t)q * BM * BN));
@@ -494,7 +500,7 @@ __global__ void __launch_bounds__(ADD_THREADS) probe_add_kernel(ProbeParams P) {
       }
 #pragma unroll
       for (int q = 1; q <= D; ++q) act += (double)((x[q][0] * x[q][0] + x[q][1] * x[q][1]) + (x[q][2] * x[q][2] + x[q][3] * x[q][3]));
-      if (EXACT) sq += (double)welford_row<4>(P, P.first_batch + g, (size_t)r0 * P.d_in + col, x[0]);
+      if (EXACT) sq += (double)welford_row<4>(P, P.first_batch + g, tile, row, q0, x[0]);
     }
   }
   tile_sums<ADD_THREADS>(P, EXACT, blockIdx.x, act, sq, s_sum);
