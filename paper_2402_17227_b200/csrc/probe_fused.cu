@@ -2,16 +2,17 @@
 //
 // The gradient of a batch is a sum over its data, G_s = sum_n D_n with D_n = dY_n^T X_n, and a draw of SampleA only
 // weights the terms: G_act,j = sum_n (keep_jn / p_jn) D_n.  The product kernel therefore forms every D_n once, in a
-// fresh TMEM accumulator, and the epilogue warps add it to G_s and, weighted with c_jn = keep_jn / p_jn - 1, to the
-// differences G_act,j - G_s of up to four draws in fp32 registers; V_act needs nothing but the squares of these, and G_s
-// goes straight into the running mean and squared deviation of V_s.  (Running sums in TMEM with summation by parts save the
+// fresh TMEM accumulator, and the epilogue warps add it to G_s and, weighted with w_jn = keep_jn / p_jn where that is not 0, to
+// G_act,j of up to four draws in fp32 registers; V_act needs nothing but the squares of G_act,j - G_s, and G_s goes straight
+// into the running mean and squared deviation of V_s.  (Draws past the first four, whose pass does not form G_s, add up the
+// differences with keep_jn / p_jn - 1.)  (Running sums in TMEM with summation by parts save the
 // registers of G_s, but lose the small data, whose weights 1 / p are large, in the rounding of the large ones.)
 // No draw packs rows or has a product of its own:
 // M batches of M draws cost M products instead of M + rho M^2, and the results carry no rounding of rescaled rows.
 //
 // Four launches serve up to four batches: norms of the rows of dY and X (which also gathers the sampled columns of dY), one
-// CTA per draw for p, mask and c, one CTA per draw for Eq. 3 (beside the product, on the side stream), the product.
-// Measured on B200: 4096 rows, 768 -> 3072, M = 4: 664 -> 203 us; 16384 rows, 4096 -> 128 of 11008, M = 2: 521 -> 241 us.
+// CTA per draw for p, mask and w, one CTA per draw for Eq. 3 (beside the product, on the side stream), the product.
+// Measured on B200: 4096 rows, 768 -> 3072, M = 4: 664 -> 179 us; 16384 rows, 4096 -> 128 of 11008, M = 2: 521 -> 241 us.
 #include <atomic>
 
 #include "rows.cuh"
@@ -38,7 +39,7 @@ struct ProbeGroup {
   const __nv_bfloat16* dY[PG]; const __nv_bfloat16* X[PG];
   float* a; float* b;              // [batch][R] row square-norms of dY and X
   float* p;                        // [batch][M][N] keep probabilities
-  float* c;                        // [batch][pass][N][PD] keep / p - 1 (0 past the last draw)
+  float* w;                        // [batch][pass][N][PD] keep / p (1 past the last draw)
   __nv_bfloat16* sub;              // [batch][R][k] sampled columns of dY
 };
 
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(256) probe_norms_kernel(const __grid_constant_
 // ------------------------------------------------------------------------------------ the draws
 struct DrawParams {
   const float* a; const float* b;  // [batch][R]
-  float* p; float* c;              // as in ProbeGroup
+  float* p; float* w;              // as in ProbeGroup
   double* sparsity;                // [2][batch of the probe] p_lo, p_hi
   double* vw;                      // [batch of the probe][M] Eq. 3
   int32_t* status;
@@ -105,8 +106,8 @@ struct DrawParams {
   uint64_t seed;
 };
 
-// Where c of (batch g, draw j, datum n) is.
-__device__ __forceinline__ size_t c_index(const DrawParams& P, int g, int j, int n) {
+// Where w of (batch g, draw j, datum n) is.
+__device__ __forceinline__ size_t w_index(const DrawParams& P, int g, int j, int n) {
   return (((size_t)g * P.passes + j / PD) * P.N + n) * PD + j % PD;
 }
 
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(DRAW_THREADS) probe_draw_kernel(DrawParams P) 
   pdl_wait();
   pdl_trigger();
   if (j >= P.M && j < PD * P.passes) {
-    for (int n = threadIdx.x; n < P.N; n += DRAW_THREADS) P.c[c_index(P, g, j, n)] = 0.f;
+    for (int n = threadIdx.x; n < P.N; n += DRAW_THREADS) P.w[w_index(P, g, j, n)] = 1.f;
     return;
   }
   __syncthreads();
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(DRAW_THREADS) probe_draw_kernel(DrawParams P) 
       const int n = lane + 32 * i;
       if (n < P.N) {
         P.p[o + n] = v[i];
-        P.c[c_index(P, g, j, n)] = bernoulli_keep(v[i], seed, 0u, (uint64_t)n) ? 1.0f / v[i] - 1.0f : -1.0f;
+        P.w[w_index(P, g, j, n)] = bernoulli_keep(v[i], seed, 0u, (uint64_t)n) ? 1.0f / v[i] : 0.f;
       }
     }
     return;
@@ -183,11 +184,11 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) probe_vw_kernel(DrawParams P)
   const float* b = P.b + (size_t)g * n;
   for (int i = tid; i < n; i += SAMPLER_THREADS) {
     const int d = i / P.T;
-    s_w[i] = P.c[c_index(P, g, j, d)] >= 0.f ? sqrtf(a[i]) * sqrtf(b[i]) / P.p[o + d] : 0.f;
+    s_w[i] = P.w[w_index(P, g, j, d)] > 0.f ? sqrtf(a[i]) * sqrtf(b[i]) / P.p[o + d] : 0.f;
   }
   float dummy = 0.f;
   int kept = 0;
-  for (int i = tid; i < P.N; i += SAMPLER_THREADS) kept += P.c[c_index(P, g, j, i)] >= 0.f ? 1 : 0;
+  for (int i = tid; i < P.N; i += SAMPLER_THREADS) kept += P.w[w_index(P, g, j, i)] > 0.f ? 1 : 0;
   fast_sum(dummy, kept, &sh, 1);
   __syncthreads();
   int mode;
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) probe_vw_kernel(DrawParams P)
 // ----------------------------------------------------------------------------------- the product
 struct ProbeMaps { CUtensorMap a[PG], b[PG]; };      // per batch: dY (or its sampled columns) and X
 struct ProbeParams {
-  const float4* c;                 // [batch][pass][N] of PD draws
+  const float4* w;                 // [batch][pass][N] of PD draws
   float* mean; float* m2;          // d_out x d_in, by tiles: running mean and squared deviation of G_s
   double* pact; double* ps;        // [tiles] sum of squares of the differences so far; sum of m2 (last batch)
   float* partial;                  // [batch][unit][1 + D][128 x 64] when a tile's data are cut into slices
@@ -408,11 +409,11 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
 #pragma unroll
           for (int j = 0; j < D; ++j) df2[j][e] = 0ull;
         }
-        const float4* cg = P.c + ((size_t)g * P.passes + P.pass) * P.N;
-        float4 next = __ldg(cg + n0);
+        const float4* wg = P.w + ((size_t)g * P.passes + P.pass) * P.N;
+        float4 next = __ldg(wg + n0);
         for (int n = n0; n < n1; ++n) {
-          const float c[4] = {next.x, next.y, next.z, next.w};
-          next = __ldg(cg + min(n + 1, n1 - 1));   // on its way while this datum is added
+          const float w[4] = {next.x, next.y, next.z, next.w};
+          next = __ldg(wg + min(n + 1, n1 - 1));   // on its way while this datum is added
           // The lanes of a warp leave together.  No call here: it would put the sums held in registers into local memory.
           ok = __all_sync(0xffffffffu, mbar_wait_spin(&acc_full[buf], buf_phase, abort_flag, P.status));
           if (!ok) break;
@@ -420,12 +421,21 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
           static_assert(CW == 32, "one load");
           uint32_t v[CW];
           tmem_ld32(tmem_base + tlane + buf * (uint32_t)PBN, v);
+          uint64_t x[CW / 2];
 #pragma unroll
-          for (int e = 0; e < CW / 2; ++e) {
-            const uint64_t x = pack2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
-            if (EXACT) gs2[e] = add2(gs2[e], x);
+          for (int e = 0; e < CW / 2; ++e) x[e] = pack2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+          // fp32-bound: 0.35 us a datum with an FMA per draw and element, of 0.62 in all; dropped data cost a draw nothing
+          if (EXACT) {
 #pragma unroll
-            for (int j = 0; j < D; ++j) df2[j][e] = fma2(pack2(c[j], c[j]), x, df2[j][e]);
+            for (int e = 0; e < CW / 2; ++e) gs2[e] = add2(gs2[e], x[e]);
+          }
+#pragma unroll
+          for (int j = 0; j < D; ++j) {
+            if (EXACT && !__any_sync(0xffffffffu, w[j] != 0.f)) continue;      // the same for the whole warp: no predicates
+            const float c = EXACT ? w[j] : w[j] - 1.0f;
+            const uint64_t cc = pack2(c, c);
+#pragma unroll
+            for (int e = 0; e < CW / 2; ++e) df2[j][e] = fma2(cc, x[e], df2[j][e]);
           }
           // one arrival per warp: the arrivals of all threads at one barrier are served one after the other
           tc_fence_before();
@@ -439,7 +449,10 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
         for (int e = 0; e < CW / 2; ++e) {
           unpack2(gs2[e], gs[2 * e], gs[2 * e + 1]);
 #pragma unroll
-          for (int j = 0; j < D; ++j) unpack2(df2[j][e], df[j][2 * e], df[j][2 * e + 1]);
+          for (int j = 0; j < D; ++j) {
+            unpack2(df2[j][e], df[j][2 * e], df[j][2 * e + 1]);
+            if (EXACT) { df[j][2 * e] -= gs[2 * e]; df[j][2 * e + 1] -= gs[2 * e + 1]; }
+          }
         }
         float* part = P.partial + ((size_t)g * P.units + u) * (1 + D) * BM * PBN + scratch_at(eg * (CW / 4), BM, row);
         if (P.S > 1) {
@@ -616,7 +629,7 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
   G.a = reinterpret_cast<float*>(take((size_t)most * R * sizeof(float)));
   G.b = reinterpret_cast<float*>(take((size_t)most * R * sizeof(float)));
   G.p = reinterpret_cast<float*>(take((size_t)most * M * d.N * sizeof(float)));
-  G.c = reinterpret_cast<float*>(take((size_t)most * passes * PD * d.N * sizeof(float)));
+  G.w = reinterpret_cast<float*>(take((size_t)most * passes * PD * d.N * sizeof(float)));
 
   ProbeParams P = {};
   P.N = d.N; P.T = d.T; P.d_in = d.d_in; P.d_out = d_out;
@@ -630,11 +643,11 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
   P.pact = reinterpret_cast<double*>(h->ws.Gact);                         // this probe keeps no gradient
   P.ps = P.pact + sums;
   P.partial = h->ws.partial_tiles;
-  P.M = M; P.c = reinterpret_cast<const float4*>(G.c); P.passes = passes;
+  P.M = M; P.w = reinterpret_cast<const float4*>(G.w); P.passes = passes;
   P.status = h->ws.status; P.wait_limit_ns = h->wait_limit_ns; P.stall_once = h->stall_once;
 
   DrawParams Q = {};
-  Q.a = G.a; Q.b = G.b; Q.p = G.p; Q.c = G.c;
+  Q.a = G.a; Q.b = G.b; Q.p = G.p; Q.w = G.w;
   Q.vw = h->ws.partial; Q.sparsity = h->ws.partial + M * M; Q.status = h->ws.status;
   Q.N = d.N; Q.T = d.T; Q.M = M; Q.passes = passes; Q.rho = rho; Q.nu = nu; Q.s_lo = s_lo; Q.s_hi = s_hi; Q.seed = seed;
 
