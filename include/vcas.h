@@ -53,7 +53,9 @@ typedef enum {
 typedef enum { VCAS_DTYPE_F32 = 0, VCAS_DTYPE_BF16 = 1 } vcas_dtype;
 
 /* Which kernels compute the two products.  AUTO picks the tensor-core (tcgen05) kernels for
- * bf16 layers whose d_in and d_out are multiples of 64, the fp32-FMA kernels otherwise. */
+ * bf16 layers whose d_in and d_out are multiples of 64; fp32 layers and other widths run on the tensor
+ * cores too, with operands cut into bf16 parts whose products are summed to fp32 precision.  FMA forces the
+ * fp32-FMA kernels. */
 typedef enum { VCAS_GEMM_AUTO = 0, VCAS_GEMM_FMA = 1, VCAS_GEMM_TENSOR = 2 } vcas_gemm_path;
 
 typedef struct {
@@ -133,7 +135,7 @@ int vcas_linear_bwd_ex(vcas_handle h, const void* X, const void* dY, const void*
  *   kept_out     [N] int32: ascending list of the data this call kept, kept_cnt_out [1] its length;
  *   skip_dropped_rows  non-zero: the rows of dX (and a_out) that belong to dropped data are left unwritten instead
  *                of being set to zero - for a consumer that takes kept_out as its alive_in and therefore never
- *                reads them (tensor-core path; the fp32 path always writes them);
+ *                reads them (bf16 tensor-core path; the others always write them);
  *   defer_join   non-zero: the call returns with its weight-gradient branch (SampleW, the kept-row operands, the
  *                dW product, which run on a stream of the handle's own) not yet joined to `stream`: dX, a_out and
  *                kept_out are ordered on `stream` as usual, but dW and the sampling record are complete only after
@@ -261,7 +263,8 @@ int vcas_variance_probe(vcas_handle h, int32_t M, const void* const* X_i, const 
  * random subset fixed here: row i gets the Philox word of counter (i, 0, 2, 0) under the key (seed low, seed
  * high), the `rows` smallest words win, ties by index - and scales V_s and V_act by d_out / rows (unbiased for
  * the sums over all rows); V_w (Eq. 3) and p_lo / p_hi need no gradient and are unchanged.  The probe's two
- * products then cost rows / d_out of their full size.  rows: a multiple of 64 (8 on the fp32-FMA path), at most
+ * products then cost rows / d_out of their full size.  rows: a multiple of 64 (8 for fp32 layers, widths that
+ * are not multiples of 64 and the fp32-FMA path), at most
  * 256 and below d_out; 0 switches the sample off (default).  Synchronous.
  */
 int vcas_set_probe_subsample(vcas_handle h, int32_t rows, uint64_t seed);
@@ -307,8 +310,8 @@ int vcas_set_tuning(vcas_handle h, int32_t dx_tile_n, int32_t dw_tile_n, int32_t
 
 /* The tilings the library chose for the two products of the handle's last sampled or dense call (the paper has
  * no counterpart): plan[0..2] = tile width, contraction slices, tile-height code (as in vcas_set_tuning) of the dX
- * product, plan[3..5] the same for the dW product (host out).  VCAS_ERR_BAD_ARG before the first call or on the
- * fp32-FMA path. */
+ * product, plan[3..5] the same for the dW product (host out).  VCAS_ERR_BAD_ARG before the first call, for fp32
+ * layers, widths that are not multiples of 64 and on the fp32-FMA path. */
 int vcas_last_plan(vcas_handle h, int32_t* plan);
 
 /* Stage timing for benchmarks (the paper has no counterpart; Sec. 6 only reports end-to-end
