@@ -99,6 +99,23 @@ __device__ __forceinline__ void finish8(const SplitParams& P, size_t row, float 
   store8(reinterpret_cast<T*>(P.out) + o, v);
 }
 
+// Four columns of an fp32 output row.
+template <int MODE>
+__device__ __forceinline__ void finish4(const SplitParams& P, int row, float sc, int col, float (&v)[4]) {
+  const size_t o = (size_t)row * P.d_in + col;
+  if (MODE == MODE_DX) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] *= sc;
+    if (P.H != nullptr) {
+      const float4 h = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(P.H) + o));
+      const float x[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] *= gelu_prime_erf(x[e]);
+    }
+  }
+  *reinterpret_cast<float4*>(reinterpret_cast<float*>(P.out) + o) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
 // Where columns 4 q .. 4 q + 3 of `row` are in a slice of a tile: eight rows of four columns fill a cache line.  The product's
 // warps (32 rows, the same columns) and the adding ones (8 rows x 32 columns) both work on whole lines; in rows of 256 columns
 // every store of the product met 32 (fp32 layer of 4096 rows, 768 -> 3072: 98 -> 88 us; bf16, 4950 rows, 776 -> 1000: 65 -> 58).
@@ -241,13 +258,15 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       }
       const int row = eq * 32 + lane, r0 = tile / W.ntiles * BM + row;
       const int col0 = tile % W.ntiles * BN + eg * CW;
-      if (!ok || r0 >= W.rows) continue;
+      constexpr bool EXCHANGE = sizeof(T) == 4;      // lanes of rows past the last take part
+      if (!ok || (!EXCHANGE && r0 >= W.rows)) continue;
       if (W.S > 1) {
+        if (EXCHANGE && r0 >= W.rows) continue;
         float* part = P.partial + (size_t)u * BM * BN + partial_at(row, eg * (CW / 4));
 #pragma unroll
         for (int e = 0; e < CW; e += 4)
           *reinterpret_cast<float4*>(part + partial_at(0, e / 4)) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
-      } else {
+      } else if constexpr (!EXCHANGE) {
         float sc = 1.0f;
         const size_t r = MODE == MODE_DX ? dx_row(P, r0, sc) : (size_t)r0;
 #pragma unroll
@@ -257,6 +276,40 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 #pragma unroll
           for (int i = 0; i < 8; ++i) v[i] = acc[e + i];
           finish8<T, MODE>(P, r, sc, col0 + e, v);
+        }
+      } else {
+        // Every eight lanes exchange their rows' pieces of four columns, so that they store 128 bytes of one row at a time (a
+        // row per lane met 32 cache lines a store: 4 x 64 rows, 256 -> 256, 35.4 -> 32.0 us).  Not in bf16 layers: rows
+        // half as long, and the exchange cost more than the lines (4950 rows, 776 -> 1000: 61 -> 67 us).
+        float sc = 1.0f;
+        int target = -1;
+        if (r0 < W.rows) target = MODE == MODE_DX ? (int)dx_row(P, r0, sc) : r0;
+#pragma unroll
+        for (int c = 0; c < CW; c += 32) {
+          if (col0 + c >= P.d_in) break;
+          float x[8][4];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) x[i / 4][i % 4] = acc[c + i];
+#pragma unroll
+          for (int bit = 1; bit < 8; bit *= 2) {
+            const bool up = (lane & bit) != 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              if (i & bit) continue;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float got = __shfl_xor_sync(0xffffffffu, up ? x[i][e] : x[i | bit][e], bit);
+                if (up) x[i][e] = got; else x[i | bit][e] = got;
+              }
+            }
+          }
+          const int col = col0 + c + (lane & 7) * 4;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int r = __shfl_sync(0xffffffffu, target, (lane & 24) + i);
+            const float f = __shfl_sync(0xffffffffu, sc, (lane & 24) + i);
+            if (r >= 0 && col < P.d_in) finish4<MODE>(P, r, f, col, x[i]);
+          }
         }
       }
     }
