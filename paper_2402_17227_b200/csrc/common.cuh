@@ -393,7 +393,7 @@ void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spar
 cudaError_t launch_layernorm_bwd(Handle* h, const void* X, const void* gamma, const void* dY, float eps, void* dX,
                                  float* a_out, bool skip_dropped, float* dgamma, float* dbeta, cudaStream_t st);
 
-// The whole probe of a tensor-path layer with one product per batch for the exact gradient and all draws (probe_fused.cu),
+// The whole probe of a tensor-path layer with one product launch for the exact gradients and all draws (probe_fused.cu),
 // and whether it applies.  d_out is that of the product: the sampled rows of the parameter gradient where they are set.
 bool probe_fused_ok(const Handle* h, int M);
 cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const void* const* dY, float rho, float nu, double s_lo,

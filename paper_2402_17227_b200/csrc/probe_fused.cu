@@ -1,46 +1,55 @@
-// The variance probe of a tensor-path layer (Alg. 1, App. D) with one product per batch.
+// The variance probe of a tensor-path layer (Alg. 1, App. D) with one product launch per group of batches.
 //
-// The gradient of a batch is a sum over its data, G_s = sum_n D_n with D_n = dY_n^T X_n, and a draw of SampleA only
-// weights the terms: G_act,j = sum_n (keep_jn / p_jn) D_n.  The product kernel therefore forms every D_n once, in a
-// fresh TMEM accumulator, and the epilogue warps add it to G_s and, weighted with w_jn = keep_jn / p_jn where that is not 0, to
-// G_act,j of up to four draws in fp32 registers; V_act needs nothing but the squares of G_act,j - G_s, and G_s goes straight
-// into the running mean and squared deviation of V_s.  (Draws past the first four, whose pass does not form G_s, add up the
-// differences with keep_jn / p_jn - 1.)  (Running sums in TMEM with summation by parts save the
-// registers of G_s, but lose the small data, whose weights 1 / p are large, in the rounding of the large ones.)
-// No draw packs rows or has a product of its own:
-// M batches of M draws cost M products instead of M + rho M^2, and the results carry no rounding of rescaled rows.
+// A unit of the product is a tile of the parameter gradient of one batch.  Its CTA forms G_s = dY^T X and beside it, from the
+// same loads of X, the gradients of the draws, G_act,j = sum over the data kept in draw j of bf16(dY_n / p_n)^T X_n, each in an
+// accumulator of its own, and adds up the squares of G_act,j - G_s: no G_act is ever written.  The rows are rescaled and
+// rounded as in the sampled backward, whose gradients V_act speaks about; p_n belongs to the batch and not to the draw, so
+// they are made once for all draws, and a draw is only the list of the data that it accumulates.
+// (G_act,j as a sum of the data's exact products weighted with 1 / p_n needs one product per batch, but its V_act was up to
+// 5e-4 off: the rounding moves all values of a datum by the same 1e-4, which does not average out.)
+// Measured on B200, against a chain of launches and a product per draw (probe.cu): 4096 rows, 768 -> 3072, M = 4: 709 -> 238 us;
+// 16384 rows, 4096 -> 128 of 11008, M = 2: 538 -> 276 us; 640 rows, 128 -> 128, M = 2, rho = 0.8: 145 -> 39 us.
 //
-// Four launches serve up to four batches: norms of the rows of dY and X (which also gathers the sampled columns of dY), one
-// CTA per draw for p, mask and w, one CTA per draw for Eq. 3 (beside the product, on the side stream), the product.
-// Measured on B200: 4096 rows, 768 -> 3072, M = 4: 664 -> 179 us; 16384 rows, 4096 -> 128 of 11008, M = 2: 521 -> 241 us.
+// Launches per group: norms of the rows of dY and X (which also gathers the sampled columns of dY), one CTA per draw for p
+// and mask, one CTA per draw for Eq. 3 (beside the product, on the side stream), the rescaled rows, the product, the moments
+// of G_s.
 #include <atomic>
 
 #include "rows.cuh"
+#include "split.cuh"
 #include "umma.cuh"
 #include "water.cuh"
 
 namespace vcas {
 namespace {
 
-constexpr int PD = 4;                        // most draws a product pass serves
+constexpr int PROBE_MIN_T = 64;              // shortest data served: one step of the contraction
 constexpr int PG = 4;                        // most batches a launch serves
-constexpr int PROBE_THREADS = 12 * 32;       // warps 0-7 accumulate, 8 loads, 9 issues, 10 and 11 fill the warpgroup
+constexpr int PROBE_THREADS = 10 * 32;       // warps 0-7 read the accumulators, 8 loads, 9 issues
 constexpr int ACC_THREADS = 256;
-constexpr int PBUFS = 8;                     // TMEM accumulators of data in flight: all 512 columns
-constexpr int PK = 128;                      // rows of a step
+constexpr int PBN = 128;                     // tile columns
+constexpr int PACC = 512 / PBN;              // accumulators in TMEM
+constexpr int PK = 64;                       // rows of a step
 constexpr int PCHUNK = 64 * PK * 2;          // 64 columns of a step
-constexpr int PBN = 64;                      // tile columns: 32 per accumulating thread and (1 + D) sums of each
-constexpr int PSTAGE = (BM + PBN) / 64 * PCHUNK;
+constexpr int PA_BYTES = BM / 64 * PCHUNK;   // 128 columns of dY, or of its rescaled rows
+constexpr int PSTAGE = 2 * PA_BYTES + PBN / 64 * PCHUNK;
 constexpr int PSTAGES = 4;
-constexpr int PSMEM = PSTAGES * PSTAGE + 1024 /*alignment slack*/ + 256 /*barriers*/;
+constexpr int PMASKS = 16384;                // bytes of the masks of a launch
+constexpr int PSMEM = PSTAGES * PSTAGE + 1024 /*alignment slack*/ + 256 /*barriers*/ + PMASKS;
 
-// What a group of batches leaves for its product
+// What a group of batches leaves for its product: a block per batch.
 struct ProbeGroup {
   const __nv_bfloat16* dY[PG]; const __nv_bfloat16* X[PG];
-  float* a; float* b;              // [batch][R] row square-norms of dY and X
-  float* p;                        // [batch][M][N] keep probabilities
-  float* w;                        // [batch][pass][N][PD] keep / p (1 past the last draw)
+  uint8_t* block[PG];
+  size_t b_at, p_at, keep_at, scaled_at;
   __nv_bfloat16* sub;              // [batch][R][k] sampled columns of dY
+  __device__ __forceinline__ float* a(int g) const { return reinterpret_cast<float*>(block[g]); }             // [R] ||dY_r||^2
+  __device__ __forceinline__ float* b(int g) const { return reinterpret_cast<float*>(block[g] + b_at); }      // [R] ||X_r||^2
+  __device__ __forceinline__ float* p(int g) const { return reinterpret_cast<float*>(block[g] + p_at); }      // [N]
+  __device__ __forceinline__ uint8_t* keep(int g) const { return block[g] + keep_at; }                        // [M][N]
+  __host__ __device__ __forceinline__ __nv_bfloat16* scaled(int g) const {                                    // [R][columns]
+    return reinterpret_cast<__nv_bfloat16*>(block[g] + scaled_at);
+  }
 };
 
 // ------------------------------------------------------------------------------------- row norms
@@ -89,44 +98,33 @@ __global__ void __launch_bounds__(256) probe_norms_kernel(const __grid_constant_
     const __nv_bfloat16* row = (y ? G.dY[g] : G.X[g]) + (size_t)r * d;
     const float s = warp_sum(PICK && y ? row_partial_pick(row, d, lane, cols, k, G.sub + ((size_t)g * R + r) * k)
                                        : row_partial<__nv_bfloat16>(row, d, lane));
-    if (lane == 0) (y ? G.a : G.b)[(size_t)g * R + r] = s;
+    if (lane == 0) (y ? G.a(g) : G.b(g))[r] = s;
   }
 }
 
 // ------------------------------------------------------------------------------------ the draws
 struct DrawParams {
-  const float* a; const float* b;  // [batch][R]
-  float* p; float* w;              // as in ProbeGroup
   double* sparsity;                // [2][batch of the probe] p_lo, p_hi
   double* vw;                      // [batch of the probe][M] Eq. 3
   int32_t* status;
-  int N, T, M, passes, first_batch;
+  int N, T, M, first_batch;
   float rho, nu;
   double s_lo, s_hi;
   uint64_t seed;
 };
 
-// Where w of (batch g, draw j, datum n) is.
-__device__ __forceinline__ size_t w_index(const DrawParams& P, int g, int j, int n) {
-  return (((size_t)g * P.passes + j / PD) * P.N + n) * PD + j % PD;
-}
-
-// CTA (j, batch), j < M: SampleA of draw j (Sec. 4.1), as in the sampled backward.  CTA (PD passes, batch): Eq. 4's sparsity.
+// CTA (j, batch), j < M: SampleA of draw j (Sec. 4.1), as in the sampled backward.  CTA (M, batch): Eq. 4's sparsity.
 constexpr int DRAW_THREADS = 512;
 template <int SLOTS>
-__global__ void __launch_bounds__(DRAW_THREADS) probe_draw_kernel(DrawParams P) {
+__global__ void __launch_bounds__(DRAW_THREADS) probe_draw_kernel(const __grid_constant__ ProbeGroup G, DrawParams P) {
   __shared__ float s_g[32 * SLOTS], s_sorted[32 * SLOTS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x, g = blockIdx.y;
   for (int n = threadIdx.x; n < 32 * SLOTS; n += DRAW_THREADS) s_g[n] = 0.f;
   pdl_wait();
   pdl_trigger();
-  if (j >= P.M && j < PD * P.passes) {
-    for (int n = threadIdx.x; n < P.N; n += DRAW_THREADS) P.w[w_index(P, g, j, n)] = 1.f;
-    return;
-  }
   __syncthreads();
   for (int n = warp; n < P.N; n += DRAW_THREADS / 32) {
-    const float s = datum_sqnorm_warp(P.a + ((size_t)g * P.N + n) * P.T, P.T, lane);
+    const float s = datum_sqnorm_warp(G.a(g) + (size_t)n * P.T, P.T, lane);
     if (lane == 0) s_g[n] = sqrtf(s);
   }
   __syncthreads();
@@ -137,13 +135,14 @@ __global__ void __launch_bounds__(DRAW_THREADS) probe_draw_kernel(DrawParams P) 
     for (int i = 0; i < SLOTS; ++i) v[i] = s_g[lane + 32 * i];
     capped_prop_warp<SLOTS>(v, (float)P.N * P.rho);
     const uint64_t seed = P.seed + (uint64_t)((P.first_batch + g) * P.M + j + 1) * 0x9E3779B97F4A7C15ull;
-    const size_t o = ((size_t)g * P.M + j) * P.N;
+    float* p = G.p(g);
+    uint8_t* keep = G.keep(g) + (size_t)j * P.N;
 #pragma unroll
     for (int i = 0; i < SLOTS; ++i) {
       const int n = lane + 32 * i;
       if (n < P.N) {
-        P.p[o + n] = v[i];
-        P.w[w_index(P, g, j, n)] = bernoulli_keep(v[i], seed, 0u, (uint64_t)n) ? 1.0f / v[i] : 0.f;
+        if (j == 0) p[n] = v[i];                     // the same in every draw
+        keep[n] = bernoulli_keep(v[i], seed, 0u, (uint64_t)n) ? 1 : 0;
       }
     }
     return;
@@ -175,20 +174,21 @@ __global__ void __launch_bounds__(DRAW_THREADS) probe_draw_kernel(DrawParams P) 
 
 // Eq. 3 of draw (j, batch) at the probabilities q = min(1, c w) of ratio nu: leverage scores of the rows of its kept data (0
 // on the others), water-filling, sum of (1 - q) / q w^2.
-__global__ void __launch_bounds__(SAMPLER_THREADS) probe_vw_kernel(DrawParams P) {
+__global__ void __launch_bounds__(SAMPLER_THREADS) probe_vw_kernel(const __grid_constant__ ProbeGroup G, DrawParams P) {
   extern __shared__ __align__(16) float s_w[];
   __shared__ WShared sh;
   const int tid = threadIdx.x, j = blockIdx.x, g = blockIdx.y, n = P.N * P.T;
-  const size_t o = ((size_t)g * P.M + j) * P.N;
-  const float* a = P.a + (size_t)g * n;
-  const float* b = P.b + (size_t)g * n;
+  const float* a = G.a(g);
+  const float* b = G.b(g);
+  const float* p = G.p(g);
+  const uint8_t* keep = G.keep(g) + (size_t)j * P.N;
   for (int i = tid; i < n; i += SAMPLER_THREADS) {
     const int d = i / P.T;
-    s_w[i] = P.w[w_index(P, g, j, d)] > 0.f ? sqrtf(a[i]) * sqrtf(b[i]) / P.p[o + d] : 0.f;
+    s_w[i] = keep[d] != 0 ? sqrtf(a[i]) * sqrtf(b[i]) / p[d] : 0.f;
   }
   float dummy = 0.f;
   int kept = 0;
-  for (int i = tid; i < P.N; i += SAMPLER_THREADS) kept += P.w[w_index(P, g, j, i)] > 0.f ? 1 : 0;
+  for (int i = tid; i < P.N; i += SAMPLER_THREADS) kept += keep[i];
   fast_sum(dummy, kept, &sh, 1);
   __syncthreads();
   int mode;
@@ -206,21 +206,98 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) probe_vw_kernel(DrawParams P)
   if (tid == 0) P.vw[(P.first_batch + g) * P.M + j] = (double)vw;
 }
 
+// --------------------------------------------------------------------------------- rescaled rows
+// bf16(dY_r / p_n) for the rows of the data that any draw kept, `cols` columns of each (the sampled ones if SUB); blockIdx.y is
+// the batch.  HBM / L2 bound: 16-byte pieces over the whole matrix, four per thread in flight.
+constexpr int SCALE_THREADS = 256;
+template <bool SUB>
+__global__ void __launch_bounds__(SCALE_THREADS) probe_scale_kernel(const __grid_constant__ ProbeGroup G, int N, int T, int M, int cols) {
+  extern __shared__ float s_scale[];           // [N] 1/p of the kept data, 0 for the others
+  pdl_wait();
+  pdl_trigger();
+  const int g = blockIdx.y;
+  for (int n = threadIdx.x; n < N; n += SCALE_THREADS) {
+    const uint8_t* keep = G.keep(g) + n;
+    int any = 0;
+    for (int j = 0; j < M; ++j) any |= keep[(size_t)j * N];
+    s_scale[n] = any != 0 ? 1.0f / G.p(g)[n] : 0.f;
+  }
+  __syncthreads();
+  const int per = T * (cols / 8), total = N * per;        // pieces of a datum, of the batch
+  const __nv_bfloat16* src = SUB ? G.sub + (size_t)g * N * T * cols : G.dY[g];
+  __nv_bfloat16* dst = G.scaled(g);
+  for (int i0 = blockIdx.x * 4 * SCALE_THREADS + threadIdx.x; i0 < total; i0 += gridDim.x * 4 * SCALE_THREADS) {
+    Vec8<__nv_bfloat16> v[4];
+    float sc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = i0 + q * SCALE_THREADS;
+      sc[q] = i < total ? s_scale[i / per] : 0.f;
+      if (sc[q] == 0.f) continue;
+      if (SUB) v[q].v = __ldcg(reinterpret_cast<const uint4*>(src) + i);      // written by a kernel of this call
+      else v[q].load(src + (size_t)i * 8);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (sc[q] == 0.f) continue;
+      float f[8];
+      v[q].get(f);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) f[e] *= sc[q];
+      store8(dst + (size_t)(i0 + q * SCALE_THREADS) * 8, f);
+    }
+  }
+}
+
 // ----------------------------------------------------------------------------------- the product
-struct ProbeMaps { CUtensorMap a[PG], b[PG]; };      // per batch: dY (or its sampled columns) and X
+struct ProbeMaps { CUtensorMap a[PG], e[PG], b[PG]; };      // per batch: dY (or its sampled columns), its rescaled rows, X
 struct ProbeParams {
-  const float4* w;                 // [batch][pass][N] of PD draws
-  float* mean; float* m2;          // d_out x d_in, by tiles: running mean and squared deviation of G_s
-  double* pact; double* ps;        // [tiles] sum of squares of the differences so far; sum of m2 (last batch)
-  float* partial;                  // [batch][unit][1 + D][128 x 64] when a tile's data are cut into slices
-  int N, T, d_in, d_out, kT, steps, S, per, ntiles, units;    // kT: steps of a datum
-  int first_batch, batches, M;
-  int pass, passes;                // the draws of this pass are pass * PD ...
-  int fresh;                       // pact starts here
+  const uint8_t* keep[PG];         // [M][N]
+  float* gs; size_t gs_stride;     // G_s of every batch, d_out x d_in, see gs_at
+  double* pact;                    // [batch][tile or part of it]: sum of squares of the differences
+  float* partial;                  // [unit][1 + M][128 x 128] when the contraction is cut into slices
+  int N, T, d_in, d_out, kT, S, ntiles, tiles, units;    // kT: steps of a datum
+  int batches, M;
   int32_t* status;
   unsigned long long wait_limit_ns;
   int stall_once;
 };
+// Unit u: a slice of the contractions of a tile of a batch.
+struct ProbeUnit { int g, tile, slice; };
+__device__ __forceinline__ ProbeUnit probe_unit(const ProbeParams& P, int u) {
+  ProbeUnit w;
+  const int t = u / P.S;
+  w.slice = u - t * P.S;
+  w.g = t / P.tiles;
+  w.tile = t - w.g * P.tiles;
+  return w;
+}
+// A unit works in rounds, as many accumulators at a time as TMEM holds: round 0 takes G_s and the first draws, the others draws
+// alone.  The draws of round r, and where the results of its accumulators go (0: G_s, 1 + j: draw j).
+__device__ __forceinline__ int round_first(int r) { return r == 0 ? 0 : r * PACC - 1; }
+__device__ __forceinline__ int round_draws(int r, int M) { return min(r == 0 ? PACC - 1 : PACC, M - round_first(r)); }
+__host__ __device__ __forceinline__ int rounds_of(int M) { return (M + PACC) / PACC; }
+// The steps of a slice of a round: `left` steps from step kb of datum n on.  Round 0 runs over all data, the others over those
+// that any of their draws kept.  mask: [N rounded up to 4] the draws of the round that kept the datum, a bit each; kept: the
+// number of data with a mask.
+struct RoundSteps { int n, kb, left; };
+__device__ __forceinline__ RoundSteps round_steps(const uint8_t* mask, int kept, int N, int kT, int r, int S, int slice) {
+  RoundSteps s;
+  const int steps = (r == 0 ? N : kept) * kT, per = (steps + S - 1) / S, c0 = min(steps, slice * per);
+  s.left = min(steps, c0 + per) - c0;
+  int k = c0 / kT;
+  s.kb = c0 - k * kT;
+  s.n = k;
+  if (r == 0 || s.left <= 0) return s;
+  s.n = 0;
+  for (;; s.n += 4) {                          // the k-th datum with a mask
+    const int c = __popc(__vcmpne4(*reinterpret_cast<const uint32_t*>(mask + s.n), 0u)) / 8;
+    if (k < c) break;
+    k -= c;
+  }
+  for (;; ++s.n)
+    if (mask[s.n] != 0 && k-- == 0) return s;
+}
 
 // Welford's update of one element of batch `i` of M: returns its final squared deviation in the last batch, else 0.
 __device__ __forceinline__ float welford(float x, int i, int M, float& mean, float& m2) {
@@ -231,112 +308,124 @@ __device__ __forceinline__ float welford(float x, int i, int M, float& mean, flo
   return i == M - 1 ? m2 : 0.f;
 }
 // Where a tile's columns 4 q .. 4 q + 3 of `row` are in a scratch tile of `rows` rows.  The threads of a warp have consecutive
-// rows, so they take 512 consecutive bytes: in rows of 64 columns an instruction met 32 cache lines, and the moments of a tile
-// and batch took 4 us in which the products could run eight data ahead at most (189 -> 176 us for 768 -> 3072, M = 4).
+// rows, so they take 512 consecutive bytes; in rows of columns an instruction would meet 32 cache lines.
 __device__ __forceinline__ size_t scratch_at(int q, int rows, int row) { return ((size_t)q * rows + row) * 4; }
-// G_s of batch i at W columns from 4 q0 on into the running moments, all loads before the first store.  m2 of the first batch
-// is 0 and not stored, neither is anything of the last.  The moments of a tile have its rows below d_out.
-template <int W>
-__device__ __forceinline__ float welford_row(const ProbeParams& P, int i, int tile, int row, int q0, const float (&x)[W]) {
-  float4 mean[W / 4], m2[W / 4];
-  const int r0 = tile / P.ntiles * BM, rows = min(BM, P.d_out - r0);
-  const size_t o = (size_t)r0 * P.d_in + (size_t)(tile % P.ntiles) * rows * PBN + scratch_at(q0, rows, row);
-  const size_t step = (size_t)rows * 4;
-#pragma unroll
-  for (int e = 0; e < W / 4; ++e) {
-    mean[e] = i > 0 ? *reinterpret_cast<const float4*>(P.mean + o + e * step) : make_float4(0.f, 0.f, 0.f, 0.f);
-    m2[e] = i > 1 ? *reinterpret_cast<const float4*>(P.m2 + o + e * step) : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  float r = 0.f;
-#pragma unroll
-  for (int e = 0; e < W / 4; ++e) {
-    r += (welford(x[4 * e], i, P.M, mean[e].x, m2[e].x) + welford(x[4 * e + 1], i, P.M, mean[e].y, m2[e].y)) +
-         (welford(x[4 * e + 2], i, P.M, mean[e].z, m2[e].z) + welford(x[4 * e + 3], i, P.M, mean[e].w, m2[e].w));
-    if (i < P.M - 1) {
-      *reinterpret_cast<float4*>(P.mean + o + e * step) = mean[e];
-      if (i > 0) *reinterpret_cast<float4*>(P.m2 + o + e * step) = m2[e];
-    }
-  }
-  return r;
+// Where columns col .. col + 3 (col a multiple of 4) of row `row` of tile row r0 are in a kept G_s, `rows` = gs_rows(r0).
+__device__ __forceinline__ int gs_rows(const ProbeParams& P, int r0) { return min(BM, P.d_out - r0); }
+__device__ __forceinline__ size_t gs_at(const ProbeParams& P, int r0, int rows, int row, int col) {
+  return (size_t)r0 * P.d_in + scratch_at(col / 4, rows, row);
 }
-// The sums of THREADS threads over a tile, added in a fixed order by thread 0.
+// The sums of THREADS threads, added in a fixed order by thread 0.
 template <int THREADS>
-__device__ __forceinline__ void tile_sums(const ProbeParams& P, bool exact, int tile, double act, double sq, double (*sh)[2]) {
+__device__ __forceinline__ void block_act(double* out, double act, double* sh) {
   act = warp_sum(act);
-  sq = warp_sum(sq);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) { sh[warp][0] = act; sh[warp][1] = sq; }
+  if (lane == 0) sh[warp] = act;
   asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
   if (threadIdx.x == 0) {
-    double t0 = 0.0, t1 = 0.0;
-    for (int w = 0; w < THREADS / 32; ++w) { t0 += sh[w][0]; t1 += sh[w][1]; }
-    P.pact[tile] = P.fresh ? t0 : P.pact[tile] + t0;
-    if (exact && P.first_batch + P.batches == P.M) P.ps[tile] = t1;
+    double t = 0.0;
+    for (int w = 0; w < THREADS / 32; ++w) t += sh[w];
+    *out = t;
   }
   asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
 }
 
-// A unit is a tile of the gradient and a contiguous range of a batch's steps, worked off batch by batch; a step is up to
-// 128 rows of one datum.  EXACT: this pass makes G_s.
-template <int D, bool EXACT>
+// Persistent CTAs; a unit is a tile of one batch's gradients, possibly with a slice of the contraction.  Bound by the bytes
+// through shared memory (operands in, and out again once per accumulator: 16 KB and 32 KB per 64 rows), for gradients of few
+// rows by X from HBM.  The loading and the issuing warp run their loops with uniform control flow, one elected lane acts, and
+// what a step does is fixed per datum: with the lists of data walked by one lane a step took 0.8 us whatever it had to do.
 __global__ void __launch_bounds__(PROBE_THREADS, 1)
-probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
+probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ ProbeParams P) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ double s_sum[ACC_THREADS / 32][2];
+  __shared__ double s_sum[ACC_THREADS / 32];
+  __shared__ uint32_t s_begun;               // the accumulators of the round that a product has written, a bit each
+  __shared__ int s_kept[PG * 16];            // [batch][round] data with a mask
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(base + PSTAGES * PSTAGE);
   uint64_t* empty = full + PSTAGES;
-  uint64_t* acc_full = empty + PSTAGES;      // [PBUFS] a datum's product is complete
-  uint64_t* acc_empty = acc_full + PBUFS;      // [PBUFS] ... has been read
-  uint32_t* tmem_holder = (uint32_t*)(acc_empty + PBUFS);
+  uint64_t* acc_full = empty + PSTAGES;      // the accumulators of a round are complete
+  uint64_t* acc_empty = acc_full + 1;        // ... have been read
+  uint32_t* tmem_holder = (uint32_t*)(acc_empty + 1);
   volatile int* abort_flag = (int*)(tmem_holder + 1);
+  uint8_t* s_mask = base + PSTAGES * PSTAGE + 256;      // [batch][round][N rounded up to 4], see round_steps
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < PSTAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    for (int i = 0; i < PBUFS; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], ACC_THREADS / 32); }
+    mbar_init(acc_full, 2);                  // the issuing lane, which has written s_begun, and its products
+    mbar_init(acc_empty, ACC_THREADS / 32);
     *abort_flag = 0;
     *reinterpret_cast<volatile unsigned long long*>(abort_flag + 5) = P.wait_limit_ns;     // read by mbar_wait
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
-  if (warp == 9) tmem_alloc(tmem_holder, PBUFS * PBN);
+  if (warp == 9) tmem_alloc(tmem_holder, 512);
+  const int rounds = rounds_of(P.M), n_pad = (P.N + 3) & ~3;
+  pdl_wait();
+  for (int i = warp; i < P.batches * rounds; i += PROBE_THREADS / 32) {
+    const int g = i / rounds, r = i - g * rounds, first = round_first(r), draws = round_draws(r, P.M);
+    const uint8_t* keep = P.keep[g] + (size_t)first * P.N;
+    int kept = 0;
+    for (int n = lane; n < n_pad; n += 32) {
+      uint32_t m = 0;
+      if (n < P.N)
+        for (int j = 0; j < draws; ++j) m |= (uint32_t)keep[(size_t)j * P.N + n] << j;
+      s_mask[i * n_pad + n] = (uint8_t)m;
+      kept += m != 0u ? 1 : 0;
+    }
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if (lane == 0) s_kept[i] = kept;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *(volatile uint32_t*)tmem_holder;
-  pdl_wait();
 
-  // The launch gives every thread 168 registers, 64512 in all.  The sums of four draws need more: the accumulating warpgroups
-  // take 2 x 128 x 224 = 57344, the third keeps 128 x 56 = 7168.
-  if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
   if (warp == 8) {
     // ------------------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      int stage = 0; uint32_t phase = 0;
-      bool ok = true, stalled = false;
-      for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
-        const int tile = u / P.S, s0 = (u - tile * P.S) * P.per, s1 = min(P.steps, s0 + P.per);
-        const int row0 = tile / P.ntiles * BM, col0 = tile % P.ntiles * PBN;
-        for (int g = 0; g < P.batches && ok; ++g) {
-          int n = s0 / P.kT, kb = s0 - n * P.kT;
-          for (int s = s0; s < s1; ++s) {
-            ok = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, P.status);
+    const bool leader = elect_one();
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true, stalled = P.stall_once == 0 || blockIdx.x != 0;
+    for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
+      const ProbeUnit w = probe_unit(P, u);
+      const int row0 = w.tile / P.ntiles * BM, col0 = w.tile % P.ntiles * PBN;
+      const CUtensorMap* ma = &maps.a[w.g];
+      const CUtensorMap* me = &maps.e[w.g];
+      const CUtensorMap* mb = &maps.b[w.g];
+      for (int r = 0; r < rounds && ok; ++r) {
+        const uint8_t* mask = s_mask + (w.g * rounds + r) * n_pad;
+        RoundSteps it = round_steps(mask, s_kept[w.g * rounds + r], P.N, P.kT, r, P.S, w.slice);
+        while (it.left > 0 && ok) {
+          const bool kept = __any_sync(0xffffffffu, mask[it.n] != 0);
+          const uint32_t bytes = PSTAGE - (r == 0 ? 0 : PA_BYTES) - (kept ? 0 : PA_BYTES);
+          const int end = min(P.kT, it.kb + it.left);
+          it.left -= end - it.kb;
+          for (int kb = it.kb; kb < end; ++kb) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&empty[stage], phase ^ 1u, abort_flag, P.status));
             if (!ok) break;
             uint8_t* sa = base + stage * PSTAGE;
-            if (P.stall_once != 0 && blockIdx.x == 0 && !stalled) {
-              stalled = true;                  // nothing will ever arrive for this stage: a wait runs out
-            } else {
-              mbar_expect_tx(&full[stage], PSTAGE);
-              tma_load_3d(sa, &maps.a[g], row0, kb * PK, n, &full[stage]);           // rows past T are zero-filled
-              tma_load_3d(sa + PCHUNK, &maps.a[g], row0 + 64, kb * PK, n, &full[stage]);
-#pragma unroll
-              for (int j = 0; j < PBN / 64; ++j)
-                tma_load_3d(sa + (2 + j) * PCHUNK, &maps.b[g], col0 + j * 64, kb * PK, n, &full[stage]);
+            if (stalled) {                       // otherwise nothing will ever arrive for this stage: a wait runs out
+              if (leader) {
+                mbar_expect_tx(&full[stage], bytes);
+                if (r == 0) {
+                  tma_load_3d(sa, ma, row0, kb * PK, it.n, &full[stage]);              // rows past T are zero-filled
+                  tma_load_3d(sa + PCHUNK, ma, row0 + 64, kb * PK, it.n, &full[stage]);
+                }
+                if (kept) {
+                  tma_load_3d(sa + PA_BYTES, me, row0, kb * PK, it.n, &full[stage]);
+                  tma_load_3d(sa + PA_BYTES + PCHUNK, me, row0 + 64, kb * PK, it.n, &full[stage]);
+                }
+                tma_load_3d(sa + 2 * PA_BYTES, mb, col0, kb * PK, it.n, &full[stage]);
+                tma_load_3d(sa + 2 * PA_BYTES + PCHUNK, mb, col0 + 64, kb * PK, it.n, &full[stage]);
+              }
+              __syncwarp();
             }
+            stalled = true;
             if (++stage == PSTAGES) { stage = 0; phase ^= 1u; }
-            if (++kb == P.kT) { kb = 0; ++n; }
           }
+          it.kb = 0;
+          ++it.n;
+          if (r > 0 && it.left > 0)
+            while (mask[it.n] == 0) ++it.n;
         }
       }
     }
@@ -347,187 +436,208 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, ProbeParams P) {
     // 64-column chunks PCHUNK apart, 8 k-rows 1 KB apart, 128-byte swizzle
     constexpr uint64_t mn_major = ((uint64_t)(PCHUNK >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
     constexpr uint32_t k_step = UMMA_K * 128 >> 4;
-    const int last_rows = P.T - (P.kT - 1) * PK;
-    int stage = 0; uint32_t phase = 0, buf = 0, buf_phase = 0;
+    const int last16 = (P.T - (P.kT - 1) * PK + UMMA_K - 1) / UMMA_K;      // steps of 16 rows in the last step of a datum
+    int stage = 0; uint32_t phase = 0, acc_phase = 0;
     bool ok = true;
     for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
-      const int s0 = (u % P.S) * P.per, s1 = min(P.steps, s0 + P.per);
-      for (int g = 0; g < P.batches && ok; ++g) {
-        int kb = s0 % P.kT;
-        bool fresh = true;
-        for (int s = s0; s < s1 && ok; ++s) {
-          if (fresh) ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[buf], buf_phase ^ 1u, abort_flag, P.status));
-          ok = ok && __all_sync(0xffffffffu, mbar_wait(&full[stage], phase, abort_flag, P.status));
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t sa = smem_u32(base + stage * PSTAGE);
-          const uint64_t da = mn_major | (sa >> 4), db = mn_major | ((sa + 2 * PCHUNK) >> 4);
-          const uint32_t d = tmem_base + buf * (uint32_t)PBN;
-          auto product = [&](int k, uint32_t accumulate) {
-            umma_bf16(d, da + (uint64_t)(k * k_step), db + (uint64_t)(k * k_step), idesc, accumulate);
-          };
-          const bool ends = kb == P.kT - 1;
-          const int rows = ends ? last_rows : PK;
-          const bool done = ends || s == s1 - 1;
-          if (leader) {
-            product(0, fresh ? 0u : 1u);
-            if (rows == PK) {
+      const ProbeUnit w = probe_unit(P, u);
+      for (int r = 0; r < rounds && ok; ++r) {
+        const uint8_t* mask = s_mask + (w.g * rounds + r) * n_pad;
+        RoundSteps it = round_steps(mask, s_kept[w.g * rounds + r], P.N, P.kT, r, P.S, w.slice);
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_empty, acc_phase ^ 1u, abort_flag, P.status));
+        if (!ok) break;
+        tc_fence_after();
+        uint32_t begun = 0;
+        while (it.left > 0 && ok) {
+          const uint32_t m = __reduce_or_sync(0xffffffffu, (uint32_t)mask[it.n]), todo = r == 0 ? m << 1 | 1u : m;
+          const int end = min(P.kT, it.kb + it.left);
+          it.left -= end - it.kb;
+          for (int kb = it.kb; kb < end; ++kb) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&full[stage], phase, abort_flag, P.status));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t sa = smem_u32(base + stage * PSTAGE) >> 4;
+            const uint64_t de = mn_major | (sa + (PA_BYTES >> 4)), db = mn_major | (sa + (2 * PA_BYTES >> 4));
+            const uint64_t d0 = r == 0 ? mn_major | sa : de;
+            const int k16 = kb == P.kT - 1 ? last16 : PK / UMMA_K;
 #pragma unroll
-              for (int k = 1; k < PK / UMMA_K; ++k) product(k, 1u);
-            } else {                           // the steps of 16 rows that hold any
-              for (int k = 1; k * UMMA_K < rows; ++k) product(k, 1u);
+            for (int a = 0; a < PACC; ++a) {
+              if ((todo >> a & 1u) == 0u) continue;
+              const uint64_t dop = a == 0 ? d0 : de;
+              const uint32_t d = tmem_base + (uint32_t)(a * PBN);
+#pragma unroll
+              for (int k = 0; k < PK / UMMA_K; ++k)        // only the steps of 16 rows that hold any
+                if (leader && k < k16)
+                  umma_bf16(d, dop + (uint64_t)(k * k_step), db + (uint64_t)(k * k_step), idesc, k > 0 ? 1u : begun >> a & 1u);
             }
-            umma_commit(&empty[stage]);
-            if (done) umma_commit(&acc_full[buf]);
+            if (leader) umma_commit(&empty[stage]);
+            begun |= todo;
+            if (++stage == PSTAGES) { stage = 0; phase ^= 1u; }
           }
-          if (done && ++buf == PBUFS) { buf = 0; buf_phase ^= 1u; }
-          fresh = ends;
-          kb = ends ? 0 : kb + 1;
-          if (++stage == PSTAGES) { stage = 0; phase ^= 1u; }
-        }
-      }
-    }
-  }
-  } else {
-    // ------------------------------------------------------------------ accumulation and output
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
-    const int eq = warp & 3, eg = warp >> 2;       // TMEM lane quarter, half of the columns
-    constexpr int CW = PBN / 2;
-    const uint32_t tlane = ((uint32_t)(eq * 32) << 16) + (uint32_t)(eg * CW);
-    uint32_t buf = 0, buf_phase = 0;
-    bool ok = true;
-    for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
-      const int tile = u / P.S, s0 = (u - tile * P.S) * P.per, s1 = min(P.steps, s0 + P.per);
-      const int n0 = s0 / P.kT, n1 = (s1 - 1) / P.kT + 1;
-      const int row = eq * 32 + lane, r0 = tile / P.ntiles * BM + row;
-      double act = 0.0, sq = 0.0;
-      for (int g = 0; g < P.batches; ++g) {
-        uint64_t gs2[CW / 2], df2[D][CW / 2];      // two columns per register pair and instruction
-#pragma unroll
-        for (int e = 0; e < CW / 2; ++e) {
-          gs2[e] = 0ull;
-#pragma unroll
-          for (int j = 0; j < D; ++j) df2[j][e] = 0ull;
-        }
-        const float4* wg = P.w + ((size_t)g * P.passes + P.pass) * P.N;
-        float4 next = __ldg(wg + n0);
-        for (int n = n0; n < n1; ++n) {
-          const float w[4] = {next.x, next.y, next.z, next.w};
-          next = __ldg(wg + min(n + 1, n1 - 1));   // on its way while this datum is added
-          // The lanes of a warp leave together.  No call here: it would put the sums held in registers into local memory.
-          ok = __all_sync(0xffffffffu, mbar_wait_spin(&acc_full[buf], buf_phase, abort_flag, P.status));
-          if (!ok) break;
-          tc_fence_after();
-          static_assert(CW == 32, "one load");
-          uint32_t v[CW];
-          tmem_ld32(tmem_base + tlane + buf * (uint32_t)PBN, v);
-          uint64_t x[CW / 2];
-#pragma unroll
-          for (int e = 0; e < CW / 2; ++e) x[e] = pack2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
-          // fp32-bound: 0.35 us a datum with an FMA per draw and element, of 0.62 in all; dropped data cost a draw nothing
-          if (EXACT) {
-#pragma unroll
-            for (int e = 0; e < CW / 2; ++e) gs2[e] = add2(gs2[e], x[e]);
-          }
-#pragma unroll
-          for (int j = 0; j < D; ++j) {
-            if (EXACT && !__any_sync(0xffffffffu, w[j] != 0.f)) continue;      // the same for the whole warp: no predicates
-            const float c = EXACT ? w[j] : w[j] - 1.0f;
-            const uint64_t cc = pack2(c, c);
-#pragma unroll
-            for (int e = 0; e < CW / 2; ++e) df2[j][e] = fma2(cc, x[e], df2[j][e]);
-          }
-          // one arrival per warp: the arrivals of all threads at one barrier are served one after the other
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&acc_empty[buf]);
-          if (++buf == PBUFS) { buf = 0; buf_phase ^= 1u; }
+          it.kb = 0;
+          ++it.n;
+          if (r > 0 && it.left > 0)
+            while (mask[it.n] == 0) ++it.n;
         }
         if (!ok) break;
-        float gs[CW], df[D][CW];
-#pragma unroll
-        for (int e = 0; e < CW / 2; ++e) {
-          unpack2(gs2[e], gs[2 * e], gs[2 * e + 1]);
-#pragma unroll
-          for (int j = 0; j < D; ++j) {
-            unpack2(df2[j][e], df[j][2 * e], df[j][2 * e + 1]);
-            if (EXACT) { df[j][2 * e] -= gs[2 * e]; df[j][2 * e + 1] -= gs[2 * e + 1]; }
-          }
+        if (leader) {
+          *(volatile uint32_t*)&s_begun = begun;
+          mbar_arrive(acc_full);
+          umma_commit(acc_full);
         }
-        float* part = P.partial + ((size_t)g * P.units + u) * (1 + D) * BM * PBN + scratch_at(eg * (CW / 4), BM, row);
-        if (P.S > 1) {
+        __syncwarp();
+        acc_phase ^= 1u;
+      }
+    }
+  } else {
+    // --------------------------------------------------------------------------------- the sums
+    const int eq = warp & 3, eg = warp >> 2;       // TMEM lane quarter, half of the columns
+    constexpr int CW = PBN / 2;
+    const uint32_t taddr = tmem_base + ((uint32_t)(eq * 32) << 16) + (uint32_t)(eg * CW);
+    const int row = eq * 32 + lane;
+    uint32_t acc_phase = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
+      const ProbeUnit w = probe_unit(P, u);
+      const int r0 = w.tile / P.ntiles * BM, col0 = w.tile % P.ntiles * PBN + eg * CW;
+      float gs[CW];
+      double act = 0.0;
+      for (int r = 0; r < rounds; ++r) {
+        // The lanes of a warp leave together.  No call here: it would put G_s into local memory.
+        ok = __all_sync(0xffffffffu, mbar_wait_spin(acc_full, acc_phase, abort_flag, P.status));
+        if (!ok) break;
+        acc_phase ^= 1u;
+        tc_fence_after();
+        const uint32_t begun = *(volatile uint32_t*)&s_begun;
+        const int accs = round_draws(r, P.M) + (r == 0 ? 1 : 0), first = r == 0 ? 0 : 1 + round_first(r);
+        for (int a = 0; a < accs; ++a) {
+          const bool any = __any_sync(0xffffffffu, (begun >> a & 1u) != 0u);      // the same for the whole warp: no predicates
+          float* part = P.partial + ((size_t)u * (1 + P.M) + first + a) * BM * PBN + scratch_at(eg * (CW / 4), BM, row);
+          float t = 0.f;
 #pragma unroll
-          for (int e = 0; e < CW; e += 4) {
-            if (EXACT) *reinterpret_cast<float4*>(part + scratch_at(e / 4, BM, 0)) = make_float4(gs[e], gs[e + 1], gs[e + 2], gs[e + 3]);
+          for (int h = 0; h < CW / 32; ++h) {
+            uint32_t v[32];
+            if (any) {
+              tmem_ld32(taddr + (uint32_t)(a * PBN + h * 32), v);
+            } else {
 #pragma unroll
-            for (int j = 0; j < D; ++j)
-              *reinterpret_cast<float4*>(part + (size_t)(1 + j) * BM * PBN + scratch_at(e / 4, BM, 0)) = make_float4(df[j][e], df[j][e + 1], df[j][e + 2], df[j][e + 3]);
+              for (int e = 0; e < 32; ++e) v[e] = 0u;
+            }
+            if (P.S > 1) {
+#pragma unroll
+              for (int e = 0; e < 32; e += 4)
+                *reinterpret_cast<uint4*>(part + scratch_at(h * 8 + e / 4, BM, 0)) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+            } else if (first + a == 0) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) gs[h * 32 + e] = __uint_as_float(v[e]);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) {
+                const float x = __uint_as_float(v[e]) - gs[h * 32 + e];
+                t = fmaf(x, x, t);
+              }
+            }
           }
-        } else if (r0 < P.d_out) {
+          act += (double)t;
+        }
+        // one arrival per warp: the arrivals of all threads at one barrier are served one after the other
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty);
+        if (r == 0 && P.S == 1 && r0 + row < P.d_out) {
+          const int rows = gs_rows(P, r0);
+          float* out = P.gs + w.g * P.gs_stride + gs_at(P, r0, rows, row, col0);
 #pragma unroll
-          for (int j = 0; j < D; ++j) {
-            float t = 0.f;
-#pragma unroll
-            for (int e = 0; e < CW; ++e) t = fmaf(df[j][e], df[j][e], t);
-            act += (double)t;
-          }
-          if (EXACT) sq += (double)welford_row<CW>(P, P.first_batch + g, tile, row, eg * (CW / 4), gs);
+          for (int e = 0; e < CW; e += 4, out += rows * 4)
+            if (col0 + e < P.d_in) *reinterpret_cast<float4*>(out) = make_float4(gs[e], gs[e + 1], gs[e + 2], gs[e + 3]);
         }
       }
       if (!ok) break;
-      if (P.S == 1) tile_sums<ACC_THREADS>(P, EXACT, tile, act, sq, s_sum);
+      if (P.S == 1) block_act<ACC_THREADS>(P.pact + w.g * P.tiles + w.tile, act, s_sum);
     }
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  // Not before all warps are here: the first thread to say so speaks for the CTA, and the CTAs of the kernel that adds slices
-  // would wait on the SMs left to Eq. 3, whose CTAs need all of an SM's registers (20 us at the end of a probe).
+  // Not before all warps are here: the first thread to say so speaks for the CTA, and the CTAs of the next kernel would wait on
+  // the SMs left to Eq. 3, whose CTAs need half of an SM's registers (20 us at the end of a probe).
   pdl_trigger();
-  if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem_base, PBUFS * PBN); }
+  if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem_base, 512); }
 }
 
-// Sliced tiles: four CTAs per tile add the slices in order and finish as the product's epilogue does; a CTA's sums are
-// kept like those of a tile.
-constexpr int ADD_PARTS = 4, ADD_THREADS = 256;
-template <int D, bool EXACT>
+// Sliced tiles: sixteen CTAs per tile and batch add the slices in order and finish as the product's epilogue does.
+constexpr int ADD_PARTS = 16, ADD_THREADS = 256;
 __global__ void __launch_bounds__(ADD_THREADS) probe_add_kernel(ProbeParams P) {
   constexpr int BN = PBN;
-  __shared__ double s_sum[ADD_THREADS / 32][2];
+  __shared__ double s_sum[ADD_THREADS / 32];
   pdl_wait();
-  const int tile = blockIdx.x / ADD_PARTS, rows = BM / ADD_PARTS, first = blockIdx.x % ADD_PARTS * rows;
-  double act = 0.0, sq = 0.0;
+  pdl_trigger();
+  const int t = blockIdx.x / ADD_PARTS, rows = BM / ADD_PARTS, first = blockIdx.x % ADD_PARTS * rows;
+  const int g = t / P.tiles, tile = t - g * P.tiles, r0 = tile / P.ntiles * BM;
+  double act = 0.0;
   for (int i = threadIdx.x; i < rows * BN / 4; i += ADD_THREADS) {
-    const int row = first + i % rows, q0 = i / rows;
-    if (tile / P.ntiles * BM + row >= P.d_out) continue;
-    for (int g = 0; g < P.batches; ++g) {
-      float x[1 + D][4] = {};
+    const int row = first + i % rows, q = i / rows, col = tile % P.ntiles * BN + q * 4;
+    if (r0 + row >= P.d_out || col >= P.d_in) continue;
+    float4 gs = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int ph = 0; ph <= P.M; ++ph) {
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
       for (int s = 0; s < P.S; ++s) {
-        const float* part = P.partial + ((size_t)g * P.units + tile * P.S + s) * (1 + D) * BM * BN + scratch_at(q0, BM, row);
-#pragma unroll
-        for (int q = EXACT ? 0 : 1; q <= D; ++q) {
-          const float4 v = __ldcg(reinterpret_cast<const float4*>(part + (size_t)q * BM * BN));
-          x[q][0] += v.x; x[q][1] += v.y; x[q][2] += v.z; x[q][3] += v.w;
-        }
+        const float* part = P.partial + ((size_t)(t * P.S + s) * (1 + P.M) + ph) * BM * BN + scratch_at(q, BM, row);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(part));
+        x.x += v.x; x.y += v.y; x.z += v.z; x.w += v.w;
       }
-#pragma unroll
-      for (int q = 1; q <= D; ++q) act += (double)((x[q][0] * x[q][0] + x[q][1] * x[q][1]) + (x[q][2] * x[q][2] + x[q][3] * x[q][3]));
-      if (EXACT) sq += (double)welford_row<4>(P, P.first_batch + g, tile, row, q0, x[0]);
+      if (ph == 0) {
+        gs = x;
+        *reinterpret_cast<float4*>(P.gs + g * P.gs_stride + gs_at(P, r0, gs_rows(P, r0), row, col)) = x;
+      } else {
+        const float dx = x.x - gs.x, dy = x.y - gs.y, dz = x.z - gs.z, dw = x.w - gs.w;
+        act += (double)((dx * dx + dy * dy) + (dz * dz + dw * dw));
+      }
     }
   }
-  tile_sums<ADD_THREADS>(P, EXACT, blockIdx.x, act, sq, s_sum);
+  block_act<ADD_THREADS>(P.pact + blockIdx.x, act, s_sum);
+}
+
+// The G_s of a group's batches into the running moments, four elements a thread: HBM / L2 bound.  m2 of the first batch is 0 and
+// not stored, neither is anything of the last, whose squared deviations are summed per CTA in a fixed order.
+constexpr int MOMENT_THREADS = 256;
+__global__ void __launch_bounds__(MOMENT_THREADS) probe_moments_kernel(const float* gs, size_t gs_stride, float* mean, float* m2, long n4,
+                                                                       int first, int batches, int M, double* ps) {
+  __shared__ double s_sum[MOMENT_THREADS / 32];
+  pdl_wait();
+  const bool last = first + batches == M;
+  double sq = 0.0;
+  for (long i = (long)blockIdx.x * MOMENT_THREADS + threadIdx.x; i < n4; i += (long)gridDim.x * MOMENT_THREADS) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, x[PG];
+#pragma unroll
+    for (int g = 0; g < PG; ++g)
+      if (g < batches) x[g] = reinterpret_cast<const float4*>(gs + g * gs_stride)[i];
+    if (first > 0) a = reinterpret_cast<float4*>(mean)[i];
+    if (first > 1) b = reinterpret_cast<float4*>(m2)[i];
+#pragma unroll
+    for (int g = 0; g < PG; ++g)
+      if (g < batches)
+        sq += (double)((welford(x[g].x, first + g, M, a.x, b.x) + welford(x[g].y, first + g, M, a.y, b.y)) +
+                       (welford(x[g].z, first + g, M, a.z, b.z) + welford(x[g].w, first + g, M, a.w, b.w)));
+    if (!last) {
+      reinterpret_cast<float4*>(mean)[i] = a;
+      reinterpret_cast<float4*>(m2)[i] = b;
+    }
+  }
+  if (last) block_act<MOMENT_THREADS>(ps + blockIdx.x, sq, s_sum);
 }
 
 // Alg. 1's averages from the tiles' and draws' sums, in a fixed order.
-__global__ void __launch_bounds__(1024) probe_final_kernel(const double* __restrict__ pact, const double* __restrict__ ps, int tiles,
+__global__ void __launch_bounds__(1024) probe_final_kernel(const double* __restrict__ pact, int np, const double* __restrict__ ps, int ns,
                                                            const double* __restrict__ vw, const double* __restrict__ sparsity, int M,
                                                            double scale, float* V_s, float* V_act, float* V_w, float* p_lo,
                                                            float* p_hi) {
   __shared__ double sh[3][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double t[3] = {0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < tiles; i += 1024) { t[0] += pact[i]; t[1] += ps[i]; }
+  for (int i = threadIdx.x; i < np; i += 1024) t[0] += pact[i];
+  for (int i = threadIdx.x; i < ns; i += 1024) t[1] += ps[i];
   for (int i = threadIdx.x; i < M * M; i += 1024) t[2] += vw[i];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -559,33 +669,18 @@ bool datum_map(CUtensorMap* m, const void* p, int d, int T, int N) {
   return make_map(m, p, 3, dims, strides, box);
 }
 
-// Tiles of a pass and the slices of their data: as many as fill the CTAs once.
-void probe_tiling(ProbeParams& P, int ctas) {
-  P.ntiles = (P.d_in + PBN - 1) / PBN;
-  const int tiles = (P.d_out + BM - 1) / BM * P.ntiles;
-  P.S = ctas / tiles;
-  if (P.S > P.steps / 4) P.S = P.steps / 4;
-  if (P.S < 1) P.S = 1;
-  P.per = (P.steps + P.S - 1) / P.S;
-  P.S = (P.steps + P.per - 1) / P.per;                                    // no empty slice
-  P.units = tiles * P.S;
-}
-// entries of pact and ps that a pass writes
-int probe_sums(const ProbeParams& P) { return P.S > 1 ? P.units / P.S * ADD_PARTS : P.units; }
-
-template <int D, bool EXACT>
 cudaError_t run_probe(Handle* h, const ProbeMaps& maps, const ProbeParams& P, int ctas, cudaStream_t st) {
   static std::atomic<bool> attr_set[64];
   if (!attr_set[h->device].load(std::memory_order_acquire)) {
-    const cudaError_t e = cudaFuncSetAttribute(probe_kernel<D, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
+    const cudaError_t e = cudaFuncSetAttribute(probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
     if (e != cudaSuccess) return e;
     attr_set[h->device].store(true, std::memory_order_release);
   }
-  cudaError_t e = launch_after(probe_kernel<D, EXACT>, dim3((unsigned)(P.units < ctas ? P.units : ctas)), dim3(PROBE_THREADS),
-                               PSMEM, st, maps, P);
+  cudaError_t e = launch_after(probe_kernel, dim3((unsigned)(P.units < ctas ? P.units : ctas)), dim3(PROBE_THREADS), PSMEM,
+                               st, maps, P);
   h->launches += 1;
   if (e == cudaSuccess && P.S > 1) {
-    e = launch_after(probe_add_kernel<D, EXACT>, dim3((unsigned)(P.units / P.S * ADD_PARTS)), dim3(ADD_THREADS), 0, st, P);
+    e = launch_after(probe_add_kernel, dim3((unsigned)(P.units / P.S * ADD_PARTS)), dim3(ADD_THREADS), 0, st, P);
     h->launches += 1;
   }
   return e;
@@ -593,10 +688,10 @@ cudaError_t run_probe(Handle* h, const ProbeMaps& maps, const ProbeParams& P, in
 
 }  // namespace
 
-// Shorter data would leave the steps of 128 rows mostly empty, and every datum costs a pass of the epilogue over its tile;
+// Shorter data would leave the steps of 64 rows partly empty, and every datum costs a pass of the epilogue over its tile;
 // the scores of Eq. 3 must fit a CTA's shared memory.
 bool probe_fused_ok(const Handle* h, int M) {
-  return h->tensor_path && h->desc.T >= 64 && (long)h->desc.N * h->desc.T <= SAMPLE_W_SMEM_ROWS && M * (M + 2) <= PARTIAL_SLOTS;
+  return h->tensor_path && h->desc.T >= PROBE_MIN_T && (long)h->desc.N * h->desc.T <= SAMPLE_W_SMEM_ROWS && M * (M + 2) <= PARTIAL_SLOTS;
 }
 
 cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const void* const* dY, float rho, float nu, double s_lo,
@@ -613,43 +708,60 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
                                     SAMPLE_W_SMEM_ROWS * (int)sizeof(float)));
     attr_set[h->device].store(true, std::memory_order_release);
   }
-  // What a group's batches leave for its product lies in packG and packX, which are neighbours and which this probe does not
-  // need otherwise (R rows of d_out + d_in bf16: at least one batch fits, since the sampled rows are fewer than d_out).
-  const int passes = (M + PD - 1) / PD;
-  const size_t scratch = (size_t)h->R_pad * (d.d_out + d.d_in) * 2;
-  const size_t per_batch = (size_t)R * (2 * sizeof(float) + 2 * (size_t)sub) + (size_t)(M + passes * PD) * d.N * sizeof(float) + 1280;
-  int most = (int)(scratch / per_batch);
-  if (most < 1) return cudaErrorInvalidValue;
-  if (most > PG) most = PG;
-  if (most > M) most = M;
   ProbeGroup G = {};
-  uint8_t* cur = reinterpret_cast<uint8_t*>(h->ws.packG);
-  auto take = [&](size_t bytes) { uint8_t* q = cur; cur += (bytes + 255) / 256 * 256; return q; };
-  G.sub = reinterpret_cast<__nv_bfloat16*>(take((size_t)most * R * sub * 2));
-  G.a = reinterpret_cast<float*>(take((size_t)most * R * sizeof(float)));
-  G.b = reinterpret_cast<float*>(take((size_t)most * R * sizeof(float)));
-  G.p = reinterpret_cast<float*>(take((size_t)most * M * d.N * sizeof(float)));
-  G.w = reinterpret_cast<float*>(take((size_t)most * passes * PD * d.N * sizeof(float)));
+  const int cols = d_out;
+  auto up = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+  G.b_at = up((size_t)R * sizeof(float));
+  G.p_at = G.b_at + up((size_t)R * sizeof(float));
+  G.keep_at = G.p_at + up((size_t)d.N * sizeof(float));
+  G.scaled_at = G.keep_at + up((size_t)M * d.N);
+  const size_t block = G.scaled_at + up((size_t)R * cols * 2);
+  G.sub = reinterpret_cast<__nv_bfloat16*>(h->sub_dY);
 
   ProbeParams P = {};
   P.N = d.N; P.T = d.T; P.d_in = d.d_in; P.d_out = d_out;
+  P.M = M;
   P.kT = (d.T + PK - 1) / PK;
-  P.steps = d.N * P.kT;
-  const int ctas = h->num_sms > 2 * PD ? h->num_sms - PD : h->num_sms;    // Eq. 3's CTAs run beside the product
-  // all passes have the same tiles, so that their sums add up entry by entry
-  probe_tiling(P, ctas);
-  const int sums = probe_sums(P);
-  P.mean = h->ws.mean; P.m2 = h->ws.m2;
-  P.pact = reinterpret_cast<double*>(h->ws.Gact);                         // this probe keeps no gradient
-  P.ps = P.pact + sums;
+  const int ctas = h->num_sms > 8 ? h->num_sms - 4 : h->num_sms;          // Eq. 3's CTAs run beside the product
+  P.ntiles = (d.d_in + PBN - 1) / PBN;
+  P.tiles = (d_out + BM - 1) / BM * P.ntiles;
+  // slices of the contraction: as many as fill the CTAs once, of eight steps at least, and as the workspace holds
+  auto slices = [&](int batches) {
+    const int units = P.tiles * batches;
+    long S = ctas / units;
+    if (S > (long)d.N * P.kT / 8) S = (long)d.N * P.kT / 8;
+    const long room = 3l * h->max_units * (BM * 256) / ((long)(1 + M) * BM * PBN * units);
+    if (S > room) S = room;
+    return (int)(S < 1 ? 1 : S);
+  };
+  // A group's blocks and its G_s lie where this probe needs nothing else.  The blocks: the compact operands of the two
+  // workspace sets (each packG and packX, neighbours: R rows of d_out + d_in bf16, which hold one at least) and, if no
+  // contraction is cut, the partial tiles.  G_s: Gs and Gact and, if one group is all there is, the moments behind them.
+  const size_t elems = (size_t)d_out * d.d_in;
+  P.gs = h->ws.Gs; P.gs_stride = (size_t)(h->ws.Gact - h->ws.Gs);
+  P.pact = reinterpret_cast<double*>(h->ws2.Gact);
   P.partial = h->ws.partial_tiles;
-  P.M = M; P.w = reinterpret_cast<const float4*>(G.w); P.passes = passes;
+  int most = 0;
+  auto place = [&](void* region, size_t bytes, int limit) {
+    for (size_t at = 0; at + block <= bytes && most < limit; at += block) G.block[most++] = reinterpret_cast<uint8_t*>(region) + at;
+  };
+  const size_t arena = (size_t)h->R_pad * (d.d_out + d.d_in) * 2;
+  const int limit = sub > 0 && SUB_MAX / sub < PG ? SUB_MAX / sub : PG;
+  place(h->ws.packG, arena, limit);
+  place(h->ws2.packG, arena, limit);
+  if (M <= limit && most < M && slices(M) == 1) place(h->ws.partial_tiles, 3 * (size_t)h->max_units * BM * 256 * sizeof(float), M);
+  if (most < 1) return cudaErrorInvalidValue;
+  if (most > M) most = M;
+  while (most > 1 && most * rounds_of(M) * ((d.N + 3) & ~3) > PMASKS) --most;      // M < 64, N < 897: one batch fits
+  if (most < M && most > 2) most = 2;                // the moments keep their place
+  int sums = 0;                                      // entries of pact so far
+  double* ps = h->ws2.partial;
+  const int moment_ctas = (int)(elems / 4 / MOMENT_THREADS + 1 < 592 ? elems / 4 / MOMENT_THREADS + 1 : 592);
   P.status = h->ws.status; P.wait_limit_ns = h->wait_limit_ns; P.stall_once = h->stall_once;
 
   DrawParams Q = {};
-  Q.a = G.a; Q.b = G.b; Q.p = G.p; Q.w = G.w;
   Q.vw = h->ws.partial; Q.sparsity = h->ws.partial + M * M; Q.status = h->ws.status;
-  Q.N = d.N; Q.T = d.T; Q.M = M; Q.passes = passes; Q.rho = rho; Q.nu = nu; Q.s_lo = s_lo; Q.s_hi = s_hi; Q.seed = seed;
+  Q.N = d.N; Q.T = d.T; Q.M = M; Q.rho = rho; Q.nu = nu; Q.s_lo = s_lo; Q.s_hi = s_hi; Q.seed = seed;
 
   cudaStream_t side = h->side_stream;
   for (int i0 = 0; i0 < M; i0 += most) {
@@ -658,7 +770,7 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
     for (int g = 0; g < batches; ++g) {
       G.dY[g] = (const __nv_bfloat16*)dY[i0 + g]; G.X[g] = (const __nv_bfloat16*)X[i0 + g];
       if (!datum_map(&maps.a[g], sub > 0 ? (const void*)(G.sub + (size_t)g * R * sub) : dY[i0 + g], d_out, d.T, d.N) ||
-          !datum_map(&maps.b[g], X[i0 + g], d.d_in, d.T, d.N))
+          !datum_map(&maps.e[g], G.scaled(g), d_out, d.T, d.N) || !datum_map(&maps.b[g], X[i0 + g], d.d_in, d.T, d.N))
         return cudaErrorInvalidValue;
     }
     if (i0 > 0) PROBE_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));       // Eq. 3 of the group before reads its scratch
@@ -668,28 +780,39 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
     else probe_norms_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(G, batches, R, d.d_out, d.d_in, nullptr, 0);
     PROBE_CUDA(cudaGetLastError());
     Q.first_batch = i0;
-    const dim3 draw_grid((unsigned)(PD * passes + 1), (unsigned)batches);
+    const dim3 draw_grid((unsigned)(M + 1), (unsigned)batches);
     const dim3 threads(DRAW_THREADS);
-    PROBE_CUDA(d.N <= 32    ? launch_after(probe_draw_kernel<1>, draw_grid, threads, 0, st, Q)
-               : d.N <= 64  ? launch_after(probe_draw_kernel<2>, draw_grid, threads, 0, st, Q)
-               : d.N <= 128 ? launch_after(probe_draw_kernel<4>, draw_grid, threads, 0, st, Q)
-               : d.N <= 256 ? launch_after(probe_draw_kernel<8>, draw_grid, threads, 0, st, Q)
-                            : launch_after(probe_draw_kernel<32>, draw_grid, threads, 0, st, Q));
+    PROBE_CUDA(d.N <= 32    ? launch_after(probe_draw_kernel<1>, draw_grid, threads, 0, st, G, Q)
+               : d.N <= 64  ? launch_after(probe_draw_kernel<2>, draw_grid, threads, 0, st, G, Q)
+               : d.N <= 128 ? launch_after(probe_draw_kernel<4>, draw_grid, threads, 0, st, G, Q)
+               : d.N <= 256 ? launch_after(probe_draw_kernel<8>, draw_grid, threads, 0, st, G, Q)
+                            : launch_after(probe_draw_kernel<32>, draw_grid, threads, 0, st, G, Q));
     PROBE_CUDA(cudaEventRecord(h->ev_fork, st));
     PROBE_CUDA(cudaStreamWaitEvent(side, h->ev_fork, 0));
-    PROBE_CUDA(launch_maybe_after(false, probe_vw_kernel, dim3((unsigned)M, (unsigned)batches), dim3(SAMPLER_THREADS), vw_smem, side, Q));
+    PROBE_CUDA(launch_maybe_after(false, probe_vw_kernel, dim3((unsigned)M, (unsigned)batches), dim3(SAMPLER_THREADS), vw_smem, side, G, Q));
     PROBE_CUDA(cudaEventRecord(h->ev_join, side));
-    h->launches += 3;
-    P.first_batch = i0; P.batches = batches;
-    for (P.pass = 0; P.pass < passes; ++P.pass) {
-      P.fresh = i0 == 0 && P.pass == 0;
-      PROBE_CUDA(M == 2         ? run_probe<2, true>(h, maps, P, ctas, st)
-                 : P.pass == 0 ? run_probe<PD, true>(h, maps, P, ctas, st)
-                                : run_probe<PD, false>(h, maps, P, ctas, st));
-    }
+    const long pieces = (long)R * (cols / 8);
+    long scale_blocks = (pieces + 4 * SCALE_THREADS - 1) / (4 * SCALE_THREADS);
+    if (scale_blocks > 8l * h->num_sms / batches) scale_blocks = 8l * h->num_sms / batches;
+    const dim3 scale_grid((unsigned)scale_blocks, (unsigned)batches);
+    const size_t scale_smem = (size_t)d.N * sizeof(float);
+    PROBE_CUDA(sub > 0 ? launch_after(probe_scale_kernel<true>, scale_grid, dim3(SCALE_THREADS), scale_smem, st, G, d.N, d.T, M, cols)
+                       : launch_after(probe_scale_kernel<false>, scale_grid, dim3(SCALE_THREADS), scale_smem, st, G, d.N, d.T, M, cols));
+    h->launches += 4;
+    P.batches = batches;
+    P.S = slices(batches);
+    P.units = P.tiles * batches * P.S;
+    for (int g = 0; g < batches; ++g) P.keep[g] = G.block[g] + G.keep_at;
+    PROBE_CUDA(run_probe(h, maps, P, ctas, st));
+    const int parts = P.tiles * batches * (P.S > 1 ? ADD_PARTS : 1);
+    sums += parts;
+    P.pact += parts;
+    PROBE_CUDA(launch_after(probe_moments_kernel, dim3((unsigned)moment_ctas), dim3(MOMENT_THREADS), 0, st, (const float*)P.gs,
+                            P.gs_stride, h->ws.mean, h->ws.m2, (long)(elems / 4), i0, batches, M, ps));
+    h->launches += 1;
   }
   PROBE_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
-  probe_final_kernel<<<1, 1024, 0, st>>>(P.pact, P.ps, sums, Q.vw, Q.sparsity, M, scale, V_s, V_act, V_w, p_lo, p_hi);
+  probe_final_kernel<<<1, 1024, 0, st>>>(reinterpret_cast<const double*>(h->ws2.Gact), sums, ps, moment_ctas, Q.vw, Q.sparsity, M, scale, V_s, V_act, V_w, p_lo, p_hi);
   h->launches += 1;
 #undef PROBE_CUDA
   return cudaGetLastError();
