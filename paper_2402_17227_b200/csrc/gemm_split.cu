@@ -131,12 +131,14 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   uint64_t* empty = full + C::STAGES;
   uint64_t* acc_full = empty + C::STAGES;      // [2] the accumulator of a stage is complete
   uint64_t* acc_empty = acc_full + 2;          // [2] ... has been read
-  uint32_t* tmem_holder = (uint32_t*)(acc_empty + 2);
+  uint64_t* done = acc_empty + 2;              // see drain_products
+  uint32_t* tmem_holder = (uint32_t*)(done + 1);
   volatile int* abort_flag = (int*)(tmem_holder + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int i = 0; i < C::STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], ACC_WARPS); }
+    mbar_init(done, 1);
     *abort_flag = 0;
     *reinterpret_cast<volatile unsigned long long*>(abort_flag + 5) = P.wait_limit_ns;     // read by mbar_wait
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -153,7 +155,7 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   if (warp == 8) {
     // ------------------------------------------------------------------------- TMA producer
     if (lane == 0) {
-      int stage = 0; uint32_t phase = 0;
+      int stage = 0; uint32_t phase = 0, filled = 0;
       bool ok = true, stalled = false;
       for (int u = blockIdx.x; u < W.units && ok; u += gridDim.x) {
         const int tile = u / W.S, slice = u - tile * W.S;
@@ -180,9 +182,11 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             for (int j = 0; j < 4 * PB; ++j)
               tma_load_3d(sb + j * C::CHUNK, &tmB, col0 + (j & 3) * 64, k * C::KS, j >> 2, &full[stage]);
           }
+          ++filled;
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
       }
+      drain_loads(full, C::STAGES, stage, phase, filled, abort_flag, P.status);
     }
   } else if (warp == 9) {
     // --------------------------------------------------------------------------- MMA issuer
@@ -224,6 +228,7 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
       }
+      drain_products(done, abort_flag, P.status);
     }
   } else {
     // ----------------------------------------------------------- fp32 accumulation and output

@@ -58,6 +58,7 @@ struct SmemLayout {
   uint8_t* epi;       // [8 warps][32 rows][128 B] staging for bulk / TMA stores
   uint8_t* hbuf;      // GELU: [8 warps][32 rows][128 B] pre-activations of a warp's next chunk
   uint64_t* h_full;   // GELU: [8 warps]
+  uint64_t* done;     // see drain_products
 };
 
 template <int BN, int MH, bool GELU>
@@ -76,7 +77,8 @@ __device__ __forceinline__ SmemLayout carve(uint8_t* raw) {
   s.q_full = bars + 2 * C::STAGES + 4;
   s.q_empty = bars + 2 * C::STAGES + 4 + QD;
   s.h_full = bars + 2 * C::STAGES + 4 + 2 * QD;
-  s.tmem_holder = (uint32_t*)(s.h_full + (GELU ? 8 : 0));
+  s.done = s.h_full + (GELU ? 8 : 0);
+  s.tmem_holder = (uint32_t*)(s.done + 1);
   s.abort_flag = (int*)(s.tmem_holder + 1);
   s.flag = s.abort_flag + 1;
   s.tile_q = s.flag + 1;
@@ -92,6 +94,7 @@ __device__ __forceinline__ uint32_t setup(const SmemLayout& s, int warp, int tid
     for (int i = 0; i < 2; ++i) { mbar_init(&s.tmem_full[i], 1); mbar_init(&s.tmem_empty[i], EPI_THREADS); }
     if (GELU)
       for (int i = 0; i < 8; ++i) mbar_init(&s.h_full[i], 1);
+    mbar_init(s.done, 1);
     if (with_queue)
       for (int i = 0; i < QD; ++i) { mbar_init(&s.q_full[i], 1); mbar_init(&s.q_empty[i], EPI_THREADS + 1); }
     *s.abort_flag = 0;
@@ -335,7 +338,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   if (warp == 4) {
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
-      int stage = 0; uint32_t phase = 0;
+      int stage = 0; uint32_t phase = 0, filled = 0;
       bool ok = true, stalled = false;
       int qi = 0; uint32_t qph = 0;
       // next unit of this CTA, or -1 (see KIND above)
@@ -373,6 +376,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           uint8_t* sa = s.stages + stage * C::STAGE_BYTES;
           if (P.stall_once != 0 && blockIdx.x == 0 && !stalled) {
             stalled = true;                    // nothing will ever arrive for this stage: the MMA role's wait runs out
+            ++filled;
             if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
             continue;
           }
@@ -390,6 +394,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
           for (int j = 0; j < BN / 64; ++j)
             tma_load_2d(sa + C::AT_BYTES + j * CHUNK_BYTES, &tmB, c1 * BN + j * 64, kb * BK, &s.full[stage]);
+          ++filled;
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
       }
@@ -399,6 +404,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           if (atomicAdd(P.sched + 1, 1) == (int)gridDim.x - 1) { P.sched[0] = 0; P.sched[1] = 0; }
         }
       }
+      drain_loads(s.full, C::STAGES, stage, phase, filled, abort_flag, P.status);
     }
   } else if (warp == 5) {
     // ------------------------------------------------------------------ MMA issuer
@@ -458,6 +464,8 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (!ok) break;
         if (leader) umma_commit(&s.tmem_full[buf]);
       }
+      if (leader) drain_products(s.done, abort_flag, P.status);
+      __syncwarp();
     }
   } else {
     // -------------------------------------------------------------------- epilogue
@@ -568,10 +576,12 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           }
         }
       };
+      bool has_h = false;
       if constexpr (GELU) {
         int first = eg;
         while (first < MH * (BN / 64) && col0 + first % (BN / 64) * 64 >= P.d_in) first += 2;
-        if (first < MH * (BN / 64)) load_h(first);
+        has_h = first < MH * (BN / 64);
+        if (has_h) load_h(first);
       }
       bool got = mbar_wait(&s.tmem_full[buf], use, abort_flag, P.status);
       if constexpr (!LEAN) {
@@ -584,8 +594,16 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             "selp.u32 %0, 1, 0, q;\n\t}"
             : "=r"(all) : "r"(got ? 1u : 0u) : "memory");
         got = all != 0;
+      } else {
+        got = __all_sync(0xffffffffu, got);      // the lanes of a warp read TMEM together or not at all
       }
-      if (!got) { ok = false; break; }
+      if (!got) {
+        if constexpr (GELU) {                    // the pre-activations on their way
+          if (has_h) mbar_wait(&s.h_full[eg * 4 + eq], h_phase, abort_flag, P.status);
+        }
+        ok = false;
+        break;
+      }
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(eq * 32) << 16) + (uint32_t)(buf * BN);
       if constexpr (LEAN) {

@@ -345,7 +345,8 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
   uint64_t* empty = full + PSTAGES;
   uint64_t* acc_full = empty + PSTAGES;      // the accumulators of a round are complete
   uint64_t* acc_empty = acc_full + 1;        // ... have been read
-  uint32_t* tmem_holder = (uint32_t*)(acc_empty + 1);
+  uint64_t* done = acc_empty + 1;            // see drain_products
+  uint32_t* tmem_holder = (uint32_t*)(done + 1);
   volatile int* abort_flag = (int*)(tmem_holder + 1);
   uint8_t* s_mask = base + PSTAGES * PSTAGE + 256;      // [batch][round][N rounded up to 4], see round_steps
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -353,6 +354,7 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
     for (int i = 0; i < PSTAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(acc_full, 2);                  // the issuing lane, which has written s_begun, and its products
     mbar_init(acc_empty, ACC_THREADS / 32);
+    mbar_init(done, 1);
     *abort_flag = 0;
     *reinterpret_cast<volatile unsigned long long*>(abort_flag + 5) = P.wait_limit_ns;     // read by mbar_wait
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -383,7 +385,7 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
   if (warp == 8) {
     // ------------------------------------------------------------------------- TMA producer
     const bool leader = elect_one();
-    int stage = 0; uint32_t phase = 0;
+    int stage = 0; uint32_t phase = 0, filled = 0;
     bool ok = true, stalled = P.stall_once == 0 || blockIdx.x != 0;
     for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
       const ProbeUnit w = probe_unit(P, u);
@@ -420,6 +422,7 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
               __syncwarp();
             }
             stalled = true;
+            ++filled;
             if (++stage == PSTAGES) { stage = 0; phase ^= 1u; }
           }
           it.kb = 0;
@@ -429,6 +432,7 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
         }
       }
     }
+    drain_loads(full, PSTAGES, stage, phase, filled, abort_flag, P.status);
   } else if (warp == 9) {
     // --------------------------------------------------------------------------- MMA issuer
     const bool leader = elect_one();
@@ -489,6 +493,8 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
         acc_phase ^= 1u;
       }
     }
+    if (leader) drain_products(done, abort_flag, P.status);
+    __syncwarp();
   } else {
     // --------------------------------------------------------------------------------- the sums
     const int eq = warp & 3, eg = warp >> 2;       // TMEM lane quarter, half of the columns

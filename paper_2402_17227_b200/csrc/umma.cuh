@@ -72,6 +72,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return mbar_wait_slow(bar, parity, abort_flag, status);
 }
 
+// What a role does before it leaves, so that a CTA that gave up does not hand back shared memory or TMEM under copies and
+// products still in flight (else they are complete already).  Bounded like every wait.
+// The loads of the stages filled last; (stage, phase) would be the next of `filled`.
+__device__ __forceinline__ void drain_loads(uint64_t* full, int stages, int stage, uint32_t phase, uint32_t filled,
+                                            volatile int* abort_flag, int32_t* status) {
+  for (int i = 0; i < stages && (uint32_t)i < filled; ++i) {
+    if (stage == 0) { stage = stages; phase ^= 1u; }
+    mbar_wait(&full[--stage], phase, abort_flag, status);
+  }
+}
+
 // true in one lane of a converged warp
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
@@ -128,6 +139,11 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint
 // the mbarrier gets one arrival when all tcgen05.mma issued so far by this thread have finished
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// The products that this thread issued; `bar` is used for nothing else.
+__device__ __forceinline__ void drain_products(uint64_t* bar, volatile int* abort_flag, int32_t* status) {
+  umma_commit(bar);
+  mbar_wait(bar, 0, abort_flag, status);
 }
 // 32 lanes x 32 consecutive fp32 columns: thread i of the warp gets lane (base + i)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
