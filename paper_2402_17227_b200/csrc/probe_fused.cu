@@ -254,7 +254,7 @@ struct ProbeMaps { CUtensorMap a[PG], e[PG], b[PG]; };      // per batch: dY (or
 struct ProbeParams {
   const uint8_t* keep[PG];         // [M][N]
   float* gs; size_t gs_stride;     // G_s of every batch, d_out x d_in, see gs_at
-  double* pact;                    // [batch][tile or part of it]: sum of squares of the differences
+  double* pact;                    // [batch][tile][warp or part of it]: sum of squares of the differences
   float* partial;                  // [unit][1 + M][128 x 128] when the contraction is cut into slices
   int N, T, d_in, d_out, kT, S, ntiles, tiles, units;    // kT: steps of a datum
   int batches, M;
@@ -337,7 +337,6 @@ __device__ __forceinline__ void block_act(double* out, double act, double* sh) {
 __global__ void __launch_bounds__(PROBE_THREADS, 1)
 probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ ProbeParams P) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ double s_sum[ACC_THREADS / 32];
   __shared__ uint32_t s_begun;               // the accumulators of the round that a product has written, a bit each
   __shared__ int s_kept[PG * 16];            // [batch][round] data with a mask
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -559,7 +558,10 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
         }
       }
       if (!ok) break;
-      if (P.S == 1) block_act<ACC_THREADS>(P.pact + w.g * P.tiles + w.tile, act, s_sum);
+      if (P.S == 1) {      // a sum per warp: at a barrier of the eight those that gave up would be missed for good
+        act = warp_sum(act);
+        if (lane == 0) P.pact[(w.g * P.tiles + w.tile) * (ACC_THREADS / 32) + warp] = act;
+      }
     }
   }
   __syncwarp();
@@ -810,7 +812,7 @@ cudaError_t launch_probe_fused(Handle* h, int M, const void* const* X, const voi
     P.units = P.tiles * batches * P.S;
     for (int g = 0; g < batches; ++g) P.keep[g] = G.block[g] + G.keep_at;
     PROBE_CUDA(run_probe(h, maps, P, ctas, st));
-    const int parts = P.tiles * batches * (P.S > 1 ? ADD_PARTS : 1);
+    const int parts = P.tiles * batches * (P.S > 1 ? ADD_PARTS : ACC_THREADS / 32);
     sums += parts;
     P.pact += parts;
     PROBE_CUDA(launch_after(probe_moments_kernel, dim3((unsigned)moment_ctas), dim3(MOMENT_THREADS), 0, st, (const float*)P.gs,

@@ -45,3 +45,23 @@ def test_wait_runs_out_and_handle_recovers(shape, tuning):
         assert torch.equal(dXd, ref_dXd) and torch.equal(dWd, ref_dWd)
     assert layer.device_status() == 0
     layer.close(); clean.close()
+
+
+def test_probe_whose_warps_give_up_one_by_one():
+    """Unsliced tiles of 57344 rows: the warps that wait for a complete accumulator run out of their limit in the middle of the
+    products, each by itself.  The kernel returns, the time-out is reported and the handle recovers."""
+    vbuild.build()
+    N, T, d_in, d_out = 28, 2048, 1024, 1280
+    case = inputs.LayerCase("gp", N, T, d_in, d_out, BF16, 0.5, 0.5, 0.5, 0.5)
+    batches = [inputs.make_layer(case, batch=b, device="cuda") for b in range(2)]
+    layer = vb.Layer(N, T, d_in, d_out, BF16, vb.GEMM_TENSOR)
+    run = lambda: layer.variance_probe([b[0] for b in batches], [b[1] for b in batches], batches[0][2], 0.5, 0.5, 0.75, 3)
+    ref = run().clone()
+    assert layer.device_status() == 0
+    for limit in (1_000, 20_000, 100_000):
+        layer.set_wait_limit(limit, stall_once=False)
+        run()
+        assert layer.device_status() in (0, -6)
+        layer.set_wait_limit(2_000_000_000, stall_once=False)
+        assert torch.equal(run(), ref) and layer.device_status() == 0
+    layer.close()
