@@ -118,6 +118,12 @@ int copy_out(Handle* h, float* g, float* p, float* w, float* q, int32_t* idxA, i
   return VCAS_OK;
 }
 
+// The split products move 16 bytes at a time.  A caller's tensor that does not start on such a boundary (a view into a flat
+// gradient buffer, say) is multiplied by the fp32-FMA kernels, which read and write single elements.
+bool aligned16(const void* a, const void* b, const void* c, const void* d = nullptr) {
+  return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 15) == 0;
+}
+
 // SampleW, the kept-row list with its compact operands, and dW over those rows into `out`; follows SampleA
 // on the workspace set that h->ws currently names.  first_programmatic: the first kernel is launched as a
 // dependent of the kernel before it in `st` (false when its inputs arrive through an event).
@@ -125,10 +131,11 @@ int sample_w_and_dw(Handle* h, const void* X, const void* dY, const SamplerArgs&
                     const Plan* plan, float* out, cudaStream_t st) {
   VCAS_CUDA(launch_scores_x(h, X, a, first_programmatic, st));
   VCAS_CUDA(launch_sample_w(h, a, st));
-  VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path || h->split_path, st));
+  const bool split = h->split_path && aligned16(X, dY, out);
+  VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path || split, st));
   const float keep = a.sample_w ? a.rho * a.nu : a.rho;
   const int hint = (int)(keep * (float)(h->desc.N * h->desc.T)) + 1;
-  if (h->split_path) {
+  if (split) {
     VCAS_CUDA(launch_split_dw(h, dY, X, false, hint, out, true, st));
   } else if (h->tensor_path) {
     VCAS_CUDA(launch_umma_dw(h, h->ws.packG, h->ws.packX, h->R_pad, h->ws.counts + 1, hint, plan, out, st));
@@ -159,7 +166,7 @@ inline void mark_dense(Handle* h, int k, cudaStream_t st) {
 // dX of a sampled call by the products that leave its row square-norms to a pass of their own
 int plain_dx(Handle* h, const void* dY, const void* W, float rho, const void* Hpre, void* dX, float* a_out, bool programmatic,
              cudaStream_t st) {
-  if (h->split_path) {
+  if (h->split_path && aligned16(dY, W, Hpre, dX)) {
     const bool fp32 = h->desc.dtype == VCAS_DTYPE_F32;
     VCAS_CUDA(launch_split_prep(h, dY, false, fp32 ? W : nullptr, h->ws.packW, h->desc.d_out, h->desc.d_in, dX, programmatic, st));
     VCAS_CUDA(launch_split_dx(h, dY, W, false, rho, Hpre, dX, st));
@@ -171,9 +178,9 @@ int plain_dx(Handle* h, const void* dY, const void* W, float rho, const void* Hp
 }
 
 // plan: the tiling made for a call whose dX product runs beside it (nullptr: planned alone)
-// y_ready: split path of an fp32 layer, the parts of dY are in place
-int dense_dw(Handle* h, const void* X, const void* dY, const Plan* plan, bool y_ready, float* out, cudaStream_t st) {
-  if (h->split_path) {
+// split: by the split products; y_ready: the parts of an fp32 layer's dY are in place
+int dense_dw(Handle* h, const void* X, const void* dY, const Plan* plan, bool split, bool y_ready, float* out, cudaStream_t st) {
+  if (split) {
     const int R = h->desc.N * h->desc.T;
     const bool fp32 = h->desc.dtype == VCAS_DTYPE_F32;
     if (fp32) VCAS_CUDA(launch_split_prep(h, y_ready ? nullptr : dY, true, X, h->ws.packX, R, h->desc.d_in, nullptr, false, st));
@@ -327,9 +334,10 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
     }
     mark(h, 3, st);
     mark(h, 6, st);
-    VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path || h->split_path, st));
+    const bool split = h->split_path && aligned16(X, dY, dW);
+    VCAS_CUDA(launch_emit_pack(h, dY, X, a, h->tensor_path || split, st));
     mark(h, 4, st);
-    if (h->split_path) {
+    if (split) {
       VCAS_CUDA(launch_split_dw(h, dY, X, false, hint, dW, false, st));
     } else if (h->tensor_path) {
       VCAS_CUDA(launch_umma_dw(h, h->ws.packG, h->ws.packX, h->R_pad, h->ws.counts + 1, hint, &pw, dW, st));
@@ -446,8 +454,9 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
   cudaStream_t st = S(stream);
   if (join_pending(h, st) != VCAS_OK) return VCAS_ERR_CUDA;
   cudaStream_t sw = st;
-  const bool fork = (h->tensor_path || h->split_path) && !h->prof_enabled;
-  const bool cut = h->split_path && h->desc.dtype == VCAS_DTYPE_F32;
+  const bool split = h->split_path && aligned16(X, dY, dW) && aligned16(W, Hpre, dX);
+  const bool fork = (h->tensor_path || split) && !h->prof_enabled;
+  const bool cut = split && h->desc.dtype == VCAS_DTYPE_F32;
   mark_dense(h, 0, st);
   if (cut) VCAS_CUDA(launch_split_prep(h, dY, true, W, h->ws.packW, h->desc.d_out, h->desc.d_in, nullptr, false, st));
   if (fork) {
@@ -457,7 +466,7 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
   }
   Plan px = {256, 1, 1}, pw = {256, 1, 1};
   if (h->tensor_path) plan_products(h, true, 1.0f, h->desc.N * h->desc.T, 0, false, Hpre != nullptr, &px, &pw);
-  if (h->split_path) {
+  if (split) {
     VCAS_CUDA(launch_split_dx(h, dY, W, true, 1.0f, Hpre, dX, st));
   } else if (h->tensor_path) {
     VCAS_CUDA(launch_umma_dx(h, dY, W, true, 1.0f, Hpre, dX, nullptr, false, 0, &px, st));
@@ -466,7 +475,7 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
   }
   mark_dense(h, 1, st);
   mark_dense(h, 3, sw);
-  const int rc = dense_dw(h, X, dY, h->tensor_path ? &pw : nullptr, cut, dW, sw);
+  const int rc = dense_dw(h, X, dY, h->tensor_path ? &pw : nullptr, split, cut, dW, sw);
   mark_dense(h, 2, sw);
   if (fork) {
     VCAS_CUDA(cudaEventRecord(h->ev_join, sw));
@@ -543,7 +552,7 @@ int vcas_variance_probe(vcas_handle hh, int32_t M, const void* const* X_i, const
       VCAS_CUDA(launch_gather_cols(h, dY_i[i], h->desc.d_out, h->sub_rows, h->sub_k, h->sub_dY, st));
       dYp = h->sub_dY;
     }
-    int rc = dense_dw(hp, X_i[i], dYp, nullptr, false, h->ws.Gs, st);   // G_s,i
+    int rc = dense_dw(hp, X_i[i], dYp, nullptr, h->split_path && aligned16(X_i[i], dYp, nullptr), false, h->ws.Gs, st);   // G_s,i
     if (rc != VCAS_OK) return rc;
     VCAS_CUDA(launch_probe_welford(hp, i, st));
     SamplerArgs a = sampler_args(rho, nu, 0);
