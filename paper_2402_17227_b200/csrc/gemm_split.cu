@@ -2,7 +2,7 @@
 // layers and for bf16 layers whose widths are not multiples of 64:
 //   dX[rows of kept data] = (1/p_n) dY[rows] W                   (App. E; zero rows for dropped data)
 //   dW = G_tilde^T X over the kept rows                           (Sec. 4.2)
-// An fp32 operand is cut into three bf16 parts, x = x1 + x2 + x3 exactly (split.cuh), once, by a pass of its own; the
+// An fp32 operand is cut into three bf16 parts, x = x1 + x2 + x3 (split.cuh), once, by a pass of its own; the
 // product is the sum of the part products down to 2^-18: x1y1, x1y2, x2y1, x2y2, x1y3, x3y1 (what is left out is below
 // 2^-26 of |x||y|).  A bf16 operand is its own single part; the rescaled rows of dY that enter a sampled dW product are
 // formed in fp32 and cut into three.
@@ -383,7 +383,7 @@ __device__ __forceinline__ void prep_row(const T* src, __nv_bfloat16* dst, size_
     if constexpr (CUT) {
       float f[8];
       v[q].get(f);
-      store_parts3(f, dst + c, stride);
+      store_parts3<true>(f, dst + c, stride);
     } else {
       *reinterpret_cast<uint4*>(dst + c) = v[q].v;
     }

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) f[e] *= sc;
               }
-              store_parts3(f, dst, g ? P.g_stride : P.x_stride);
+              store_parts3<sizeof(E) == 4>(f, dst, g ? P.g_stride : P.x_stride);      // a bf16 X is a single part
               continue;
             }
           }

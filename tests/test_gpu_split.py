@@ -3,6 +3,7 @@
 Tolerances: fp32 results within 1e-6 of the float64 oracle (the parts are exact, products below 2^-26 are left out,
 sums of a stage of 32 or 64 terms are truncated to 24 bits and added up in fp32: measured below 4e-7); a bf16 layer's dW,
 whose rescaled rows are not rounded to bf16, meets the same, its dX carries one bf16 rounding (2^-9 / sqrt(3) of its norm)."""
+import numpy as np
 import pytest
 import torch
 
@@ -56,7 +57,7 @@ def test_split_products_match_oracle(dtype, shape):
 
 @pytest.mark.parametrize("value", [float("inf"), float("nan"), 3.4e38])
 def test_split_products_of_values_without_a_finite_bf16_part(value):
-    """An infinite, NaN or nearly overflowing weight gives what fp32 arithmetic gives: only its own column is not finite."""
+    """An infinite or NaN weight, or one whose products overflow, leaves only its own column not finite."""
     vbuild.build()
     N, T, d_in, d_out = 2, 40, 72, 64
     X, dY, W = inputs.make_layer(inputs.LayerCase("t", N, T, d_in, d_out, F32, 1.0, 0.5, 0.5, 0.5))
@@ -102,4 +103,45 @@ def test_tensors_off_16_byte_boundaries(dtype, which):
         # a bf16 layer's dX rounds sums that differ by 1e-7 of themselves: one value in thousands falls on the other side
         assert rel_fro(gX, rX) <= (1e-6 if dtype == F32 else 1e-3) and rel_fro(gW, rW) <= 1e-6
     assert layer.device_status() == 0
+    layer.close()
+
+
+def test_nearly_overflowing_values_keep_their_products():
+    """3.4e38 rounds to infinity in bf16; its products with small values are those of fp32 arithmetic all the same (1e-6)."""
+    vbuild.build()
+    N, T, d_in, d_out = 2, 40, 72, 64
+    X, dY, W = inputs.make_layer(inputs.LayerCase("t", N, T, d_in, d_out, F32, 1.0, 0.5, 0.5, 0.5))
+    dY, W, X = dY / dY.abs().max() / 80, W.clone(), X.clone()
+    W[5, 7], W[6, 9], X[3, 11] = 3.4e38, -3.4028234e38, 3.3999e38
+    layer = vb.Layer(N, T, d_in, d_out, F32)
+    dX, dW = layer.dense_bwd(X.cuda(), dY.cuda(), W.cuda())
+    rX, rW = np64(dY) @ np64(W), np64(dY).T @ np64(X)
+    for got, ref in ((np64(dX), rX), (np64(dW), rW)):
+        assert np.isfinite(got).all() and (np.abs(got - ref) <= 1e-6 * np.abs(ref).max(0)).all()
+    layer.close()
+
+
+def same_kind(got, ref):
+    """Infinities of the same sign, NaN where NaN, finite where finite."""
+    return (np.isnan(got) == np.isnan(ref)).all() and (np.isinf(got) == np.isinf(ref)).all() and \
+        (np.sign(got[np.isinf(ref)]) == np.sign(ref[np.isinf(ref)])).all()
+
+
+@pytest.mark.parametrize("sampled", [True, False])
+@pytest.mark.parametrize("dtype", [F32, BF16])
+def test_infinite_operands(dtype, sampled):
+    """Infinities on one or both sides of a product: what IEEE arithmetic gives, inf inf = inf and inf 0 = NaN among it.  At
+    ratio 1 every row is kept with scale 1, so the parts of a bf16 layer's rows past the first are 0."""
+    vbuild.build()
+    N, T, d_in, d_out = 2, 40, 72, 72
+    X, dY, W = inputs.make_layer(inputs.LayerCase("t", N, T, d_in, d_out, dtype, 1.0, 0.5, 0.5, 0.5))
+    X, dY, W = X.clone(), dY.clone(), W.clone()
+    X[50, 3], W[5, 7], dY[20, 8] = float("inf"), float("-inf"), 0.0
+    if not sampled:                      # an infinite row norm leaves no probabilities
+        dY[3, 5], dY[4, 6], X[4, 9] = float("inf"), float("-inf"), float("inf")
+    layer = vb.Layer(N, T, d_in, d_out, dtype)
+    args = X.cuda(), dY.cuda(), W.cuda()
+    dX, dW = layer.linear_bwd(*args, 1.0, 1.0, 3) if sampled else layer.dense_bwd(*args)
+    with np.errstate(invalid="ignore"):
+        assert same_kind(np64(dX), np64(dY) @ np64(W)) and same_kind(np64(dW), np64(dY).T @ np64(X))
     layer.close()
