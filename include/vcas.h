@@ -54,8 +54,9 @@ typedef enum { VCAS_DTYPE_F32 = 0, VCAS_DTYPE_BF16 = 1 } vcas_dtype;
 
 /* Which kernels compute the two products.  AUTO picks the tensor-core (tcgen05) kernels for
  * bf16 layers whose d_in and d_out are multiples of 64; fp32 layers and other widths run on the tensor
- * cores too, with operands cut into bf16 parts whose products are summed to fp32 precision.  FMA forces the
- * fp32-FMA kernels. */
+ * cores too, with operands cut into bf16 parts whose products are summed to fp32 precision (if the workspace for
+ * these does not fit the device, and for tensors that are not 16-byte aligned, on the fp32-FMA kernels).  FMA
+ * forces the fp32-FMA kernels. */
 typedef enum { VCAS_GEMM_AUTO = 0, VCAS_GEMM_FMA = 1, VCAS_GEMM_TENSOR = 2 } vcas_gemm_path;
 
 typedef struct {

@@ -252,7 +252,16 @@ int vcas_create(vcas_handle* out, const vcas_layer_desc* desc, const vcas_config
   h->max_units = h->split_path ? split_max_units(*desc, h->num_sms) : 2 * h->num_sms;
   if ((h->tensor_path || h->split_path) && major != 10) { delete h; return VCAS_ERR_CUDA; }
   h->bytes = layout(h, nullptr);
-  if (cudaMalloc(&h->base, h->bytes) != cudaSuccess) {
+  cudaError_t got = cudaMalloc(&h->base, h->bytes);
+  if (got != cudaSuccess && h->split_path) {
+    // the cut operands (12 bytes per element of dY and X in an fp32 layer) do not fit: the FMA kernels need none
+    cudaGetLastError();
+    h->split_path = false;
+    h->max_units = 2 * h->num_sms;
+    h->bytes = layout(h, nullptr);
+    got = cudaMalloc(&h->base, h->bytes);
+  }
+  if (got != cudaSuccess) {
     cudaGetLastError();
     delete h;
     return VCAS_ERR_WORKSPACE;

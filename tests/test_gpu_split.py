@@ -145,3 +145,11 @@ def test_infinite_operands(dtype, sampled):
     with np.errstate(invalid="ignore"):
         assert same_kind(np64(dX), np64(dY) @ np64(W)) and same_kind(np64(dW), np64(dY).T @ np64(X))
     layer.close()
+
+
+def test_layer_whose_parts_do_not_fit_the_device():
+    """Rows for 190 GB of parts: the handle is made all the same, with the workspace of the FMA kernels."""
+    vbuild.build()
+    layer = vb.Layer(512, 2048, 4096, 11008, F32)
+    assert layer.workspace_bytes() < 8 * 2**30
+    layer.close()
