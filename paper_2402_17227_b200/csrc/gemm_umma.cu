@@ -967,7 +967,10 @@ void best_pair(const Cand* c1, int n1, int ctas1, const Cand* c2, int n2, int ct
     const bool split1 = c1[i].plan.mh == 3;
     const long g1 = split1 || c1[i].units > ctas1 ? ctas1 : c1[i].units;
     // The kernels in front of the second product share the SMs with the first: on the BERT-base layer the call takes 31 us
-    // with 30 CTAs of the first product and 34 with 120, although these finish earlier.
+    // with 30 CTAs of the first product and 34 with 120, although these finish earlier.  Over seven layer shapes at eight
+    // ratio pairs the chosen pair is 1.2 % off the best of 42 forced ones on average and 7.8 % at worst; without this term
+    // 1.7 % and 9.2 %.  It only decides among the pairs of small layers: limited to the latencies of those kernels (4 us
+    // at most) it gives the same pairs in 55 of the 56.
     offset = alone_offset * (1.0 + 0.25 * (double)g1 / num_sms);
     const double d1 = (split1 ? c1[i].alone : (double)((c1[i].units + g1 - 1) / g1) * c1[i].unit) + KERNEL_US;
     for (int j = 0; j < n2; ++j) {
