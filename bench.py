@@ -642,6 +642,27 @@ def kernel_run(args):
     layer.close()
 
 
+def shortened(v):
+    """The same report in fewer characters, so that the one line it goes into stays within 12 KB: numbers to four digits, lists
+    of like records as a table, long lists of numbers by their ends."""
+    if isinstance(v, float):
+        return float(f"{v:.4g}")
+    if isinstance(v, dict):
+        return {k: shortened(x) for k, x in v.items()}
+    if isinstance(v, list) and len(v) > 2 and all(isinstance(x, dict) for x in v):
+        def flat(d, prefix=""):
+            return {k2: x2 for k, x in d.items() for k2, x2 in (flat(x, prefix + k + ".") if isinstance(x, dict) else
+                                                                {prefix + k: x}).items()}
+        rows = [flat(shortened(x)) for x in v]
+        if all(list(r) == list(rows[0]) for r in rows):
+            return {"columns": list(rows[0]), "rows": [list(r.values()) for r in rows]}
+    if isinstance(v, list) and len(v) > 16 and all(isinstance(x, (int, float)) for x in v):
+        return {"first": shortened(v[0]), "last": shortened(v[-1]), "min": shortened(min(v)), "max": shortened(max(v)), "count": len(v)}
+    if isinstance(v, (list, tuple)):
+        return [shortened(x) for x in v]
+    return v
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -967,7 +988,9 @@ def main():
     }
     if not args.no_cpu_baseline and world == 1:
         line["cpu_baseline"] = cpu_baseline(case, RHO, NU, reps=3)
-    print(json.dumps(line))
+    for key in ("stages", "other_workloads", "roofline", "adaptation_state"):
+        line[key] = shortened(line[key])
+    print(json.dumps(line, separators=(",", ":")))
     if world > 1:
         dist.destroy_process_group()
 

@@ -320,7 +320,7 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     }
   }
   __syncwarp();
-  pdl_trigger();       // not earlier: the adding CTAs would hold the SMs that the call's other branch needs
+  pdl_trigger();       // by each warp as it leaves its loop; the loading warp, the first to be done, speaks for the CTA
   tc_fence_before();
   __syncthreads();
   if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem_base, 2 * BN); }

@@ -50,7 +50,7 @@ struct SmemLayout {
   uint64_t* tmem_full;
   uint64_t* tmem_empty;
   uint64_t* q_full;   // work queue (unsliced instance): slot holds a work item
-  uint64_t* q_empty;  // ... slot has been read by the MMA thread and the 128 epilogue threads
+  uint64_t* q_empty;  // ... slot has been read by the MMA warp and the 256 epilogue threads
   uint32_t* tmem_holder;
   int* abort_flag;
   int* flag;          // epilogue broadcast slot

@@ -696,8 +696,9 @@ cudaError_t run_probe(Handle* h, const ProbeMaps& maps, const ProbeParams& P, in
 
 }  // namespace
 
-// Shorter data would leave the steps of 64 rows partly empty, and every datum costs a pass of the epilogue over its tile;
-// the scores of Eq. 3 must fit a CTA's shared memory.
+// Shorter data leave the steps of 64 rows partly empty.  4096 rows, 768 -> 3072, M = 4, here and draw by draw: 244 and 709 us
+// with T = 128, 267 and 690 with 64, 417 and 667 with 32, 733 and 697 with 16; 512 rows, 256 -> 256, M = 2: 37 and 119 with
+// 32, 38 and 121 with 16.  The line at whole steps is on the safe side.  The scores of Eq. 3 must fit a CTA's shared memory.
 bool probe_fused_ok(const Handle* h, int M) {
   return h->tensor_path && h->desc.T >= PROBE_MIN_T && (long)h->desc.N * h->desc.T <= SAMPLE_W_SMEM_ROWS && M * (M + 2) <= PARTIAL_SLOTS;
 }

@@ -1,7 +1,8 @@
 // Keep probabilities, Philox Bernoulli masks and compaction for SampleA and SampleW
 // (Sec. 4.1, 4.2).  Everything stays on the device: the kept counts are written to the workspace
 // and read by the product kernels.  The stage is a chain of small kernels:
-//   sample_a_kernel   one CTA: ||G_n||_F, p_n, mask, kept / dropped data (the dX product can start here);
+//   sample_a_kernel   ||G_n||_F on a few CTAs, the last of which draws: p_n, mask, kept / dropped data (the dX product can
+//                     start here);
 //   scores_x_kernel   (score.cu) many CTAs: leverage scores and uniforms of the rows of kept data;
 //   sample_w_kernel   one CTA, scores in shared memory: the water-filling for q = min(1, c w) - a handful
 //                     of block-wide sums - then the masks' counts per chunk of 32 rows and their prefix sums;
