@@ -4,11 +4,12 @@
 // same loads of X, the gradients of the draws, G_act,j = sum over the data kept in draw j of bf16(dY_n / p_n)^T X_n, each in an
 // accumulator of its own, and adds up the squares of G_act,j - G_s: no G_act is ever written.  The rows are rescaled and
 // rounded as in the sampled backward, whose gradients V_act speaks about; p_n belongs to the batch and not to the draw, so
-// they are made once for all draws, and a draw is only the list of the data that it accumulates.
+// they are made once for all draws, and a draw is only the list of the data that it accumulates.  The accumulators are added
+// up in fp32 registers every 1024 rows: tcgen05 truncates, and over 32768 rows in TMEM V_s lost 7e-5 of itself (2e-6 so).
 // (G_act,j as a sum of the data's exact products weighted with 1 / p_n needs one product per batch, but its V_act was up to
 // 5e-4 off: the rounding moves all values of a datum by the same 1e-4, which does not average out.)
-// Measured on B200, against a chain of launches and a product per draw (probe.cu): 4096 rows, 768 -> 3072, M = 4: 709 -> 238 us;
-// 16384 rows, 4096 -> 128 of 11008, M = 2: 538 -> 276 us; 640 rows, 128 -> 128, M = 2, rho = 0.8: 145 -> 39 us.
+// Measured on B200, against a chain of launches and a product per draw (probe.cu): 4096 rows, 768 -> 3072, M = 4: 709 -> 254 us;
+// 16384 rows, 4096 -> 128 of 11008, M = 2: 538 -> 283 us; 640 rows, 128 -> 128, M = 2, rho = 0.8: 145 -> 39 us.
 //
 // Launches per group: norms of the rows of dY and X (which also gathers the sampled columns of dY), one CTA per draw for p
 // and mask, one CTA per draw for Eq. 3 (beside the product, on the side stream), the rescaled rows, the product, the moments
@@ -25,16 +26,17 @@ namespace {
 
 constexpr int PROBE_MIN_T = 64;              // shortest data served: one step of the contraction
 constexpr int PG = 4;                        // most batches a launch serves
-constexpr int PROBE_THREADS = 10 * 32;       // warps 0-7 read the accumulators, 8 loads, 9 issues
+constexpr int PROBE_THREADS = 12 * 32;       // warps 0-7 add up, 8 loads, 9 issues, 10 and 11 fill the warpgroup
 constexpr int ACC_THREADS = 256;
 constexpr int PBN = 128;                     // tile columns
-constexpr int PACC = 512 / PBN;              // accumulators in TMEM
+constexpr int PD = 2;                        // draws of a round
+constexpr int FLUSH = 16;                    // steps that an accumulator takes before fp32 registers add it up
 constexpr int PK = 64;                       // rows of a step
 constexpr int PCHUNK = 64 * PK * 2;          // 64 columns of a step
 constexpr int PA_BYTES = BM / 64 * PCHUNK;   // 128 columns of dY, or of its rescaled rows
 constexpr int PSTAGE = 2 * PA_BYTES + PBN / 64 * PCHUNK;
 constexpr int PSTAGES = 4;
-constexpr int PMASKS = 16384;                // bytes of the masks of a launch
+constexpr int PMASKS = 28672;                // bytes of the masks of a launch
 constexpr int PSMEM = PSTAGES * PSTAGE + 1024 /*alignment slack*/ + 256 /*barriers*/ + PMASKS;
 
 // What a group of batches leaves for its product: a block per batch.
@@ -272,11 +274,9 @@ __device__ __forceinline__ ProbeUnit probe_unit(const ProbeParams& P, int u) {
   w.tile = t - w.g * P.tiles;
   return w;
 }
-// A unit works in rounds, as many accumulators at a time as TMEM holds: round 0 takes G_s and the first draws, the others draws
-// alone.  The draws of round r, and where the results of its accumulators go (0: G_s, 1 + j: draw j).
-__device__ __forceinline__ int round_first(int r) { return r == 0 ? 0 : r * PACC - 1; }
-__device__ __forceinline__ int round_draws(int r, int M) { return min(r == 0 ? PACC - 1 : PACC, M - round_first(r)); }
-__host__ __device__ __forceinline__ int rounds_of(int M) { return (M + PACC) / PACC; }
+// A unit works in rounds, two draws at a time, the first beside G_s: the sums that the registers hold.
+__device__ __forceinline__ int round_draws(int r, int M) { return min(PD, M - PD * r); }
+__host__ __device__ __forceinline__ int rounds_of(int M) { return (M + PD - 1) / PD; }
 // The steps of a slice of a round: `left` steps from step kb of datum n on.  Round 0 runs over all data, the others over those
 // that any of their draws kept.  mask: [N rounded up to 4] the draws of the round that kept the datum, a bit each; kept: the
 // number of data with a mask.
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(PROBE_THREADS, 1)
 probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ ProbeParams P) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_begun;               // the accumulators of the round that a product has written, a bit each
-  __shared__ int s_kept[PG * 16];            // [batch][round] data with a mask
+  __shared__ int s_kept[PG * 32];            // [batch][round] data with a mask
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(base + PSTAGES * PSTAGE);
   uint64_t* empty = full + PSTAGES;
@@ -363,8 +363,8 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
   const int rounds = rounds_of(P.M), n_pad = (P.N + 3) & ~3;
   pdl_wait();
   for (int i = warp; i < P.batches * rounds; i += PROBE_THREADS / 32) {
-    const int g = i / rounds, r = i - g * rounds, first = round_first(r), draws = round_draws(r, P.M);
-    const uint8_t* keep = P.keep[g] + (size_t)first * P.N;
+    const int g = i / rounds, r = i - g * rounds, draws = round_draws(r, P.M);
+    const uint8_t* keep = P.keep[g] + (size_t)(PD * r) * P.N;
     int kept = 0;
     for (int n = lane; n < n_pad; n += 32) {
       uint32_t m = 0;
@@ -381,6 +381,10 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
   tc_fence_after();
   const uint32_t tmem_base = *(volatile uint32_t*)tmem_holder;
 
+  // The launch gives every thread 168 registers, 64512 in all.  Three sums of 64 columns need more: the two accumulating
+  // warpgroups take 2 x 128 x 224 = 57344, the third keeps 128 x 56 = 7168.
+  if (warp >= 8) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
   if (warp == 8) {
     // ------------------------------------------------------------------------- TMA producer
     const bool leader = elect_one();
@@ -451,22 +455,38 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
         if (!ok) break;
         tc_fence_after();
         uint32_t begun = 0;
+        int taken = 0;
+        auto hand_over = [&]() {                 // the accumulators, complete when the products so far are
+          if (leader) {
+            *(volatile uint32_t*)&s_begun = begun;
+            mbar_arrive(acc_full);
+            umma_commit(acc_full);
+          }
+          __syncwarp();
+          acc_phase ^= 1u;
+        };
         while (it.left > 0 && ok) {
-          const uint32_t m = __reduce_or_sync(0xffffffffu, (uint32_t)mask[it.n]), todo = r == 0 ? m << 1 | 1u : m;
+          const uint32_t m = __reduce_or_sync(0xffffffffu, (uint32_t)mask[it.n]), todo = m << 1 | (r == 0 ? 1u : 0u);
           const int end = min(P.kT, it.kb + it.left);
           it.left -= end - it.kb;
           for (int kb = it.kb; kb < end; ++kb) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&full[stage], phase, abort_flag, P.status));
+            if (taken == FLUSH) {
+              hand_over();
+              ok = __all_sync(0xffffffffu, mbar_wait(acc_empty, acc_phase ^ 1u, abort_flag, P.status));
+              begun = 0;
+              taken = 0;
+            }
+            ++taken;
+            ok = ok && __all_sync(0xffffffffu, mbar_wait(&full[stage], phase, abort_flag, P.status));
             if (!ok) break;
             tc_fence_after();
             const uint32_t sa = smem_u32(base + stage * PSTAGE) >> 4;
             const uint64_t de = mn_major | (sa + (PA_BYTES >> 4)), db = mn_major | (sa + (2 * PA_BYTES >> 4));
-            const uint64_t d0 = r == 0 ? mn_major | sa : de;
             const int k16 = kb == P.kT - 1 ? last16 : PK / UMMA_K;
 #pragma unroll
-            for (int a = 0; a < PACC; ++a) {
+            for (int a = 0; a < 1 + PD; ++a) {
               if ((todo >> a & 1u) == 0u) continue;
-              const uint64_t dop = a == 0 ? d0 : de;
+              const uint64_t dop = a == 0 ? mn_major | sa : de;
               const uint32_t d = tmem_base + (uint32_t)(a * PBN);
 #pragma unroll
               for (int k = 0; k < PK / UMMA_K; ++k)        // only the steps of 16 rows that hold any
@@ -483,19 +503,15 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
             while (mask[it.n] == 0) ++it.n;
         }
         if (!ok) break;
-        if (leader) {
-          *(volatile uint32_t*)&s_begun = begun;
-          mbar_arrive(acc_full);
-          umma_commit(acc_full);
-        }
-        __syncwarp();
-        acc_phase ^= 1u;
+        hand_over();
       }
     }
     if (leader) drain_products(done, abort_flag, P.status);
     __syncwarp();
+  }
   } else {
     // --------------------------------------------------------------------------------- the sums
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
     const int eq = warp & 3, eg = warp >> 2;       // TMEM lane quarter, half of the columns
     constexpr int CW = PBN / 2;
     const uint32_t taddr = tmem_base + ((uint32_t)(eq * 32) << 16) + (uint32_t)(eg * CW);
@@ -505,56 +521,69 @@ probe_kernel(const __grid_constant__ ProbeMaps maps, const __grid_constant__ Pro
     for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
       const ProbeUnit w = probe_unit(P, u);
       const int r0 = w.tile / P.ntiles * BM, col0 = w.tile % P.ntiles * PBN + eg * CW;
-      float gs[CW];
+      float sum[1 + PD][CW];                       // G_s and the draws of a round
       double act = 0.0;
+#pragma unroll
+      for (int e = 0; e < CW; ++e) sum[0][e] = 0.f;
       for (int r = 0; r < rounds; ++r) {
-        // The lanes of a warp leave together.  No call here: it would put G_s into local memory.
-        ok = __all_sync(0xffffffffu, mbar_wait_spin(acc_full, acc_phase, abort_flag, P.status));
-        if (!ok) break;
-        acc_phase ^= 1u;
-        tc_fence_after();
-        const uint32_t begun = *(volatile uint32_t*)&s_begun;
-        const int accs = round_draws(r, P.M) + (r == 0 ? 1 : 0), first = r == 0 ? 0 : 1 + round_first(r);
-        for (int a = 0; a < accs; ++a) {
-          const bool any = __any_sync(0xffffffffu, (begun >> a & 1u) != 0u);      // the same for the whole warp: no predicates
-          float* part = P.partial + ((size_t)u * (1 + P.M) + first + a) * BM * PBN + scratch_at(eg * (CW / 4), BM, row);
-          float t = 0.f;
 #pragma unroll
-          for (int h = 0; h < CW / 32; ++h) {
-            uint32_t v[32];
-            if (any) {
-              tmem_ld32(taddr + (uint32_t)(a * PBN + h * 32), v);
-            } else {
+        for (int a = 1; a <= PD; ++a)
 #pragma unroll
-              for (int e = 0; e < 32; ++e) v[e] = 0u;
-            }
-            if (P.S > 1) {
+          for (int e = 0; e < CW; ++e) sum[a][e] = 0.f;
+        int parts = (round_steps(s_mask + (w.g * rounds + r) * n_pad, s_kept[w.g * rounds + r], P.N, P.kT, r, P.S, w.slice).left + FLUSH - 1) / FLUSH;
+        do {
+          // The lanes of a warp leave together.  No call here: it would put the sums into local memory.
+          ok = __all_sync(0xffffffffu, mbar_wait_spin(acc_full, acc_phase, abort_flag, P.status));
+          if (!ok) break;
+          acc_phase ^= 1u;
+          tc_fence_after();
+          const uint32_t begun = *(volatile uint32_t*)&s_begun;
 #pragma unroll
-              for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<uint4*>(part + scratch_at(h * 8 + e / 4, BM, 0)) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-            } else if (first + a == 0) {
+          for (int a = 0; a <= PD; ++a) {
+            if (!__any_sync(0xffffffffu, (begun >> a & 1u) != 0u)) continue;      // the same for the whole warp: no predicates
 #pragma unroll
-              for (int e = 0; e < 32; ++e) gs[h * 32 + e] = __uint_as_float(v[e]);
-            } else {
+            for (int h = 0; h < CW / 16; ++h) {
+              uint32_t v[16];
+              tmem_ld16(taddr + (uint32_t)(a * PBN + h * 16), v);
 #pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                const float x = __uint_as_float(v[e]) - gs[h * 32 + e];
-                t = fmaf(x, x, t);
-              }
+              for (int e = 0; e < 16; ++e) sum[a][h * 16 + e] += __uint_as_float(v[e]);
             }
           }
-          act += (double)t;
-        }
-        // one arrival per warp: the arrivals of all threads at one barrier are served one after the other
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(acc_empty);
-        if (r == 0 && P.S == 1 && r0 + row < P.d_out) {
-          const int rows = gs_rows(P, r0);
-          float* out = P.gs + w.g * P.gs_stride + gs_at(P, r0, rows, row, col0);
+          // one arrival per warp: the arrivals of all threads at one barrier are served one after the other
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_empty);
+        } while (--parts > 0);
+        if (!ok) break;
+        const int draws = round_draws(r, P.M);
+        if (P.S > 1) {
 #pragma unroll
-          for (int e = 0; e < CW; e += 4, out += rows * 4)
-            if (col0 + e < P.d_in) *reinterpret_cast<float4*>(out) = make_float4(gs[e], gs[e + 1], gs[e + 2], gs[e + 3]);
+          for (int a = 0; a <= PD; ++a) {
+            if (a == 0 ? r > 0 : a > draws) continue;
+            float* part = P.partial + ((size_t)u * (1 + P.M) + (a == 0 ? 0 : PD * r + a)) * BM * PBN + scratch_at(eg * (CW / 4), BM, row);
+#pragma unroll
+            for (int e = 0; e < CW; e += 4)
+              *reinterpret_cast<float4*>(part + scratch_at(e / 4, BM, 0)) = make_float4(sum[a][e], sum[a][e + 1], sum[a][e + 2], sum[a][e + 3]);
+          }
+        } else {
+#pragma unroll
+          for (int a = 1; a <= PD; ++a) {
+            if (a > draws) break;
+            float t = 0.f;
+#pragma unroll
+            for (int e = 0; e < CW; ++e) {
+              const float x = sum[a][e] - sum[0][e];
+              t = fmaf(x, x, t);
+            }
+            act += (double)t;
+          }
+          if (r == 0 && r0 + row < P.d_out) {
+            const int rows = gs_rows(P, r0);
+            float* out = P.gs + w.g * P.gs_stride + gs_at(P, r0, rows, row, col0);
+#pragma unroll
+            for (int e = 0; e < CW; e += 4, out += rows * 4)
+              if (col0 + e < P.d_in) *reinterpret_cast<float4*>(out) = make_float4(sum[0][e], sum[0][e + 1], sum[0][e + 2], sum[0][e + 3]);
+          }
         }
       }
       if (!ok) break;
@@ -696,9 +725,9 @@ cudaError_t run_probe(Handle* h, const ProbeMaps& maps, const ProbeParams& P, in
 
 }  // namespace
 
-// Shorter data leave the steps of 64 rows partly empty.  4096 rows, 768 -> 3072, M = 4, here and draw by draw: 244 and 709 us
-// with T = 128, 267 and 690 with 64, 417 and 667 with 32, 733 and 697 with 16; 512 rows, 256 -> 256, M = 2: 37 and 119 with
-// 32, 38 and 121 with 16.  The line at whole steps is on the safe side.  The scores of Eq. 3 must fit a CTA's shared memory.
+// Shorter data leave the steps of 64 rows partly empty.  4096 rows, 768 -> 3072, M = 4, here and draw by draw: 251 and 709 us
+// with T = 128, 276 and 690 with 64, 438 and 653 with 32, 794 and 687 with 16; 512 rows, 256 -> 256, M = 2: 37 and 119 with
+// 32, 39 and 121 with 16.  The line at whole steps is on the safe side.  The scores of Eq. 3 must fit a CTA's shared memory.
 bool probe_fused_ok(const Handle* h, int M) {
   return h->tensor_path && h->desc.T >= PROBE_MIN_T && (long)h->desc.N * h->desc.T <= SAMPLE_W_SMEM_ROWS && M * (M + 2) <= PARTIAL_SLOTS;
 }

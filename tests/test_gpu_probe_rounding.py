@@ -36,3 +36,17 @@ def test_v_act_of_rounded_rows(N, T, d_in, d_out, M, rows, rho):
     assert np.array_equal(layer.variance_probe(Xs, dYs, W, rho, 0.5, 0.75, 42).cpu().numpy(), out)
     assert layer.device_status() == 0
     layer.close()
+
+
+def test_long_contractions_do_not_drift():
+    """Accumulation in TMEM truncates, 2^-25 of the sum per 16 rows on average: over the 32768 rows of these unsliced tiles V_s
+    would lose 6e-5 (twice the gradient's share).  Sums of 1024 rows, added up in fp32, lose 2e-6 each: bound 1e-5."""
+    vbuild.build()
+    N, T, d_in, d_out = 16, 2048, 512, 4096
+    case = inputs.LayerCase("pl", N, T, d_in, d_out, torch.bfloat16, 0.0, 1.0, 0.3, 0.3)
+    batches = [inputs.make_layer(case, batch=b, device="cuda") for b in range(2)]
+    layer = vb.Layer(N, T, d_in, d_out, torch.bfloat16, vb.GEMM_TENSOR)
+    out = layer.variance_probe([b[0] for b in batches], [b[1] for b in batches], batches[0][2], 0.3, 0.5, 0.75, 42)
+    G = [b[1].double().T @ b[0].double() for b in batches]
+    assert float(out[0]) == pytest.approx(float(((G[0] - G[1]) ** 2).sum()) / 2, rel=1e-5)
+    layer.close()
