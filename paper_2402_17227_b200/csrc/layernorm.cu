@@ -242,8 +242,7 @@ __global__ void __launch_bounds__(256) ln_row_kernel(LnParams P) {
       for (int e = 0; e < VN; ++e) zero[e] = 0.f;
       L::pack(zero, z);
       for (int j = lane; j < nv; j += 32) reinterpret_cast<V*>((T*)P.dX + r * d)[j] = z;
-      if (P.a_out != nullptr)
-        for (int j = lane; j < P.a_parts; j += 32) P.a_out[r * P.a_parts + j] = 0.f;
+      if (P.a_out != nullptr && lane < P.a_parts) P.a_out[r * P.a_parts + lane] = 0.f;
       continue;
     }
     const int k = c / Tn;
@@ -297,12 +296,14 @@ __global__ void __launch_bounds__(256) ln_row_kernel(LnParams P) {
       reinterpret_cast<V*>((T*)P.dX + r * d)[j] = ov;
     }
     sq = warp_sum(sq);
+    // the first 32 parts; a loop over all of them here left fewer loads in flight above (8192 columns in fp32: 90 us, not 78)
     if (lane == 0) {
       P.mu[r] = mean;
       P.rstd[r] = rstd;
+      if (P.a_out != nullptr) P.a_out[r * P.a_parts] = sq;
+    } else if (P.a_out != nullptr && lane < P.a_parts) {
+      P.a_out[r * P.a_parts + lane] = 0.f;
     }
-    if (P.a_out != nullptr)
-      for (int j = lane; j < P.a_parts; j += 32) P.a_out[r * P.a_parts + j] = j == 0 ? sq : 0.f;
   }
 }
 
@@ -363,6 +364,29 @@ __global__ void __launch_bounds__(ADD_WARPS * 32) ln_add_kernel(LnParams P, int 
   }
 }
 
+// The few row ranges of wide rows: one thread per column, the ranges in order.  (ln_add_kernel's CTAs of 1024 threads, 32 columns
+// each, took 2 to 5 us longer for 8200 columns of 17 ranges.)  And the parts of the rows' square-norms past the 32 that the row
+// kernel writes, which are 0.
+__global__ void __launch_bounds__(256) ln_range_add_kernel(LnParams P, int ranges) {
+  pdl_wait();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, which = i / P.d, col = i - which * P.d;
+  if (P.a_out != nullptr && P.a_parts > 32) {
+    const int more = P.a_parts - 32, kept = P.counts[0] * P.T;
+    const long total = (long)(P.skip_dropped ? kept : P.N * P.T) * more;
+    for (long e = i; e < total; e += (long)gridDim.x * blockDim.x) {
+      const int c = (int)(e / more), m = c < kept ? c : c - kept, k = m / P.T;
+      const size_t r = (size_t)(c < kept ? P.idxA : P.dropA)[k] * P.T + (m - k * P.T);
+      P.a_out[r * P.a_parts + 32 + (e - (long)c * more)] = 0.f;
+    }
+  }
+  if (which > 1) return;
+  const float* src = P.partial + (size_t)which * ranges * P.d + col;
+  float t = 0.f;
+#pragma unroll 8
+  for (int r = 0; r < ranges; ++r) t += __ldcg(src + (size_t)r * P.d);
+  (which == 0 ? P.dgamma : P.dbeta)[col] = t;
+}
+
 template <typename T, int G>
 cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
   // Two CTAs per SM, fewer when there are fewer rows than row groups or the scratch (4 d^2 floats) is small
@@ -388,7 +412,7 @@ cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
   const long blocks = (rows + 7) / 8 < (1l << 20) ? (rows + 7) / 8 : (1l << 20);
   cudaError_t e = launch_after(ln_row_kernel<T>, dim3((unsigned)blocks), dim3(256), 0, st, P);
   if (e == cudaSuccess) e = launch_after(ln_col_kernel<T>, dim3(col_blocks, chunks), dim3(256), 0, st, P);
-  if (e == cudaSuccess) e = launch_after(ln_add_kernel, dim3(2 * ((P.d + 31) / 32)), dim3(ADD_WARPS * 32), 0, st, P, chunks);
+  if (e == cudaSuccess) e = launch_after(ln_range_add_kernel, dim3((unsigned)((2l * P.d + 255) / 256)), dim3(256), 0, st, P, chunks);
   h->launches += 3;
   return e != cudaSuccess ? e : cudaGetLastError();
 }
