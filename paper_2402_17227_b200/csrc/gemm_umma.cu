@@ -387,13 +387,9 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
               tma_load_3d(sa + hh * A_BYTES, &tmA, kb * BK, c0 * BMT + hh * BM, n, &s.full[stage]);
           } else {
             mbar_expect_tx(&s.full[stage], C::STAGE_BYTES);
-#pragma unroll
-            for (int j = 0; j < BMT / 64; ++j)
-              tma_load_2d(sa + j * CHUNK_BYTES, &tmA, c0 * BMT + j * 64, kb * BK, &s.full[stage]);
+            tma_load_3d(sa, &tmA, 0, kb * BK, c0 * (BMT / 64), &s.full[stage]);
           }
-#pragma unroll
-          for (int j = 0; j < BN / 64; ++j)
-            tma_load_2d(sa + C::AT_BYTES + j * CHUNK_BYTES, &tmB, c1 * BN + j * 64, kb * BK, &s.full[stage]);
+          tma_load_3d(sa + C::AT_BYTES, &tmB, 0, kb * BK, c1 * (BN / 64), &s.full[stage]);
           ++filled;
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -829,13 +825,13 @@ __global__ void __launch_bounds__(REDUCE_THREADS) slice_reduce_kernel(GemmParams
 // ------------------------------------------------------------------------------ host side
 // Tile shape and number of contraction slices from a small cost model of the kernel instances (per
 // unit of work, so independent of the layer's shape), fitted to serialised stage times of every tiling
-// on eight layer shapes on B200: a k-block costs about 0.385 / 0.32 / 0.28 us for 256 / 128 / 64 wide
-// 128-row tiles (four products of 0.08 us each at the clock under load; the rest is the hand-over of a stage, so narrow
-// tiles only pay off when they fill more SMs); a unit costs about 2 us of set-up, pipeline fill and output store; a sliced
+// on eight layer shapes on B200: a k-block costs about 0.36 / 0.27 / 0.265 us for 256 / 128 / 64 wide
+// 128-row tiles (0.385 / 0.32 / 0.28 with a load per 64 columns; four products of 0.08 us each at the clock under load; the
+// rest is the fill and the hand-over of a stage, so narrow tiles only pay off when they fill more SMs); a unit costs about 2 us of set-up, pipeline fill and output store; a sliced
 // unit stores its partial tile instead, and the reduction launch that follows adds the slices on all SMs: together
 // about 4 us and 0.05 us per 256-wide unit for the traffic of the partial tiles; a 256 x 256 tile (mh = 2) costs about
 // 0.62 us per k-block for twice the work, and 4.5 us per tile, whose epilogue nothing overlaps.
-constexpr double KB_US[3] = {0.385, 0.32, 0.28}, UNIT_US = 2.0, KB2_US = 0.62, UNIT2_US = 4.5;
+constexpr double KB_US[3] = {0.36, 0.27, 0.265}, UNIT_US = 2.0, KB2_US = 0.62, UNIT2_US = 4.5;
 inline double sliced_us(long units, int bn) { return 4.0 + 0.05 * (double)units * bn / 256.0; }
 struct Cand {
   Plan plan;
@@ -1062,9 +1058,10 @@ cudaError_t run_gemm(Handle* h, const CUtensorMap& a, const CUtensorMap& b, cons
   }
 }
 
+// a1: A for a second launch of 128-row tiles
 template <int MODE>
-cudaError_t run_gemm_bn(Handle* h, const Plan& plan, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
-                        const CUtensorMap& hm, const GemmParams& P, long max_items, int ctas, bool pdl, cudaStream_t st) {
+cudaError_t run_gemm_bn(Handle* h, const Plan& plan, const CUtensorMap& a, const CUtensorMap& a1, const CUtensorMap& b,
+                        const CUtensorMap& c, const CUtensorMap& hm, const GemmParams& P, long max_items, int ctas, bool pdl, cudaStream_t st) {
   if (plan.mh == 3) {
     // whole waves of 256-row tiles, then the remaining tiles as 128-row tiles with a sliced contraction
     // (both launches derive the same division from the device-resident counts)
@@ -1076,7 +1073,7 @@ cudaError_t run_gemm_bn(Handle* h, const Plan& plan, const CUtensorMap& a, const
     if (e != cudaSuccess) return e;
     Q.part = 2;
     Q.split_k = 0;
-    return run_gemm<MODE, 256, 1>(h, a, b, c, hm, Q, (long)ctas, ctas, true, st);
+    return run_gemm<MODE, 256, 1>(h, a1, b, c, hm, Q, (long)ctas, ctas, true, st);
   }
   if (plan.mh == 2) return run_gemm<MODE, 256, 2>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
   switch (plan.bn) {
@@ -1084,6 +1081,17 @@ cudaError_t run_gemm_bn(Handle* h, const Plan& plan, const CUtensorMap& a, const
     case 128: return run_gemm<MODE, 128, 1>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
     default: return run_gemm<MODE, 64, 1>(h, a, b, c, hm, P, max_items, ctas, pdl, st);
   }
+}
+
+// An MN-major operand [rows of the contraction][cols], cols a multiple of 64, as [chunk of 64 columns][row][64]: one load of
+// BK rows x `tile` columns writes its chunks one after the other, as the products' descriptors want them.  With a load per
+// chunk the loading thread issued five or six a stage and was what the 128-row tiles waited for: of 16384 rows, 1024 x 4096,
+// dW took 675 cycles a k-block and now 620 (115 -> 104 us); 4096 rows, 768 x 3072: 36 -> 31 us.
+bool mn_map(CUtensorMap* m, const void* base, int cols, long rows, int tile) {
+  const uint64_t dims[3] = {64, (uint64_t)rows, (uint64_t)(cols / 64)};
+  const uint64_t strides[2] = {(uint64_t)cols * 2, 128};
+  const uint32_t box[3] = {64, BK, (uint32_t)(tile / 64)};
+  return make_map(m, base, 3, dims, strides, box);
 }
 
 void common_params(Handle* h, GemmParams& P, int which) {
@@ -1195,12 +1203,6 @@ cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense,
     if (!make_map(&tmA, dY, 3, dims, strides, box)) return cudaErrorInvalidValue;
   }
   {
-    const uint64_t dims[2] = {(uint64_t)d.d_in, (uint64_t)d.d_out};
-    const uint64_t strides[1] = {(uint64_t)d.d_in * 2};
-    const uint32_t box[2] = {64, BK};
-    if (!make_map(&tmB, W, 2, dims, strides, box)) return cudaErrorInvalidValue;
-  }
-  {
     const uint64_t dims[3] = {(uint64_t)d.d_in, (uint64_t)d.T, (uint64_t)d.N};
     const uint64_t strides[2] = {(uint64_t)d.d_in * 2, (uint64_t)d.T * d.d_in * 2};
     const uint32_t box[3] = {64, (uint32_t)(d.T < 32 ? d.T : 32), 1};
@@ -1230,28 +1232,17 @@ cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense,
                                   rn ? 256 : h->tune_dx_tile_n, rn ? 1 : h->tune_dx_split_k, g.rem_ok && !rn, H != nullptr, cands);
     plan = apply_tile_m(h->tune_dx_tile_m, best_alone(cands, n), g.rem_ok && !rn);
   }
+  if (!mn_map(&tmB, W, d.d_in, d.d_out, plan.bn)) return cudaErrorInvalidValue;
   P.split_k = plan.split;
   // upper bound of work items: every datum kept and split, or every datum a zero tile
   const long max_items = (long)d.N * (plan.mh >= 2 ? chunks2 : chunks) * ((d.d_in + plan.bn - 1) / plan.bn) * plan.split;
-  return run_gemm_bn<MODE_DX>(h, plan, tmA, tmB, tmC, tmH, P, max_items, ctas, true, st);
+  return run_gemm_bn<MODE_DX>(h, plan, tmA, tmA, tmB, tmC, tmH, P, max_items, ctas, true, st);
 }
 
 cudaError_t launch_umma_dw(Handle* h, const void* A_rows, const void* B_rows, int rows_capacity, const int32_t* cnt,
                            int cnt_hint, const Plan* pair_plan, float* dW, cudaStream_t st) {
   const vcas_layer_desc& d = h->desc;
   CUtensorMap tmA, tmB, tmC;
-  {
-    const uint64_t dims[2] = {(uint64_t)d.d_out, (uint64_t)rows_capacity};
-    const uint64_t strides[1] = {(uint64_t)d.d_out * 2};
-    const uint32_t box[2] = {64, BK};
-    if (!make_map(&tmA, A_rows, 2, dims, strides, box)) return cudaErrorInvalidValue;
-  }
-  {
-    const uint64_t dims[2] = {(uint64_t)d.d_in, (uint64_t)rows_capacity};
-    const uint64_t strides[1] = {(uint64_t)d.d_in * 2};
-    const uint32_t box[2] = {64, BK};
-    if (!make_map(&tmB, B_rows, 2, dims, strides, box)) return cudaErrorInvalidValue;
-  }
   {
     const uint64_t dims[2] = {(uint64_t)d.d_in, (uint64_t)d.d_out};
     const uint64_t strides[1] = {(uint64_t)d.d_in * 4};
@@ -1272,9 +1263,14 @@ cudaError_t launch_umma_dw(Handle* h, const void* A_rows, const void* B_rows, in
                                   h->tune_dw_tile_n, h->tune_dw_split_k, rem_ok, false, cands);
     plan = apply_tile_m(h->tune_dw_tile_m, best_alone(cands, n), rem_ok);
   }
+  // the 128-row tiles that follow whole waves of 256-row ones have a map of their own for A
+  CUtensorMap tmA1;
+  if (!mn_map(&tmA, A_rows, d.d_out, rows_capacity, plan.mh >= 2 ? 2 * BM : BM) || !mn_map(&tmB, B_rows, d.d_in, rows_capacity, plan.bn) ||
+      (plan.mh == 3 && !mn_map(&tmA1, A_rows, d.d_out, rows_capacity, BM)))
+    return cudaErrorInvalidValue;
   P.split_k = plan.split;
   const long max_items = (plan.mh >= 2 ? mtiles2 : mtiles) * ((d.d_in + plan.bn - 1) / plan.bn) * plan.split;
-  return run_gemm_bn<MODE_DW>(h, plan, tmA, tmB, tmC, tmC, P, max_items, h->num_sms, true, st);
+  return run_gemm_bn<MODE_DW>(h, plan, tmA, plan.mh == 3 ? tmA1 : tmA, tmB, tmC, tmC, P, max_items, h->num_sms, true, st);
 }
 
 }  // namespace vcas
