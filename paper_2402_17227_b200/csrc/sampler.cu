@@ -299,13 +299,99 @@ struct SampleWParams {
   float nu;
   int sample_w, accumulate_vw;
   int smem_rows;                            // scores that fit the kernel's shared memory
+  int rows;                                 // N T: entries of wc and uc
 };
 
-// SampleW's single-CTA part (Sec. 4.2, Eq. 3).  The n = T * (#kept data) scores sit in shared memory (in
-// global memory beyond smem_rows: same code, slower loads).  1. c with sum_r min(1, c w_r) = nu * n by
-// water-filling: every round is one pass over the scores and one block-wide sum.  2. Eq. 3 at these
-// probabilities (probe only).  3. The number of kept rows in every chunk of 32 rows, and the exclusive
-// prefix sums of these counts: emit_pack_kernel then places every chunk's rows without looking at others.
+// SampleW's single-CTA part (Sec. 4.2, Eq. 3) over the n = T * (#kept data) scores.  1. c with sum_r min(1, c w_r) = nu * n by
+// water-filling: every round is one pass over the scores and one block-wide sum.  2. Eq. 3 at these probabilities (probe only).
+// 3. The number of kept rows in every chunk of 32 rows, and the exclusive prefix sums of these counts: emit_pack_kernel then
+// places every chunk's rows without looking at others.
+//
+// Bound by latencies, not by data.  Up to 16384 scores sit in registers, score j of a thread being entry tid + 1024 j, so that
+// a warp's j-th scores are chunk warp + 32 j; they and their uniforms are read before the number of them is known, which takes
+// one memory latency for all three, and the counts stay in shared memory until they are summed up.  (With the scores in shared
+// memory, the uniforms read when they were needed and the counts written to memory and read back, 1200 scores took 9 us and
+// now 6: 4096 rows, 768 -> 3072, 46.1 -> 44.5 us the call; 960 rows of an fp32 layer, 368 -> 80, 39.5 -> 37.)
+template <int SLOTS>
+__device__ __forceinline__ void sample_w_regs(const SampleWParams& P, const float (&wv)[SLOTS], const uint32_t (&uv)[SLOTS],
+                                              int cntA, int n, WShared* sh, int* s_cnt) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = P.T;
+  int mode = Q_GIVEN;
+  float c = 0.f;
+  if (P.q_in == nullptr && !water_fill_regs<SLOTS>(wv, P.nu * (float)T * (float)cntA, sh, mode, c) && tid == 0)
+    atomicExch(P.status, (int32_t)VCAS_ERR_INTERNAL);
+  const int nchunks = (n + 31) >> 5;
+  float vw = 0.f;
+#pragma unroll
+  for (int j = 0; j < SLOTS; ++j) {
+    const int i = tid + SAMPLER_THREADS * j, ch = warp + 32 * j;
+    if (ch < nchunks) {                            // warp-uniform
+      bool keep = false;
+      if (i < n) {
+        const int k = P.q_in != nullptr ? i / T : 0;
+        const float q = q_of(mode, c, wv[j], P.q_in, P.q_in != nullptr ? P.idxA[k] * T + (i - k * T) : 0);
+        keep = row_kept(P.sample_w, q, uv[j]);
+        if (q > 0.f) vw += (1.0f - q) / q * wv[j] * wv[j];
+      }
+      const unsigned b = __ballot_sync(0xffffffffu, keep);
+      if (lane == 0) s_cnt[ch] = __popc(b);
+    }
+  }
+  __syncthreads();      // the counts are in place, the reduction buffers free again
+  if (P.accumulate_vw) {      // Eq. 3 at these probabilities
+    int dummy = 0;
+    fast_sum(vw, dummy, sh, 0);
+    if (tid == 0) P.acc[1] += (double)vw;
+  }
+  // exclusive prefix sums over the chunk counts (32 SLOTS of them at most): a thread per chunk
+  const int mine = tid < nchunks ? s_cnt[tid] : 0;
+  int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) sh->scan[warp] = incl;
+  __syncthreads();
+  const int wt = sh->scan[lane];
+  const int base = incl - mine + __reduce_add_sync(0xffffffffu, lane < warp ? wt : 0);
+  const int total = __reduce_add_sync(0xffffffffu, wt);
+  if (tid < nchunks) P.chunk_off[tid] = base;
+  if (tid == 0) {
+    P.counts[1] = total;
+    P.fix[0] = c;
+    P.fix[1] = (float)mode;
+  }
+}
+// The scores of the rows that may be among the kept data's (`rows` of them in memory), and their uniforms.
+template <int SLOTS>
+__device__ __forceinline__ void sample_w_small(const SampleWParams& P, WShared* sh, int* s_cnt) {
+  float wv[SLOTS];
+  uint32_t uv[SLOTS];
+#pragma unroll
+  for (int j = 0; j < SLOTS; ++j) {
+    const int i = threadIdx.x + SAMPLER_THREADS * j;
+    wv[j] = i < P.rows ? __ldcg(P.wc + i) : 0.f;
+    uv[j] = i < P.rows && P.sample_w ? __ldcg(P.uc + i) : 0u;
+  }
+  const int cntA = __ldcg(P.counts), n = cntA * P.T;
+#pragma unroll
+  for (int j = 0; j < SLOTS; ++j)
+    if (threadIdx.x + SAMPLER_THREADS * j >= n) wv[j] = 0.f;
+  sample_w_regs<SLOTS>(P, wv, uv, cntA, n, sh, s_cnt);
+}
+
+template <int SLOTS>
+__global__ void __launch_bounds__(SAMPLER_THREADS) sample_w_small_kernel(SampleWParams P) {
+  __shared__ WShared sh;
+  __shared__ int s_cnt[32 * SLOTS];
+  pdl_wait();      // the scores come from the kernel before this one
+  pdl_trigger();
+  sample_w_small<SLOTS>(P, &sh, s_cnt);
+}
+
+// The same for more scores: in shared memory, or in global memory beyond smem_rows (same code, slower loads).
 __global__ void __launch_bounds__(SAMPLER_THREADS) sample_w_kernel(SampleWParams P) {
   extern __shared__ __align__(16) float s_w[];
   __shared__ WShared sh;
@@ -636,6 +722,18 @@ cudaError_t launch_sample_w(Handle* h, const SamplerArgs& a, cudaStream_t st) {
   const Workspace& ws = h->ws;
   const vcas_layer_desc& d = h->desc;
   const long R = (long)d.N * d.T;
+  SampleWParams P;
+  P.wc = ws.wc; P.uc = ws.uc; P.q_in = a.q_in; P.idxA = ws.idxA;
+  P.counts = ws.counts; P.chunk_off = ws.chunk_off; P.fix = ws.fix; P.acc = ws.acc; P.status = ws.status;
+  P.T = d.T; P.nu = a.nu; P.sample_w = a.sample_w; P.accumulate_vw = a.accumulate_vw;
+  P.smem_rows = 0;
+  P.rows = (int)R;
+  h->launches += 1;
+  const dim3 threads(SAMPLER_THREADS);
+  if (R <= 2 * SAMPLER_THREADS) return launch_after(sample_w_small_kernel<2>, dim3(1), threads, 0, st, P);
+  if (R <= 4 * SAMPLER_THREADS) return launch_after(sample_w_small_kernel<4>, dim3(1), threads, 0, st, P);
+  if (R <= 8 * SAMPLER_THREADS) return launch_after(sample_w_small_kernel<8>, dim3(1), threads, 0, st, P);
+  if (R <= 16 * SAMPLER_THREADS) return launch_after(sample_w_small_kernel<16>, dim3(1), threads, 0, st, P);
   // shared memory for the scores: enough for every row when that fits, else the kernel reads global memory
   // whenever the kept rows exceed it
   int rows = (int)(R < SAMPLE_W_SMEM_ROWS ? R : SAMPLE_W_SMEM_ROWS);
@@ -653,13 +751,8 @@ cudaError_t launch_sample_w(Handle* h, const SamplerArgs& a, cudaStream_t st) {
       attr_set[dev].store(true, std::memory_order_release);
     }
   }
-  SampleWParams P;
-  P.wc = ws.wc; P.uc = ws.uc; P.q_in = a.q_in; P.idxA = ws.idxA;
-  P.counts = ws.counts; P.chunk_off = ws.chunk_off; P.fix = ws.fix; P.acc = ws.acc; P.status = ws.status;
-  P.T = d.T; P.nu = a.nu; P.sample_w = a.sample_w; P.accumulate_vw = a.accumulate_vw;
   P.smem_rows = rows;
-  const cudaError_t e = launch_after(sample_w_kernel, dim3(1), dim3(SAMPLER_THREADS), smem, st, P);
-  h->launches += 1;
+  const cudaError_t e = launch_after(sample_w_kernel, dim3(1), threads, smem, st, P);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

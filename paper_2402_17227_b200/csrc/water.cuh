@@ -48,16 +48,9 @@ __device__ __forceinline__ void fast_sum(float& s, int& c, WShared* sh, int pari
   c = __reduce_add_sync(0xffffffffu, sh->part_i[parity][lane]);
 }
 
-// c with sum_i min(1, c w_i) = budget over the n scores w by SAMPLER_THREADS threads: every round is one pass over the
-// scores and one block-wide sum.  Returns false if it has not converged after WATER_ROUNDS rounds.
-__device__ __forceinline__ bool water_fill(const float* w, int n, float budget, WShared* sh, int& mode, float& c) {
-  const int tid = threadIdx.x;
-  float S = 0.f;
-  int nz = 0;
-  for (int i = tid; i < n; i += SAMPLER_THREADS) {
-    const float x = w[i];
-    if (x > 0.f) { S += x; ++nz; }
-  }
+// The fixed point itself; part(c, Su, ks): sum of the positive scores with c w < 1 and number of the others of a thread.
+template <typename Part>
+__device__ __forceinline__ bool water_rounds(float S, int nz, float budget, WShared* sh, int& mode, float& c, Part part) {
   int parity = 0;
   fast_sum(S, nz, sh, parity); parity ^= 1;
   c = 0.f;
@@ -69,12 +62,7 @@ __device__ __forceinline__ bool water_fill(const float* w, int n, float budget, 
   for (int iter = 0; iter < WATER_ROUNDS; ++iter) {
     float Su = 0.f;
     int ks = 0;
-    for (int i = tid; i < n; i += SAMPLER_THREADS) {
-      const float x = w[i];
-      if (x > 0.f) {
-        if (c * x >= 1.0f) ++ks; else Su += x;
-      }
-    }
+    part(c, Su, ks);
     fast_sum(Su, ks, sh, parity); parity ^= 1;
     if (ks == k) return true;
     k = ks;
@@ -84,6 +72,42 @@ __device__ __forceinline__ bool water_fill(const float* w, int n, float budget, 
     }
   }
   return false;
+}
+
+// c with sum_i min(1, c w_i) = budget over the n scores w by SAMPLER_THREADS threads: every round is one pass over the
+// scores and one block-wide sum.  Returns false if it has not converged after WATER_ROUNDS rounds.
+__device__ __forceinline__ bool water_fill(const float* w, int n, float budget, WShared* sh, int& mode, float& c) {
+  const int tid = threadIdx.x;
+  float S = 0.f;
+  int nz = 0;
+  for (int i = tid; i < n; i += SAMPLER_THREADS) {
+    const float x = w[i];
+    if (x > 0.f) { S += x; ++nz; }
+  }
+  return water_rounds(S, nz, budget, sh, mode, c, [&](float at, float& Su, int& ks) {
+    for (int i = tid; i < n; i += SAMPLER_THREADS) {
+      const float x = w[i];
+      if (x > 0.f) {
+        if (at * x >= 1.0f) ++ks; else Su += x;
+      }
+    }
+  });
+}
+// The same over scores in registers, 0 where there are none.
+template <int SLOTS>
+__device__ __forceinline__ bool water_fill_regs(const float (&w)[SLOTS], float budget, WShared* sh, int& mode, float& c) {
+  float S = 0.f;
+  int nz = 0;
+#pragma unroll
+  for (int j = 0; j < SLOTS; ++j)
+    if (w[j] > 0.f) { S += w[j]; ++nz; }
+  return water_rounds(S, nz, budget, sh, mode, c, [&](float at, float& Su, int& ks) {
+#pragma unroll
+    for (int j = 0; j < SLOTS; ++j)
+      if (w[j] > 0.f) {
+        if (at * w[j] >= 1.0f) ++ks; else Su += w[j];
+      }
+  });
 }
 
 }  // namespace
