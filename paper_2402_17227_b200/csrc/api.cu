@@ -337,7 +337,7 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
     VCAS_CUDA(launch_sample_w(h, a, st));
     mark(h, 2, st);
     if (h->tensor_path) {
-      VCAS_CUDA(launch_umma_dx(h, dY, W, false, a.rho, Hpre, dX, a_out, skip_dropped, spare, &px, st));
+      VCAS_CUDA(launch_umma_dx(h, dY, W, false, a.rho, Hpre, dX, a_out, skip_dropped, spare, &px, true, st));
     } else if (plain_dx(h, dY, W, a.rho, Hpre, dX, a_out, false, st) != VCAS_OK) {
       return VCAS_ERR_CUDA;
     }
@@ -355,19 +355,28 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
     }
     mark(h, 5, st);
   } else {
-    // The dX product needs SampleA only: on `st`, the row norms of dY, SampleA and the dX product follow one
-    // another as programmatic dependent launches.  Everything SampleW needs (the norms of the kept rows of X,
-    // the water-filling, the kept-row list and the compact operands) and the dW product run beside the dX
-    // product on the handle's side stream and are joined back before the call's work ends on `st`.
+    // Both products need SampleA; dW also needs what SampleW needs (the norms of the kept rows of X, the water-filling, the
+    // kept-row list and the compact operands).  The two branches run side by side, one on `st`, where its kernels follow the
+    // row norms of dY and SampleA as programmatic dependent launches, the other on the handle's side stream, joined back
+    // before the call's work ends on `st`.
     VCAS_CUDA(launch_rownorm_dy(h, dY, a, st));
     VCAS_CUDA(launch_sample_a(h, a, a.a_in == nullptr, st));
     VCAS_CUDA(cudaEventRecord(h->ev_fork, st));
     VCAS_CUDA(cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
-    if (h->tensor_path) VCAS_CUDA(launch_umma_dx(h, dY, W, false, a.rho, Hpre, dX, a_out, skip_dropped, spare, &px, st));
-    else if (plain_dx(h, dY, W, a.rho, Hpre, dX, a_out, true, st) != VCAS_OK) return VCAS_ERR_CUDA;
-    const int rc = sample_w_and_dw(h, X, dY, a, false, &pw, dW, h->side_stream);
+    // The branch on `st` is the one that ends last.  Small layers: dW's, whose kernels are a chain of latencies (on the side
+    // stream and on `st`: 1.1 GFLOP of dX, 1024 x 1024: 27.0 and 26.1 us; fp32, 0.8, 512 x 512: 33.2 and 31.8; 3.8, 776 x 1000:
+    // 57.8 and 56.4).  Larger ones: dX's (fp32, 7.2, 768 x 768: 47.6 and 49.1; bf16, 24, 768 x 3072: 84 and 89; 554,
+    // 4096 x 11008: 530 and 536).  A call whose join is deferred leaves its dW branch to the side stream.
+    const double dx_flops = 2.0 * a.rho * h->desc.N * h->desc.T * (double)h->desc.d_in * h->desc.d_out *
+                            (h->desc.dtype == VCAS_DTYPE_F32 ? 6.0 : 1.0);
+    const bool dw_first = !defer_join && dx_flops <= 4e9;
+    cudaStream_t sx = dw_first ? h->side_stream : st, sw = dw_first ? st : h->side_stream;
+    if (h->tensor_path) VCAS_CUDA(launch_umma_dx(h, dY, W, false, a.rho, Hpre, dX, a_out, skip_dropped, spare, &px, !dw_first, sx));
+    else if (plain_dx(h, dY, W, a.rho, Hpre, dX, a_out, !dw_first, sx) != VCAS_OK) return VCAS_ERR_CUDA;
+    if (dw_first) VCAS_CUDA(cudaEventRecord(h->ev_join, sx));
+    const int rc = sample_w_and_dw(h, X, dY, a, dw_first, &pw, dW, sw);
     if (rc != VCAS_OK) return rc;
-    VCAS_CUDA(cudaEventRecord(h->ev_join, h->side_stream));
+    if (!dw_first) VCAS_CUDA(cudaEventRecord(h->ev_join, sw));
     if (defer_join) h->join_pending = true;       // dW and the sampling record are complete only after vcas_join
     else VCAS_CUDA(cudaStreamWaitEvent(st, h->ev_join, 0));
   }
@@ -478,7 +487,7 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
   if (split) {
     VCAS_CUDA(launch_split_dx(h, dY, W, true, 1.0f, Hpre, dX, st));
   } else if (h->tensor_path) {
-    VCAS_CUDA(launch_umma_dx(h, dY, W, true, 1.0f, Hpre, dX, nullptr, false, 0, &px, st));
+    VCAS_CUDA(launch_umma_dx(h, dY, W, true, 1.0f, Hpre, dX, nullptr, false, 0, &px, true, st));
   } else {
     VCAS_CUDA(launch_fma_dx(h, dY, W, nullptr, Hpre, dX, st));
   }

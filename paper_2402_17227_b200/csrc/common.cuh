@@ -375,9 +375,10 @@ cudaError_t launch_split_dw(Handle* h, const void* dY, const void* X, bool dense
 // (nullptr: chosen here, for this product alone)
 // a_out: optional [R][a_out_parts(d_in)] partial row square-norms of the stored dX, written by the epilogue
 // skip_dropped: the rows of dropped data are not written (a consumer with the kept-data list never reads them)
+// programmatic: launched as a dependent of the kernel before it in the stream
 cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense, float rho_hint,
                            const void* H, void* dX, float* a_out, bool skip_dropped, int spare_sms,
-                           const Plan* pair_plan, cudaStream_t st);
+                           const Plan* pair_plan, bool programmatic, cudaStream_t st);
 inline int a_out_parts(int d_in) { return 2 * ((d_in + 255) / 256); }    // one per 256-column tile and epilogue group
 // dW = A_rows^T B_rows over the first *cnt rows (A_rows [rows, d_out], B_rows [rows, d_in], bf16)
 // cnt_hint: the expected *cnt, used on the host to pick the tiling

@@ -1193,7 +1193,7 @@ void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spar
 
 cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense, float rho_hint, const void* H,
                            void* dX, float* a_out, bool skip_dropped, int spare_sms, const Plan* pair_plan,
-                           cudaStream_t st) {
+                           bool programmatic, cudaStream_t st) {
   const vcas_layer_desc& d = h->desc;
   CUtensorMap tmA, tmB, tmC, tmH;
   {
@@ -1236,7 +1236,7 @@ cudaError_t launch_umma_dx(Handle* h, const void* dY, const void* W, bool dense,
   P.split_k = plan.split;
   // upper bound of work items: every datum kept and split, or every datum a zero tile
   const long max_items = (long)d.N * (plan.mh >= 2 ? chunks2 : chunks) * ((d.d_in + plan.bn - 1) / plan.bn) * plan.split;
-  return run_gemm_bn<MODE_DX>(h, plan, tmA, tmA, tmB, tmC, tmH, P, max_items, ctas, true, st);
+  return run_gemm_bn<MODE_DX>(h, plan, tmA, tmA, tmB, tmC, tmH, P, max_items, ctas, programmatic, st);
 }
 
 cudaError_t launch_umma_dw(Handle* h, const void* A_rows, const void* B_rows, int rows_capacity, const int32_t* cnt,
