@@ -823,16 +823,17 @@ __global__ void __launch_bounds__(REDUCE_THREADS) slice_reduce_kernel(GemmParams
 }
 
 // ------------------------------------------------------------------------------ host side
-// Tile shape and number of contraction slices from a small cost model of the kernel instances (per
-// unit of work, so independent of the layer's shape), fitted to serialised stage times of every tiling
-// on eight layer shapes on B200: a k-block costs about 0.36 / 0.27 / 0.265 us for 256 / 128 / 64 wide
-// 128-row tiles (0.385 / 0.32 / 0.28 with a load per 64 columns; four products of 0.08 us each at the clock under load; the
-// rest is the fill and the hand-over of a stage, so narrow tiles only pay off when they fill more SMs); a unit costs about 2 us of set-up, pipeline fill and output store; a sliced
-// unit stores its partial tile instead, and the reduction launch that follows adds the slices on all SMs: together
-// about 4 us and 0.05 us per 256-wide unit for the traffic of the partial tiles; a 256 x 256 tile (mh = 2) costs about
-// 0.62 us per k-block for twice the work, and 4.5 us per tile, whose epilogue nothing overlaps.
-constexpr double KB_US[3] = {0.36, 0.27, 0.265}, UNIT_US = 2.0, KB2_US = 0.62, UNIT2_US = 4.5;
-inline double sliced_us(long units, int bn) { return 4.0 + 0.05 * (double)units * bn / 256.0; }
+// Tile shape and number of contraction slices from a small cost model of the kernel instances (per unit of work, so
+// independent of the layer's shape).  Its constants are fitted to the times of whole calls on B200: 14 layer shapes, 1024 to
+// 16384 rows, at eight ratio pairs, 63 forced pairs of tilings each.  Over these the chosen pair is 1.1 % off the best on
+// average and 7 % at worst (1.5 % and 11 % with constants fitted to serialised stages only).  A k-block costs about 0.34 /
+// 0.29 / 0.25 us for 256 / 128 / 64 wide 128-row tiles (four products of 0.08 us each at the clock under load; the rest is
+// the fill and the hand-over of a stage, so narrow tiles only pay off when they fill more SMs); a unit costs about 2 us of
+// set-up, pipeline fill and output store; a sliced unit stores its partial tile instead, and the reduction launch that follows
+// adds the slices on all SMs: together about 3 us and 0.065 us per 256-wide unit for the traffic of the partial tiles; a 256 x
+// 256 tile (mh = 2) costs about 0.65 us per k-block for twice the work, and 2.5 us per tile, whose epilogue nothing overlaps.
+constexpr double KB_US[3] = {0.335, 0.29, 0.245}, UNIT_US = 2.0, KB2_US = 0.65, UNIT2_US = 2.5;
+inline double sliced_us(long units, int bn) { return 3.2 + 0.065 * (double)units * bn / 256.0; }
 struct Cand {
   Plan plan;
   long units;      // (tile, slice) units
@@ -879,7 +880,7 @@ int enumerate_plans(long row_tiles128, long row_tiles256, int n_extent, int kblo
         if (sp < 1) sp = 1;
         // the second launch always runs the sliced instance (its tiles go through the slice exchange even when
         // a contraction ends up in one slice), and costs a launch of its own
-        const double tail = (double)((kblocks + sp - 1) / sp) * KB_US[0] + sliced_us(2 * frac * sp, 256) + 4.0;
+        const double tail = (double)((kblocks + sp - 1) / sp) * KB_US[0] + sliced_us(2 * frac * sp, 256) + 5.2;
         if (n < MAX_CANDS) out[n++] = {{256, 1, 3}, units, wave, (double)(units / num_sms) * wave + tail};
       }
     }
@@ -910,7 +911,7 @@ Plan best_alone(const Cand* c, int n) {
 // up and draws units until none are left.  (Measured on the BERT-base layer: a dense call takes 63 us when the
 // two grids together exceed the SMs and every unit of the second waits for the first, 52 us when the dW product
 // runs as 36 tiles of 256 x 256 beside the 96 CTAs of the dX product.)
-constexpr double KERNEL_US = 4.0;   // launch ramp and exit of a product kernel, on top of its units (timeline measurements)
+constexpr double KERNEL_US = 3.3;   // launch ramp and exit of a product kernel, on top of its units
 
 // Finish time of the second product: `units` units of `unit` us each, ready at `ready`, on the SMs the first
 // product (g1 CTAs, `units1` units of `unit1` us) leaves free.
@@ -963,11 +964,8 @@ void best_pair(const Cand* c1, int n1, int ctas1, const Cand* c2, int n2, int ct
     const bool split1 = c1[i].plan.mh == 3;
     const long g1 = split1 || c1[i].units > ctas1 ? ctas1 : c1[i].units;
     // The kernels in front of the second product share the SMs with the first: on the BERT-base layer the call takes 31 us
-    // with 30 CTAs of the first product and 34 with 120, although these finish earlier.  Over seven layer shapes at eight
-    // ratio pairs the chosen pair is 1.2 % off the best of 42 forced ones on average and 7.8 % at worst; without this term
-    // 1.7 % and 9.2 %.  It only decides among the pairs of small layers: limited to the latencies of those kernels (4 us
-    // at most) it gives the same pairs in 55 of the 56.
-    offset = alone_offset * (1.0 + 0.25 * (double)g1 / num_sms);
+    // with 30 CTAs of the first product and 34 with 120, although these finish earlier.
+    offset = alone_offset * (1.0 + 0.32 * (double)g1 / num_sms);
     const double d1 = (split1 ? c1[i].alone : (double)((c1[i].units + g1 - 1) / g1) * c1[i].unit) + KERNEL_US;
     for (int j = 0; j < n2; ++j) {
       const bool split2 = c2[j].plan.mh == 3;
@@ -1163,15 +1161,15 @@ void plan_products(Handle* h, bool dense, float rho_hint, int cnt_hint, int spar
     const int nw = enumerate_plans((d.d_out + BM - 1) / BM, (d.d_out + 2 * BM - 1) / (2 * BM), d.d_in, kb_w, h->num_sms,
                                    h->max_units, h->tune_dw_tile_n, h->tune_dw_split_k, rem_w, false, cw);
     // A sampled dW product becomes ready later than the dX product by the time of the kernels in front of it
-    // on the side stream (fitted to their ncu durations on three layer shapes): the norms of the kept rows of X
+    // on the side stream (fitted with the costs of the products): the norms of the kept rows of X
     // (HBM-bound), SampleW's single-CTA fixed point over the rows of kept data, and the emit + pack pass, which
     // moves the kept rows of both operands twice.  The dense products start together.
     double offset = 0.0;
     if (!dense) {
       const double rows_a = (double)rho_hint * d.N * d.T;
-      const double scores_us = 4.0 + rows_a * d.d_in * 2.0 / 3.5e6;
-      const double sample_w_us = 6.0 + rows_a * 0.0013;
-      const double pack_us = 6.0 + 2.0 * (double)cnt_hint * (d.d_in + d.d_out) * 2.0 / 3.0e6;
+      const double scores_us = 3.3 + rows_a * d.d_in * 2.0 / 4.0e6;
+      const double sample_w_us = 5.6 + rows_a * 0.00096;
+      const double pack_us = 4.3 + 2.0 * (double)cnt_hint * (d.d_in + d.d_out) * 2.0 / 3.8e6;
       offset = scores_us + sample_w_us + pack_us;
     }
     Plan px, pw;
