@@ -81,14 +81,14 @@ __device__ __forceinline__ size_t dx_row(const SplitParams& P, int c, float& sc)
   sc = P.scaleA != nullptr ? P.scaleA[n] : 1.0f;
   return (size_t)n * P.T + (c - k * P.T);
 }
-// Eight consecutive columns of one output row: rescaled, times GELU', stored.
-template <typename T, int MODE>
+// Eight consecutive columns of one output row: rescaled, times GELU' (GELU: there may be one), stored.
+template <typename T, int MODE, bool GELU>
 __device__ __forceinline__ void finish8(const SplitParams& P, size_t row, float sc, int col, float (&v)[8]) {
   const size_t o = row * (size_t)P.d_in + col;
   if (MODE == MODE_DW) { store8(reinterpret_cast<float*>(P.out) + o, v); return; }
 #pragma unroll
   for (int e = 0; e < 8; ++e) v[e] *= sc;
-  if (P.H != nullptr) {
+  if (GELU && P.H != nullptr) {
     Vec8<T> h;
     h.load(reinterpret_cast<const T*>(P.H) + o);
     float x[8];
@@ -100,13 +100,13 @@ __device__ __forceinline__ void finish8(const SplitParams& P, size_t row, float 
 }
 
 // Four columns of an fp32 output row.
-template <int MODE>
+template <int MODE, bool GELU>
 __device__ __forceinline__ void finish4(const SplitParams& P, int row, float sc, int col, float (&v)[4]) {
   const size_t o = (size_t)row * P.d_in + col;
   if (MODE == MODE_DX) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) v[e] *= sc;
-    if (P.H != nullptr) {
+    if (GELU && P.H != nullptr) {
       const float4 h = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(P.H) + o));
       const float x[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
@@ -121,7 +121,11 @@ __device__ __forceinline__ void finish4(const SplitParams& P, int row, float sc,
 // every store of the product met 32 (fp32 layer of 4096 rows, 768 -> 3072: 98 -> 88 us; bf16, 4950 rows, 776 -> 1000: 65 -> 58).
 __device__ __forceinline__ size_t partial_at(int row, int q) { return (((size_t)(row / 8) * (BN / 4) + q) * 8 + row % 8) * 4; }
 
-template <typename T, int MODE, int PA, int PB>
+// GELU: an instance of its own.  The factor's code stands in the unrolled output loop 128 times, and jumping over it cost a
+// tile more in instruction fetches than its products took: the output of a first 128 x 256 tile of fp32 was 17000 to 34000
+// cycles, of a later one 12000, and is 7200 (fp32: 15834 rows, 368 -> 856 at ratio 0.3, 107.4 -> 101.9 us the call; dense, 9728 rows,
+// 64 -> 944, 83.1 -> 79.5; bf16, 4950 rows, 776 -> 1000, 58.5 -> 57.8).
+template <typename T, int MODE, int PA, int PB, bool GELU>
 __global__ void __launch_bounds__(SPLIT_THREADS, 1)
 split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, SplitParams P) {
   using C = SplitCfg<PA, PB>;
@@ -280,7 +284,7 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           float v[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) v[i] = acc[e + i];
-          finish8<T, MODE>(P, r, sc, col0 + e, v);
+          finish8<T, MODE, GELU>(P, r, sc, col0 + e, v);
         }
       } else {
         // Every eight lanes exchange their rows' pieces of four columns, so that they store 128 bytes of one row at a time (a
@@ -313,7 +317,7 @@ split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           for (int i = 0; i < 8; ++i) {
             const int r = __shfl_sync(0xffffffffu, target, (lane & 24) + i);
             const float f = __shfl_sync(0xffffffffu, sc, (lane & 24) + i);
-            if (r >= 0 && col < P.d_in) finish4<MODE>(P, r, f, col, x[i]);
+            if (r >= 0 && col < P.d_in) finish4<MODE, GELU>(P, r, f, col, x[i]);
           }
         }
       }
@@ -352,7 +356,7 @@ __global__ void __launch_bounds__(ADD_THREADS) split_add_kernel(SplitParams P) {
     }
     float sc = 1.0f;
     const size_t r = MODE == MODE_DX ? dx_row(P, row, sc) : (size_t)row;
-    finish8<T, MODE>(P, r, sc, col, v);
+    finish8<T, MODE, true>(P, r, sc, col, v);
   }
 }
 
@@ -436,22 +440,22 @@ int split_slices(const Handle* h, long tiles, int k, double kblock_us) {
   return best;
 }
 
-template <typename T, int MODE, int PA, int PB>
+template <typename T, int MODE, int PA, int PB, bool GELU = false>
 cudaError_t run_split(Handle* h, const CUtensorMap& a, const CUtensorMap& b, SplitParams& P, long exp_tiles, long max_tiles,
                       int k, long max_rows, bool programmatic, cudaStream_t st) {
   static std::atomic<bool> attr_set[64];
   using C = SplitCfg<PA, PB>;
   if (h->device < 0 || h->device >= 64) return cudaErrorInvalidDevice;
   if (!attr_set[h->device].load(std::memory_order_acquire)) {
-    const cudaError_t e = cudaFuncSetAttribute(split_kernel<T, MODE, PA, PB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               C::SMEM_BYTES);
+    const cudaError_t e = cudaFuncSetAttribute(split_kernel<T, MODE, PA, PB, GELU>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     attr_set[h->device].store(true, std::memory_order_release);
   }
   P.slices = split_slices(h, exp_tiles, k, PA * PB == 9 ? 1.7 : (PA * PB == 3 ? 0.9 : 0.55));
   long grid = max_tiles * P.slices;
   if (grid > h->num_sms) grid = h->num_sms;
-  cudaError_t e = launch_maybe_after(programmatic, split_kernel<T, MODE, PA, PB>, dim3((unsigned)grid), dim3(SPLIT_THREADS),
+  cudaError_t e = launch_maybe_after(programmatic, split_kernel<T, MODE, PA, PB, GELU>, dim3((unsigned)grid), dim3(SPLIT_THREADS),
                                      C::SMEM_BYTES, st, a, b, P);
   h->launches += 1;
   if (e == cudaSuccess && P.slices > 1) {
@@ -536,6 +540,10 @@ cudaError_t launch_split_dx(Handle* h, const void* dY, const void* W, bool dense
   const long max_tiles = (R + BM - 1) / BM * nt;
   const long exp_rows = dense ? R : (long)((double)rho_hint * (double)R) + 1;
   const long exp_tiles = (exp_rows + BM - 1) / BM * nt;
+  if (Hpre != nullptr) {
+    if (fp32) return run_split<float, MODE_DX, 3, 3, true>(h, a, b, P, exp_tiles, max_tiles, d.d_out, R, true, st);
+    return run_split<__nv_bfloat16, MODE_DX, 1, 1, true>(h, a, b, P, exp_tiles, max_tiles, d.d_out, R, !dense, st);
+  }
   if (fp32) return run_split<float, MODE_DX, 3, 3>(h, a, b, P, exp_tiles, max_tiles, d.d_out, R, true, st);
   return run_split<__nv_bfloat16, MODE_DX, 1, 1>(h, a, b, P, exp_tiles, max_tiles, d.d_out, R, !dense, st);
 }
