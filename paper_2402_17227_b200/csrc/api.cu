@@ -359,8 +359,7 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
     // kept-row list and the compact operands).  The two branches run side by side, one on `st`, where its kernels follow the
     // row norms of dY and SampleA as programmatic dependent launches, the other on the handle's side stream, joined back
     // before the call's work ends on `st`.
-    VCAS_CUDA(launch_rownorm_dy(h, dY, a, st));
-    VCAS_CUDA(launch_sample_a(h, a, a.a_in == nullptr, st));
+    VCAS_CUDA(launch_norms_sample_a(h, dY, a, st));
     VCAS_CUDA(cudaEventRecord(h->ev_fork, st));
     VCAS_CUDA(cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
     // The branch on `st` is the one that ends last.  Small layers: dW's, whose kernels are a chain of latencies (on the side
@@ -437,8 +436,7 @@ int vcas_layernorm_bwd(vcas_handle hh, const void* X, const void* gamma, const v
   }
   cudaStream_t st = S(stream);
   if (join_pending(h, st) != VCAS_OK) return VCAS_ERR_CUDA;
-  VCAS_CUDA(launch_rownorm_dy(h, dY, a, st));
-  VCAS_CUDA(launch_sample_a(h, a, a.a_in == nullptr, st));
+  VCAS_CUDA(launch_norms_sample_a(h, dY, a, st));
   VCAS_CUDA(launch_layernorm_bwd(h, X, gamma, dY, eps, dX, a_out, skip, dgamma, dbeta, st));
   return VCAS_OK;
 }
@@ -512,8 +510,7 @@ int vcas_score(vcas_handle hh, const void* X, const void* dY, float rho, float n
   cudaStream_t st = S(stream);
   if (join_pending(h, st) != VCAS_OK) return VCAS_ERR_CUDA;
   const SamplerArgs a = sampler_args(rho, nu, seed);
-  VCAS_CUDA(launch_rownorm_dy(h, dY, a, st));
-  VCAS_CUDA(launch_sample_a(h, a, true, st));
+  VCAS_CUDA(launch_norms_sample_a(h, dY, a, st));
   VCAS_CUDA(launch_scores_x(h, X, a, true, st));
   VCAS_CUDA(launch_sample_w(h, a, st));
   VCAS_CUDA(launch_emit_pack(h, dY, X, a, false, st));

@@ -1,6 +1,7 @@
 // Keep probabilities, Philox Bernoulli masks and compaction for SampleA and SampleW
 // (Sec. 4.1, 4.2).  Everything stays on the device: the kept counts are written to the workspace
 // and read by the product kernels.  The stage is a chain of small kernels:
+//   norms_sample_a_kernel  of few rows: their norms (else score.cu) and what follows in one launch;
 //   sample_a_kernel   ||G_n||_F on a few CTAs, the last of which draws: p_n, mask, kept / dropped data (the dX product can
 //                     start here);
 //   scores_x_kernel   (score.cu) many CTAs: leverage scores and uniforms of the rows of kept data;
@@ -10,6 +11,7 @@
 // Only the scalar fixed point and a scan over R/32 counts run on a single SM.
 #include <atomic>
 
+#include "rows.cuh"
 #include "split.cuh"
 #include "water.cuh"
 
@@ -167,6 +169,32 @@ __device__ __forceinline__ float datum_sqnorm_cta(const float* an, int len, floa
   return r;
 }
 
+// The number of alive data.  A caller's list is not trusted: a length outside [0, N] or an entry outside [0, N) is reported as
+// VCAS_ERR_BAD_ARG in the status word and not followed.
+__device__ __forceinline__ int alive_data(const SampleAParams& P) {
+  if (P.alive == nullptr) return P.N;
+  const int nd = *P.alive_cnt;
+  if (nd >= 0 && nd <= P.N) return nd;
+  if (threadIdx.x == 0 && blockIdx.x == 0) atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
+  return min(max(nd, 0), P.N);
+}
+// p, the masks and the lists from the data's norms, by the first warp of a CTA; the others store the norms.
+template <int SLOTS>
+__device__ __forceinline__ void draw_a(const SampleAParams& P, const float* s_g) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp == 0) {
+    SampleAOut o;
+    o.p = P.p; o.scaleA = P.scaleA; o.idxA = P.idxA; o.dropA = P.dropA; o.idx_copy = P.kept_out;
+    const int kept = sample_a_warp<SLOTS>(s_g, P.N, P.rho, P.p_in, P.seed, o, lane);
+    if (lane == 0) {
+      P.counts[0] = kept;
+      if (P.kept_cnt_out != nullptr) *P.kept_cnt_out = kept;
+    }
+  } else {
+    for (int n = threadIdx.x - 32; n < P.N; n += SAMPLE_A_THREADS - 32) P.g[n] = s_g[n];
+  }
+}
+
 // SampleA (Sec. 4.1) for N <= 32 * SLOTS data.  The CTAs share the data (only the alive ones are read; the others have norm
 // 0): one warp sums a datum's T row square-norms, or, where a producer's partial sums make that many more, a CTA.  The CTA
 // that finishes last finds p, draws the masks and writes the lists in one warp, whose lanes hold SLOTS data each: the
@@ -180,16 +208,7 @@ __global__ void __launch_bounds__(SAMPLE_A_THREADS) sample_a_kernel(SampleAParam
   pdl_wait();      // the row norms come from the kernel before this one
   pdl_trigger();   // the dX product kernel may set itself up meanwhile
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // a caller's list of alive data is not trusted: a length outside [0, N] or an entry outside [0, N) is reported
-  // as VCAS_ERR_BAD_ARG in the status word and not followed
-  int nd = P.N;
-  if (P.alive != nullptr) {
-    nd = *P.alive_cnt;
-    if (nd < 0 || nd > P.N) {
-      if (threadIdx.x == 0 && blockIdx.x == 0) atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
-      nd = min(max(nd, 0), P.N);
-    }
-  }
+  const int nd = alive_data(P);
   const int len = P.T * P.a_parts;
   if (len <= SAMPLE_A_WARP_LEN) {
     for (int k = blockIdx.x * (SAMPLE_A_THREADS / 32) + warp; k < nd; k += gridDim.x * (SAMPLE_A_THREADS / 32)) {
@@ -222,17 +241,50 @@ __global__ void __launch_bounds__(SAMPLE_A_THREADS) sample_a_kernel(SampleAParam
     else atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
   }
   __syncthreads();
-  if (warp == 0) {
-    SampleAOut o;
-    o.p = P.p; o.scaleA = P.scaleA; o.idxA = P.idxA; o.dropA = P.dropA; o.idx_copy = P.kept_out;
-    const int kept = sample_a_warp<SLOTS>(s_g, P.N, P.rho, P.p_in, P.seed, o, lane);
-    if (lane == 0) {
-      P.counts[0] = kept;
-      if (P.kept_cnt_out != nullptr) *P.kept_cnt_out = kept;
-    }
-  } else {
-    for (int n = threadIdx.x - 32; n < P.N; n += SAMPLE_A_THREADS - 32) P.g[n] = s_g[n];
+  draw_a<SLOTS>(P, s_g);
+}
+
+// Row square-norms of dY and SampleA of N <= 32 data in one launch, for few rows: a warp per row, and the CTA that finishes last
+// sums up the data, a warp each, and draws.  The sums are those of the two kernels, in the same order.  Saves a launch, 2.5 to
+// 3.4 us on the host, and its start on the GPU (whole calls, two launches and one: 2048 rows of 4096, 55.3 and 51.0 us; of 3072,
+// 38.9 and 36.8; of 1000, 41.8 and 40.8; 3200 of 4096, 50.5 and 46.3; 256 of 256, 25.8 and 23.5).  With more rows the wait for
+// the last CTA takes back what it saves (4096 of 3072: 40.7 and 39.6 in bf16, 90.0 and 90.6 in fp32; of 256, 31.2 and 31.6; 8192:
+// 46.9 and 48.7), and with more data their sums by one CTA cost more (100 of 16 rows: 28.9 and 35.0).
+constexpr int FUSED_MAX_N = 32, FUSED_MAX_ROWS = 3200;
+template <typename T>
+__global__ void __launch_bounds__(SAMPLE_A_THREADS) norms_sample_a_kernel(const T* __restrict__ dY, int d_out, float* __restrict__ a,
+                                                                          SampleAParams P) {
+  __shared__ float s_g[FUSED_MAX_N];
+  __shared__ int s_last;
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = gridDim.x * (SAMPLE_A_THREADS / 32);
+  const int nd = alive_data(P);
+  for (int c = blockIdx.x * (SAMPLE_A_THREADS / 32) + warp; c < nd * P.T; c += warps) {
+    const int k = c / P.T, n = P.alive != nullptr ? P.alive[k] : k;
+    if ((unsigned)n >= (unsigned)P.N) continue;          // reported below
+    const int r = n * P.T + (c - k * P.T);
+    const float sq = warp_sum(row_partial<T>(dY + (size_t)r * d_out, d_out, lane));
+    if (lane == 0) a[r] = sq;
   }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(P.ticket, 1) == (int)gridDim.x - 1;
+  if (threadIdx.x < FUSED_MAX_N) s_g[threadIdx.x] = 0.f;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (threadIdx.x == 0) *P.ticket = 0;
+  for (int k = warp; k < nd; k += SAMPLE_A_THREADS / 32) {
+    const int n = P.alive != nullptr ? P.alive[k] : k;
+    if ((unsigned)n >= (unsigned)P.N) {
+      if (lane == 0) atomicExch(P.status, (int32_t)VCAS_ERR_BAD_ARG);
+      continue;
+    }
+    const float s = datum_sqnorm_warp(a + (size_t)n * P.T, P.T, lane);
+    if (lane == 0) s_g[n] = sqrtf(s);
+  }
+  __syncthreads();
+  draw_a<1>(P, s_g);
 }
 
 // The same for batches of more than 1024 data: one CTA over global memory.
@@ -683,7 +735,8 @@ mask_kernel(const float* __restrict__ p, int n, uint64_t seed, int sampler, uint
 
 }  // namespace
 
-cudaError_t launch_sample_a(Handle* h, const SamplerArgs& a, bool programmatic, cudaStream_t st) {
+namespace {
+SampleAParams sample_a_params(const Handle* h, const SamplerArgs& a) {
   const Workspace& ws = h->ws;
   const vcas_layer_desc& d = h->desc;
   SampleAParams P;
@@ -695,6 +748,33 @@ cudaError_t launch_sample_a(Handle* h, const SamplerArgs& a, bool programmatic, 
   P.kept_out = a.kept_out; P.kept_cnt_out = a.kept_cnt_out;
   P.status = ws.status;
   P.gk = ws.gk; P.ticket = ws.counts + 5;
+  return P;
+}
+
+template <typename T>
+cudaError_t run_norms_sample_a(Handle* h, const void* dY, const SampleAParams& P, cudaStream_t st) {
+  const vcas_layer_desc& d = h->desc;
+  const dim3 grid((unsigned)((d.N * d.T + SAMPLE_A_THREADS / 32 - 1) / (SAMPLE_A_THREADS / 32))), threads(SAMPLE_A_THREADS);
+  const T* y = reinterpret_cast<const T*>(dY);
+  norms_sample_a_kernel<T><<<grid, threads, 0, st>>>(y, d.d_out, h->ws.a, P);
+  h->launches += 1;
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_norms_sample_a(Handle* h, const void* dY, const SamplerArgs& a, cudaStream_t st) {
+  const vcas_layer_desc& d = h->desc;
+  if (a.a_in != nullptr || (long)d.N * d.T > FUSED_MAX_ROWS || d.N > FUSED_MAX_N || d.T > SAMPLE_A_WARP_LEN) {
+    const cudaError_t e = launch_rownorm_dy(h, dY, a, st);
+    return e != cudaSuccess ? e : launch_sample_a(h, a, a.a_in == nullptr, st);
+  }
+  const SampleAParams P = sample_a_params(h, a);
+  return d.dtype == VCAS_DTYPE_BF16 ? run_norms_sample_a<__nv_bfloat16>(h, dY, P, st) : run_norms_sample_a<float>(h, dY, P, st);
+}
+
+cudaError_t launch_sample_a(Handle* h, const SamplerArgs& a, bool programmatic, cudaStream_t st) {
+  const vcas_layer_desc& d = h->desc;
+  const SampleAParams P = sample_a_params(h, a);
   const int per_cta = d.T * P.a_parts <= SAMPLE_A_WARP_LEN ? SAMPLE_A_THREADS / 32 : 1;
   int ctas = (d.N + per_cta - 1) / per_cta;
   const int cap = h->num_sms > 0 ? h->num_sms : 148;

@@ -86,8 +86,7 @@ extern "C" int vcas_score_static(int32_t N, int32_t T, int32_t d_in, int32_t d_o
   // The array keeps the previous call's contents: the counters and accumulators start at zero.
   if (cudaMemsetAsync(tail, 0, kTailBytes, st) != cudaSuccess) return VCAS_ERR_CUDA;
   const SamplerArgs a = sampler_args(rho, nu, seed);
-  if (launch_rownorm_dy(&h, dY, a, st) != cudaSuccess) return VCAS_ERR_CUDA;
-  if (launch_sample_a(&h, a, true, st) != cudaSuccess) return VCAS_ERR_CUDA;
+  if (launch_norms_sample_a(&h, dY, a, st) != cudaSuccess) return VCAS_ERR_CUDA;
   if (launch_scores_x(&h, X, a, true, st) != cudaSuccess) return VCAS_ERR_CUDA;
   if (launch_sample_w(&h, a, st) != cudaSuccess) return VCAS_ERR_CUDA;
   if (launch_emit_pack(&h, dY, X, a, false, st) != cudaSuccess) return VCAS_ERR_CUDA;
