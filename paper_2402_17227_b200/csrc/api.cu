@@ -111,13 +111,6 @@ size_t layout(Handle* h, uint8_t* base) {
   return (size_t)(cur - base);
 }
 
-// programmatic: behind the kernel before it in `st`
-int copy_out(Handle* h, float* g, float* p, float* w, float* q, int32_t* idxA, int32_t* cntA, int32_t* idxW,
-             int32_t* cntW, bool programmatic, cudaStream_t st) {
-  VCAS_CUDA(launch_copy_out(h, g, p, w, q, idxA, cntA, idxW, cntW, programmatic, st));
-  return VCAS_OK;
-}
-
 // The split products move 16 bytes at a time.  A caller's tensor that does not start on such a boundary (a view into a flat
 // gradient buffer, say) is multiplied by the fp32-FMA kernels, which read and write single elements.
 bool aligned16(const void* a, const void* b, const void* c, const void* d = nullptr) {
@@ -513,15 +506,16 @@ int vcas_score(vcas_handle hh, const void* X, const void* dY, float rho, float n
   VCAS_CUDA(launch_norms_sample_a(h, dY, a, st));
   VCAS_CUDA(launch_scores_x(h, X, a, true, st));
   VCAS_CUDA(launch_sample_w(h, a, st));
-  VCAS_CUDA(launch_emit_pack(h, dY, X, a, false, st));
-  return copy_out(h, g, p, w, q, idxA, cntA, idxW, cntW, true, st);
+  VCAS_CUDA(launch_emit_record(h, a, g, p, w, q, idxA, cntA, idxW, cntW, st));
+  return VCAS_OK;
 }
 
 int vcas_last_sampling(vcas_handle hh, float* g, float* p, float* w, float* q, int32_t* idxA, int32_t* cntA,
                        int32_t* idxW, int32_t* cntW, vcas_stream stream) {
   if (hh == nullptr) return VCAS_ERR_BAD_ARG;
   if (join_pending(H(hh), S(stream)) != VCAS_OK) return VCAS_ERR_CUDA;
-  return copy_out(H(hh), g, p, w, q, idxA, cntA, idxW, cntW, false, S(stream));
+  VCAS_CUDA(launch_copy_out(H(hh), g, p, w, q, idxA, cntA, idxW, cntW, S(stream)));
+  return VCAS_OK;
 }
 
 int vcas_mask_from_probs(vcas_handle hh, const float* p, int32_t n, uint64_t seed, int32_t sampler_id,

@@ -379,9 +379,12 @@ cudaError_t launch_scores_x(Handle* h, const void* X, const SamplerArgs& a, bool
 cudaError_t launch_sample_w(Handle* h, const SamplerArgs& a, cudaStream_t st);
 // kept-row list, 1/(p q), q and w by global row and, with pack, the compact bf16 operands of the dW product
 cudaError_t launch_emit_pack(Handle* h, const void* dY, const void* X, const SamplerArgs& a, bool pack, cudaStream_t st);
+// the same without packing, and the sampling record into the caller's arrays (each may be nullptr)
+cudaError_t launch_emit_record(Handle* h, const SamplerArgs& a, float* g, float* p, float* w, float* q, int32_t* idxA,
+                               int32_t* cntA, int32_t* idxW, int32_t* cntW, cudaStream_t st);
 // the sampling record of the workspace into the caller's arrays (each may be nullptr), in one launch
 cudaError_t launch_copy_out(Handle* h, float* g, float* p, float* w, float* q, int32_t* idxA, int32_t* cntA, int32_t* idxW,
-                            int32_t* cntW, bool programmatic, cudaStream_t st);
+                            int32_t* cntW, cudaStream_t st);
 cudaError_t launch_mask_from_probs(Handle* h, const float* p, int n, uint64_t seed, int sampler,
                                    uint8_t* keep, int32_t* idx, int32_t* cnt, cudaStream_t st);
 

@@ -7,7 +7,7 @@
 //   scores_x_kernel   (score.cu) many CTAs: leverage scores and uniforms of the rows of kept data;
 //   sample_w_kernel   one CTA, scores in shared memory: the water-filling for q = min(1, c w) - a handful
 //                     of block-wide sums - then the masks' counts per chunk of 32 rows and their prefix sums;
-//   emit_pack_kernel  many CTAs: kept-row list, 1/(p q), and the compact operands of the dW product.
+//   emit_pack_kernel  many CTAs: kept-row list, 1/(p q), and the compact operands of the dW product (emit_rows_kernel: without).
 // Only the scalar fixed point and a scan over R/32 counts run on a single SM.
 #include <atomic>
 
@@ -549,7 +549,7 @@ struct EmitParams {
   const int32_t* counts; const int32_t* chunk_off; const float* fix;
   float* w; float* q; float* scaleW; int32_t* idxW;
   const void* dY; const void* X;                         // operands to pack
-  __nv_bfloat16* packG; __nv_bfloat16* packX;            // compact operands (nullptr: no packing)
+  __nv_bfloat16* packG; __nv_bfloat16* packX;            // compact operands
   size_t g_stride, x_stride;                             // elements between the parts of a cut operand
   int N, T, d_in, d_out;
   int sample_w;
@@ -567,6 +567,79 @@ __device__ __forceinline__ uint4 scale8(const uint4& v, float sc) {
   }
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
+// What emit_rows_kernel hands out of the sampling record (see vcas_score); null pointers: not asked for.
+struct RecordOut {
+  float* g; float* p; float* w; float* q;
+  int32_t* idxA; int32_t* cntA; int32_t* idxW; int32_t* cntW;
+};
+// The kept rows of a chunk of 32 compact rows, one per lane: its place j among the chunk's and pos among all, its factor; how many.
+struct ChunkRow { bool keep; int r, j, pos, count; float w, q, sc; };
+__device__ __forceinline__ ChunkRow chunk_row(const EmitParams& P, int ch, int lane, int n, int mode, float c) {
+  ChunkRow o = {};
+  const int i = (ch << 5) + lane;
+  float sa = 0.f;
+  if (i < n) {
+    const int k = i / P.T;
+    const int nd = P.idxA[k];
+    o.r = nd * P.T + (i - k * P.T);
+    o.w = P.wc[i];
+    o.q = q_of(mode, c, o.w, P.q_in, o.r);
+    o.keep = row_kept(P.sample_w, o.q, P.sample_w ? P.uc[i] : 0u);
+    sa = P.scaleA[nd];
+  }
+  const unsigned b = __ballot_sync(0xffffffffu, o.keep);
+  o.count = __popc(b);
+  o.j = __popc(b & ((1u << lane) - 1u));
+  if (o.keep) {
+    o.pos = P.chunk_off[ch] + o.j;
+    o.sc = P.sample_w ? sa / o.q : sa;
+  }
+  return o;
+}
+constexpr int EMIT_THREADS = 256;
+// Without operands to pack: a warp per chunk, and the record into the caller's arrays.  Latency-bound; with an emitting
+// launch of a CTA per chunk and a copying one, a scoring call of 16384 rows of 4096 and 1024 columns took 126.4 us, now 121.9.
+__global__ void __launch_bounds__(EMIT_THREADS) emit_rows_kernel(EmitParams P, const float* g, const float* p, RecordOut O) {
+  pdl_wait();      // c and the chunk offsets come from the kernel before this one
+  pdl_trigger();
+  const int tid = blockIdx.x * EMIT_THREADS + threadIdx.x, threads = gridDim.x * EMIT_THREADS, lane = threadIdx.x & 31;
+  const int cntA = P.counts[0], cntW = P.counts[1], T = P.T, n = cntA * T;
+  const float c = P.fix[0];
+  const int mode = (int)P.fix[1];
+  for (int ch = tid >> 5; ch < (n + 31) >> 5; ch += threads >> 5) {
+    const ChunkRow o = chunk_row(P, ch, lane, n, mode, c);
+    if ((ch << 5) + lane < n) {
+      P.w[o.r] = o.w;
+      P.q[o.r] = o.q;
+      if (O.w != nullptr) O.w[o.r] = o.w;
+      if (O.q != nullptr) O.q[o.r] = o.q;
+    }
+    if (o.keep) {
+      P.idxW[o.pos] = o.r;
+      P.scaleW[o.pos] = o.sc;
+      if (O.idxW != nullptr) O.idxW[o.pos] = o.r;
+    }
+  }
+  // rows of dropped data
+  for (int i = tid; i < (P.N - cntA) * T; i += threads) {
+    const int k = i / T;
+    const int r = P.dropA[k] * T + (i - k * T);
+    P.w[r] = 0.f;
+    P.q[r] = 0.f;
+    if (O.w != nullptr) O.w[r] = 0.f;
+    if (O.q != nullptr) O.q[r] = 0.f;
+  }
+  for (int i = tid; i < P.N; i += threads) {
+    if (O.g != nullptr) O.g[i] = g[i];
+    if (O.p != nullptr) O.p[i] = p[i];
+    if (O.idxA != nullptr && i < cntA) O.idxA[i] = P.idxA[i];
+  }
+  if (tid == 0) {
+    if (O.cntA != nullptr) *O.cntA = cntA;
+    if (O.cntW != nullptr) *O.cntW = cntW;
+  }
+}
+
 // One CTA per (chunk of 32 compact rows, part) (grid-strided): the chunk's kept rows go to positions
 // chunk_off[ch]... of the ascending kept-row list with their rescale factors 1/(p_n q_r); q and w are written by
 // global row (by part 0); the operands of the chunk's kept rows j with j % parts == part are packed for the dW
@@ -574,7 +647,6 @@ __device__ __forceinline__ uint4 scale8(const uint4& v, float sc) {
 // multiple of 64 (the product's last k-block then adds nothing).
 // CUT: the operands for the products of gemm_split.cu: the rescaled rows of dY are kept to fp32 precision in three bf16
 // parts, and the rows of an fp32 X likewise (a bf16 X is its own single part).
-constexpr int EMIT_THREADS = 256;
 template <typename E, bool CUT>
 __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   __shared__ int s_r[32], s_pos[32], s_cnt;
@@ -588,84 +660,65 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   const float c = P.fix[0];
   const int mode = (int)P.fix[1];
   const int nchunks = (n + 31) >> 5;
-  const bool pack = P.packG != nullptr;
-  const int parts = pack ? P.parts : 1;
+  const int parts = P.parts;
   for (int u = blockIdx.x; u < nchunks * parts; u += gridDim.x) {
     const int ch = u / parts, part = u - ch * parts;
     if (warp == 0) {
-      const int i = (ch << 5) + lane;
-      bool keep = false;
-      float q = 0.f, wv = 0.f, sa = 0.f;
-      int r = 0;
-      if (i < n) {
-        const int k = i / T;
-        const int nd = P.idxA[k];
-        r = nd * T + (i - k * T);
-        wv = P.wc[i];
-        q = q_of(mode, c, wv, P.q_in, r);
-        keep = row_kept(P.sample_w, q, P.sample_w ? P.uc[i] : 0u);
-        sa = P.scaleA[nd];
-        if (part == 0) { P.w[r] = wv; P.q[r] = q; }
+      const ChunkRow o = chunk_row(P, ch, lane, n, mode, c);
+      if (part == 0 && (ch << 5) + lane < n) { P.w[o.r] = o.w; P.q[o.r] = o.q; }
+      if (o.keep) {
+        if (part == 0) { P.idxW[o.pos] = o.r; P.scaleW[o.pos] = o.sc; }
+        s_r[o.j] = o.r; s_pos[o.j] = o.pos; s_sc[o.j] = o.sc;
       }
-      const unsigned b = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
-        const int j = __popc(b & ((1u << lane) - 1u));
-        const int pos = P.chunk_off[ch] + j;
-        const float sc = P.sample_w ? sa / q : sa;
-        if (part == 0) { P.idxW[pos] = r; P.scaleW[pos] = sc; }
-        s_r[j] = r; s_pos[j] = pos; s_sc[j] = sc;
-      }
-      if (lane == 0) s_cnt = __popc(b);
+      if (lane == 0) s_cnt = o.count;
     }
-    if (pack) {
-      __syncthreads();
-      // This part's rows j = part, part + parts, ...  A row's 16-byte pieces (first those of dY, then those of X)
-      // are cut into segments of 128; a warp takes (row, segment) items in turn and moves a segment with four
-      // independent loads per lane in flight.  One integer division per 2 KB moved, none per piece.
-      const int m = s_cnt;
-      const int mp = m > part ? (m - part + parts - 1) / parts : 0;
-      const int vo = P.d_out / 8, vt = vo + P.d_in / 8;
-      const int nseg = (vt + 127) >> 7;
-      for (int item = warp; item < mp * nseg; item += EMIT_THREADS / 32) {
-        const int jj = item / nseg, seg = item - jj * nseg;
-        const int j = part + jj * parts;
-        const size_t r = (size_t)s_r[j], pos = (size_t)s_pos[j];
-        const float sc = s_sc[j];
-        const E* srcG = reinterpret_cast<const E*>(P.dY) + r * P.d_out;
-        const E* srcX = reinterpret_cast<const E*>(P.X) + r * P.d_in - (size_t)P.d_out;
-        __nv_bfloat16* dstG = P.packG + pos * P.d_out;
-        __nv_bfloat16* dstX = P.packX + pos * P.d_in - (size_t)P.d_out;
-        const int p0 = (seg << 7) + lane;
-        Vec8<E> v[4];
+    __syncthreads();
+    // This part's rows j = part, part + parts, ...  A row's 16-byte pieces (first those of dY, then those of X)
+    // are cut into segments of 128; a warp takes (row, segment) items in turn and moves a segment with four
+    // independent loads per lane in flight.  One integer division per 2 KB moved, none per piece.
+    const int m = s_cnt;
+    const int mp = m > part ? (m - part + parts - 1) / parts : 0;
+    const int vo = P.d_out / 8, vt = vo + P.d_in / 8;
+    const int nseg = (vt + 127) >> 7;
+    for (int item = warp; item < mp * nseg; item += EMIT_THREADS / 32) {
+      const int jj = item / nseg, seg = item - jj * nseg;
+      const int j = part + jj * parts;
+      const size_t r = (size_t)s_r[j], pos = (size_t)s_pos[j];
+      const float sc = s_sc[j];
+      const E* srcG = reinterpret_cast<const E*>(P.dY) + r * P.d_out;
+      const E* srcX = reinterpret_cast<const E*>(P.X) + r * P.d_in - (size_t)P.d_out;
+      __nv_bfloat16* dstG = P.packG + pos * P.d_out;
+      __nv_bfloat16* dstX = P.packX + pos * P.d_in - (size_t)P.d_out;
+      const int p0 = (seg << 7) + lane;
+      Vec8<E> v[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int piece = p0 + 32 * q;
-          if (piece < vt) v[q].load((piece < vo ? srcG : srcX) + piece * 8);
-        }
+      for (int q = 0; q < 4; ++q) {
+        const int piece = p0 + 32 * q;
+        if (piece < vt) v[q].load((piece < vo ? srcG : srcX) + piece * 8);
+      }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int piece = p0 + 32 * q;
-          if (piece >= vt) break;
-          const bool g = piece < vo;
-          __nv_bfloat16* dst = (g ? dstG : dstX) + piece * 8;
-          if constexpr (CUT) {
-            if (sizeof(E) == 4 || g) {
-              float f[8];
-              v[q].get(f);
-              if (g) {
+      for (int q = 0; q < 4; ++q) {
+        const int piece = p0 + 32 * q;
+        if (piece >= vt) break;
+        const bool g = piece < vo;
+        __nv_bfloat16* dst = (g ? dstG : dstX) + piece * 8;
+        if constexpr (CUT) {
+          if (sizeof(E) == 4 || g) {
+            float f[8];
+            v[q].get(f);
+            if (g) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) f[e] *= sc;
-              }
-              store_parts3<sizeof(E) == 4>(f, dst, g ? P.g_stride : P.x_stride);      // a bf16 X is a single part
-              continue;
+              for (int e = 0; e < 8; ++e) f[e] *= sc;
             }
+            store_parts3<sizeof(E) == 4>(f, dst, g ? P.g_stride : P.x_stride);      // a bf16 X is a single part
+            continue;
           }
-          if constexpr (sizeof(E) == 2)
-            *reinterpret_cast<uint4*>(dst) = g ? scale8(v[q].v, sc) : v[q].v;
         }
+        if constexpr (sizeof(E) == 2)
+          *reinterpret_cast<uint4*>(dst) = g ? scale8(v[q].v, sc) : v[q].v;
       }
-      __syncthreads();
     }
+    __syncthreads();
   }
   // rows of dropped data
   const int ndrop_rows = (P.N - cntA) * T;
@@ -676,19 +729,17 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
     P.q[r] = 0.f;
   }
   // zero rows up to the next multiple of 64
-  if (pack) {
-    const int padded = (cntW + 63) / 64 * 64;
-    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-    for (int k = cntW + (int)blockIdx.x; k < padded; k += gridDim.x) {
+  const int padded = (cntW + 63) / 64 * 64;
+  const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+  for (int k = cntW + (int)blockIdx.x; k < padded; k += gridDim.x) {
 #pragma unroll
-      for (int part = 0; part < (CUT ? 3 : 1); ++part)
-        for (int i = tid; i < P.d_out / 8; i += EMIT_THREADS)
-          reinterpret_cast<uint4*>(P.packG + part * P.g_stride + (size_t)k * P.d_out)[i] = z;
+    for (int part = 0; part < (CUT ? 3 : 1); ++part)
+      for (int i = tid; i < P.d_out / 8; i += EMIT_THREADS)
+        reinterpret_cast<uint4*>(P.packG + part * P.g_stride + (size_t)k * P.d_out)[i] = z;
 #pragma unroll
-      for (int part = 0; part < (CUT && sizeof(E) == 4 ? 3 : 1); ++part)
-        for (int i = tid; i < P.d_in / 8; i += EMIT_THREADS)
-          reinterpret_cast<uint4*>(P.packX + part * P.x_stride + (size_t)k * P.d_in)[i] = z;
-    }
+    for (int part = 0; part < (CUT && sizeof(E) == 4 ? 3 : 1); ++part)
+      for (int i = tid; i < P.d_in / 8; i += EMIT_THREADS)
+        reinterpret_cast<uint4*>(P.packX + part * P.x_stride + (size_t)k * P.d_in)[i] = z;
   }
 }
 
@@ -702,7 +753,6 @@ struct CopyParams {
   int N, R;
 };
 __global__ void __launch_bounds__(256) copy_out_kernel(CopyParams P) {
-  pdl_wait();
   for (int i = blockIdx.x * 256 + threadIdx.x; i < P.R; i += gridDim.x * 256) {
     if (P.ow != nullptr) P.ow[i] = P.w[i];
     if (P.oq != nullptr) P.oq[i] = P.q[i];
@@ -836,32 +886,54 @@ cudaError_t launch_sample_w(Handle* h, const SamplerArgs& a, cudaStream_t st) {
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_emit_pack(Handle* h, const void* dY, const void* X, const SamplerArgs& a, bool pack, cudaStream_t st) {
+namespace {
+EmitParams emit_params(const Handle* h, const SamplerArgs& a) {
   const Workspace& ws = h->ws;
   const vcas_layer_desc& d = h->desc;
-  EmitParams P;
+  EmitParams P = {};
   P.wc = ws.wc; P.uc = ws.uc; P.q_in = a.q_in; P.scaleA = ws.scaleA; P.idxA = ws.idxA; P.dropA = ws.dropA;
   P.counts = ws.counts; P.chunk_off = ws.chunk_off; P.fix = ws.fix;
   P.w = ws.w; P.q = ws.q; P.scaleW = ws.scaleW; P.idxW = ws.idxW;
-  P.dY = dY; P.X = X;
-  P.g_stride = (size_t)h->R_pad * d.d_out; P.x_stride = (size_t)h->R_pad * d.d_in;
-  P.packG = pack ? ws.packG : nullptr;
-  P.packX = pack ? ws.packX : nullptr;
   P.N = d.N; P.T = d.T; P.d_in = d.d_in; P.d_out = d.d_out;
   P.sample_w = a.sample_w;
-  // The number of chunks with kept rows is only known on the device.  With packing, the grid has eight CTAs per
-  // SM and the rows of a chunk are shared among as many CTAs as the expected number of chunks leaves room for.
+  return P;
+}
+}  // namespace
+
+cudaError_t launch_emit_record(Handle* h, const SamplerArgs& a, float* g, float* p, float* w, float* q, int32_t* idxA,
+                               int32_t* cntA, int32_t* idxW, int32_t* cntW, cudaStream_t st) {
+  RecordOut O;
+  O.g = g; O.p = p; O.w = w; O.q = q; O.idxA = idxA; O.cntA = cntA; O.idxW = idxW; O.cntW = cntW;
+  const long rows = (long)h->desc.N * h->desc.T, cap = (long)(h->num_sms > 0 ? h->num_sms : 148) * 8;
+  long blocks = (rows + EMIT_THREADS - 1) / EMIT_THREADS;
+  if (blocks > cap) blocks = cap;
+  const cudaError_t e = launch_after(emit_rows_kernel, dim3((unsigned)blocks), dim3(EMIT_THREADS), 0, st, emit_params(h, a),
+                                     (const float*)h->ws.g, (const float*)h->ws.p, O);
+  h->launches += 1;
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_emit_pack(Handle* h, const void* dY, const void* X, const SamplerArgs& a, bool pack, cudaStream_t st) {
+  if (!pack) return launch_emit_record(h, a, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, st);
+  const Workspace& ws = h->ws;
+  const vcas_layer_desc& d = h->desc;
+  EmitParams P = emit_params(h, a);
+  P.dY = dY; P.X = X;
+  P.g_stride = (size_t)h->R_pad * d.d_out; P.x_stride = (size_t)h->R_pad * d.d_in;
+  P.packG = ws.packG; P.packX = ws.packX;
+  // The number of chunks with kept rows is only known on the device.  The grid has eight CTAs per SM and the rows of a
+  // chunk are shared among as many CTAs as the expected number of chunks leaves room for.
   const long R = (long)d.N * d.T;
   const long cap = (long)(h->num_sms > 0 ? h->num_sms : 148) * 8;
   long expected = (long)((double)a.rho * (double)R / 32.0) + 1;
-  long parts = pack ? cap / expected : 1;
+  long parts = cap / expected;
   if (parts < 1) parts = 1;
   if (parts > 16) parts = 16;
   P.parts = (int)parts;
   long blocks = ((R + 31) / 32) * parts;
   if (blocks > cap) blocks = cap;
   const dim3 grid((unsigned)blocks), threads(EMIT_THREADS);
-  const cudaError_t e = !(pack && h->split_path) ? launch_after(emit_pack_kernel<__nv_bfloat16, false>, grid, threads, 0, st, P)
+  const cudaError_t e = !h->split_path           ? launch_after(emit_pack_kernel<__nv_bfloat16, false>, grid, threads, 0, st, P)
       : d.dtype == VCAS_DTYPE_F32                ? launch_after(emit_pack_kernel<float, true>, grid, threads, 0, st, P)
                                                  : launch_after(emit_pack_kernel<__nv_bfloat16, true>, grid, threads, 0, st, P);
   h->launches += 1;
@@ -869,7 +941,7 @@ cudaError_t launch_emit_pack(Handle* h, const void* dY, const void* X, const Sam
 }
 
 cudaError_t launch_copy_out(Handle* h, float* g, float* p, float* w, float* q, int32_t* idxA, int32_t* cntA, int32_t* idxW,
-                            int32_t* cntW, bool programmatic, cudaStream_t st) {
+                            int32_t* cntW, cudaStream_t st) {
   const Workspace& ws = h->ws;
   CopyParams P;
   P.g = ws.g; P.p = ws.p; P.w = ws.w; P.q = ws.q; P.idxA = ws.idxA; P.idxW = ws.idxW; P.counts = ws.counts;
@@ -877,9 +949,9 @@ cudaError_t launch_copy_out(Handle* h, float* g, float* p, float* w, float* q, i
   P.N = h->desc.N; P.R = h->desc.N * h->desc.T;
   int blocks = (P.R + 255) / 256;
   if (blocks > 592) blocks = 592;
-  const cudaError_t e = launch_maybe_after(programmatic, copy_out_kernel, dim3((unsigned)blocks), dim3(256), 0, st, P);
+  copy_out_kernel<<<(unsigned)blocks, 256, 0, st>>>(P);
   h->launches += 1;
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return cudaGetLastError();
 }
 
 cudaError_t launch_mask_from_probs(Handle* h, const float* p, int n, uint64_t seed, int sampler,

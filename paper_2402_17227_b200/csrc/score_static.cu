@@ -89,8 +89,6 @@ extern "C" int vcas_score_static(int32_t N, int32_t T, int32_t d_in, int32_t d_o
   if (launch_norms_sample_a(&h, dY, a, st) != cudaSuccess) return VCAS_ERR_CUDA;
   if (launch_scores_x(&h, X, a, true, st) != cudaSuccess) return VCAS_ERR_CUDA;
   if (launch_sample_w(&h, a, st) != cudaSuccess) return VCAS_ERR_CUDA;
-  if (launch_emit_pack(&h, dY, X, a, false, st) != cudaSuccess) return VCAS_ERR_CUDA;
-
-  if (launch_copy_out(&h, g, p, w, q, idxA, cntA, idxW, cntW, true, st) != cudaSuccess) return VCAS_ERR_CUDA;
+  if (launch_emit_record(&h, a, g, p, w, q, idxA, cntA, idxW, cntW, st) != cudaSuccess) return VCAS_ERR_CUDA;
   return VCAS_OK;
 }
