@@ -207,6 +207,20 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 // ---------------------------------------------------------------------------------------
 // SampleA inside one warp (Sec. 4.1), shared by the sampling kernel and the tail of the row-norm kernel.
 // ---------------------------------------------------------------------------------------
+// A lane's values t, t + 32, ... < T, V of them at most: whole groups of four by sum, what is left over on s0.
+template <int V>
+__device__ __forceinline__ void datum_rest(const float* an, int T, int t, float& s0, float& s1, float& s2, float& s3) {
+  float v[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) v[k] = t + 32 * k < T ? __ldcg(an + t + 32 * k) : 0.f;
+#pragma unroll
+  for (int k = 0; k < V; k += 4) {
+    const bool four = t + 32 * k + 96 < T;
+    s0 += v[k];
+    s1 += four ? v[k + 1] : 0.f; s2 += four ? v[k + 2] : 0.f; s3 += four ? v[k + 3] : 0.f;
+    if (!four) s0 = (s0 + v[k + 1]) + v[k + 2];
+  }
+}
 // Sum of the T squared row norms of one datum by one warp, in a fixed order, result in every lane.  Up to
 // sixteen independent loads per lane are in flight (a dependent chain of T/32 loads would cost a memory
 // latency each: 8192 rows in 32 data, 768 -> 768, the call 46.6 us with the rest's loads in turn and 45.9 at once).  The
@@ -221,17 +235,9 @@ __device__ __forceinline__ float datum_sqnorm_warp(const float* an, int T, int l
 #pragma unroll
     for (int k = 0; k < 16; k += 4) { s0 += v[k]; s1 += v[k + 1]; s2 += v[k + 2]; s3 += v[k + 3]; }
   }
-  // the rest, loaded at once as well: whole groups of four by accumulator, what a lane has left over on s0
-  float v[16];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) v[k] = t + 32 * k < T ? __ldcg(an + t + 32 * k) : 0.f;
-#pragma unroll
-  for (int k = 0; k < 16; k += 4) {
-    const bool four = t + 32 * k + 96 < T;
-    s0 += v[k];
-    s1 += four ? v[k + 1] : 0.f; s2 += four ? v[k + 2] : 0.f; s3 += four ? v[k + 3] : 0.f;
-    if (!four) s0 = (s0 + v[k + 1]) + v[k + 2];
-  }
+  // the rest, of at most 128 values or of more, loaded at once as well
+  if (t - lane + 128 >= T) datum_rest<4>(an, T, t, s0, s1, s2, s3);
+  else datum_rest<16>(an, T, t, s0, s1, s2, s3);
   return warp_sum((s0 + s1) + (s2 + s3));
 }
 
