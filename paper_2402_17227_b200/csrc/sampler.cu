@@ -572,27 +572,38 @@ struct RecordOut {
   float* g; float* p; float* w; float* q;
   int32_t* idxA; int32_t* cntA; int32_t* idxW; int32_t* cntW;
 };
-// The kept rows of a chunk of 32 compact rows, one per lane: its place j among the chunk's and pos among all, its factor; how many.
-struct ChunkRow { bool keep; int r, j, pos, count; float w, q, sc; };
-__device__ __forceinline__ ChunkRow chunk_row(const EmitParams& P, int ch, int lane, int n, int mode, float c) {
-  ChunkRow o = {};
+// A compact row of a chunk of 32, one per lane, as the kernels before SampleW left it.  The first chunk of a CTA is read before the
+// wait for SampleW, which started when they had ended and then let this grid start (whole calls: 192 rows, 128 -> 192, 22.6 -> 21.5 us
+// on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2).
+struct ChunkIn { bool in; int r; float w, sa; uint32_t u; };
+__device__ __forceinline__ ChunkIn chunk_in(const EmitParams& P, int ch, int lane, int n) {
+  ChunkIn o = {};
   const int i = (ch << 5) + lane;
-  float sa = 0.f;
-  if (i < n) {
+  o.in = i < n;
+  if (o.in) {
     const int k = i / P.T;
     const int nd = P.idxA[k];
     o.r = nd * P.T + (i - k * P.T);
     o.w = P.wc[i];
-    o.q = q_of(mode, c, o.w, P.q_in, o.r);
-    o.keep = row_kept(P.sample_w, o.q, P.sample_w ? P.uc[i] : 0u);
-    sa = P.scaleA[nd];
+    o.u = P.sample_w ? P.uc[i] : 0u;
+    o.sa = P.scaleA[nd];
+  }
+  return o;
+}
+// Of a kept row: its place j among the chunk's and pos among all, its factor.  The number of them in every lane.
+struct ChunkRow { bool keep; int j, pos, count; float q, sc; };
+__device__ __forceinline__ ChunkRow chunk_row(const EmitParams& P, const ChunkIn& x, int ch, int lane, int mode, float c) {
+  ChunkRow o = {};
+  if (x.in) {
+    o.q = q_of(mode, c, x.w, P.q_in, x.r);
+    o.keep = row_kept(P.sample_w, o.q, x.u);
   }
   const unsigned b = __ballot_sync(0xffffffffu, o.keep);
   o.count = __popc(b);
   o.j = __popc(b & ((1u << lane) - 1u));
   if (o.keep) {
     o.pos = P.chunk_off[ch] + o.j;
-    o.sc = P.sample_w ? sa / o.q : sa;
+    o.sc = P.sample_w ? x.sa / o.q : x.sa;
   }
   return o;
 }
@@ -600,24 +611,27 @@ constexpr int EMIT_THREADS = 256;
 // Without operands to pack: a warp per chunk, and the record into the caller's arrays.  Latency-bound; with an emitting
 // launch of a CTA per chunk and a copying one, a scoring call of 16384 rows of 4096 and 1024 columns took 126.4 us, now 121.9.
 __global__ void __launch_bounds__(EMIT_THREADS) emit_rows_kernel(EmitParams P, const float* g, const float* p, RecordOut O) {
+  const int tid = blockIdx.x * EMIT_THREADS + threadIdx.x, threads = gridDim.x * EMIT_THREADS, lane = threadIdx.x & 31;
+  const int cntA = P.counts[0], T = P.T, n = cntA * T;
+  ChunkIn x = chunk_in(P, tid >> 5, lane, n);
   pdl_wait();      // c and the chunk offsets come from the kernel before this one
   pdl_trigger();
-  const int tid = blockIdx.x * EMIT_THREADS + threadIdx.x, threads = gridDim.x * EMIT_THREADS, lane = threadIdx.x & 31;
-  const int cntA = P.counts[0], cntW = P.counts[1], T = P.T, n = cntA * T;
+  const int cntW = __ldcg(P.counts + 1);
   const float c = P.fix[0];
   const int mode = (int)P.fix[1];
   for (int ch = tid >> 5; ch < (n + 31) >> 5; ch += threads >> 5) {
-    const ChunkRow o = chunk_row(P, ch, lane, n, mode, c);
-    if ((ch << 5) + lane < n) {
-      P.w[o.r] = o.w;
-      P.q[o.r] = o.q;
-      if (O.w != nullptr) O.w[o.r] = o.w;
-      if (O.q != nullptr) O.q[o.r] = o.q;
+    if (ch != tid >> 5) x = chunk_in(P, ch, lane, n);
+    const ChunkRow o = chunk_row(P, x, ch, lane, mode, c);
+    if (x.in) {
+      P.w[x.r] = x.w;
+      P.q[x.r] = o.q;
+      if (O.w != nullptr) O.w[x.r] = x.w;
+      if (O.q != nullptr) O.q[x.r] = o.q;
     }
     if (o.keep) {
-      P.idxW[o.pos] = o.r;
+      P.idxW[o.pos] = x.r;
       P.scaleW[o.pos] = o.sc;
-      if (O.idxW != nullptr) O.idxW[o.pos] = o.r;
+      if (O.idxW != nullptr) O.idxW[o.pos] = x.r;
     }
   }
   // rows of dropped data
@@ -651,24 +665,27 @@ template <typename E, bool CUT>
 __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   __shared__ int s_r[32], s_pos[32], s_cnt;
   __shared__ float s_sc[32];
-  pdl_wait();      // c and the chunk offsets come from the kernel before this one
-  pdl_trigger();   // the dW product kernel may set itself up; it waits for this grid before loading
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cntA = P.counts[0], cntW = P.counts[1];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, parts = P.parts;
+  const int cntA = P.counts[0];
   const int T = P.T;
   const int n = cntA * T;
+  ChunkIn x = {};
+  if (warp == 0) x = chunk_in(P, (int)blockIdx.x / parts, lane, n);
+  pdl_wait();      // c and the chunk offsets come from the kernel before this one
+  pdl_trigger();   // the dW product kernel may set itself up; it waits for this grid before loading
+  const int cntW = __ldcg(P.counts + 1);
   const float c = P.fix[0];
   const int mode = (int)P.fix[1];
   const int nchunks = (n + 31) >> 5;
-  const int parts = P.parts;
   for (int u = blockIdx.x; u < nchunks * parts; u += gridDim.x) {
     const int ch = u / parts, part = u - ch * parts;
     if (warp == 0) {
-      const ChunkRow o = chunk_row(P, ch, lane, n, mode, c);
-      if (part == 0 && (ch << 5) + lane < n) { P.w[o.r] = o.w; P.q[o.r] = o.q; }
+      if (u != (int)blockIdx.x) x = chunk_in(P, ch, lane, n);
+      const ChunkRow o = chunk_row(P, x, ch, lane, mode, c);
+      if (part == 0 && x.in) { P.w[x.r] = x.w; P.q[x.r] = o.q; }
       if (o.keep) {
-        if (part == 0) { P.idxW[o.pos] = o.r; P.scaleW[o.pos] = o.sc; }
-        s_r[o.j] = o.r; s_pos[o.j] = o.pos; s_sc[o.j] = o.sc;
+        if (part == 0) { P.idxW[o.pos] = x.r; P.scaleW[o.pos] = o.sc; }
+        s_r[o.j] = x.r; s_pos[o.j] = o.pos; s_sc[o.j] = o.sc;
       }
       if (lane == 0) s_cnt = o.count;
     }
