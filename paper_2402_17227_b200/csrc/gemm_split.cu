@@ -427,13 +427,13 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_kernel(PrepParams P) {
 // ------------------------------------------------------------------------------------ host side
 // Slices of the contraction from the expected number of tiles and k-blocks: the fewest microseconds of waves x
 // (k-blocks per slice x cost + set-up) under the measured cost of a k-block.
-int split_slices(const Handle* h, long tiles, int k, double kblock_us) {
+int split_slices(const Handle* h, int sms, long tiles, int k, double kblock_us) {
   const int kb = k > BK ? (k + BK - 1) / BK : 1;
   int best = 1;
   double best_t = 1e30;
   for (int s = 1; s <= MAX_SPLIT && (s == 1 || kb / s >= 2); ++s) {
     if (tiles * s > h->max_units) break;
-    const double waves = (double)((tiles * s + h->num_sms - 1) / h->num_sms);
+    const double waves = (double)((tiles * s + sms - 1) / sms);
     const double t = waves * ((double)((kb + s - 1) / s) * kblock_us + 1.5) + (s > 1 ? 3.5 + 0.3 * s : 0.0);
     if (t < best_t - 1e-9) { best_t = t; best = s; }
   }
@@ -452,9 +452,12 @@ cudaError_t run_split(Handle* h, const CUtensorMap& a, const CUtensorMap& b, Spl
     if (e != cudaSuccess) return e;
     attr_set[h->device].store(true, std::memory_order_release);
   }
-  P.slices = split_slices(h, exp_tiles, k, PA * PB == 9 ? 1.7 : (PA * PB == 3 ? 0.9 : 0.55));
+  // A sampled dX leaves one SM to SampleW, whose CTA does not fit beside one of these and would wait for a product to end
+  // (fp32, 8192 rows, 512 -> 512: 67.5 and 66.8 us the call; 8192, 256 -> 1024: 54.6 and 54.1; 2048, 768 -> 3072: 78.2 and 77.7).
+  const int sms = MODE == MODE_DX && P.counts != nullptr && h->num_sms > 1 ? h->num_sms - 1 : h->num_sms;
+  P.slices = split_slices(h, sms, exp_tiles, k, PA * PB == 9 ? 1.7 : (PA * PB == 3 ? 0.9 : 0.55));
   long grid = max_tiles * P.slices;
-  if (grid > h->num_sms) grid = h->num_sms;
+  if (grid > sms) grid = sms;
   cudaError_t e = launch_maybe_after(programmatic, split_kernel<T, MODE, PA, PB, GELU>, dim3((unsigned)grid), dim3(SPLIT_THREADS),
                                      C::SMEM_BYTES, st, a, b, P);
   h->launches += 1;
