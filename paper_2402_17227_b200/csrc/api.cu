@@ -161,7 +161,11 @@ int plain_dx(Handle* h, const void* dY, const void* W, float rho, const void* Hp
              cudaStream_t st) {
   if (h->split_path && aligned16(dY, W, Hpre, dX)) {
     const bool fp32 = h->desc.dtype == VCAS_DTYPE_F32;
-    VCAS_CUDA(launch_split_prep(h, dY, false, fp32 ? W : nullptr, h->ws.packW, h->desc.d_out, h->desc.d_in, dX, programmatic, st));
+    // Behind SampleA the weight is cut while that runs, where dX ends the call: from 14 GFLOP of part products on (fp32, 14.5,
+    // 768 -> 1536: 57.7 and 56.8 us; 29, 768 -> 3072: 78.5 and 76.7; 35, 768 -> 3072: 90.0 and 88.0).  Where dW's branch ends it,
+    // a product that starts earlier keeps the SMs from that branch's X norms (10, 768 -> 768: 55.6 and 60.3; 7.2: 45.7 and 48.1).
+    const bool early = programmatic && 12.0 * rho * h->desc.N * h->desc.T * (double)h->desc.d_in * h->desc.d_out > 14e9;
+    VCAS_CUDA(launch_split_prep(h, dY, false, fp32 ? W : nullptr, h->ws.packW, h->desc.d_out, h->desc.d_in, dX, programmatic, early, st));
     VCAS_CUDA(launch_split_dx(h, dY, W, false, rho, Hpre, dX, st));
   } else {
     VCAS_CUDA(launch_fma_dx(h, dY, W, h->ws.scaleA, Hpre, dX, st));
@@ -176,7 +180,7 @@ int dense_dw(Handle* h, const void* X, const void* dY, const Plan* plan, bool sp
   if (split) {
     const int R = h->desc.N * h->desc.T;
     const bool fp32 = h->desc.dtype == VCAS_DTYPE_F32;
-    if (fp32) VCAS_CUDA(launch_split_prep(h, y_ready ? nullptr : dY, true, X, h->ws.packX, R, h->desc.d_in, nullptr, false, st));
+    if (fp32) VCAS_CUDA(launch_split_prep(h, y_ready ? nullptr : dY, true, X, h->ws.packX, R, h->desc.d_in, nullptr, false, false, st));
     VCAS_CUDA(launch_split_dw(h, dY, X, true, R, out, fp32, st));
   } else if (h->tensor_path) {
     VCAS_CUDA(launch_umma_dw(h, dY, X, h->desc.N * h->desc.T, h->ws.counts + 2, h->desc.N * h->desc.T, plan, out, st));
@@ -467,7 +471,7 @@ int vcas_dense_bwd_ex(vcas_handle hh, const void* X, const void* dY, const void*
   const bool fork = (h->tensor_path || split) && !h->prof_enabled;
   const bool cut = split && h->desc.dtype == VCAS_DTYPE_F32;
   mark_dense(h, 0, st);
-  if (cut) VCAS_CUDA(launch_split_prep(h, dY, true, W, h->ws.packW, h->desc.d_out, h->desc.d_in, nullptr, false, st));
+  if (cut) VCAS_CUDA(launch_split_prep(h, dY, true, W, h->ws.packW, h->desc.d_out, h->desc.d_in, nullptr, false, false, st));
   if (fork) {
     VCAS_CUDA(cudaEventRecord(h->ev_fork, st));
     VCAS_CUDA(cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));

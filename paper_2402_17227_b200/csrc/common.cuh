@@ -403,9 +403,10 @@ cudaError_t launch_fma_dw(Handle* h, const void* dY, const void* X, const int32_
 // products of fp32 layers and of odd widths on the tensor cores, operands cut into bf16 parts
 int split_max_units(const vcas_layer_desc& d, int num_sms);      // (tile, slice) units their workspace holds
 // What they read: the rows of dY of kept data, compact (dense: all rows) into packY, a whole matrix M into Mp, and zeros in
-// the rows of dX_zero of dropped data; each may be nullptr.  programmatic: launched as a dependent of the kernel before it.
+// the rows of dX_zero of dropped data; each may be nullptr.  programmatic: launched as a dependent of the kernel before it; early: M is cut before that
+// has ended (it must not be that kernel's, and nothing before in the call reads Mp).
 cudaError_t launch_split_prep(Handle* h, const void* dY, bool dense, const void* M, __nv_bfloat16* Mp, int m_rows, int m_d,
-                              void* dX_zero, bool programmatic, cudaStream_t st);
+                              void* dX_zero, bool programmatic, bool early, cudaStream_t st);
 // dX from packY and packW (bf16: from packY, or dY itself when dense, and W)
 cudaError_t launch_split_dx(Handle* h, const void* dY, const void* W, bool dense, float rho_hint, const void* H, void* dX,
                             cudaStream_t st);

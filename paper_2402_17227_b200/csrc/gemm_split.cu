@@ -393,27 +393,40 @@ __device__ __forceinline__ void prep_row(const T* src, __nv_bfloat16* dst, size_
     }
   }
 }
-template <typename T>
+// EARLY: the matrix is cut before the wait for the kernel before, in an instance of its own: the others, whose code is short
+// enough that more of it costs them 0.5 us, take it behind the rows, which the product needs first.
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(PREP_THREADS) prep_kernel(PrepParams P) {
   constexpr bool CUT = sizeof(T) == 4;
-  pdl_wait();
-  pdl_trigger();
   const int lane = threadIdx.x & 31;
-  const int cntA = P.idxA != nullptr ? P.counts[0] : P.N;
   const int yseg = (P.d_out + PREP_ELEMS - 1) / PREP_ELEMS, mseg = (P.m_d + PREP_ELEMS - 1) / PREP_ELEMS,
             zseg = (P.d_in + PREP_ELEMS - 1) / PREP_ELEMS;
-  const int n_y = P.Y != nullptr ? cntA * P.T * yseg : 0, n_m = P.M != nullptr ? P.m_rows * mseg : 0,
-            n_z = P.dX != nullptr ? (P.N - cntA) * P.T * zseg : 0;
   const int warps = gridDim.x * (PREP_THREADS / 32);
-  for (int i = blockIdx.x * (PREP_THREADS / 32) + (threadIdx.x >> 5); i < n_y + n_m + n_z; i += warps) {
+  const int all_m = P.M != nullptr ? P.m_rows * mseg : 0, n_m = EARLY ? 0 : all_m;
+  int i = blockIdx.x * (PREP_THREADS / 32) + (threadIdx.x >> 5);
+  auto cut_m = [&](int item) {
+    const int r = item / mseg, first = (item - r * mseg) * PREP_ELEMS;
+    prep_row<T, CUT>(reinterpret_cast<const T*>(P.M) + (size_t)r * P.m_d, P.Mp + (size_t)r * P.m_d, P.m_stride, P.m_d, first, lane);
+  };
+  if constexpr (EARLY) {
+    pdl_trigger();
+    for (; i < all_m; i += warps) cut_m(i);
+    i -= all_m;
+    pdl_wait();
+  } else {
+    pdl_wait();
+    pdl_trigger();
+  }
+  const int cntA = P.idxA != nullptr ? P.counts[0] : P.N;
+  const int n_y = P.Y != nullptr ? cntA * P.T * yseg : 0, n_z = P.dX != nullptr ? (P.N - cntA) * P.T * zseg : 0;
+  for (; i < n_y + n_m + n_z; i += warps) {
     if (i < n_y) {
       const int c = i / yseg, first = (i - c * yseg) * PREP_ELEMS;
       const int k = c / P.T;
       const size_t r = (size_t)(P.idxA != nullptr ? P.idxA[k] : k) * P.T + (c - k * P.T);
       prep_row<T, CUT>(reinterpret_cast<const T*>(P.Y) + r * P.d_out, P.Yp + (size_t)c * P.d_out, P.y_stride, P.d_out, first, lane);
-    } else if (i < n_y + n_m) {
-      const int r = (i - n_y) / mseg, first = (i - n_y - r * mseg) * PREP_ELEMS;
-      prep_row<T, CUT>(reinterpret_cast<const T*>(P.M) + (size_t)r * P.m_d, P.Mp + (size_t)r * P.m_d, P.m_stride, P.m_d, first, lane);
+    } else if (!EARLY && i < n_y + n_m) {
+      cut_m(i - n_y);
     } else {
       const int c = (i - n_y - n_m) / zseg, first = (i - n_y - n_m - c * zseg) * PREP_ELEMS;
       const int k = c / P.T;
@@ -502,7 +515,7 @@ int split_max_units(const vcas_layer_desc& d, int num_sms) {
 }
 
 cudaError_t launch_split_prep(Handle* h, const void* dY, bool dense, const void* M, __nv_bfloat16* Mp, int m_rows, int m_d,
-                              void* dX_zero, bool programmatic, cudaStream_t st) {
+                              void* dX_zero, bool programmatic, bool early, cudaStream_t st) {
   const vcas_layer_desc& d = h->desc;
   PrepParams P = {};
   P.Y = dY; P.Yp = h->ws.packY; P.y_stride = (size_t)h->R_pad * d.d_out;
@@ -517,9 +530,10 @@ cudaError_t launch_split_prep(Handle* h, const void* dY, bool dense, const void*
   long blocks = (items + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
   const long cap = (long)h->num_sms * 16;
   if (blocks > cap) blocks = cap;
-  const cudaError_t e = d.dtype == VCAS_DTYPE_F32
-      ? launch_maybe_after(programmatic, prep_kernel<float>, dim3((unsigned)blocks), dim3(PREP_THREADS), 0, st, P)
-      : launch_maybe_after(programmatic, prep_kernel<__nv_bfloat16>, dim3((unsigned)blocks), dim3(PREP_THREADS), 0, st, P);
+  const dim3 grid((unsigned)blocks), threads(PREP_THREADS);
+  const cudaError_t e = d.dtype != VCAS_DTYPE_F32 ? launch_maybe_after(programmatic, prep_kernel<__nv_bfloat16, false>, grid, threads, 0, st, P)
+      : early                                     ? launch_maybe_after(programmatic, prep_kernel<float, true>, grid, threads, 0, st, P)
+                                                  : launch_maybe_after(programmatic, prep_kernel<float, false>, grid, threads, 0, st, P);
   h->launches += 1;
   return e != cudaSuccess ? e : cudaGetLastError();
 }
