@@ -5,8 +5,8 @@
 //   sample_a_kernel   ||G_n||_F on a few CTAs, the last of which draws: p_n, mask, kept / dropped data (the dX product can
 //                     start here);
 //   scores_x_kernel   (score.cu) many CTAs: leverage scores and uniforms of the rows of kept data;
-//   sample_w_kernel   one CTA, scores in shared memory: the water-filling for q = min(1, c w) - a handful
-//                     of block-wide sums - then the masks' counts per chunk of 32 rows and their prefix sums;
+//   sample_w_small_kernel, sample_w_kernel  one CTA, scores in registers or in shared memory: the water-filling for q = min(1, c w)
+//                     - a handful of block-wide sums - then the masks' counts per chunk of 32 rows and their prefix sums;
 //   emit_pack_kernel  many CTAs: kept-row list, 1/(p q), and the compact operands of the dW product (emit_rows_kernel: without).
 // Only the scalar fixed point and a scan over R/32 counts run on a single SM.
 #include <atomic>
