@@ -138,6 +138,9 @@ __device__ __forceinline__ bool bernoulli_keep(float p, uint64_t seed, uint32_t 
 // before it in the stream is still running; it must call pdl_wait() before it touches anything that
 // kernel writes (the wait returns once that grid has completed and its writes are visible).
 // pdl_trigger() in the earlier kernel lets the dependent grid be scheduled from that point on.
+// Reading ahead: before its own wait a kernel may read what kernels further back wrote only if every CTA of the kernel between
+// calls pdl_wait() before pdl_trigger(); their writes are then complete when its first CTA starts.  It reads them past
+// L1 (__ldcg), whose lines only the wait is specified to make current.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

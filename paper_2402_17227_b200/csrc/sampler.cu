@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) sample_w_small_kernel(SampleW
   __shared__ WShared sh;
   __shared__ int s_cnt[32 * SLOTS];
   pdl_wait();      // the scores come from the kernel before this one
-  pdl_trigger();
+  pdl_trigger();   // not before the wait: the emitting kernel reads them ahead
   sample_w_small<SLOTS>(P, &sh, s_cnt);
 }
 
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(SAMPLER_THREADS) sample_w_kernel(SampleWParams
   extern __shared__ __align__(16) float s_w[];
   __shared__ WShared sh;
   pdl_wait();      // the scores come from the kernel before this one
-  pdl_trigger();
+  pdl_trigger();   // not before the wait: the emitting kernel reads them ahead
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cntA = P.counts[0];
   const int T = P.T;
@@ -572,8 +572,8 @@ struct RecordOut {
   float* g; float* p; float* w; float* q;
   int32_t* idxA; int32_t* cntA; int32_t* idxW; int32_t* cntW;
 };
-// A compact row of a chunk of 32, one per lane, as the kernels before SampleW left it.  The first chunk of a CTA is read before the
-// wait for SampleW, which started when they had ended and then let this grid start (whole calls: 192 rows, 128 -> 192, 22.6 -> 21.5 us
+// A compact row of a chunk of 32, one per lane, as the kernels before SampleW left it.  The first chunk of a CTA is read ahead (see
+// pdl_wait), before the wait for SampleW, which started when they had ended and then let this grid start (whole calls: 192 rows, 128 -> 192, 22.6 -> 21.5 us
 // on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2).
 struct ChunkIn { bool in; int r; float w, sa; uint32_t u; };
 __device__ __forceinline__ ChunkIn chunk_in(const EmitParams& P, int ch, int lane, int n) {
@@ -582,11 +582,11 @@ __device__ __forceinline__ ChunkIn chunk_in(const EmitParams& P, int ch, int lan
   o.in = i < n;
   if (o.in) {
     const int k = i / P.T;
-    const int nd = P.idxA[k];
+    const int nd = __ldcg(P.idxA + k);
     o.r = nd * P.T + (i - k * P.T);
-    o.w = P.wc[i];
-    o.u = P.sample_w ? P.uc[i] : 0u;
-    o.sa = P.scaleA[nd];
+    o.w = __ldcg(P.wc + i);
+    o.u = P.sample_w ? __ldcg(P.uc + i) : 0u;
+    o.sa = __ldcg(P.scaleA + nd);
   }
   return o;
 }
@@ -612,7 +612,7 @@ constexpr int EMIT_THREADS = 256;
 // launch of a CTA per chunk and a copying one, a scoring call of 16384 rows of 4096 and 1024 columns took 126.4 us, now 121.9.
 __global__ void __launch_bounds__(EMIT_THREADS) emit_rows_kernel(EmitParams P, const float* g, const float* p, RecordOut O) {
   const int tid = blockIdx.x * EMIT_THREADS + threadIdx.x, threads = gridDim.x * EMIT_THREADS, lane = threadIdx.x & 31;
-  const int cntA = P.counts[0], T = P.T, n = cntA * T;
+  const int cntA = __ldcg(P.counts), T = P.T, n = cntA * T;
   ChunkIn x = chunk_in(P, tid >> 5, lane, n);
   pdl_wait();      // c and the chunk offsets come from the kernel before this one
   pdl_trigger();
@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   __shared__ int s_r[32], s_pos[32], s_cnt;
   __shared__ float s_sc[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, parts = P.parts;
-  const int cntA = P.counts[0];
+  const int cntA = __ldcg(P.counts);
   const int T = P.T;
   const int n = cntA * T;
   ChunkIn x = {};
