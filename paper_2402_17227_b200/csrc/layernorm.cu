@@ -90,7 +90,8 @@ __device__ __forceinline__ void group_sum(float (&v)[3], int n, float* slot, int
 // stores one partial sum per column.  (With a second, column-wise pass over the rows the call on 16384 x 1024 at ratio 0.5
 // took 87 us, 17 for the rows and 40 for the columns, one dependent load at a time.)
 // Bound by instructions as much as by bytes: the values are widened once and worked on in pairs (f32x2), gamma is widened once
-// for all rows, 1/p and 1/sigma are factored out of the sums.  A row is also a chain of a memory latency and two reductions, so
+// for all rows.  1/sigma multiplies x - mean and the sum in brackets one after the other: as one factor 1/sigma^2 it left fp32's range
+// for x of 1e17 or 1e-18 (16384 x 1024, ratio 0.5 and 1: 32.4 and 39.9 us so, 32.9 and 41.2 now).  A row is also a chain of a memory latency and two reductions, so
 // the next row's loads are issued before the present one is worked on, and the zero rows of dropped data go out while the first
 // is on its way.  (A row in four vectors a lane, widened in each pass and not loaded ahead: that call 37.1 us, now 35.8; at
 // ratio 1 48.1 and 43.2; 4096 columns 116 and 108, 2048 rows of 8192 56.9 and 50.0; 1408, of 2048 a group holds, 53.8 and 54.8.)
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
     group_sum<G>(sums, 1, s_slot[group], gw, group);
     const float mean = sums[0] * inv_d;
     // variance, and the two row sums of g_hat = G_hat * gamma that the Jacobian needs
-    const uint64_t nmean = pack2(-mean, -mean);
+    const uint64_t nmean = pack2(-mean, -mean), scale = pack2(sc, sc);
     p0 = 0;
 #pragma unroll
     for (int q = 0; q < LN_VPL; ++q)
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
 #pragma unroll
         for (int e = 0; e < VN / 2; ++e) {
           x[q][e] = add2(x[q][e], nmean);
+          g[q][e] = mul2(g[q][e], scale);
           const uint64_t gh = mul2(g[q][e], w[q][e]);
           p0 = fma2(x[q][e], x[q][e], p0);
           p1 = add2(p1, gh);
@@ -200,10 +202,8 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
     sums[0] = halves(p0); sums[1] = halves(p1); sums[2] = halves(p2);
     group_sum<G>(sums, 3, s_slot[group], gw, group);
     const float rstd = rsqrtf(sums[0] * inv_d + P.eps);
-    const float m1 = sc * sums[1] * inv_d, m2 = sc * sums[2] * rstd * inv_d;     // mean(g_hat), mean(g_hat * x_hat)
-    // dX = (g_hat - m1 - x_hat m2) / sigma
-    const float f0 = sc * rstd, f1 = -m1 * rstd, f2 = -m2 * rstd * rstd;
-    const uint64_t s0 = pack2(f0, f0), s1 = pack2(f1, f1), s2 = pack2(f2, f2), s3 = pack2(sc, sc);
+    const float m1 = sums[1] * inv_d, m2 = sums[2] * rstd * inv_d;     // mean(g_hat), mean(g_hat * x_hat)
+    const uint64_t nm1 = pack2(-m1, -m1), nm2 = pack2(-m2, -m2), inv = pack2(rstd, rstd);
     float sq[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int q = 0; q < LN_VPL; ++q)
@@ -211,10 +211,11 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
         float o[VN];
 #pragma unroll
         for (int e = 0; e < VN / 2; ++e) {
-          const uint64_t gs = mul2(g[q][e], s0);
-          unpack2(fma2(x[q][e], s2, fma2(gs, w[q][e], s1)), o[2 * e], o[2 * e + 1]);
-          ag[q][e] = fma2(gs, x[q][e], ag[q][e]);
-          ab[q][e] = fma2(g[q][e], s3, ab[q][e]);
+          const uint64_t xh = mul2(x[q][e], inv);
+          // dX = (g_hat - m1 - x_hat m2) / sigma
+          unpack2(mul2(fma2(xh, nm2, fma2(g[q][e], w[q][e], nm1)), inv), o[2 * e], o[2 * e + 1]);
+          ag[q][e] = fma2(g[q][e], xh, ag[q][e]);
+          ab[q][e] = add2(ab[q][e], g[q][e]);
         }
         V ov;
         sq[0] += L::pack(o, ov, P.a_out != nullptr);
