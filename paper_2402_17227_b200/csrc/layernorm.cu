@@ -60,9 +60,6 @@ struct LnParams {
   float eps;
 };
 
-constexpr int LN_VPL = 2;          // 16-byte vectors of a row that a lane holds
-template <int G> constexpr int LN_WARPS = G > 8 ? G : G == 3 ? 9 : 8;      // of a CTA with G warps per row
-
 // Sum of one float over the G warps of a row group, in a fixed order; result in every lane.  slot: G floats per group.
 template <int G>
 __device__ __forceinline__ void group_sum(float (&v)[3], int n, float* slot, int gw, int group) {
@@ -84,22 +81,24 @@ __device__ __forceinline__ void group_sum(float (&v)[3], int n, float* slot, int
   }
 }
 
-// G warps per row, two vectors of it a lane, the kept rows dealt out to the row groups of the grid in turn.  The row's
+// G warps per row, VPL vectors of it a lane, the kept rows dealt out to the row groups of the grid in turn.  The row's
 // statistics, dX and its share of the column sums dgamma = sum_r G_hat_r x_hat_r, dbeta = sum_r G_hat_r come from one read of X
 // and dY; a lane keeps the column sums of its columns in registers over all its rows, the CTA adds its groups in order and
 // stores one partial sum per column.  (With a second, column-wise pass over the rows the call on 16384 x 1024 at ratio 0.5
 // took 87 us, 17 for the rows and 40 for the columns, one dependent load at a time.)
 // Bound by instructions as much as by bytes: the values are widened once and worked on in pairs (f32x2), gamma is widened once
-// for all rows.  1/sigma multiplies x - mean and the sum in brackets one after the other: as one factor 1/sigma^2 it left fp32's range
-// for x of 1e17 or 1e-18 (16384 x 1024, ratio 0.5 and 1: 32.4 and 39.9 us so, 32.9 and 41.2 now).  A row is also a chain of a memory latency and two reductions, so
-// the next row's loads are issued before the present one is worked on, and the zero rows of dropped data go out while the first
-// is on its way.  (A row in four vectors a lane, widened in each pass and not loaded ahead: that call 37.1 us, now 35.8; at
-// ratio 1 48.1 and 43.2; 4096 columns 116 and 108, 2048 rows of 8192 56.9 and 50.0; 1408, of 2048 a group holds, 53.8 and 54.8.)
-template <typename T, int G>
-__global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnParams P) {
+// for all rows.  1/sigma multiplies x - mean and the sum in brackets one after the other: as one factor 1/sigma^2 it left fp32's
+// range for x of 1e17 or 1e-18 (16384 x 4096, ratio 0.5 and 1: 102.3 and 137.5 us so, 102.9 and 139.8 now).  A row is also a chain
+// of a memory latency and two reductions, so the next row's loads are issued before the present one is worked on, and the zero
+// rows of dropped data go out while the first is on its way.  (A row in four vectors a lane, widened in each pass and not loaded
+// ahead: bf16, 16384 x 1024, ratio 0.5 35.2 us the call, now 32.6; ratio 1 43.9 and 39.2; 4096 columns 107 and 103, 2048 rows of
+// 8192 53.5 and 39.2; fp32, 16384 x 4096 156 and 149.)
+template <typename T, int G, int VPL, int WARPS, int CTAS>
+__global__ void __launch_bounds__(WARPS * 32, CTAS) ln_kernel(LnParams P) {
   using L = Ld<T>;
   using V = typename L::V;
-  constexpr int VN = L::N, WARPS = LN_WARPS<G>, GROUPS = WARPS / G;
+  constexpr int VN = L::N, GROUPS = WARPS / G;
+  static_assert(GROUPS * G == WARPS && (G == 1 || GROUPS < 16), "whole groups, a named barrier each");
   __shared__ float s_slot[GROUPS][G * 3];
   extern __shared__ float s_col[];                   // [GROUPS][2][32 * G * VN] column sums on their way to the CTA's sum
   pdl_wait();      // the kept data come from the SampleA kernel
@@ -110,8 +109,8 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
   const int nv = d / VN;
   const float inv_d = 1.0f / (float)d;
   const int v0 = gw * 32 + lane;                     // this lane's vectors: v0, v0 + 32 G
-  bool has[LN_VPL];
-  uint64_t w[LN_VPL][VN / 2], ag[LN_VPL][VN / 2], ab[LN_VPL][VN / 2];
+  bool has[VPL];
+  uint64_t w[VPL][VN / 2], ag[VPL][VN / 2], ab[VPL][VN / 2];
   auto widen = [](const V& v, uint64_t (&o)[VN / 2]) {
     float f[VN];
     L::unpack(v, f);
@@ -119,14 +118,14 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
     for (int e = 0; e < VN / 2; ++e) o[e] = pack2(f[2 * e], f[2 * e + 1]);
   };
 #pragma unroll
-  for (int q = 0; q < LN_VPL; ++q) {
+  for (int q = 0; q < VPL; ++q) {
     has[q] = v0 + q * 32 * G < nv;
 #pragma unroll
     for (int e = 0; e < VN / 2; ++e) { w[q][e] = 0; ag[q][e] = 0; ab[q][e] = 0; }
     if (has[q]) widen(__ldg(reinterpret_cast<const V*>((const T*)P.gamma) + v0 + q * 32 * G), w[q]);
   }
   const int groups = gridDim.x * GROUPS, me = blockIdx.x * GROUPS + group;
-  V xn[LN_VPL], gn[LN_VPL];                          // the next row, its number and 1/p
+  V xn[VPL], gn[VPL];                          // the next row, its number and 1/p
   size_t rn = 0;
   float scn = 0.f;
   int k = me / Tn, t = me - k * Tn;                  // the row to be loaded next: token t of the k-th kept datum
@@ -141,10 +140,10 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
     const V* xv = reinterpret_cast<const V*>((const T*)P.X + rn * d);
     const V* gv = reinterpret_cast<const V*>((const T*)P.dY + rn * d);
 #pragma unroll
-    for (int q = 0; q < LN_VPL; ++q)
+    for (int q = 0; q < VPL; ++q)
       if (has[q]) xn[q] = __ldg(xv + v0 + q * 32 * G);
 #pragma unroll
-    for (int q = 0; q < LN_VPL; ++q)
+    for (int q = 0; q < VPL; ++q)
       if (has[q]) gn[q] = __ldg(gv + v0 + q * 32 * G);
   };
   if (me < kept_rows) fetch();
@@ -166,16 +165,16 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
   for (int c = me; c < kept_rows; c += groups) {
     const size_t r = rn;
     const float sc = scn;
-    uint64_t x[LN_VPL][VN / 2], g[LN_VPL][VN / 2];
+    uint64_t x[VPL][VN / 2], g[VPL][VN / 2];
 #pragma unroll
-    for (int q = 0; q < LN_VPL; ++q)
+    for (int q = 0; q < VPL; ++q)
       if (has[q]) { widen(xn[q], x[q]); widen(gn[q], g[q]); }
     if (c + groups < kept_rows) fetch();
     float sums[3] = {0.f, 0.f, 0.f};
     auto halves = [](uint64_t v) { float a, b; unpack2(v, a, b); return a + b; };
     uint64_t p0 = 0, p1 = 0, p2 = 0;
 #pragma unroll
-    for (int q = 0; q < LN_VPL; ++q)
+    for (int q = 0; q < VPL; ++q)
       if (has[q]) {
 #pragma unroll
         for (int e = 0; e < VN / 2; ++e) p0 = add2(p0, x[q][e]);
@@ -187,7 +186,7 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
     const uint64_t nmean = pack2(-mean, -mean), scale = pack2(sc, sc);
     p0 = 0;
 #pragma unroll
-    for (int q = 0; q < LN_VPL; ++q)
+    for (int q = 0; q < VPL; ++q)
       if (has[q]) {
 #pragma unroll
         for (int e = 0; e < VN / 2; ++e) {
@@ -206,7 +205,7 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
     const uint64_t nm1 = pack2(-m1, -m1), nm2 = pack2(-m2, -m2), inv = pack2(rstd, rstd);
     float sq[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-    for (int q = 0; q < LN_VPL; ++q)
+    for (int q = 0; q < VPL; ++q)
       if (has[q]) {
         float o[VN];
 #pragma unroll
@@ -230,7 +229,7 @@ __global__ void __launch_bounds__(LN_WARPS<G> * 32, G > 8 ? 1 : 2) ln_kernel(LnP
   // the CTA's column sums, groups in order
   constexpr int W = 32 * G * VN;                     // columns of one q
 #pragma unroll
-  for (int q = 0; q < LN_VPL; ++q) {
+  for (int q = 0; q < VPL; ++q) {
     if (q * 32 * G >= nv) break;
     __syncthreads();
 #pragma unroll
@@ -422,16 +421,16 @@ __global__ void __launch_bounds__(256) ln_range_add_kernel(LnParams P, int range
   (which == 0 ? P.dgamma : P.dbeta)[col] = t;
 }
 
-template <typename T, int G>
-cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
-  // Two CTAs per SM (of sixteen warps: one), fewer when there are fewer rows than row groups or the scratch (4 d^2 floats) is small
-  constexpr int WARPS = LN_WARPS<G>;
-  long blocks = (rows + WARPS / G - 1) / (WARPS / G);
-  const int most = (G > 8 ? 1 : 2) * h->num_sms;
-  if (blocks > most) blocks = most;
+// WARPS warps a CTA, CTAS CTAs per SM
+template <typename T, int G, int VPL, int WARPS, int CTAS>
+cudaError_t run_rows(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
+  // fewer when there are fewer rows than row groups or the scratch (4 d^2 floats) is small
+  constexpr int GROUPS = WARPS / G;
+  long blocks = (rows + GROUPS - 1) / GROUPS;
+  if (blocks > CTAS * h->num_sms) blocks = CTAS * h->num_sms;
   if (blocks > 2l * P.d) blocks = 2l * P.d;
   const size_t smem = (size_t)WARPS * 2 * 32 * Ld<T>::N * sizeof(float);
-  cudaError_t e = launch_after(ln_kernel<T, G>, dim3((unsigned)blocks), dim3(WARPS * 32), smem, st, P);
+  cudaError_t e = launch_after(ln_kernel<T, G, VPL, WARPS, CTAS>, dim3((unsigned)blocks), dim3(WARPS * 32), smem, st, P);
   if (e == cudaSuccess)
     e = launch_after(ln_add_kernel, dim3(2 * ((P.d + 31) / 32)), dim3(ADD_WARPS * 32), 0, st, P, (int)blocks);
   h->launches += 2;
@@ -439,16 +438,35 @@ cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
 }
 template <typename T>
 cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
-  const int per_warp = 32 * LN_VPL * Ld<T>::N;       // columns one warp can hold
-  if (P.d <= per_warp) return run_ln<T, 1>(h, P, rows, st);
-  if (P.d <= 2 * per_warp) return run_ln<T, 2>(h, P, rows, st);
-  // 768 columns in fp32 (4096 rows: 19.7 us the call with a fourth, idle warp a row, 18.6 so); nine warps leave a bf16 row too
-  // few registers (16384 x 1408: 66 us)
-  if constexpr (sizeof(T) == 4)
-    if (P.d <= 3 * per_warp) return run_ln<T, 3>(h, P, rows, st);
-  if (P.d <= 4 * per_warp) return run_ln<T, 4>(h, P, rows, st);
-  if (P.d <= 8 * per_warp) return run_ln<T, 8>(h, P, rows, st);
-  if (P.d <= 16 * per_warp) return run_ln<T, 16>(h, P, rows, st);
+  // The 16-byte vectors of a row decide; a group holds 32 G VPL.  Groups that fit leave no warp with a half-empty row to wait
+  // for (powers of two of two vectors a lane, 16384 rows at ratio 0.5 and so: bf16, 576 columns 31.1 and 29.0 us, 1088 47.4 and
+  // 41.3, 2560 81.1 and 69.9; fp32, 320 25.2 and 23.6, 1280 72.2 and 61.8, 2560 124 and 104).  Three and four vectors a lane have
+  // registers for the next row in fp32 only, in bf16 three with twelve warps an SM; in fp32 they beat more warps a row, which wait for
+  // one another (4096 columns by sixteen warps 158 us, by eight 149).  One CTA an SM halves the column sums to be added up (bf16,
+  // 2048 rows of 2048 18.8 and 17.8 us); fp32, 2048 columns: in CTAs of one row group, four an SM, 2048 rows take 21.9 us, in one
+  // CTA 19.7; 16384 rows at ratio 1 98.8 and 106.3.
+  const int nv = P.d / Ld<T>::N;
+  if constexpr (sizeof(T) == 2) {
+    if (nv <= 64) return run_rows<T, 1, 2, 8, 2>(h, P, rows, st);
+    if (nv <= 96) return run_rows<T, 1, 3, 12, 1>(h, P, rows, st);
+    if (nv <= 128) return run_rows<T, 2, 2, 16, 1>(h, P, rows, st);
+    if (nv <= 192) return run_rows<T, 3, 2, 12, 1>(h, P, rows, st);
+    if (nv <= 256) return run_rows<T, 4, 2, 16, 1>(h, P, rows, st);
+    if (nv <= 320) return run_rows<T, 5, 2, 15, 1>(h, P, rows, st);
+    if (nv <= 512) return run_rows<T, 8, 2, 8, 2>(h, P, rows, st);
+    if (nv <= 1024) return run_rows<T, 16, 2, 16, 1>(h, P, rows, st);
+  } else {
+    if (nv <= 64) return run_rows<T, 1, 2, 8, 2>(h, P, rows, st);
+    if (nv <= 96) return run_rows<T, 1, 3, 8, 2>(h, P, rows, st);
+    if (nv <= 128) return run_rows<T, 2, 2, 8, 2>(h, P, rows, st);
+    if (nv <= 192) return run_rows<T, 2, 3, 8, 2>(h, P, rows, st);
+    if (nv <= 256) return run_rows<T, 4, 2, 8, 2>(h, P, rows, st);
+    if (nv <= 384) return run_rows<T, 4, 3, 16, 1>(h, P, rows, st);
+    if (nv <= 480) return run_rows<T, 5, 3, 15, 1>(h, P, rows, st);
+    if (nv <= 512) return rows > 4096 ? run_rows<T, 4, 4, 4, 4>(h, P, rows, st) : run_rows<T, 8, 2, 16, 1>(h, P, rows, st);
+    if (nv <= 768) return run_rows<T, 8, 3, 8, 2>(h, P, rows, st);
+    if (nv <= 1024) return run_rows<T, 8, 4, 8, 2>(h, P, rows, st);
+  }
   const int col_blocks = (P.d + 255) / 256;
   const int chunks = 4 * h->num_sms > col_blocks ? 4 * h->num_sms / col_blocks : 1;
   const long blocks = (rows + 7) / 8 < (1l << 20) ? (rows + 7) / 8 : (1l << 20);

@@ -1,5 +1,5 @@
 """LayerNorm behind SampleA with several rows per row group (each loaded while the one before is worked on), at the widths of the
-groups of one to four warps, dropped rows written or left.  Tolerances: one bf16 rounding of dX (2^-9 / sqrt(3) of its norm) and
+groups of one to sixteen warps, dropped rows written or left.  Tolerances: one bf16 rounding of dX (2^-9 / sqrt(3) of its norm) and
 fp32 sums; the column sums add up to 6000 rows in fp32, in a tree of row groups, CTAs and ranges of them."""
 import numpy as np
 import pytest
@@ -15,7 +15,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
-@pytest.mark.parametrize("N,T,d", [(30, 200, 256), (30, 200, 264), (7, 857, 768), (30, 100, 776), (2500, 2, 64)])
+@pytest.mark.parametrize("N,T,d", [(30, 200, 256), (30, 200, 264), (7, 857, 768), (30, 100, 776), (2500, 2, 64), (30, 200, 512),
+                                   (25, 100, 1032), (9, 200, 1544), (10, 100, 2000), (42, 100, 2000), (9, 100, 2056), (9, 100, 4096),
+                                   (9, 100, 4104)])
 def test_rows_loaded_ahead(dtype, N, T, d):
     vbuild.build()
     X, dY, _ = inputs.make_layer(inputs.LayerCase("ln", N, T, d, d, dtype, 0.5, 0.5, 0.5, 0.5), d_out=d)

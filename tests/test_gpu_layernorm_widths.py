@@ -1,6 +1,6 @@
-"""LayerNorm behind SampleA at the widths where a row changes from one, two, four or eight warps to the two-pass kernels,
-with few and many rows, against the oracle.  Tolerances as derived for the narrower widths: one bf16 rounding of dX
-(2^-9 / sqrt(3) of its norm) and fp32 sums; the column sums add up to 300 rows in fp32."""
+"""LayerNorm behind SampleA at the widths where a row changes from one to sixteen warps and to the two-pass kernels, with few
+and many rows, against the oracle.  Tolerances as derived for the narrower widths: one bf16 rounding of dX (2^-9 / sqrt(3) of its
+norm) and fp32 sums; the column sums add up to 300 rows in fp32."""
 import numpy as np
 import pytest
 import torch
