@@ -164,6 +164,8 @@ int plain_dx(Handle* h, const void* dY, const void* W, float rho, const void* Hp
     // Behind SampleA the weight is cut while that runs, where dX ends the call: from 14 GFLOP of part products on (fp32, 14.5,
     // 768 -> 1536: 57.7 and 56.8 us; 29, 768 -> 3072: 78.5 and 76.7; 35, 768 -> 3072: 90.0 and 88.0).  Where dW's branch ends it,
     // a product that starts earlier keeps the SMs from that branch's X norms (10, 768 -> 768: 55.6 and 60.3; 7.2: 45.7 and 48.1).
+    // The same line where the join is deferred and the next layer's dX follows (stacks of two and four layers, 2048 to 8192 rows,
+    // 512 to 1024 columns: 0.99 to 1.05 times as long with the weight cut behind SampleA, 1.01 in the middle).
     const bool early = programmatic && 12.0 * rho * h->desc.N * h->desc.T * (double)h->desc.d_in * h->desc.d_out > 14e9;
     VCAS_CUDA(launch_split_prep(h, dY, false, fp32 ? W : nullptr, h->ws.packW, h->desc.d_out, h->desc.d_in, dX, programmatic, early, st));
     VCAS_CUDA(launch_split_dx(h, dY, W, false, rho, Hpre, dX, st));
@@ -319,8 +321,8 @@ int run_sampled(Handle* h, const void* X, const void* dY, const void* W, const S
                 void* dX, float* dW, float* a_out, bool skip_dropped, bool defer_join, cudaStream_t st) {
   if (join_pending(h, st) != VCAS_OK) return VCAS_ERR_CUDA;
   const int hint = (int)(a.rho * a.nu * (float)(h->desc.N * h->desc.T)) + 1;
-  // The sampled dX grid leaves one SM free: SampleW's single-CTA kernel, which runs beside it on the side
-  // stream, needs a whole SM's shared memory.
+  // The sampled dX grid leaves one SM free for SampleW's single CTA, which runs beside it on the other stream: up to 16384 rows the
+  // registers of its 1024 threads (32 each, or 64) do not fit beside a dX CTA (320 threads of 104), beyond them its shared memory.
   const int spare = 1;
   Plan px = {256, 1, 1}, pw = {256, 1, 1};
   if (h->tensor_path) plan_products(h, false, a.rho, hint, spare, a_out != nullptr, Hpre != nullptr, &px, &pw);

@@ -466,7 +466,10 @@ cudaError_t run_split(Handle* h, const CUtensorMap& a, const CUtensorMap& b, Spl
     attr_set[h->device].store(true, std::memory_order_release);
   }
   // A sampled dX leaves one SM to SampleW, whose CTA does not fit beside one of these and would wait for a product to end
-  // (fp32, 8192 rows, 512 -> 512: 67.5 and 66.8 us the call; 8192, 256 -> 1024: 54.6 and 54.1; 2048, 768 -> 3072: 78.2 and 77.7).
+  // (fp32, 8192 rows, 512 -> 512: 67.5 and 66.8 us the call; 8192, 256 -> 1024: 54.6 and 54.1; 2048, 768 -> 3072: 78.2 and 77.7).  Also
+  // where that makes a wave more: of 4700 rows, 148 tiles, dX alone takes 52 us on all SMs and 81 on one less (fp32, 1024 -> 1024;
+  // bf16, 1000 -> 3000: 50 and 78), but the call 116 and 105 (145 and 136), as the dW branch is not held up.  With stage
+  // profiling, where nothing runs beside it, too: the stages timed are the call's, bit for bit.
   const int sms = MODE == MODE_DX && P.counts != nullptr && h->num_sms > 1 ? h->num_sms - 1 : h->num_sms;
   P.slices = split_slices(h, sms, exp_tiles, k, PA * PB == 9 ? 1.7 : (PA * PB == 3 ? 0.9 : 0.55));
   long grid = max_tiles * P.slices;

@@ -249,7 +249,9 @@ __global__ void __launch_bounds__(SAMPLE_A_THREADS) sample_a_kernel(SampleAParam
 // 3.4 us on the host, and its start on the GPU (whole calls, two launches and one: 2048 rows of 4096, 55.3 and 51.0 us; of 3072,
 // 38.9 and 36.8; of 1000, 41.8 and 40.8; 3200 of 4096, 50.5 and 46.3; 256 of 256, 25.8 and 23.5).  With more rows the wait for
 // the last CTA takes back what it saves (4096 of 3072: 40.7 and 39.6 in bf16, 90.0 and 90.6 in fp32; of 256, 31.2 and 31.6; 8192:
-// 46.9 and 48.7), and with more data their sums by one CTA cost more (100 of 16 rows: 28.9 and 35.0).
+// 46.9 and 48.7), and with more data their sums by one CTA cost more (100 of 16 rows: 28.9 and 35.0).  LayerNorm and scoring calls
+// gain the launch on the host (LayerNorm, 256 to 3072 rows of 256 to 1024: 18.2 and 16.0 us; eight scoring calls 0.97 to 1.00 of the
+// time, 1576 rows of 768 1.04, the kernels alone 0.94 for 2048 rows of 3072 to 1.07 for 2048 of 1024 in fp32).
 constexpr int FUSED_MAX_N = 32, FUSED_MAX_ROWS = 3200;
 template <typename T>
 __global__ void __launch_bounds__(SAMPLE_A_THREADS) norms_sample_a_kernel(const T* __restrict__ dY, int d_out, float* __restrict__ a,
@@ -574,7 +576,7 @@ struct RecordOut {
 };
 // A compact row of a chunk of 32, one per lane, as the kernels before SampleW left it.  The first chunk of a CTA is read ahead (see
 // pdl_wait), before the wait for SampleW, which started when they had ended and then let this grid start (whole calls: 192 rows, 128 -> 192, 22.6 -> 21.5 us
-// on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2).
+// on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2, of which the loads past L1 took back 0.4).
 struct ChunkIn { bool in; int r; float w, sa; uint32_t u; };
 __device__ __forceinline__ ChunkIn chunk_in(const EmitParams& P, int ch, int lane, int n) {
   ChunkIn o = {};
