@@ -446,26 +446,31 @@ cudaError_t run_ln(Handle* h, const LnParams& P, long rows, cudaStream_t st) {
   // 2048 rows of 2048 18.8 and 17.8 us); fp32, 2048 columns: in CTAs of one row group, four an SM, 2048 rows take 21.9 us, in one
   // CTA 19.7; 16384 rows at ratio 1 98.8 and 106.3.
   const int nv = P.d / Ld<T>::N;
+  // Few rows, of which a group has one at most: more and smaller CTAs start sooner (256 rows of 768 in bf16, the kernels alone: by
+  // two warps a row in CTAs of eight 10.4 us, by one in CTAs of twelve 11.3; 512 rows of 3072 in fp32 by sixteen warps 14.2, by eight
+  // 15.6; up to 2048 rows of 4096 so).
+  const bool few = rows <= 512;
   if constexpr (sizeof(T) == 2) {
     if (nv <= 64) return run_rows<T, 1, 2, 8, 2>(h, P, rows, st);
+    if (nv <= 128 && few) return run_rows<T, 2, 2, 8, 2>(h, P, rows, st);
     if (nv <= 96) return run_rows<T, 1, 3, 12, 1>(h, P, rows, st);
     if (nv <= 128) return run_rows<T, 2, 2, 16, 1>(h, P, rows, st);
     if (nv <= 192) return run_rows<T, 3, 2, 12, 1>(h, P, rows, st);
-    if (nv <= 256) return run_rows<T, 4, 2, 16, 1>(h, P, rows, st);
+    if (nv <= 256) return few ? run_rows<T, 4, 2, 8, 2>(h, P, rows, st) : run_rows<T, 4, 2, 16, 1>(h, P, rows, st);
     if (nv <= 320) return run_rows<T, 5, 2, 15, 1>(h, P, rows, st);
     if (nv <= 512) return run_rows<T, 8, 2, 8, 2>(h, P, rows, st);
     if (nv <= 1024) return run_rows<T, 16, 2, 16, 1>(h, P, rows, st);
   } else {
     if (nv <= 64) return run_rows<T, 1, 2, 8, 2>(h, P, rows, st);
-    if (nv <= 96) return run_rows<T, 1, 3, 8, 2>(h, P, rows, st);
+    if (nv <= 96 && !few) return run_rows<T, 1, 3, 8, 2>(h, P, rows, st);
     if (nv <= 128) return run_rows<T, 2, 2, 8, 2>(h, P, rows, st);
     if (nv <= 192) return run_rows<T, 2, 3, 8, 2>(h, P, rows, st);
     if (nv <= 256) return run_rows<T, 4, 2, 8, 2>(h, P, rows, st);
-    if (nv <= 384) return run_rows<T, 4, 3, 16, 1>(h, P, rows, st);
-    if (nv <= 480) return run_rows<T, 5, 3, 15, 1>(h, P, rows, st);
+    if (nv <= 384 && !few) return run_rows<T, 4, 3, 16, 1>(h, P, rows, st);
+    if (nv <= 480 && !few) return run_rows<T, 5, 3, 15, 1>(h, P, rows, st);
     if (nv <= 512) return rows > 4096 ? run_rows<T, 4, 4, 4, 4>(h, P, rows, st) : run_rows<T, 8, 2, 16, 1>(h, P, rows, st);
-    if (nv <= 768) return run_rows<T, 8, 3, 8, 2>(h, P, rows, st);
-    if (nv <= 1024) return run_rows<T, 8, 4, 8, 2>(h, P, rows, st);
+    if (nv <= 768 && !few) return run_rows<T, 8, 3, 8, 2>(h, P, rows, st);
+    if (nv <= 1024) return rows > 2048 ? run_rows<T, 8, 4, 8, 2>(h, P, rows, st) : run_rows<T, 16, 2, 16, 1>(h, P, rows, st);
   }
   const int col_blocks = (P.d + 255) / 256;
   const int chunks = 4 * h->num_sms > col_blocks ? 4 * h->num_sms / col_blocks : 1;

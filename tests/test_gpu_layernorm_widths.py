@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
-@pytest.mark.parametrize("N,T,d", [(1, 1, 8), (5, 60, 512), (5, 60, 520), (4, 33, 1024), (4, 33, 1032), (3, 21, 2056), (3, 21, 4104),
+@pytest.mark.parametrize("N,T,d", [(1, 1, 8), (5, 60, 512), (5, 60, 520), (4, 33, 1024), (4, 33, 1032), (4, 33, 2000), (3, 21, 2056), (2, 9, 4096), (3, 21, 4104),
                                    (2, 9, 8192), (2, 9, 8200)])
 def test_layernorm_bwd_at_every_row_group_size(dtype, N, T, d):
     vbuild.build()
