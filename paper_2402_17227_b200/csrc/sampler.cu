@@ -554,6 +554,7 @@ struct EmitParams {
   __nv_bfloat16* packG; __nv_bfloat16* packX;            // compact operands
   size_t g_stride, x_stride;                             // elements between the parts of a cut operand
   int N, T, d_in, d_out;
+  int ahead;                                             // CTAs that read their first chunk ahead
   int sample_w;
   int parts;                                             // CTAs that share the packing of one chunk's rows
 };
@@ -576,19 +577,23 @@ struct RecordOut {
 };
 // A compact row of a chunk of 32, one per lane, as the kernels before SampleW left it.  The first chunk of a CTA is read ahead (see
 // pdl_wait), before the wait for SampleW, which started when they had ended and then let this grid start (whole calls: 192 rows, 128 -> 192, 22.6 -> 21.5 us
-// on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2, of which the loads past L1 took back 0.4).
+// on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2, of which the loads past L1 took back 0.4).  Of a
+// packing grid only the CTAs that may be there by then do so, three an SM; the others read after the wait, and find in L1
+// what the chunk's other CTAs have read (4096 rows, 768 -> 3072: with every CTA past L1 44.6 us, so 43.9; 16384, 1024 -> 1024: 71.8 and 70.1).
 struct ChunkIn { bool in; int r; float w, sa; uint32_t u; };
+template <bool AHEAD>
 __device__ __forceinline__ ChunkIn chunk_in(const EmitParams& P, int ch, int lane, int n) {
+  auto read = [](const auto* p) { return AHEAD ? __ldcg(p) : *p; };
   ChunkIn o = {};
   const int i = (ch << 5) + lane;
   o.in = i < n;
   if (o.in) {
     const int k = i / P.T;
-    const int nd = __ldcg(P.idxA + k);
+    const int nd = read(P.idxA + k);
     o.r = nd * P.T + (i - k * P.T);
-    o.w = __ldcg(P.wc + i);
-    o.u = P.sample_w ? __ldcg(P.uc + i) : 0u;
-    o.sa = __ldcg(P.scaleA + nd);
+    o.w = read(P.wc + i);
+    o.u = P.sample_w ? read(P.uc + i) : 0u;
+    o.sa = read(P.scaleA + nd);
   }
   return o;
 }
@@ -610,19 +615,20 @@ __device__ __forceinline__ ChunkRow chunk_row(const EmitParams& P, const ChunkIn
   return o;
 }
 constexpr int EMIT_THREADS = 256;
+constexpr int EMIT_AHEAD = 3;      // CTAs per SM that fit in every instance (80 registers)
 // Without operands to pack: a warp per chunk, and the record into the caller's arrays.  Latency-bound; with an emitting
 // launch of a CTA per chunk and a copying one, a scoring call of 16384 rows of 4096 and 1024 columns took 126.4 us, now 121.9.
 __global__ void __launch_bounds__(EMIT_THREADS) emit_rows_kernel(EmitParams P, const float* g, const float* p, RecordOut O) {
   const int tid = blockIdx.x * EMIT_THREADS + threadIdx.x, threads = gridDim.x * EMIT_THREADS, lane = threadIdx.x & 31;
   const int cntA = __ldcg(P.counts), T = P.T, n = cntA * T;
-  ChunkIn x = chunk_in(P, tid >> 5, lane, n);
+  ChunkIn x = chunk_in<true>(P, tid >> 5, lane, n);
   pdl_wait();      // c and the chunk offsets come from the kernel before this one
   pdl_trigger();
   const int cntW = __ldcg(P.counts + 1);
   const float c = P.fix[0];
   const int mode = (int)P.fix[1];
   for (int ch = tid >> 5; ch < (n + 31) >> 5; ch += threads >> 5) {
-    if (ch != tid >> 5) x = chunk_in(P, ch, lane, n);
+    if (ch != tid >> 5) x = chunk_in<false>(P, ch, lane, n);
     const ChunkRow o = chunk_row(P, x, ch, lane, mode, c);
     if (x.in) {
       P.w[x.r] = x.w;
@@ -668,13 +674,18 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   __shared__ int s_r[32], s_pos[32], s_cnt;
   __shared__ float s_sc[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, parts = P.parts;
-  const int cntA = __ldcg(P.counts);
+  const bool ahead = (int)blockIdx.x < P.ahead;
   const int T = P.T;
-  const int n = cntA * T;
+  int cntA = 0;
   ChunkIn x = {};
-  if (warp == 0) x = chunk_in(P, (int)blockIdx.x / parts, lane, n);
+  if (ahead) {
+    cntA = __ldcg(P.counts);
+    if (warp == 0) x = chunk_in<true>(P, (int)blockIdx.x / parts, lane, cntA * T);
+  }
   pdl_wait();      // c and the chunk offsets come from the kernel before this one
   pdl_trigger();   // the dW product kernel may set itself up; it waits for this grid before loading
+  if (!ahead) cntA = P.counts[0];
+  const int n = cntA * T;
   const int cntW = __ldcg(P.counts + 1);
   const float c = P.fix[0];
   const int mode = (int)P.fix[1];
@@ -682,7 +693,7 @@ __global__ void __launch_bounds__(EMIT_THREADS) emit_pack_kernel(EmitParams P) {
   for (int u = blockIdx.x; u < nchunks * parts; u += gridDim.x) {
     const int ch = u / parts, part = u - ch * parts;
     if (warp == 0) {
-      if (u != (int)blockIdx.x) x = chunk_in(P, ch, lane, n);
+      if (!ahead || u != (int)blockIdx.x) x = chunk_in<false>(P, ch, lane, n);
       const ChunkRow o = chunk_row(P, x, ch, lane, mode, c);
       if (part == 0 && x.in) { P.w[x.r] = x.w; P.q[x.r] = o.q; }
       if (o.keep) {
@@ -951,6 +962,7 @@ cudaError_t launch_emit_pack(Handle* h, const void* dY, const void* X, const Sam
   P.parts = (int)parts;
   long blocks = ((R + 31) / 32) * parts;
   if (blocks > cap) blocks = cap;
+  P.ahead = (int)(cap / 8) * EMIT_AHEAD;
   const dim3 grid((unsigned)blocks), threads(EMIT_THREADS);
   const cudaError_t e = !h->split_path           ? launch_after(emit_pack_kernel<__nv_bfloat16, false>, grid, threads, 0, st, P)
       : d.dtype == VCAS_DTYPE_F32                ? launch_after(emit_pack_kernel<float, true>, grid, threads, 0, st, P)

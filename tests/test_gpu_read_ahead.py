@@ -28,10 +28,12 @@ def test_order_and_loads_in_the_sources():
     for name in ("sample_w_small_kernel", "sample_w_kernel"):
         k = body(src, name)
         assert 0 < k.index("pdl_wait()") < k.index("pdl_trigger()"), name
-    memory = re.compile(r"(?<!__ldcg\()P\.(idxA|dropA|wc|uc|scaleA|counts|w|q|fix|chunk_off)\b(?! !=)")
-    assert not memory.findall(body(src, "chunk_in"))
+    memory = re.compile(r"(?<!__ldcg\()(?<!read\()P\.(idxA|dropA|wc|uc|scaleA|counts|w|q|fix|chunk_off)\b(?! !=)")
+    k = body(src, "chunk_in")
+    assert not memory.findall(k) and "return AHEAD ? __ldcg(p) : *p;" in k
     for name in ("emit_rows_kernel", "emit_pack_kernel"):
-        assert not memory.findall(body(src, name).split("pdl_wait()")[0]), name
+        before = body(src, name).split("pdl_wait()")[0]
+        assert not memory.findall(before) and "chunk_in<true>(" in before and "chunk_in<false>(" not in before, name
 
 
 @pytest.mark.gpu
