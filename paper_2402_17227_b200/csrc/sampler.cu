@@ -576,10 +576,11 @@ struct RecordOut {
   int32_t* idxA; int32_t* cntA; int32_t* idxW; int32_t* cntW;
 };
 // A compact row of a chunk of 32, one per lane, as the kernels before SampleW left it.  The first chunk of a CTA is read ahead (see
-// pdl_wait), before the wait for SampleW, which started when they had ended and then let this grid start (whole calls: 192 rows, 128 -> 192, 22.6 -> 21.5 us
-// on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2, of which the loads past L1 took back 0.4).  Of a
-// packing grid only the CTAs that may be there by then do so, three an SM; the others read after the wait, and find in L1
-// what the chunk's other CTAs have read (4096 rows, 768 -> 3072: with every CTA past L1 44.6 us, so 43.9; 16384, 1024 -> 1024: 71.8 and 70.1).
+// pdl_wait), before the wait for SampleW, which started when they had ended and then let this grid start (whole calls: 192 rows,
+// 128 -> 192, 22.6 -> 21.5 us on the GPU; 256 rows, 256 -> 256, 21.3 -> 20.5; 8192 rows, 256 -> 1024, 40.9 -> 40.2, of which the
+// loads past L1 took back 0.4).  Of a packing grid only the CTAs that may be there by then do so, three an SM; the others read
+// after the wait, and find in L1 what the chunk's other CTAs have read (4096 rows, 768 -> 3072: with every CTA past L1 44.6 us, so
+// 43.9; 16384, 1024 -> 1024: 71.8 and 70.1).
 struct ChunkIn { bool in; int r; float w, sa; uint32_t u; };
 template <bool AHEAD>
 __device__ __forceinline__ ChunkIn chunk_in(const EmitParams& P, int ch, int lane, int n) {
